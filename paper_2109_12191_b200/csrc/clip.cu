@@ -33,7 +33,7 @@ struct SegTable {
 // example e of the step adds sd * z_e(g), sd = sigma*C/sqrt(|B|), to its clipped gradient before the sum.
 struct ExampleNoise {
     float sd;
-    unsigned long long seed, step;
+    NoiseStream ns;
     uint32_t example0;               // index within the step of this chunk's first example
 };
 
@@ -357,7 +357,7 @@ scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable tab, const flo
 // transcendental work of B*P normals, not by memory.
 __global__ void __launch_bounds__(256)
 scale_accumulate_noised_kernel(const __grid_constant__ SegTable tab, const float *__restrict__ factor, int B, int L,
-                               int per_layer, const ExampleNoise nz) {
+                               int per_layer, const __grid_constant__ ExampleNoise nz) {
     __shared__ float f_sh[256];
     const int seg = find_seg(tab, blockIdx.x);
     const long long P = tab.P[seg];
@@ -389,7 +389,7 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable tab, const float
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         float z[4];
-                        example_normals4(nz.seed, nz.step, nz.example0 + (uint32_t)(n0 + n + u), block, z);
+                        example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n + u), block, z);
                         const float f = f_sh[n + u];
                         s.x += fmaf(f, v[u].x, nz.sd * z[0]); s.y += fmaf(f, v[u].y, nz.sd * z[1]);
                         s.z += fmaf(f, v[u].z, nz.sd * z[2]); s.w += fmaf(f, v[u].w, nz.sd * z[3]);
@@ -398,7 +398,7 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable tab, const float
                 for (; n < nb; ++n) {
                     const float4 v = __ldcs(reinterpret_cast<const float4 *>(g + (long long)n * P));
                     float z[4];
-                    example_normals4(nz.seed, nz.step, nz.example0 + (uint32_t)(n0 + n), block, z);
+                    example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n), block, z);
                     const float f = f_sh[n];
                     s.x += fmaf(f, v.x, nz.sd * z[0]); s.y += fmaf(f, v.y, nz.sd * z[1]);
                     s.z += fmaf(f, v.z, nz.sd * z[2]); s.w += fmaf(f, v.w, nz.sd * z[3]);
@@ -426,7 +426,7 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable tab, const float
                     if (c0 + i < P) {
                         const unsigned long long gi = (unsigned long long)(goff + c0 + i);
                         float z[4];
-                        example_normals4(nz.seed, nz.step, nz.example0 + (uint32_t)(n0 + n), (uint32_t)(gi >> 2), z);
+                        example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n), (uint32_t)(gi >> 2), z);
                         s[q] += fmaf(f, g[i], nz.sd * z[gi & 3]);
                     }
                 }
@@ -658,7 +658,7 @@ extern "C" dp_status dp_clip_accumulate_noised(int mode, int B, int L, const flo
                                         workspace_bytes, cuda_stream);
     dp::ExampleNoise nz;
     nz.sd = (float)((double)sigma * (double)C / sqrt((double)total_batch));
-    nz.seed = seed; nz.step = step; nz.example0 = (uint32_t)example0;
+    nz.ns = dp::noise_stream(seed, step); nz.example0 = (uint32_t)example0;
     dp::ClipVariant var;
     var.noise = &nz;
     var.goff_l = param_offset_l;

@@ -6,28 +6,47 @@
 
 namespace dp {
 
-// Thread t owns Philox block first_block + t, i.e. global indices 4*(first_block+t) .. +3;
-// local index = global - param_offset.  VEC: param_offset % 4 == 0, so a block is one float4.
+// A thread block covers kNoiseTile parameters, i.e. kNoiseTile/4 Philox blocks from global index 4*(param_offset/4) on;
+// local index = global - param_offset.  VEC: param_offset % 4 == 0, so a Philox block is one float4.
+// What bounds the kernel is the issue rate (some 45 instructions a normal, of which a third Philox), not the 8 bytes a
+// parameter it moves: two blocks a thread halve the index arithmetic and give the ten-round chain a second one to
+// overlap with.  25.6 M parameters: 62 us with one block a thread and the library's logf / sincospif.
+constexpr int kNoiseTile = 2048;
+
 template <bool VEC>
 __global__ void __launch_bounds__(256)
 noise_average_kernel(const float *acc, float *out, long long P,   // out may alias acc
-                     unsigned long long param_offset, unsigned long long n_blocks,
-                     float noise_std, float inv_batch, unsigned long long seed, unsigned long long step) {
-    const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n_blocks) return;
-    const unsigned long long block = (param_offset >> 2) + t;
-    float z[4] = {0.f, 0.f, 0.f, 0.f};
-    if (noise_std != 0.0f) normals4(seed, step, block, z);
-    const long long i0 = (long long)(4ull * block - param_offset);   // may be negative for the first block
-    if (VEC && i0 + 3 < P) {
-        const float4 a = __ldcs(reinterpret_cast<const float4 *>(acc + i0));
-        float4 r;
-        r.x = (a.x + noise_std * z[0]) * inv_batch;
-        r.y = (a.y + noise_std * z[1]) * inv_batch;
-        r.z = (a.z + noise_std * z[2]) * inv_batch;
-        r.w = (a.w + noise_std * z[3]) * inv_batch;
-        __stcs(reinterpret_cast<float4 *>(out + i0), r);
-    } else {
+                     unsigned long long param_offset, float noise_std, float inv_batch,
+                     const __grid_constant__ NoiseStream ns) {
+    const unsigned long long block0 = (param_offset >> 2) + (unsigned long long)blockIdx.x * (kNoiseTile / 4);
+    const long long tile0 = (long long)(4ull * block0 - param_offset);       // may be negative for the first tile
+    if (VEC && tile0 + kNoiseTile <= P) {
+        const float4 *src = reinterpret_cast<const float4 *>(acc + tile0) + threadIdx.x;
+        float4 *dst = reinterpret_cast<float4 *>(out + tile0) + threadIdx.x;
+        float4 a[2];
+        a[0] = __ldcs(src); a[1] = __ldcs(src + 256);                        // on their way while the noise is worked out
+        float z[2][4] = {};
+        if (noise_std != 0.0f) {
+            normals4(ns, block0 + threadIdx.x, z[0]);
+            normals4(ns, block0 + threadIdx.x + 256, z[1]);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            float4 r;
+            r.x = (a[u].x + noise_std * z[u][0]) * inv_batch;
+            r.y = (a[u].y + noise_std * z[u][1]) * inv_batch;
+            r.z = (a[u].z + noise_std * z[u][2]) * inv_batch;
+            r.w = (a[u].w + noise_std * z[u][3]) * inv_batch;
+            __stcs(dst + 256 * u, r);
+        }
+        return;
+    }
+#pragma unroll 1
+    for (int u = 0; u < 2; ++u) {
+        const long long i0 = tile0 + 4 * (threadIdx.x + 256 * u);
+        if (i0 >= P) return;
+        float z[4] = {0.f, 0.f, 0.f, 0.f};
+        if (noise_std != 0.0f) normals4(ns, block0 + threadIdx.x + 256 * u, z);
 #pragma unroll
         for (int lane = 0; lane < 4; ++lane) {
             const long long i = i0 + lane;
@@ -38,16 +57,39 @@ noise_average_kernel(const float *acc, float *out, long long P,   // out may ali
 
 // Noise, average and the parameter update in one pass: g = (acc + std*z) / |B|;  m <- mu*m + g (when a momentum
 // buffer is given);  theta <- theta - lr*m (or - lr*g).  Same thread-to-Philox-block mapping as above.
+// VEC: param_offset % 4 == 0 and 16-byte aligned buffers, so the four parameters of a block are one 16-byte access to
+// each array (20 bytes a parameter with momentum).
+template <bool VEC>
 __global__ void __launch_bounds__(256)
 noise_average_sgd_kernel(const float *acc, long long P, unsigned long long param_offset, unsigned long long n_blocks,
-                         float noise_std, float inv_batch, unsigned long long seed, unsigned long long step, float lr,
-                         float mu, float *theta, float *mom, float *g_out) {
+                         float noise_std, float inv_batch, const __grid_constant__ NoiseStream ns, float lr, float mu,
+                         float *theta, float *mom, float *g_out) {
     const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_blocks) return;
     const unsigned long long block = (param_offset >> 2) + t;
-    float z[4] = {0.f, 0.f, 0.f, 0.f};
-    if (noise_std != 0.0f) normals4(seed, step, block, z);
     const long long i0 = (long long)(4ull * block - param_offset);
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    if (VEC && i0 + 3 < P) {
+        // the loads are on their way while the noise is worked out
+        const float4 a = __ldcs(reinterpret_cast<const float4 *>(acc + i0));
+        float4 th = *reinterpret_cast<const float4 *>(theta + i0);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (mom) v = *reinterpret_cast<const float4 *>(mom + i0);
+        if (noise_std != 0.0f) normals4(ns, block, z);
+        const float4 g = make_float4((a.x + noise_std * z[0]) * inv_batch, (a.y + noise_std * z[1]) * inv_batch,
+                                     (a.z + noise_std * z[2]) * inv_batch, (a.w + noise_std * z[3]) * inv_batch);
+        if (mom) {
+            v = make_float4(fmaf(mu, v.x, g.x), fmaf(mu, v.y, g.y), fmaf(mu, v.z, g.z), fmaf(mu, v.w, g.w));
+            *reinterpret_cast<float4 *>(mom + i0) = v;
+        } else {
+            v = g;
+        }
+        th = make_float4(fmaf(-lr, v.x, th.x), fmaf(-lr, v.y, th.y), fmaf(-lr, v.z, th.z), fmaf(-lr, v.w, th.w));
+        *reinterpret_cast<float4 *>(theta + i0) = th;
+        if (g_out) *reinterpret_cast<float4 *>(g_out + i0) = g;
+        return;
+    }
+    if (noise_std != 0.0f) normals4(ns, block, z);
 #pragma unroll
     for (int lane = 0; lane < 4; ++lane) {
         const long long i = i0 + lane;
@@ -61,20 +103,20 @@ noise_average_sgd_kernel(const float *acc, long long P, unsigned long long param
 }
 
 __global__ void philox_raw_kernel(uint32_t *out4, long long n_blocks, unsigned long long first_block,
-                                  unsigned long long seed, unsigned long long step) {
+                                  const __grid_constant__ NoiseStream ns) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_blocks) return;
-    const Words4 w = philox_block(seed, step, first_block + (unsigned long long)t);
+    const Words4 w = philox_block(ns, first_block + (unsigned long long)t);
     reinterpret_cast<uint4 *>(out4)[t] = make_uint4(w.w0, w.w1, w.w2, w.w3);
 }
 
 __global__ void noise_z_kernel(float *z, long long count, unsigned long long first_index,
-                               unsigned long long n_blocks, unsigned long long seed, unsigned long long step) {
+                               unsigned long long n_blocks, const __grid_constant__ NoiseStream ns) {
     const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_blocks) return;
     const unsigned long long block = (first_index >> 2) + t;
     float v[4];
-    normals4(seed, step, block, v);
+    normals4(ns, block, v);
     const long long i0 = (long long)(4ull * block - first_index);
 #pragma unroll
     for (int lane = 0; lane < 4; ++lane) {
@@ -85,13 +127,13 @@ __global__ void noise_z_kernel(float *z, long long count, unsigned long long fir
 
 // z[t] = normal of example `example`'s stream at global index first_index + t (one thread per Philox block)
 __global__ void example_noise_z_kernel(float *z, long long count, unsigned long long first_index,
-                                       unsigned long long n_blocks, uint32_t example, unsigned long long seed,
-                                       unsigned long long step) {
+                                       unsigned long long n_blocks, uint32_t example,
+                                       const __grid_constant__ NoiseStream ns) {
     const unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_blocks) return;
     const unsigned long long block = (first_index >> 2) + t;
     float v[4];
-    example_normals4(seed, step, example, (uint32_t)block, v);
+    example_normals4(ns, example, (uint32_t)block, v);
     const long long i0 = (long long)(4ull * block - first_index);
 #pragma unroll
     for (int lane = 0; lane < 4; ++lane) {
@@ -115,14 +157,13 @@ extern "C" dp_status dp_noise_average(const float *acc, long long P, long long p
     const unsigned long long n_blocks = ((off & 3ull) + (unsigned long long)P + 3ull) >> 2;
     const float noise_std = (sigma == 0.0f) ? 0.0f : sigma * C;
     const float inv_batch = 1.0f / (float)total_batch;
-    const unsigned long long grid = (n_blocks + 255) / 256;
+    const unsigned long long grid = (n_blocks + dp::kNoiseTile / 4 - 1) / (dp::kNoiseTile / 4);
     if (grid > 0x7fffffffull) return DP_ERR_UNSUPPORTED;
+    const dp::NoiseStream ns = dp::noise_stream(seed, step);
     if ((off & 3ull) == 0)
-        dp::noise_average_kernel<true><<<(unsigned)grid, 256, 0, stream>>>(acc, out, P, off, n_blocks, noise_std,
-                                                                          inv_batch, seed, step);
+        dp::noise_average_kernel<true><<<(unsigned)grid, 256, 0, stream>>>(acc, out, P, off, noise_std, inv_batch, ns);
     else
-        dp::noise_average_kernel<false><<<(unsigned)grid, 256, 0, stream>>>(acc, out, P, off, n_blocks, noise_std,
-                                                                           inv_batch, seed, step);
+        dp::noise_average_kernel<false><<<(unsigned)grid, 256, 0, stream>>>(acc, out, P, off, noise_std, inv_batch, ns);
     DP_LAUNCH_CHECK("noise_average_kernel");
     return DP_OK;
 }
@@ -141,8 +182,10 @@ extern "C" dp_status dp_noise_average_sgd(const float *acc, long long P, long lo
     const unsigned long long n_blocks = ((off & 3ull) + (unsigned long long)P + 3ull) >> 2;
     const unsigned long long grid = (n_blocks + 255) / 256;
     if (grid > 0x7fffffffull) return DP_ERR_UNSUPPORTED;
-    dp::noise_average_sgd_kernel<<<(unsigned)grid, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        acc, P, off, n_blocks, (sigma == 0.0f) ? 0.0f : sigma * C, 1.0f / (float)total_batch, seed, step, lr, momentum,
+    const bool vec = (off & 3ull) == 0 && dp::aligned(acc, 16) && dp::aligned(theta, 16) && dp::aligned(momentum_buf, 16) &&
+                     dp::aligned(g_out, 16);
+    (vec ? dp::noise_average_sgd_kernel<true> : dp::noise_average_sgd_kernel<false>)<<<(unsigned)grid, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
+        acc, P, off, n_blocks, (sigma == 0.0f) ? 0.0f : sigma * C, 1.0f / (float)total_batch, dp::noise_stream(seed, step), lr, momentum,
         theta, momentum_buf, g_out);
     DP_LAUNCH_CHECK("noise_average_sgd_kernel");
     return DP_OK;
@@ -154,7 +197,7 @@ extern "C" dp_status dp_debug_philox_raw(unsigned int *out4, long long n_blocks,
     const long long grid = (n_blocks + 255) / 256;
     if (grid > 0x7fffffffll) return DP_ERR_UNSUPPORTED;
     dp::philox_raw_kernel<<<(unsigned)grid, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        out4, n_blocks, (unsigned long long)first_block, seed, step);
+        out4, n_blocks, (unsigned long long)first_block, dp::noise_stream(seed, step));
     DP_LAUNCH_CHECK("philox_raw_kernel");
     return DP_OK;
 }
@@ -167,7 +210,7 @@ extern "C" dp_status dp_debug_noise_z(float *z, long long count, long long first
     const unsigned long long grid = (n_blocks + 255) / 256;
     if (grid > 0x7fffffffull) return DP_ERR_UNSUPPORTED;
     dp::noise_z_kernel<<<(unsigned)grid, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(z, count, off, n_blocks,
-                                                                                         seed, step);
+                                                                                         dp::noise_stream(seed, step));
     DP_LAUNCH_CHECK("noise_z_kernel");
     return DP_OK;
 }
@@ -181,7 +224,7 @@ extern "C" dp_status dp_debug_example_noise_z(float *z, long long count, long lo
     const unsigned long long grid = (n_blocks + 255) / 256;
     if (grid > 0x7fffffffull) return DP_ERR_UNSUPPORTED;
     dp::example_noise_z_kernel<<<(unsigned)grid, 256, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        z, count, off, n_blocks, (uint32_t)example, seed, step);
+        z, count, off, n_blocks, (uint32_t)example, dp::noise_stream(seed, step));
     DP_LAUNCH_CHECK("example_noise_z_kernel");
     return DP_OK;
 }

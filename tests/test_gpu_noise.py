@@ -113,3 +113,27 @@ def test_fused_sgd_update_matches_oracle_over_several_steps(P, off, mu):
     out = torch.empty(P, device="cuda")
     b.check(b.dp_noise_average(dev(acc), P, off, sigma, C, total, 21, 2, out))
     np.testing.assert_array_equal(out.cpu().numpy(), g_out.cpu().numpy())
+
+
+@pytest.mark.parametrize("P,off,shift", [(2047, 0, 0), (2048, 4, 0), (2049, 0, 0), (6147, 0, 0), (4096, 2, 0), (1030, 0, 1), (1, 0, 0), (5, 8, 3)])
+def test_update_and_average_at_the_edges_of_their_tiles(P, off, shift):
+    """Whole and ragged tiles, tensors that start at any parameter index and buffers that start at any float."""
+    b = B()
+    rng = np.random.default_rng(P)
+    acc, theta0 = rng.standard_normal(P).astype(np.float32), rng.standard_normal(P).astype(np.float32)
+    buf = {k: torch.zeros(P + shift + 4, device="cuda") for k in ("acc", "theta", "mom", "g")}
+    view = {k: v[shift:shift + P] for k, v in buf.items()}
+    view["acc"].copy_(dev(acc)); view["theta"].copy_(dev(theta0))
+    b.check(b.dp_noise_average_sgd(view["acc"], P, off, 0.7, 1.3, 9, 5, 6, 0.1, 0.5, view["theta"], view["mom"], view["g"]))
+    ref = oracle.noise_average(acc.astype(np.float64), off, 0.7, 1.3, 9, 5, 6)
+    ref_theta, ref_m = theta0.astype(np.float64), np.zeros(P)
+    oracle.sgd_update(ref, 0.1, 0.5, ref_theta, ref_m)
+    for got, want in ((view["g"], ref), (view["theta"], ref_theta), (view["mom"], ref_m)):
+        assert np.max(np.abs(got.cpu().numpy() - want)) <= 2e-6
+    for k in buf:
+        assert not buf[k][shift + P:].any() and not buf[k][:shift].any()
+    if shift == 0:
+        out = torch.full((P + 4,), float("nan"), device="cuda")
+        b.check(b.dp_noise_average(view["acc"], P, off, 0.7, 1.3, 9, 5, 6, out))
+        assert torch.isnan(out[P:]).all()
+        np.testing.assert_array_equal(out[:P].cpu().numpy(), view["g"].cpu().numpy())
