@@ -148,6 +148,30 @@ DP_API dp_status dp_per_example_wgrad(const dp_layer_desc *desc, const void *X, 
                                int epilogue, float C_l, float *acc_w, float *acc_b, float *clip_out,
                                void *workspace, size_t workspace_bytes, void *cuda_stream);
 
+/* The calls of dp_per_example_wgrad that make up one chunk, handed over together: layers of one kind then share their
+ * launches, which keeps the whole GPU busy with layers that are small one by one (a chunk of few examples) and spares
+ * the host a call and a launch or more per layer.  Results are those of the single calls (other summation orders).
+ *
+ * dp_batch_create plans n layers, descs[i] with epilogue epilogues[i], once (host memory only; it may be used from any
+ *   thread, by one run at a time per workspace).  dp_batch_destroy frees the plan; runs already enqueued are not affected.
+ * dp_batch_workspace_bytes: device scratch of a run; prepare it once with dp_workspace_init, dp_wgrad_check reports it.
+ * dp_batch_run: the n calls with the buffers io[i] (host array, fields as the arguments of dp_per_example_wgrad; C_l for
+ *   every DP_EPI_CLIP_ACCUM layer).  The outputs of different layers must not overlap.
+ * dp_set_sm_target does not apply: a batch is planned for the whole GPU.
+ * Errors as for dp_per_example_wgrad; on DP_ERR_INVALID_ARG and DP_ERR_WORKSPACE nothing has been launched. */
+typedef struct dp_batch dp_batch;
+typedef struct {
+    const void *X, *dY;
+    float *G_w, *G_b, *sqnorm;
+    long long sqnorm_stride;
+    float *acc_w, *acc_b, *clip_out;
+} dp_layer_io;
+DP_API dp_status dp_batch_create(int n, const dp_layer_desc *descs, const int *epilogues, dp_batch **out);
+DP_API void dp_batch_destroy(dp_batch *batch);
+DP_API size_t dp_batch_workspace_bytes(const dp_batch *batch);
+DP_API dp_status dp_batch_run(const dp_batch *batch, const dp_layer_io *io, float C_l, void *workspace,
+                              size_t workspace_bytes, void *cuda_stream);
+
 /* The clipped sum of one layer with the factors already known: acc_w += sum_n factor_w[n*factor_stride] * g_w,n and
  * acc_b += sum_n factor_b[n*factor_stride] * g_b,n, the per-example gradients formed on the fly and never written
  * (section 2: the sum over the batch of clip(g_j, C), whose factor min(1, C/||g_j||) needs every layer's norm first).

@@ -31,12 +31,18 @@ EXPORTS = ["dp_layer_groups", "dp_workspace_bytes", "dp_per_example_wgrad", "dp_
            "dp_clip_static_scratch_bytes", "dp_noise_average_sgd", "dp_clip_accumulate_noised",
            "dp_debug_example_noise_z", "dp_clip_accumulate_grouped", "dp_clip_accumulate_micro",
            "dp_per_example_wgrad_scaled", "dp_clip_factors", "dp_scale_accumulate", "dp_workspace_init",
-           "dp_debug_set_wait_polls", "dp_set_sm_target", "dp_debug_set_single_pass"]
+           "dp_debug_set_wait_polls", "dp_set_sm_target", "dp_debug_set_single_pass", "dp_batch_create",
+           "dp_batch_destroy", "dp_batch_workspace_bytes", "dp_batch_run"]
 
 
 class dp_layer_desc(ctypes.Structure):
     _fields_ = [(n, ctypes.c_int) for n in ("kind", "dtype", "B", "C_in", "H", "W", "K_out", "R", "S",
                                             "stride", "pad", "has_bias", "bias_separate", "impl")]
+
+
+class dp_layer_io(ctypes.Structure):
+    _fields_ = ([(n, ctypes.c_void_p) for n in ("X", "dY", "G_w", "G_b", "sqnorm")] + [("sqnorm_stride", ctypes.c_longlong)] +
+                [(n, ctypes.c_void_p) for n in ("acc_w", "acc_b", "clip_out")])
 
 
 class DpError(RuntimeError):
@@ -87,6 +93,10 @@ _lib.dp_noise_average_sgd.argtypes = [_vp, _ll, _ll, _f, _f, _ll, _ull, _ull, _f
 _lib.dp_noise_average_sgd.restype = _i
 _lib.dp_debug_philox_raw.argtypes = [_vp, _ll, _ll, _ull, _ull, _vp]; _lib.dp_debug_philox_raw.restype = _i
 _lib.dp_debug_noise_z.argtypes = [_vp, _ll, _ll, _ull, _ull, _vp]; _lib.dp_debug_noise_z.restype = _i
+_lib.dp_batch_create.argtypes = [_i, _dp, ctypes.POINTER(_i), ctypes.POINTER(_vp)]; _lib.dp_batch_create.restype = _i
+_lib.dp_batch_destroy.argtypes = [_vp]; _lib.dp_batch_destroy.restype = None
+_lib.dp_batch_workspace_bytes.argtypes = [_vp]; _lib.dp_batch_workspace_bytes.restype = _sz
+_lib.dp_batch_run.argtypes = [_vp, _vp, _f, _vp, _sz, _vp]; _lib.dp_batch_run.restype = _i
 _lib.dp_wgrad_check.argtypes = [_vp, _vp]; _lib.dp_wgrad_check.restype = _i
 _lib.dp_workspace_init.argtypes = [_vp, _sz, _vp]; _lib.dp_workspace_init.restype = _i
 _lib.dp_debug_set_wait_polls.argtypes = [_ll]; _lib.dp_debug_set_wait_polls.restype = None
@@ -245,6 +255,31 @@ def dp_noise_average_sgd(acc, P, param_offset, sigma, C, total_batch, seed, step
                          g_out=None, stream=None):
     return _lib.dp_noise_average_sgd(_ptr(acc), P, param_offset, sigma, C, total_batch, seed, step, lr, momentum,
                                      _ptr(theta), _ptr(momentum_buf), _ptr(g_out), _stream(stream))
+
+
+class Batch:
+    """A dp_batch and its dp_layer_io table.  set() fills in the buffers a layer keeps from run to run, run() the inputs."""
+
+    def __init__(self, descs, epilogues):
+        n = len(descs)
+        self._handle = _vp()
+        check(_lib.dp_batch_create(n, (dp_layer_desc * n)(*descs), (_i * n)(*epilogues), ctypes.byref(self._handle)), "dp_batch_create")
+        self.n, self.io = n, (dp_layer_io * n)()
+        self.workspace_bytes = _lib.dp_batch_workspace_bytes(self._handle)
+
+    def set(self, i, **buffers):
+        for name, v in buffers.items():
+            setattr(self.io[i], name, v if name == "sqnorm_stride" else _ptr(v))
+
+    def run(self, inputs, C_l, workspace, stream=None):
+        """inputs: (X, dY) of every layer, in order."""
+        for io, (X, dY) in zip(self.io, inputs, strict=True):
+            io.X, io.dY = _ptr(X), _ptr(dY)
+        return _lib.dp_batch_run(self._handle, self.io, C_l, _ptr(workspace), _nbytes(workspace), _stream(stream))
+
+    def __del__(self):
+        if getattr(self, "_handle", None) and _lib is not None:       # (module globals go first at interpreter exit)
+            _lib.dp_batch_destroy(self._handle)
 
 
 def dp_debug_philox_raw(out4, n_blocks, first_block, seed, step, stream=None):

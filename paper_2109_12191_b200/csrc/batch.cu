@@ -1,0 +1,245 @@
+// A batch of layer calls: the layers of one chunk handed over together, so that layers of one kind share their launches.
+// The plan (which layer goes where, its tiling and scratch) is made once; a run fills in the buffers and launches.
+#include "batch.cuh"
+#include "wgrad_tc.cuh"
+#include <algorithm>
+#include <mutex>
+#include <new>
+#include <vector>
+
+using namespace dp;
+
+struct dp_batch {
+    struct Item {
+        dp_layer_desc desc;
+        int epi;
+        WgradPlan plan;
+        int group, slot;             // table of its kind and place in it; group < 0: a call of its own
+        size_t scratch;              // byte offset of the layer's own scratch (factors, finished per-example gradients)
+    };
+    std::vector<Item> items;
+    std::vector<AffineGroup> affine;             // shapes filled in, buffers per run
+    std::vector<int> affine_dtype;
+    size_t affine_partial = 0;                   // byte offset of the pixel-chunk partials
+    std::vector<ConvJob> convs;                  // geometry filled in, buffers per run
+    std::vector<int> conv_item;                  // item of every conv
+    double walk = 0.0;                           // conv_batch_walk() of all of them
+    size_t singles = 0;                          // byte offset of the scratch the single calls share
+    size_t total = 0;
+    // Streams and events of the runs, made on the first run's device; host threads take turns at enqueueing.
+    mutable std::mutex mu;
+    mutable int device = -1;
+    mutable cudaStream_t side[BatchStreams::kCount] = {};
+    mutable cudaEvent_t fork = nullptr, gram_done = nullptr, done[BatchStreams::kCount] = {};
+};
+
+namespace dp {
+
+// The side streams of a batch, or false where this device is not the one they were made on or they cannot be had.
+static bool side_streams(const dp_batch &b) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    if (b.device >= 0) return b.device == dev;
+    bool ok = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&b.gram_done, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 1; ok && i < BatchStreams::kCount; ++i)
+        ok = cudaStreamCreateWithFlags(&b.side[i], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&b.done[i], cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) { (void)cudaGetLastError(); return false; }
+    b.device = dev;
+    return true;
+}
+
+static void plan_affine(dp_batch &b, size_t &off) {
+    size_t partial_floats = 0;
+    for (int dt = 0; dt < 2; ++dt) {
+        const int dtype = dt == 0 ? DP_BF16 : DP_F32;
+        for (auto &it : b.items) {
+            const dp_layer_desc &d = it.desc;
+            if (d.kind != DP_LAYER_NORM_AFFINE || storage_type(&d) != dtype || !affine_batch_eligible(dtype, d.C_in)) continue;
+            if (b.affine.empty() || b.affine_dtype.back() != dtype || b.affine.back().n == kGroupLayers) {
+                AffineGroup fresh = {};
+                b.affine.push_back(fresh);
+                b.affine_dtype.push_back(dtype);
+            }
+            AffineGroup &g = b.affine.back();
+            it.group = (int)b.affine.size() - 1;
+            it.slot = g.n++;
+            AffineSeg &s = g.seg[it.slot];
+            affine_batch_shape(dtype, d.B, d.H * d.W, d.C_in, s);
+            s.clip = it.epi == DP_EPI_CLIP_ACCUM;
+            s.separate = groups_of(&d) == 2;
+            s.part_off = (long long)partial_floats;
+            partial_floats += (size_t)d.B * s.chunks * 2 * d.C_in;
+            // [factors][dgamma][dbeta] unless the caller takes the gradients
+            it.scratch = off;
+            off = round_up(off + sizeof(float) * 2 * d.B, 256);
+            if (it.epi != DP_EPI_STORE_NORM) off = round_up(off + sizeof(float) * 2 * (size_t)d.B * d.C_in, 256);
+        }
+    }
+    b.affine_partial = off;
+    off = round_up(off + sizeof(float) * partial_floats, 1024);
+}
+
+static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l, char *ws, cudaStream_t st) {
+    if (b.affine.empty()) return DP_OK;
+    std::vector<AffineGroup> groups = b.affine;
+    for (size_t i = 0; i < b.items.size(); ++i) {
+        const dp_batch::Item &it = b.items[i];
+        if (it.desc.kind != DP_LAYER_NORM_AFFINE || it.group < 0) continue;
+        AffineSeg &s = groups[it.group].seg[it.slot];
+        s.X = io[i].X; s.dY = io[i].dY;
+        s.sqnorm = io[i].sqnorm; s.sq_stride = io[i].sqnorm_stride; s.clip_out = io[i].clip_out;
+        s.acc_w = io[i].acc_w; s.acc_b = io[i].acc_b;
+        s.factor = reinterpret_cast<float *>(ws + it.scratch);
+        if (it.epi == DP_EPI_STORE_NORM) {
+            s.dgamma = io[i].G_w; s.dbeta = io[i].G_b;
+        } else {
+            s.dgamma = reinterpret_cast<float *>(ws + it.scratch + round_up(sizeof(float) * 2 * it.desc.B, 256));
+            s.dbeta = s.dgamma + (size_t)it.desc.B * it.desc.C_in;
+        }
+    }
+    for (size_t k = 0; k < groups.size(); ++k) {
+        groups[k].C_l = C_l;
+        groups[k].partial = reinterpret_cast<float *>(ws + b.affine_partial);
+        const dp_status rc = launch_affine_batch(b.affine_dtype[k], groups[k], st);
+        if (rc != DP_OK) return rc;
+    }
+    return DP_OK;
+}
+
+static void plan_convs(dp_batch &b, size_t &off) {
+    for (size_t i = 0; i < b.items.size(); ++i) {
+        dp_batch::Item &it = b.items[i];
+        const dp_layer_desc &d = it.desc;
+        if (d.kind != DP_LAYER_CONV2D || !it.plan.use_tc || (int)b.convs.size() >= kWsCounters) continue;
+        ConvJob j = {};
+        j.g = geom_of(&d); j.dtype = d.dtype; j.epi = it.epi;
+        j.kind = conv_batch_kind(d.dtype, j.g, it.epi, d.has_bias != 0);
+        if (j.kind == kConvSingle) continue;
+        j.separate = groups_of(&d) == 2;
+        it.group = 0; it.slot = (int)b.convs.size();
+        b.convs.push_back(j);
+        b.conv_item.push_back((int)i);
+    }
+    if (b.convs.empty()) return;
+    b.walk = conv_batch_walk(b.convs);
+    BatchPlanning planning(b.walk);
+    for (size_t k = 0; k < b.convs.size(); ++k) {
+        dp_batch::Item &it = b.items[b.conv_item[k]];
+        make_layer_plan(&it.desc, it.epi, it.plan);          // scratch sizes of the tiling a batch uses
+        b.convs[k].slots = it.plan.slots; b.convs[k].w_slots = it.plan.w_slots;
+        it.scratch = off;
+        off = round_up(off + it.plan.total - kWsHeaderBytes, 1024);
+    }
+}
+
+static dp_status run_convs(const dp_batch &b, const dp_layer_io *io, float C_l, char *ws, const BatchStreams &streams,
+                           const std::function<dp_status()> &join) {
+    const cudaStream_t st = streams.s[BatchStreams::kMain];
+    std::vector<ConvJob> jobs = b.convs;
+    for (size_t k = 0; k < jobs.size(); ++k) {
+        const dp_batch::Item &it = b.items[b.conv_item[k]];
+        const dp_layer_io &o = io[b.conv_item[k]];
+        ConvJob &j = jobs[k];
+        char *base = ws + it.scratch - kWsHeaderBytes;       // the plan's offsets count from a header
+        j.X = o.X; j.dY = o.dY; j.G_w = o.G_w; j.acc_w = o.acc_w;
+        j.partial = reinterpret_cast<float *>(base + it.plan.partial_off);
+        j.factor = reinterpret_cast<float *>(base + it.plan.factor_off);
+        j.tc_workspace = base + it.plan.tc_off;
+        j.counter = reinterpret_cast<int *>(ws + kWsCounterOffset) + k;
+        j.clip = TcInlineClip{C_l, o.sqnorm, o.sqnorm_stride, o.clip_out};
+        if (it.desc.has_bias) {
+            float *db = it.epi == DP_EPI_STORE_NORM ? o.G_b : reinterpret_cast<float *>(base + it.plan.db_off);
+            const dp_status rc = launch_bias(storage_type(&it.desc), o.dY, j.g, db, j.partial, it.plan.slots, it.plan.w_slots, st);
+            if (rc != DP_OK) return rc;
+        }
+    }
+    return launch_conv_batch(jobs, b.walk, reinterpret_cast<int *>(ws), streams, join);
+}
+
+}  // namespace dp
+
+extern "C" dp_status dp_batch_create(int n, const dp_layer_desc *descs, const int *epilogues, dp_batch **out) {
+    if (n <= 0 || !descs || !epilogues || !out) return DP_ERR_INVALID_ARG;
+    *out = nullptr;
+    for (int i = 0; i < n; ++i) {
+        if (!valid_desc(&descs[i]) || epilogues[i] < 0 || epilogues[i] > 2) return DP_ERR_INVALID_ARG;
+        if (groups_of(&descs[i]) < 1) return DP_ERR_INVALID_ARG;
+    }
+    dp_batch *b = new (std::nothrow) dp_batch;
+    if (!b) return DP_ERR_CUDA;
+    b->items.resize(n);
+    for (int i = 0; i < n; ++i) {
+        dp_batch::Item &it = b->items[i];
+        it.desc = descs[i]; it.epi = epilogues[i]; it.group = it.slot = -1; it.scratch = 0;
+        make_layer_plan(&it.desc, it.epi, it.plan);
+        if (it.desc.impl == DP_IMPL_TENSOR_CORE && !it.plan.use_tc) { delete b; return DP_ERR_UNSUPPORTED; }
+    }
+    size_t off = kWsHeaderBytes;
+    plan_convs(*b, off);
+    plan_affine(*b, off);
+    b->singles = off;
+    size_t most = 0;
+    for (const auto &it : b->items)
+        if (it.group < 0 && it.plan.total > most) most = it.plan.total;
+    b->total = most > kWsHeaderBytes ? round_up(off + most - kWsHeaderBytes, 256) : off;
+    *out = b;
+    return DP_OK;
+}
+
+extern "C" void dp_batch_destroy(dp_batch *b) {
+    if (!b) return;
+    for (int i = 0; i < BatchStreams::kCount; ++i) {
+        if (b->done[i]) cudaEventDestroy(b->done[i]);
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
+    if (b->gram_done) cudaEventDestroy(b->gram_done);
+    delete b;
+}
+
+extern "C" size_t dp_batch_workspace_bytes(const dp_batch *b) { return b ? b->total : 0; }
+
+extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, float C_l, void *workspace, size_t workspace_bytes,
+                                  void *cuda_stream) {
+    if (!b || !io) return DP_ERR_INVALID_ARG;
+    const int n = (int)b->items.size();
+    for (int i = 0; i < n; ++i) {
+        const LayerBuffers buf = {io[i].X, io[i].dY, io[i].G_w, io[i].G_b, io[i].sqnorm, io[i].sqnorm_stride, io[i].acc_w, io[i].acc_b, io[i].clip_out};
+        const dp_status rc = check_layer(&b->items[i].desc, b->items[i].epi, buf, C_l);
+        if (rc != DP_OK) return rc;
+    }
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < b->total) return DP_ERR_WORKSPACE;
+    char *ws = static_cast<char *>(workspace);
+    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    std::lock_guard<std::mutex> lock(b->mu);
+    // The launches of different kinds are independent: memory-bound normalisation layers and the blocks of small launches
+    // fill what the tensor-core launches leave idle.
+    BatchStreams streams;
+    const bool forked = n > 1 && side_streams(*b);
+    for (int i = 0; i < BatchStreams::kCount; ++i) streams.s[i] = forked && i ? b->side[i] : st;
+    streams.gram_done = forked ? b->gram_done : nullptr;
+    if (forked) {
+        DP_CUDA_TRY(cudaEventRecord(b->fork, st));
+        for (int i = 1; i < BatchStreams::kCount; ++i) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->fork, 0));
+    }
+    auto join = [&]() -> dp_status {
+        if (!forked) return DP_OK;
+        for (int i = 1; i < BatchStreams::kCount; ++i) {
+            DP_CUDA_TRY(cudaEventRecord(b->done[i], streams.s[i]));
+            DP_CUDA_TRY(cudaStreamWaitEvent(st, b->done[i], 0));
+        }
+        return DP_OK;
+    };
+    dp_status rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
+    for (int i = 0; i < n && rc == DP_OK; ++i) {
+        const dp_batch::Item &it = b->items[i];
+        if (it.group >= 0) continue;
+        const LayerBuffers buf = {io[i].X, io[i].dY, io[i].G_w, io[i].G_b, io[i].sqnorm, io[i].sqnorm_stride, io[i].acc_w, io[i].acc_b, io[i].clip_out};
+        rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kAffine]);
+    }
+    if (rc == DP_OK) return run_convs(*b, io, C_l, ws, streams, join);
+    (void)join();                        // a launch failed: whatever is enqueued still comes before what follows
+    return rc;
+}

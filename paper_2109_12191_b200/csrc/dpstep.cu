@@ -1,6 +1,6 @@
 // Host side of dp_per_example_wgrad: argument checks, workspace layout, and the choice between
 // the tcgen05 tensor-core kernel and the CUDA-core kernels.
-#include "wgrad_simple.cuh"
+#include "layer.cuh"
 #include "wgrad_tc.cuh"
 #include <math.h>
 #include <stdio.h>
@@ -43,7 +43,7 @@ int sm_count() {
     return v;
 }
 
-static bool valid_desc(const dp_layer_desc *d) {
+bool valid_desc(const dp_layer_desc *d) {
     if (!d) return false;
     if (d->kind != DP_LAYER_DENSE && d->kind != DP_LAYER_CONV2D && d->kind != DP_LAYER_NORM_AFFINE) return false;
     if (d->dtype != DP_F32 && d->dtype != DP_BF16 && d->dtype != DP_TF32) return false;
@@ -60,7 +60,7 @@ static bool valid_desc(const dp_layer_desc *d) {
     return true;
 }
 
-static ConvGeom geom_of(const dp_layer_desc *d) {
+ConvGeom geom_of(const dp_layer_desc *d) {
     ConvGeom g;
     g.B = d->B; g.H = d->H; g.W = d->W; g.Cin = d->C_in; g.Kout = d->K_out; g.R = d->R; g.S = d->S;
     g.stride = d->stride; g.pad = d->pad;
@@ -70,19 +70,7 @@ static ConvGeom geom_of(const dp_layer_desc *d) {
     return g;
 }
 
-// Element type of X and dY in memory: DP_TF32 only changes the arithmetic of the tensor-core kernel.
-static int storage_type(const dp_layer_desc *d) { return d->dtype == DP_TF32 ? DP_F32 : d->dtype; }
-
-static bool has_bias_tensor(const dp_layer_desc *d) { return d->kind == DP_LAYER_NORM_AFFINE || d->has_bias != 0; }
-static int groups_of(const dp_layer_desc *d) { return (d->bias_separate && has_bias_tensor(d)) ? 2 : 1; }
-
-struct WgradPlan {
-    bool use_tc, use_thin;
-    int slots, w_slots;
-    size_t status_off, partial_off, factor_off, db_off, chunk_off, dg_off, tc_off, total;
-};
-
-static bool make_plan(const dp_layer_desc *d, int epi, WgradPlan &pl) {
+void make_layer_plan(const dp_layer_desc *d, int epi, WgradPlan &pl) {
     const ConvGeom g = geom_of(d);
     const size_t B = (size_t)d->B;
     pl.use_tc = false;
@@ -116,7 +104,6 @@ static bool make_plan(const dp_layer_desc *d, int epi, WgradPlan &pl) {
         off = round_up(off + bytes, 256);
     }
     pl.total = off;
-    return true;
 }
 
 }  // namespace dp
@@ -128,41 +115,43 @@ extern "C" int dp_layer_groups(const dp_layer_desc *desc) { return valid_desc(de
 extern "C" size_t dp_workspace_bytes(const dp_layer_desc *desc, int epilogue) {
     if (!valid_desc(desc) || epilogue < 0 || epilogue > 2) return 0;
     WgradPlan pl;
-    make_plan(desc, epilogue, pl);
+    make_layer_plan(desc, epilogue, pl);
     return pl.total;
 }
 
 extern "C" int dp_wgrad_uses_tensor_cores(const dp_layer_desc *desc, int epilogue) {
     if (!valid_desc(desc) || epilogue < 0 || epilogue > 2) return 0;
     WgradPlan pl;
-    make_plan(desc, epilogue, pl);
+    make_layer_plan(desc, epilogue, pl);
     return pl.use_tc ? 1 : 0;
 }
 
-extern "C" dp_status dp_per_example_wgrad(const dp_layer_desc *d, const void *X, const void *dY, float *G_w, float *G_b,
-                                          float *sqnorm, long long sqnorm_stride, int epi, float C_l, float *acc_w,
-                                          float *acc_b, float *clip_out, void *workspace, size_t workspace_bytes,
-                                          void *cuda_stream) {
+namespace dp {
+
+dp_status check_layer(const dp_layer_desc *d, int epi, const LayerBuffers &io, float C_l) {
     if (!valid_desc(d) || epi < 0 || epi > 2) return DP_ERR_INVALID_ARG;
-    if (!X || !dY || !sqnorm || !aligned(X, 16) || !aligned(dY, 16) || !aligned(sqnorm, 4)) return DP_ERR_INVALID_ARG;
-    const int groups = groups_of(d);
+    if (!io.X || !io.dY || !io.sqnorm || !aligned(io.X, 16) || !aligned(io.dY, 16) || !aligned(io.sqnorm, 4)) return DP_ERR_INVALID_ARG;
     const bool bias = has_bias_tensor(d);
-    if (sqnorm_stride < groups) return DP_ERR_INVALID_ARG;
+    if (io.sqnorm_stride < groups_of(d)) return DP_ERR_INVALID_ARG;
     if (epi == DP_EPI_STORE_NORM) {
-        if (!G_w || !aligned(G_w, 16) || (bias && (!G_b || !aligned(G_b, 16)))) return DP_ERR_INVALID_ARG;
+        if (!io.G_w || !aligned(io.G_w, 16) || (bias && (!io.G_b || !aligned(io.G_b, 16)))) return DP_ERR_INVALID_ARG;
     }
     if (epi == DP_EPI_CLIP_ACCUM) {
         if (!(C_l > 0.0f)) return DP_ERR_INVALID_ARG;
-        if (!acc_w || !aligned(acc_w, 16) || (bias && (!acc_b || !aligned(acc_b, 16)))) return DP_ERR_INVALID_ARG;
-        if (clip_out && !aligned(clip_out, 4)) return DP_ERR_INVALID_ARG;
+        if (!io.acc_w || !aligned(io.acc_w, 16) || (bias && (!io.acc_b || !aligned(io.acc_b, 16)))) return DP_ERR_INVALID_ARG;
+        if (io.clip_out && !aligned(io.clip_out, 4)) return DP_ERR_INVALID_ARG;
     }
-    WgradPlan pl;
-    make_plan(d, epi, pl);
-    if (d->impl == DP_IMPL_TENSOR_CORE && !pl.use_tc) return DP_ERR_UNSUPPORTED;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < pl.total) return DP_ERR_WORKSPACE;
+    return DP_OK;
+}
 
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    char *ws = static_cast<char *>(workspace);
+dp_status run_layer(const dp_layer_desc *d, int epi, const LayerBuffers &io, float C_l, const WgradPlan &pl, char *header,
+                    char *scratch, cudaStream_t st) {
+    const void *X = io.X, *dY = io.dY;
+    float *G_w = io.G_w, *G_b = io.G_b, *sqnorm = io.sqnorm, *acc_w = io.acc_w, *acc_b = io.acc_b, *clip_out = io.clip_out;
+    const long long sqnorm_stride = io.sqnorm_stride;
+    const int groups = groups_of(d);
+    char *ws = scratch - kWsHeaderBytes;                 // the plan's offsets count from its header
+    int *status = reinterpret_cast<int *>(header + pl.status_off), *counters = reinterpret_cast<int *>(header + kWsCounterOffset);
     float *partial = reinterpret_cast<float *>(ws + pl.partial_off);
     float *factor = reinterpret_cast<float *>(ws + pl.factor_off);
     float *db_ws = reinterpret_cast<float *>(ws + pl.db_off);
@@ -192,45 +181,44 @@ extern "C" dp_status dp_per_example_wgrad(const dp_layer_desc *d, const void *X,
                 // norms only, a large gradient over a small plane, calls running side by side: from the pixel Gram matrices,
                 // without forming the gradient (far less SM time; a call that has the GPU to itself is quicker on all SMs)
                 const TcInlineClip ic = {0.f, sqnorm, sqnorm_stride, nullptr};
-                return launch_conv_gram_norm(d->dtype, X, dY, g, ic, nullptr, reinterpret_cast<int *>(ws + pl.status_off), st);
+                return launch_conv_gram_norm(d->dtype, X, dY, g, ic, nullptr, status, st);
             }
             if (pl.use_tc) {
                 // one launch: the kernel's last CTA folds the partial norms (a ticket in the workspace header)
-                const TcPublish pub = {reinterpret_cast<int *>(ws + kWsCounterOffset), pl.w_slots, groups == 2, sqnorm, sqnorm_stride, nullptr, 0.f, nullptr};
+                const TcPublish pub = {counters, pl.w_slots, groups == 2, sqnorm, sqnorm_stride, nullptr, 0.f, nullptr};
                 return launch_conv_tc(d->dtype, epi, X, dY, g, G_w, partial, pl.slots, nullptr, nullptr, ws + pl.tc_off,
-                                      reinterpret_cast<int *>(ws + pl.status_off), st, false, nullptr, &pub);
+                                      status, st, false, &pub);
             }
-            if (pl.use_tc) rc = launch_conv_tc(d->dtype, epi, X, dY, g, G_w, partial, pl.slots, nullptr, nullptr, ws + pl.tc_off, reinterpret_cast<int *>(ws + pl.status_off), st);
-            else rc = launch_conv_fma(storage_type(d), epi, X, dY, g, G_w, partial, pl.slots, nullptr, nullptr, nullptr, st);
+            rc = launch_conv_fma(storage_type(d), epi, X, dY, g, G_w, partial, pl.slots, nullptr, nullptr, nullptr, st);
             if (rc != DP_OK) return rc;
             return launch_finalize(partial, d->B, pl.slots, pl.w_slots, groups == 2, sqnorm, sqnorm_stride, 0, 0.f, factor, nullptr, st);
         }
         if (pl.use_tc && !d->has_bias && single_pass_enabled() && tc_clip_single_pass(d->dtype, g)) {
             // per-layer clipping from ONE contraction: norm, factor and scaled sum come from the same accumulators
             const TcInlineClip ic = {C_l, sqnorm, sqnorm_stride, clip_out};
-            return launch_conv_clip1(d->dtype, X, dY, g, partial, pl.slots, ic, acc_w, ws + pl.tc_off,
-                                     reinterpret_cast<int *>(ws + pl.status_off), st);
+            return launch_conv_clip1(d->dtype, X, dY, g, ic, acc_w, ws + pl.tc_off,
+                                     status, st);
         }
         // per-layer clipping: norms of every example first, then the clipped sum with the factors known
         if (pl.use_tc) {
             if (!d->has_bias && single_pass_enabled() && tc_clip_scaled_sum(d->dtype, g) && tc_gram_norm(d->dtype, g)) {
                 // small planes: norms and factors from the pixel Gram matrices, then the clipped sum as one product
                 const TcInlineClip ic = {C_l, sqnorm, sqnorm_stride, clip_out};
-                rc = launch_conv_gram_norm(d->dtype, X, dY, g, ic, factor, reinterpret_cast<int *>(ws + pl.status_off), st);
+                rc = launch_conv_gram_norm(d->dtype, X, dY, g, ic, factor, status, st);
                 if (rc != DP_OK) return rc;
                 if (tc_clip_scaled_tiles(d->dtype, g))     // enough pixels an example: scaled per example out of tensor memory
-                    return launch_conv_scaled_tiles(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, reinterpret_cast<int *>(ws + pl.status_off), st);
-                return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, reinterpret_cast<int *>(ws + pl.status_off), st);
+                    return launch_conv_scaled_tiles(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
+                return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
             }
             // the norm pass's last CTA folds the partial norms (bias slots included) into norms and factors
-            const TcPublish pub = {reinterpret_cast<int *>(ws + kWsCounterOffset), pl.w_slots, groups == 2, sqnorm, sqnorm_stride, factor, C_l, clip_out};
+            const TcPublish pub = {counters, pl.w_slots, groups == 2, sqnorm, sqnorm_stride, factor, C_l, clip_out};
             rc = launch_conv_tc(d->dtype, DP_EPI_NORM_ONLY, X, dY, g, nullptr, partial, pl.slots, nullptr, nullptr, ws + pl.tc_off,
-                                reinterpret_cast<int *>(ws + pl.status_off), st, false, nullptr, &pub);
+                                status, st, false, &pub);
             if (rc != DP_OK) return rc;
             if (!d->has_bias && single_pass_enabled() && tc_clip_scaled_sum(d->dtype, g))
-                return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, reinterpret_cast<int *>(ws + pl.status_off), st);
+                return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
             rc = launch_conv_tc(d->dtype, DP_EPI_CLIP_ACCUM, X, dY, g, nullptr, partial, pl.slots, factor, acc_w, ws + pl.tc_off,
-                                reinterpret_cast<int *>(ws + pl.status_off), st, true);
+                                status, st, true);
             if (rc != DP_OK) return rc;
             if (d->has_bias) return launch_bias_accum(db, d->B, d->K_out, factor, acc_b, st);
             return DP_OK;
@@ -239,8 +227,7 @@ extern "C" dp_status dp_per_example_wgrad(const dp_layer_desc *d, const void *X,
         if (rc != DP_OK) return rc;
         rc = launch_finalize(partial, d->B, pl.slots, pl.w_slots, groups == 2, sqnorm, sqnorm_stride, 1, C_l, factor, clip_out, st);
         if (rc != DP_OK) return rc;
-        if (pl.use_tc) rc = launch_conv_tc(d->dtype, DP_EPI_CLIP_ACCUM, X, dY, g, nullptr, partial, pl.slots, factor, acc_w, ws + pl.tc_off, reinterpret_cast<int *>(ws + pl.status_off), st, true);
-        else rc = launch_conv_fma(storage_type(d), DP_EPI_CLIP_ACCUM, X, dY, g, nullptr, partial, pl.slots, factor, acc_w, reinterpret_cast<float *>(ws + pl.tc_off), st);
+        rc = launch_conv_fma(storage_type(d), DP_EPI_CLIP_ACCUM, X, dY, g, nullptr, partial, pl.slots, factor, acc_w, reinterpret_cast<float *>(ws + pl.tc_off), st);
         if (rc != DP_OK) return rc;
         if (d->has_bias) return launch_bias_accum(db, d->B, d->K_out, factor, acc_b, st);
         return DP_OK;
@@ -268,7 +255,7 @@ extern "C" dp_status dp_per_example_wgrad(const dp_layer_desc *d, const void *X,
         float *dbt = (epi == DP_EPI_STORE_NORM) ? G_b : reinterpret_cast<float *>(ws + pl.dg_off) + (size_t)d->B * d->C_in;
         if (affine_fused_eligible(d->B))
             return launch_norm_affine_fused(storage_type(d), X, dY, d->B, d->H * d->W, d->C_in, chunk_partial, dg, dbt, factor,
-                                            reinterpret_cast<int *>(ws + kWsCounterOffset), clip, C_l, groups == 2, sqnorm,
+                                            counters, clip, C_l, groups == 2, sqnorm,
                                             sqnorm_stride, clip_out, acc_w, acc_b, st);
         rc = launch_norm_affine(storage_type(d), X, dY, d->B, d->H * d->W, d->C_in, chunk_partial, dg, dbt, partial, st);
         if (rc != DP_OK) return rc;
@@ -277,6 +264,23 @@ extern "C" dp_status dp_per_example_wgrad(const dp_layer_desc *d, const void *X,
                                             acc_w, acc_b, st);
         return launch_finalize(partial, d->B, 2, 1, groups == 2, sqnorm, sqnorm_stride, 0, 0.f, factor, nullptr, st);
     }
+}
+
+}  // namespace dp
+
+extern "C" dp_status dp_per_example_wgrad(const dp_layer_desc *d, const void *X, const void *dY, float *G_w, float *G_b,
+                                          float *sqnorm, long long sqnorm_stride, int epi, float C_l, float *acc_w,
+                                          float *acc_b, float *clip_out, void *workspace, size_t workspace_bytes,
+                                          void *cuda_stream) {
+    const LayerBuffers io = {X, dY, G_w, G_b, sqnorm, sqnorm_stride, acc_w, acc_b, clip_out};
+    const dp_status rc = check_layer(d, epi, io, C_l);
+    if (rc != DP_OK) return rc;
+    WgradPlan pl;
+    make_layer_plan(d, epi, pl);
+    if (d->impl == DP_IMPL_TENSOR_CORE && !pl.use_tc) return DP_ERR_UNSUPPORTED;
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < pl.total) return DP_ERR_WORKSPACE;
+    char *ws = static_cast<char *>(workspace);
+    return run_layer(d, epi, io, C_l, pl, ws, ws + kWsHeaderBytes, static_cast<cudaStream_t>(cuda_stream));
 }
 
 extern "C" dp_status dp_per_example_wgrad_scaled(const dp_layer_desc *d, const void *X, const void *dY,
@@ -290,7 +294,7 @@ extern "C" dp_status dp_per_example_wgrad_scaled(const dp_layer_desc *d, const v
     if (!acc_w || !aligned(acc_w, 16) || (bias && (!acc_b || !aligned(acc_b, 16)))) return DP_ERR_INVALID_ARG;
     if (!factor_b) factor_b = factor_w;
     WgradPlan pl;
-    make_plan(d, DP_EPI_CLIP_ACCUM, pl);
+    make_layer_plan(d, DP_EPI_CLIP_ACCUM, pl);
     if (d->impl == DP_IMPL_TENSOR_CORE && !pl.use_tc) return DP_ERR_UNSUPPORTED;
     if (!workspace || !aligned(workspace, 256) || workspace_bytes < pl.total) return DP_ERR_WORKSPACE;
 

@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <array>
 #include <map>
+#include <memory>
 
 namespace dp {
 
@@ -44,6 +45,7 @@ struct TcPlan {
     int OWt, OHt, tiles_w, tiles_h, Kt, k_tiles;
     int stages, stage_bytes, a_bytes;
     size_t smem;
+    double item_cycles;         // rough time of one (example, tile) item in its CTA
 };
 
 struct TcParams {
@@ -64,10 +66,7 @@ struct TcParams {
     int total_tiles;            // work items: (example, tile) pairs, or (example range, tile) pairs in mode 2
     // mode 2: item = (split, tile); the CTA walks examples [split*per_split, ...) and keeps sum_n f_n D_n in registers
     int splits, per_split;
-    const float *factor;        // [B][2], element 0 = weight factor (used when inline_factor == 0)
-    // inline_factor: the clipped-sum pass works the factor out itself from the norm pass's partial sums (partial,
-    // slots) and publishes the squared norm and the factor, which saves the separate finalising launch
-    int inline_factor;
+    const float *factor;        // [B][2], element 0 = weight factor
     float C_l;
     float *sqnorm; long long sq_stride; float *clip_out;
     float *sum_out;             // splits == 1: the accumulator (added to); else partial sums [splits][Kout*Ng]
@@ -78,7 +77,28 @@ struct TcParams {
     // space-to-depth form of a thin strided layer (s2d_st > 0): row j' of D is (r2, s2, dy, dx, c) of the regrouped
     // input and maps to column ((st*r2+dy)*s2d_S + st*s2d+dx)*s2d_Cin + c of the gradient, or to nothing
     int s2d_st, s2d_R, s2d_S, s2d_Cin;
+    // which work items a block takes (norm / store / clipped-sum kernel): block b of `blocks` starts at b * run and takes
+    // `run` items in a row, or with run == 0 every blocks-th item from b on
+    int blocks, run;
+    int cluster;                // single-pass kernel: blocks per cluster of the launch (>= tiles of one example)
 };
+
+// A launch serves up to N layers: the table of their tensor maps and parameters travels as a kernel parameter, and every
+// block finds its layer by its index (first[] ascending).  N = 1 for a call on its own.
+constexpr int kTcLayers = 48, kSsumLayers = 40;      // layers per grouped launch: a table stays below the 32 KB a launch may carry
+template <typename P, int MAPS>
+struct alignas(64) TcEntry { CUtensorMap map[MAPS]; P p; };
+template <typename P, int MAPS, int N>
+struct TcTable { int n; int first[N]; TcEntry<P, MAPS> e[N]; };
+
+template <int N>
+__device__ __forceinline__ int table_entry(const int (&first)[N], int n, int blk) {
+    if (N == 1) return 0;
+    const int lane = threadIdx.x & 31;
+    const unsigned lo = __ballot_sync(0xffffffffu, lane < n && blk >= first[lane < N ? lane : 0]);
+    const unsigned hi = __ballot_sync(0xffffffffu, lane + 32 < n && blk >= first[lane + 32 < N ? lane + 32 : 0]);
+    return __popc(lo) + __popc(hi) - 1;
+}
 
 // column of the gradient that row j of the space-to-depth product stands for, or -1 (a tap or channel that does not exist)
 __device__ __forceinline__ int s2d_column(const TcParams &p, int j) {
@@ -217,9 +237,15 @@ __device__ __forceinline__ uint32_t instr_desc(int n_cols, uint32_t fmt) {
     return (1u << 4) | (fmt << 7) | (fmt << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n_cols >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-template <bool TF32, bool CLIP>
+template <bool TF32, bool CLIP, int N>
 __global__ void __launch_bounds__(TF32 ? 480 : 224, 1)
-conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, const TcParams p) {
+conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
+    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
+    const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
+    const TcParams &p = tab.e[entry].p;
+    const int blk = (int)blockIdx.x - tab.first[entry];
+    const int item0 = p.run ? blk * p.run : blk, item_step = p.run ? 1 : p.blocks;
+    const int item_end = p.run ? min(p.total_tiles, item0 + p.run) : p.total_tiles;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], ready_bar[kMaxStages], tmem_full[2], tmem_empty[2];
     __shared__ uint32_t tmem_base_slot;
@@ -259,7 +285,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         // pixel-tile origin, so no division sits in the stage loop.
         int stage = 0; uint32_t phase = 0;
         bool live = true;
-        for (int item = blockIdx.x; item < p.total_tiles && live; item += gridDim.x) {
+        for (int item = item0; item < item_end && live; item += item_step) {
             const Item it = decode_item(p, item);
             const int mt = it.mt, nt = it.nt;
             const int a_slab0 = mt * a_slabs_tile, a_slabs = min(a_slabs_tile, p.a_ext / p.slab_ch - a_slab0);
@@ -313,7 +339,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
             const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
             const int ksteps = p.Kt / p.krows;
             constexpr uint32_t kadvance = (uint32_t)((TF32 ? 8 : 16) * kRowBytes) >> 4;   // start-address units of 16 B per MMA step
-            for (int item = blockIdx.x; item < p.total_tiles && live; item += gridDim.x) {
+            for (int item = item0; item < item_end && live; item += item_step) {
               const Item it = decode_item(p, item);
               const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
               const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, TF32 ? 2u : 1u);
@@ -377,7 +403,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         int stage = 0; uint32_t phase = 0;
         int turn = 0;                       // global stage counter modulo 2: whose stage is it
         bool live = true;
-        for (int item = blockIdx.x; item < p.total_tiles && live; item += gridDim.x) {
+        for (int item = item0; item < item_end && live; item += item_step) {
             const Item it = decode_item(p, item);
             const int a_slabs = min(a_slabs_tile, p.a_ext / p.slab_ch - it.mt * a_slabs_tile);
             const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
@@ -434,7 +460,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         uint32_t full_phase = 0;     // bit b: parity to wait for on accumulator buffer b
         int buf = 0;
         bool live = true;
-        for (int item = blockIdx.x; item < p.total_tiles && live; item += gridDim.x) {
+        for (int item = item0; item < item_end && live; item += item_step) {
             const Item it = decode_item(p, item);
             const int mt = it.mt, nt = it.nt;
             const int a_rows = min(128, p.a_ext - mt * 128);
@@ -449,7 +475,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
             float f_lane = 0.f;     // clip mode, known factors: lane l holds the factor of example n_base + l
             int n_base = it.n_lo - 32;
             for (int n = it.n_lo; n < it.n_hi; ++n) {
-                if (CLIP && !p.inline_factor && n >= n_base + 32) {
+                if (CLIP && n >= n_base + 32) {
                     n_base = n;
                     f_lane = (n + lane < it.n_hi) ? p.factor[2 * (n + lane)] : 0.f;    // one coalesced load per 32 examples
                 }
@@ -459,21 +485,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
                 tc_fence_after();
                 const uint32_t t_addr = tmem_base + (uint32_t)(buf * 256) + ((uint32_t)(q * 32) << 16);
                 if (CLIP) {
-                    float f;
-                    if (p.inline_factor) {
-                        // same summation order in every warp of every CTA, so all of them apply the identical factor
-                        double sn = 0.0;
-                        const float *pn = p.partial + (long long)n * p.slots;
-                        for (int i = lane; i < p.slots; i += 32) sn += (double)pn[i];
-                        sn = warp_sum(sn);
-                        f = clip_factor(sn, p.C_l);
-                        if (mt == 0 && nt == 0 && q == 0 && lane == 0) {
-                            p.sqnorm[n * p.sq_stride] = (float)sn;
-                            if (p.clip_out) p.clip_out[n] = f;
-                        }
-                    } else {
-                        f = __shfl_sync(0xffffffffu, f_lane, n - n_base);
-                    }
+                    const float f = __shfl_sync(0xffffffffu, f_lane, n - n_base);
 #pragma unroll
                     for (int c2 = 0; c2 < 2; ++c2) {           // columns in pairs of 32: both loads in flight before the wait
                         if (c2 * 64 < n_cols) {
@@ -543,7 +555,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
                 }
                 buf ^= 1;
             }
-            if (!CLIP && p.counters && lane == 0 && item + (int)gridDim.x >= p.total_tiles)
+            if (!CLIP && p.counters && lane == 0 && item + item_step >= item_end)
                 __threadfence();          // after this warp's last item: its partial sums are visible to the CTA that folds them
             if (CLIP && live && row_ok) {
                 // one owner per output element: add straight into the accumulator, or leave a partial sum for the fold
@@ -590,7 +602,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         __shared__ int last_cta;
         if (threadIdx.x == 0) {
             __threadfence();
-            last_cta = atomicAdd(&p.counters[0], 1) == (int)gridDim.x - 1;
+            last_cta = atomicAdd(&p.counters[0], 1) == p.blocks - 1;
             if (last_cta) p.counters[0] = 0;
         }
         __syncthreads();
@@ -693,8 +705,13 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     return false;
 }
 
+template <int N>
 __global__ void __launch_bounds__(kClipThreads, 1)
-conv_wgrad_clip1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, const TcParams p) {
+conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
+    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
+    const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
+    const TcParams &p = tab.e[entry].p;
+    const int blk = (int)blockIdx.x - tab.first[entry];
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tmem_full[2], tmem_empty[2], norm_bar[4], warp_bar[4];
     __shared__ float warp_part[4][8];                   // [example mod 4][epilogue warp]: this CTA's partial sums
@@ -708,10 +725,13 @@ conv_wgrad_clip1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
     const int cs = p.m_tiles * p.n_tiles;                 // cluster size = tiles of one example's gradient
     // With the factors known beforehand (p.factor) nothing is exchanged: the launch has no clusters and any number of tiles
     const bool known = p.factor != nullptr;
-    const int rank = known ? (int)(blockIdx.x % (unsigned)cs) : (int)cluster_rank();
+    // A cluster of the launch may hold several examples' sets of tiles (layers of different sizes share a launch): blocks
+    // [set * cs, set * cs + cs) of it are one set; blocks left over, and sets past the last example range, have no work.
+    const int sets = p.cluster / cs, crank = known ? 0 : (int)cluster_rank(), set = crank / cs;
+    const int rank = known ? blk % cs : crank - set * cs;
     const int mt = rank / p.n_tiles, nt = rank - mt * p.n_tiles;
-    const int split = (int)blockIdx.x / cs;
-    const int n_lo = split * p.per_split, n_hi = min(p.B, n_lo + p.per_split);
+    const int split = known ? blk / cs : (set < sets ? blk / p.cluster * sets + set : p.splits);
+    const int n_lo = min(p.B, split * p.per_split), n_hi = min(p.B, n_lo + p.per_split);
 
     if (threadIdx.x == 0) {
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmX)) : "memory");
@@ -938,12 +958,12 @@ conv_wgrad_clip1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
                     // this CTA expects one float from every CTA of the cluster (its own included) in this slot's phase
                     if (lane == 0) mbar_expect_tx(smem_u32(&norm_bar[slot]), (uint32_t)(cs * 4));
                     if (lane < cs)
-                        st_async_f32(map_to_cta(smem_u32(&norm_part[slot][rank]), (uint32_t)lane), cta_sq,
-                                     map_to_cta(smem_u32(&norm_bar[slot]), (uint32_t)lane));
+                        st_async_f32(map_to_cta(smem_u32(&norm_part[slot][rank]), (uint32_t)(set * cs + lane)), cta_sq,
+                                     map_to_cta(smem_u32(&norm_bar[slot]), (uint32_t)(set * cs + lane)));
                 }
             }
         }
-        if (live && row_ok) {
+        if (live && row_ok && split < p.splits) {
             // one owner per output element: add straight into the accumulator, or leave a partial sum for the fold
             const bool add = p.splits == 1;
             float *base = p.sum_out + (add ? 0ll : (long long)split * p.Kout * p.Ng);
@@ -1000,9 +1020,13 @@ conv_wgrad_clip1_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_co
 // is lost is below 2^-17 of each product) and every k-step issues two MMAs, X with hi and X with lo.  A work item is a
 // tile for a range of examples; with more than one range the tiles leave as partial sums for the fold.
 // Roles as in the kernel at the top: warp 0 / 6 TMA (the warp that loads dY loads both copies), warp 1 MMA, warps 2-5 epilogue.
+template <int N>
 __global__ void __launch_bounds__(224, 1)
-conv_wgrad_ssum_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmYhi,
-                       const __grid_constant__ CUtensorMap tmYlo, const TcParams p) {
+conv_wgrad_ssum_kernel(const __grid_constant__ TcTable<TcParams, 3, N> tab) {
+    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
+    const CUtensorMap &tmX = tab.e[entry].map[0], &tmYhi = tab.e[entry].map[1], &tmYlo = tab.e[entry].map[2];
+    const TcParams &p = tab.e[entry].p;
+    const int blk = (int)blockIdx.x - tab.first[entry];
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tmem_full[2], tmem_empty[2];
     __shared__ uint32_t tmem_base_slot;
@@ -1036,7 +1060,7 @@ conv_wgrad_ssum_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_con
         // ------------------------------------------------------------ TMA producers
         int stage = 0; uint32_t phase = 0;
         bool live = true;
-        for (int item = blockIdx.x; item < p.total_tiles && live; item += gridDim.x) {
+        for (int item = blk; item < p.total_tiles && live; item += p.blocks) {
             const Item it = decode_item(p, item);
             const int a_slab0 = it.mt * a_slabs_tile, a_slabs = min(a_slabs_tile, p.a_ext / p.slab_ch - a_slab0);
             const int b_slab0 = it.nt * b_slabs_tile, b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - b_slab0);
@@ -1090,7 +1114,7 @@ conv_wgrad_ssum_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_con
             const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
             const int ksteps = p.Kt / p.krows;
             constexpr uint32_t kadvance = (uint32_t)(16 * kRowBytes) >> 4;
-            for (int item = blockIdx.x; item < p.total_tiles && live; item += gridDim.x) {
+            for (int item = blk; item < p.total_tiles && live; item += p.blocks) {
                 const Item it = decode_item(p, item);
                 const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
                 const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, 1u);
@@ -1130,7 +1154,7 @@ conv_wgrad_ssum_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_con
         const int row = q * 32 + lane;
         uint32_t full_phase = 0;
         int buf = 0;
-        for (int item = blockIdx.x; item < p.total_tiles; item += gridDim.x) {
+        for (int item = blk; item < p.total_tiles; item += p.blocks) {
             const Item it = decode_item(p, item);
             const int mt = it.mt, nt = it.nt;
             const int a_rows = min(128, p.a_ext - mt * 128);
@@ -1212,6 +1236,7 @@ struct GramParams {
     float *sqnorm; long long sq_stride; float *factor_out; float *clip_out;
     int *status;
     uint32_t wait_polls;
+    int blocks;                 // blocks of the launch that work on this layer
 };
 
 // K-major operand of 128-byte rows with the 128-byte swizzle: 8-row groups 1024 B apart; the leading offset is unused
@@ -1228,8 +1253,13 @@ __device__ __forceinline__ uint32_t instr_desc_kmajor(int n_cols) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n_cols >> 3) << 17) | ((128u >> 4) << 24);
 }
 
+template <int N>
 __global__ void __launch_bounds__(192, 1)
-conv_gram_norm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmY, const GramParams p) {
+conv_gram_norm_kernel(const __grid_constant__ TcTable<GramParams, 2, N> tab) {
+    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
+    const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
+    const GramParams &p = tab.e[entry].p;
+    const int blk = (int)blockIdx.x - tab.first[entry];
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tmem_full[2], tmem_empty[2];
     __shared__ uint32_t tmem_base_slot;
@@ -1269,7 +1299,7 @@ conv_gram_norm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             int stage = 0; uint32_t phase = 0;
             bool live = true;
             const uint32_t tx_bytes = (uint32_t)(p.pack * p.rows * kRowBytes);
-            for (int n = blockIdx.x * p.pack; n < p.B && live; n += gridDim.x * p.pack) {
+            for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
                 for (int mt = 0; mt < p.m_tiles && live; ++mt) {
                     int tap = 0, cs = 0;
                     for (int s = 0; s < slabs; ++s) {
@@ -1296,7 +1326,7 @@ conv_gram_norm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             bool live = true;
             const uint64_t desc_base = kmajor_desc_base();
             const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
-            for (int n = blockIdx.x * p.pack; n < p.B && live; n += gridDim.x * p.pack) {
+            for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
                 for (int mt = 0; mt < p.m_tiles && live; ++mt) {
                     const int col0 = mt * 128;                       // the tile's columns start at its own first row
                     const uint32_t idesc = instr_desc_kmajor(p.pack * p.rows - col0);
@@ -1334,7 +1364,7 @@ conv_gram_norm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         int buf = 0;
         bool live = true;
         int trip = 0;
-        for (int n = blockIdx.x * p.pack; n < p.B && live; n += gridDim.x * p.pack) {
+        for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
             double acc = 0.0;
             for (int mt = 0; mt < p.m_tiles; ++mt) {
                 const int col0 = mt * 128;
@@ -1403,53 +1433,90 @@ conv_gram_norm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 }
 
 // hi[i] = bf16(f_n y[i]), lo[i] = bf16(f_n y[i] - hi[i]) for every entry of example n (eight entries per thread)
+struct SplitSeg { const __nv_bfloat16 *y; const float *factor; long long per_example, total8; __nv_bfloat16 *hi, *lo; };
+struct SplitTable { int n; int first[kTcLayers]; SplitSeg s[kTcLayers]; };
 __global__ void __launch_bounds__(256)
-scale_split_kernel(const __nv_bfloat16 *__restrict__ y, const float *__restrict__ factor, long long per_example, long long total8,
-                   __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
-    const long long i8 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i8 >= total8) return;
+scale_split_kernel(const __grid_constant__ SplitTable tab) {
+    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
+    const SplitSeg &sg = tab.s[entry];
+    const long long i8 = (long long)(blockIdx.x - tab.first[entry]) * 256 + threadIdx.x;
+    if (i8 >= sg.total8) return;
     const long long i = i8 * 8;
-    const float f = factor[2 * (i / per_example)];
+    const float f = sg.factor[2 * (i / sg.per_example)];
     __nv_bfloat16 v[8], h[8], l[8];
-    *reinterpret_cast<uint4 *>(v) = *reinterpret_cast<const uint4 *>(y + i);
+    *reinterpret_cast<uint4 *>(v) = *reinterpret_cast<const uint4 *>(sg.y + i);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         const float x = f * __bfloat162float(v[e]);
         h[e] = __float2bfloat16_rn(x);
         l[e] = __float2bfloat16_rn(x - __bfloat162float(h[e]));
     }
-    *reinterpret_cast<uint4 *>(hi + i) = *reinterpret_cast<const uint4 *>(h);
-    *reinterpret_cast<uint4 *>(lo + i) = *reinterpret_cast<const uint4 *>(l);
+    *reinterpret_cast<uint4 *>(sg.hi + i) = *reinterpret_cast<const uint4 *>(h);
+    *reinterpret_cast<uint4 *>(sg.lo + i) = *reinterpret_cast<const uint4 *>(l);
 }
 
-// acc[i] += sum over splits of part[s][i], splits in index order (P a multiple of 4, both 16-byte aligned)
-__global__ void __launch_bounds__(256)
-fold_partial_sums_kernel(const float *__restrict__ part, int splits, long long P, float *__restrict__ acc) {
-    const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-    if (i >= P) return;
-    float4 a = *reinterpret_cast<const float4 *>(acc + i);
-    for (int s = 0; s < splits; ++s) {
-        const float4 v = __ldcs(reinterpret_cast<const float4 *>(part + (long long)s * P + i));
-        a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+static dp_status launch_scale_split(const std::vector<SplitSeg> &segs, cudaStream_t stream) {
+    for (size_t i = 0; i < segs.size();) {
+        SplitTable tab;
+        long long blocks = 0;
+        for (tab.n = 0; i < segs.size() && tab.n < kTcLayers; ++i) {
+            tab.first[tab.n] = (int)blocks;
+            tab.s[tab.n++] = segs[i];
+            blocks += (segs[i].total8 + 255) / 256;
+        }
+        if (blocks > 0x7fffffffll) return DP_ERR_UNSUPPORTED;
+        scale_split_kernel<<<(unsigned)blocks, 256, 0, stream>>>(tab);
+        DP_LAUNCH_CHECK("scale_split_kernel");
     }
-    *reinterpret_cast<float4 *>(acc + i) = a;
-}
-
-__global__ void fold_partial_sums_scalar_kernel(const float *__restrict__ part, int splits, long long P, float *__restrict__ acc) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P) return;
-    float a = acc[i];
-    for (int s = 0; s < splits; ++s) a += part[(long long)s * P + i];
-    acc[i] = a;
-}
-
-dp_status launch_fold_partial_sums(const float *part, int splits, long long P, float *acc, cudaStream_t stream) {
-    if (P % 4 == 0 && aligned(part, 16) && aligned(acc, 16))
-        fold_partial_sums_kernel<<<(unsigned)((P / 4 + 255) / 256), 256, 0, stream>>>(part, splits, P, acc);
-    else
-        fold_partial_sums_scalar_kernel<<<(unsigned)((P + 255) / 256), 256, 0, stream>>>(part, splits, P, acc);
-    DP_LAUNCH_CHECK("fold_partial_sums_kernel");
     return DP_OK;
+}
+
+// acc[i] += sum over splits of part[s][i], splits in index order; vec: P a multiple of 4 and both 16-byte aligned
+struct FoldSeg { const float *part; float *acc; long long P; int splits, vec; };
+struct FoldTable { int n; int first[kTcLayers]; FoldSeg s[kTcLayers]; };
+__global__ void __launch_bounds__(256)
+fold_partial_sums_kernel(const __grid_constant__ FoldTable tab) {
+    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
+    const FoldSeg &sg = tab.s[entry];
+    const long long P = sg.P, i = ((long long)(blockIdx.x - tab.first[entry]) * 256 + threadIdx.x) * 4;
+    if (i >= P) return;
+    if (sg.vec) {
+        float4 a = *reinterpret_cast<const float4 *>(sg.acc + i);
+#pragma unroll 4
+        for (int s = 0; s < sg.splits; ++s) {
+            const float4 v = __ldcs(reinterpret_cast<const float4 *>(sg.part + (long long)s * P + i));
+            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+        }
+        *reinterpret_cast<float4 *>(sg.acc + i) = a;
+    } else {
+        for (long long k = i; k < min(P, i + 4); ++k) {
+            float a = sg.acc[k];
+            for (int s = 0; s < sg.splits; ++s) a += sg.part[(long long)s * P + k];
+            sg.acc[k] = a;
+        }
+    }
+}
+
+static FoldSeg fold_seg(const float *part, int splits, long long P, float *acc) {
+    return FoldSeg{part, acc, P, splits, (P % 4 == 0 && aligned(part, 16) && aligned(acc, 16)) ? 1 : 0};
+}
+static dp_status launch_folds(const std::vector<FoldSeg> &segs, cudaStream_t stream) {
+    for (size_t i = 0; i < segs.size();) {
+        FoldTable tab;
+        long long blocks = 0;
+        for (tab.n = 0; i < segs.size() && tab.n < kTcLayers; ++i) {
+            tab.first[tab.n] = (int)blocks;
+            tab.s[tab.n++] = segs[i];
+            blocks += (segs[i].P + 1023) / 1024;
+        }
+        if (blocks > 0x7fffffffll) return DP_ERR_UNSUPPORTED;
+        fold_partial_sums_kernel<<<(unsigned)blocks, 256, 0, stream>>>(tab);
+        DP_LAUNCH_CHECK("fold_partial_sums_kernel");
+    }
+    return DP_OK;
+}
+static dp_status launch_fold_partial_sums(const float *part, int splits, long long P, float *acc, cudaStream_t stream) {
+    return launch_folds({fold_seg(part, splits, P, acc)}, stream);
 }
 
 // Layers whose input has too few channels for a TMA slab (C_in = 3 stems) are first unfolded:
@@ -1632,13 +1699,21 @@ static double step_cycles(int dtype, int n_cols, double a_slabs_loaded, double b
 
 static TcPlan search_plan(int dtype, const ConvGeom &g, int mode);
 
+// Planning on behalf of a batch of layer calls (this thread): launches hold many layers, so every layer is tiled for
+// least SM time whatever the SM target is, and a CTA walks through at most this many cycles of one layer.
+static thread_local double tl_batch_walk = 0.0;
+BatchPlanning::BatchPlanning(double walk_cycles) : saved(tl_batch_walk) { tl_batch_walk = walk_cycles; }
+BatchPlanning::~BatchPlanning() { tl_batch_walk = saved; }
+static bool side_by_side() { return tl_batch_walk > 0.0 || sm_target_set(); }
+static int launch_sms() { return tl_batch_walk > 0.0 ? sm_count() : sm_target(); }
+
 // single-pass clipped sum: how many clusters share the batch and how many examples each walks through
 // scaled-sum product: example ranges per tile.  A launch that already has a CTA for a quarter of the SMs keeps whole
 // tiles (no partial sums to fold); fewer tiles are cut up to half of the SMs.
 static void ssum_split(int B, int tiles, int &splits, int &per_split) {
-    const int sms = sm_target();
+    const int sms = launch_sms();
     // (side by side with other calls, under an SM target, a quarter: fewer partial sums to write and fold)
-    int want = (tiles * 4 >= sms) ? 1 : (sms / (sm_target_set() ? 4 : 2)) / tiles;
+    int want = (tiles * 4 >= sms) ? 1 : (sms / (side_by_side() ? 4 : 2)) / tiles;
     if (want < 1) want = 1;
     if (want > B) want = B;
     per_split = (B + want - 1) / want;
@@ -1648,14 +1723,14 @@ static void ssum_split(int B, int tiles, int &splits, int &per_split) {
 static int max_active_clusters(int cluster_size);
 // K, NT: pixels per example and columns per tile (for a rough time of one example in one CTA)
 static void cluster_split(int B, int cluster_size, int K, int NT, int &splits, int &per_split) {
-    int want = std::min(sm_target() / cluster_size, max_active_clusters(cluster_size));
+    int want = std::min(launch_sms() / cluster_size, max_active_clusters(cluster_size));
     // A caller that set an SM target runs calls side by side: what counts then is SM time, and a cluster that walks
     // through several examples spends its start-up, its first loads and its final stores once for all of them -- up
     // to thirty-two examples (a whole chunk of the per-layer workload: one example range, nothing to fold), and not
     // beyond some 60 microseconds a launch, so that no call holds its stream up for long.
-    if (sm_target_set()) {
+    if (side_by_side()) {
         const double cycles = (K / 16.0) * std::max(NT / 2.0, 64.0) * 1.5;
-        const int per = std::max(1, std::min(kMaxExamplesPerCluster, (int)(120000.0 / cycles)));
+        const int per = std::max(1, std::min(kMaxExamplesPerCluster, (int)((tl_batch_walk > 0.0 ? tl_batch_walk : 120000.0) / cycles)));
         want = std::min(want, std::max(1, B / per));
     }
     if (want < 1) want = 1;
@@ -1668,8 +1743,8 @@ static void cluster_split(int B, int cluster_size, int K, int NT, int &splits, i
 // mode: 0 gradients are stored, 1 norms only, 2 clipped sum (running sum in registers: at most 128 columns per tile)
 static TcPlan make_plan(int dtype, const ConvGeom &g, int mode) {
     static std::mutex mu;
-    static std::map<std::array<int, 12>, TcPlan> memo;
-    const std::array<int, 12> key = {dtype, g.H, g.W, g.Cin, g.Kout, g.R, g.S, g.stride, g.pad, g.B, mode, sm_target_set() ? -sm_target() : sm_target()};
+    static std::map<std::array<int, 13>, TcPlan> memo;
+    const std::array<int, 13> key = {dtype, g.H, g.W, g.Cin, g.Kout, g.R, g.S, g.stride, g.pad, g.B, mode, side_by_side() ? -launch_sms() : launch_sms(), (int)tl_batch_walk};
     std::lock_guard<std::mutex> lock(mu);
     auto it = memo.find(key);
     if (it != memo.end()) return it->second;
@@ -1692,7 +1767,7 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
     const int krows = (dtype == DP_BF16) ? 16 : 8;
     if (g.Cin % slab_ch || g.Kout % slab_ch) return best;
     if (g.stride > 8 || g.K < 1 || g.OH > 65535) return best;
-    const int sms = sm_target();
+    const int sms = launch_sms();
     const int a_slabs_tile = 128 / slab_ch;
     const int copies = (dtype == DP_F32) ? 2 : 1;       // split tf32 keeps a hi and a lo copy of every stage
     double best_cost = 1e300;
@@ -1708,8 +1783,9 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
             if (mode == 3 && !any_tiles && m_tiles * n_tiles > kMaxCluster) continue;
             const int y_slabs = (mode == 4) ? (a_is_x ? NT / slab_ch : a_slabs_tile) : 0;     // second (lo) copy of the dY slabs
             // per-CTA share of (example, tile) units: whole waves of tiles, or in clipped-sum mode an even share of the examples
-            double waves = (mode != 2) ? (double)((total_tiles + sms - 1) / sms)
-                                       : std::max(1.0, (double)total_tiles / sms);
+            // (in a batch other layers fill the last wave)
+            double waves = (mode != 2 && tl_batch_walk == 0.0) ? (double)((total_tiles + sms - 1) / sms)
+                                       : std::max(mode == 2 ? 1.0 : 0.0, (double)total_tiles / sms);
             double sm_share = 1.0;
             if (mode == 4) {
                 int splits, per;
@@ -1761,6 +1837,7 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
                         best.k_tiles = tw * th; best.stages = stages; best.stage_bytes = stage_bytes;
                         best.a_bytes = a_slabs_tile * Kt * kRowBytes;
                         best.smem = (size_t)stages * stage_bytes + 1024;
+                        best.item_cycles = std::max(mainloop, epilogue) + 300.0;
                     }
                 }
             }
@@ -1780,7 +1857,8 @@ static bool clip1_registers_ok() {
     static int ok = -1;
     if (ok < 0) {
         cudaFuncAttributes attr;
-        ok = (cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel) == cudaSuccess && attr.numRegs == kClipRegsLaunch) ? 1 : 0;
+        ok = (cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<1>) == cudaSuccess && attr.numRegs == kClipRegsLaunch &&
+              cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<kTcLayers>) == cudaSuccess && attr.numRegs == kClipRegsLaunch) ? 1 : 0;
         if (!ok) (void)cudaGetLastError();
     }
     return ok == 1;
@@ -1801,8 +1879,8 @@ static int max_active_clusters(int cluster_size) {
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = (unsigned)cluster_size; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
         cfg.attrs = at; cfg.numAttrs = 1;
-        const bool ok = cudaFuncSetAttribute(conv_wgrad_clip1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048) == cudaSuccess &&
-                        cudaOccupancyMaxActiveClusters(&n, conv_wgrad_clip1_kernel, &cfg) == cudaSuccess && n > 0;
+        const bool ok = cudaFuncSetAttribute(conv_wgrad_clip1_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048) == cudaSuccess &&
+                        cudaOccupancyMaxActiveClusters(&n, conv_wgrad_clip1_kernel<1>, &cfg) == cudaSuccess && n > 0;
         if (!ok) (void)cudaGetLastError();
         cached[cluster_size] = ok ? n : -1;
     }
@@ -1844,7 +1922,7 @@ static bool clip1_plan(int dtype, const ConvGeom &g0, const TcProblem &pr, TcPla
 // clipped-sum mode: how many example ranges each tile is cut into so that every SM has an item
 static void clip_split(const ConvGeom &g, const TcPlan &pl, int &splits, int &per_split) {
     const int tiles = pl.m_tiles * pl.n_tiles;
-    int want = sm_target() / tiles;
+    int want = launch_sms() / tiles;
     if (want < 1) want = 1;
     if (want > g.B) want = g.B;
     per_split = (g.B + want - 1) / want;
@@ -1944,66 +2022,85 @@ static bool encode_nhwc(CUtensorMap *map, int dtype, const void *base, int C, in
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY, const ConvGeom &g_in, float *G_w,
-                         float *partial, int slots, const float *factor, float *acc_w, void *tc_workspace, int *status,
-                         cudaStream_t stream, bool second_pass, const TcInlineClip *inline_clip, const TcPublish *publish) {
-    const bool clip = epilogue == DP_EPI_CLIP_ACCUM;
-    const ConvGeom &g0 = g_in;
-    const TcProblem pr = tc_problem(dtype, g0);
-    if (!pr.ok || !encode_fn()) return DP_ERR_UNSUPPORTED;
-    const ConvGeom &g = pr.eff;
-    const TcPlan pl = make_plan(dtype, g, clip ? 2 : (epilogue == DP_EPI_STORE_NORM ? 0 : 1));
-    if (!pl.ok) return DP_ERR_UNSUPPORTED;
-    char *ws_bytes = static_cast<char *>(tc_workspace);
-    if (pr.unfold) {
-        // in a fused clip call this function runs twice (norm pass, then clipped-sum pass): the unfolded input is
-        // rebuilt only by the first of them
-        if (!(clip && second_pass)) {
-            const int vec = (dtype == DP_BF16) ? 8 : 4;
-            const long long total = (long long)g0.B * g0.OH * g0.OW * (pr.n_pad / vec);
-            const unsigned blocks = (unsigned)((total + 255) / 256);
-            const size_t row_smem = unfold_rows_smem(dtype, g0);
-            if (unfold_rows_ok(dtype, g0, pr.n_pad)) {
-                const dim3 grid_rows(g0.OH, g0.B);
-                if (dtype == DP_BF16)
-                    unfold_rows_kernel<__nv_bfloat16, 8><<<grid_rows, 256, row_smem, stream>>>(
-                        static_cast<const __nv_bfloat16 *>(X), reinterpret_cast<__nv_bfloat16 *>(ws_bytes), g0, pr.n_pad);
-                else
-                    unfold_rows_kernel<float, 4><<<grid_rows, 256, row_smem, stream>>>(
-                        static_cast<const float *>(X), reinterpret_cast<float *>(ws_bytes), g0, pr.n_pad);
-            } else if (dtype == DP_BF16)
-                unfold_small_channels_kernel<__nv_bfloat16, 8><<<blocks, 256, 0, stream>>>(
-                    static_cast<const __nv_bfloat16 *>(X), reinterpret_cast<__nv_bfloat16 *>(ws_bytes), g0, pr.n_pad, total);
-            else
-                unfold_small_channels_kernel<float, 4><<<blocks, 256, 0, stream>>>(
-                    static_cast<const float *>(X), reinterpret_cast<float *>(ws_bytes), g0, pr.n_pad, total);
-            DP_LAUNCH_CHECK("unfold_small_channels_kernel");
-        }
-        X = ws_bytes;
-    }
-    float *part_ws = reinterpret_cast<float *>(ws_bytes + unfold_bytes(dtype, g0, pr));
-    CUtensorMap tmX, tmY;
-    if (!encode_nhwc(&tmX, dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&tmY, dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
-    TcParams p;
-    p.B = g.B; p.Kout = g.Kout; p.Ng = g0.N; p.Cin = g.Cin; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
-    p.n_pad_cols = (g.N != g0.N) ? 1 : 0;
+typedef TcEntry<TcParams, 2> ConvEntry;
+typedef TcEntry<TcParams, 3> SsumEntry;
+typedef TcEntry<GramParams, 2> GramEntry;
+static_assert(sizeof(TcTable<TcParams, 3, kSsumLayers>) <= 32000 && sizeof(TcTable<TcParams, 2, kTcLayers>) <= 32000, "kernel parameters are limited to 32764 bytes");
+
+template <typename K>
+static cudaError_t allow_shared(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
+}
+// Raised once per process, for every form of the kernels at once.
+static dp_status raise_shared_limits() {
+    static std::once_flag once;
+    static cudaError_t err = cudaSuccess;
+    std::call_once(once, [] {
+        const cudaError_t all[] = {
+            allow_shared(conv_wgrad_tc_kernel<false, false, 1>), allow_shared(conv_wgrad_tc_kernel<false, true, 1>),
+            allow_shared(conv_wgrad_tc_kernel<true, false, 1>), allow_shared(conv_wgrad_tc_kernel<true, true, 1>),
+            allow_shared(conv_wgrad_tc_kernel<false, false, kTcLayers>), allow_shared(conv_wgrad_tc_kernel<true, false, kTcLayers>),
+            allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
+            allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>),
+            allow_shared(conv_gram_norm_kernel<1>), allow_shared(conv_gram_norm_kernel<kTcLayers>)};
+        for (cudaError_t e : all)
+            if (e != cudaSuccess && err == cudaSuccess) err = e;
+    });
+    return err == cudaSuccess ? DP_OK : cuda_fail(err, "cudaFuncSetAttribute");
+}
+
+// what the parameters of every kernel take from the layer and its plan
+static void fill_common(TcParams &p, int dtype, const ConvGeom &g, int Ng, const TcPlan &pl, int *status) {
+    p.B = g.B; p.Kout = g.Kout; p.Ng = Ng; p.Cin = g.Cin; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
+    p.n_pad_cols = (g.N != Ng) ? 1 : 0;
     p.slab_ch = (dtype == DP_BF16) ? 64 : 32; p.krows = (dtype == DP_BF16) ? 16 : 8;
     p.a_is_x = pl.a_is_x; p.a_ext = pl.a_ext; p.b_ext = pl.b_ext; p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.NT = pl.NT;
     p.OWt = pl.OWt; p.OHt = pl.OHt; p.tiles_w = pl.tiles_w; p.Kt = pl.Kt; p.k_tiles = pl.k_tiles;
     p.stages = pl.stages; p.stage_bytes = pl.stage_bytes; p.a_bytes = pl.a_bytes;
+    p.status = status;
+    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
+}
+
+// Layers with few input channels: the unfolded copy of X in the call's scratch.
+static dp_status unfold_input(int dtype, const void *X, const ConvGeom &g0, const TcProblem &pr, void *dst, cudaStream_t stream) {
+    const int vec = (dtype == DP_BF16) ? 8 : 4;
+    const long long total = (long long)g0.B * g0.OH * g0.OW * (pr.n_pad / vec);
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    const size_t row_smem = unfold_rows_smem(dtype, g0);
+    if (unfold_rows_ok(dtype, g0, pr.n_pad)) {
+        const dim3 grid_rows(g0.OH, g0.B);
+        if (dtype == DP_BF16)
+            unfold_rows_kernel<__nv_bfloat16, 8><<<grid_rows, 256, row_smem, stream>>>(
+                static_cast<const __nv_bfloat16 *>(X), static_cast<__nv_bfloat16 *>(dst), g0, pr.n_pad);
+        else
+            unfold_rows_kernel<float, 4><<<grid_rows, 256, row_smem, stream>>>(
+                static_cast<const float *>(X), static_cast<float *>(dst), g0, pr.n_pad);
+    } else if (dtype == DP_BF16)
+        unfold_small_channels_kernel<__nv_bfloat16, 8><<<blocks, 256, 0, stream>>>(
+            static_cast<const __nv_bfloat16 *>(X), static_cast<__nv_bfloat16 *>(dst), g0, pr.n_pad, total);
+    else
+        unfold_small_channels_kernel<float, 4><<<blocks, 256, 0, stream>>>(
+            static_cast<const float *>(X), static_cast<float *>(dst), g0, pr.n_pad, total);
+    DP_LAUNCH_CHECK("unfold_small_channels_kernel");
+    return DP_OK;
+}
+
+// Parameters of the norm / store / two-pass clipped-sum kernel for one layer; X already unfolded where the layer needs it.
+static dp_status fill_conv_tc(int dtype, int epilogue, const void *X, const void *dY, const ConvGeom &g0, const TcProblem &pr,
+                              const TcPlan &pl, float *G_w, float *partial, int slots, const float *factor, float *acc_w,
+                              void *tc_workspace, int *status, const TcPublish *publish, ConvEntry &e) {
+    const bool clip = epilogue == DP_EPI_CLIP_ACCUM;
+    const ConvGeom &g = pr.eff;
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    TcParams &p = e.p;
+    p = TcParams{};
+    fill_common(p, dtype, g, g0.N, pl, status);
     p.lo_offset = pl.stage_bytes / 2;
     p.single_pass = (dtype == DP_TF32) ? 1 : 0;
     p.mode = clip ? 2 : (epilogue == DP_EPI_STORE_NORM ? 0 : 1);
-    p.G_w = G_w; p.partial = partial; p.slots = slots; p.status = status;
-    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
+    p.G_w = G_w; p.partial = partial; p.slots = slots;
     p.splits = 1; p.per_split = g.B; p.factor = factor; p.sum_out = acc_w;
-    p.inline_factor = (clip && inline_clip) ? 1 : 0;
-    p.C_l = inline_clip ? inline_clip->C_l : 0.f;
-    p.sqnorm = inline_clip ? inline_clip->sqnorm : nullptr;
-    p.sq_stride = inline_clip ? inline_clip->sq_stride : 0;
-    p.clip_out = inline_clip ? inline_clip->clip_out : nullptr;
-    p.counters = nullptr; p.w_slots = 0; p.separate = 0; p.factor_out = nullptr;
     if (!clip && publish) {
         p.counters = publish->counters; p.w_slots = publish->w_slots; p.separate = publish->separate;
         p.sqnorm = publish->sqnorm; p.sq_stride = publish->sq_stride;
@@ -2011,28 +2108,43 @@ dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY,
     }
     if (clip) {
         clip_split(g, pl, p.splits, p.per_split);
-        if (p.splits > 1) p.sum_out = part_ws;
+        if (p.splits > 1) p.sum_out = reinterpret_cast<float *>(static_cast<char *>(tc_workspace) + unfold_bytes(dtype, g0, pr));
         p.total_tiles = p.splits * pl.m_tiles * pl.n_tiles;
     } else {
         p.total_tiles = g.B * pl.m_tiles * pl.n_tiles;
     }
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        const int bytes = kSmemBudget + 2048;
-        attr_err = cudaFuncSetAttribute(conv_wgrad_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (attr_err == cudaSuccess) attr_err = cudaFuncSetAttribute(conv_wgrad_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (attr_err == cudaSuccess) attr_err = cudaFuncSetAttribute(conv_wgrad_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (attr_err == cudaSuccess) attr_err = cudaFuncSetAttribute(conv_wgrad_tc_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    });
-    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
-    const unsigned grid = (unsigned)std::min(p.total_tiles, sm_target());
+    return DP_OK;
+}
+
+dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY, const ConvGeom &g0, float *G_w,
+                         float *partial, int slots, const float *factor, float *acc_w, void *tc_workspace, int *status,
+                         cudaStream_t stream, bool second_pass, const TcPublish *publish) {
+    const bool clip = epilogue == DP_EPI_CLIP_ACCUM;
+    const TcProblem pr = tc_problem(dtype, g0);
+    if (!pr.ok || !encode_fn()) return DP_ERR_UNSUPPORTED;
+    const TcPlan pl = make_plan(dtype, pr.eff, clip ? 2 : (epilogue == DP_EPI_STORE_NORM ? 0 : 1));
+    if (!pl.ok) return DP_ERR_UNSUPPORTED;
+    dp_status rc = raise_shared_limits();
+    if (rc != DP_OK) return rc;
+    if (pr.unfold) {
+        // in a fused clip call this function runs twice (norm pass, then clipped-sum pass): the unfolded input is
+        // rebuilt only by the first of them
+        if (!(clip && second_pass) && (rc = unfold_input(dtype, X, g0, pr, tc_workspace, stream)) != DP_OK) return rc;
+        X = tc_workspace;
+    }
+    TcTable<TcParams, 2, 1> tab;
+    tab.n = 1; tab.first[0] = 0;
+    rc = fill_conv_tc(dtype, epilogue, X, dY, g0, pr, pl, G_w, partial, slots, factor, acc_w, tc_workspace, status, publish, tab.e[0]);
+    if (rc != DP_OK) return rc;
+    TcParams &p = tab.e[0].p;
+    p.blocks = std::min(p.total_tiles, sm_target());
+    const unsigned grid = (unsigned)p.blocks;
     if (dtype == DP_BF16) {
-        if (clip) conv_wgrad_tc_kernel<false, true><<<grid, 224, pl.smem, stream>>>(tmX, tmY, p);
-        else conv_wgrad_tc_kernel<false, false><<<grid, 224, pl.smem, stream>>>(tmX, tmY, p);
+        if (clip) conv_wgrad_tc_kernel<false, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        else conv_wgrad_tc_kernel<false, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
     } else {
-        if (clip) conv_wgrad_tc_kernel<true, true><<<grid, 480, pl.smem, stream>>>(tmX, tmY, p);
-        else conv_wgrad_tc_kernel<true, false><<<grid, 480, pl.smem, stream>>>(tmX, tmY, p);
+        if (clip) conv_wgrad_tc_kernel<true, true, 1><<<grid, 480, pl.smem, stream>>>(tab);
+        else conv_wgrad_tc_kernel<true, false, 1><<<grid, 480, pl.smem, stream>>>(tab);
     }
     DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
     if (clip && p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g0.M * g0.N, acc_w, stream);
@@ -2045,44 +2157,50 @@ bool tc_clip_scaled_sum(int dtype, const ConvGeom &g0) {
     return dtype == DP_BF16 && pr.ok && !pr.unfold && encode_fn() && g0.Kout % 8 == 0 && make_plan(dtype, pr.eff, 4).ok;
 }
 
+// hi and lo copies of f_n * dY in the call's scratch, partial sums (if any) behind them
+static dp_status fill_ssum(int dtype, const void *X, const ConvGeom &g, const TcPlan &pl, float *acc_w, void *tc_workspace,
+                           int *status, SsumEntry &e) {
+    char *ws_bytes = static_cast<char *>(tc_workspace);
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, ws_bytes, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY hi)");
+    if (!encode_nhwc(&e.map[2], dtype, ws_bytes + ssum_copy_bytes(g), g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY lo)");
+    TcParams &p = e.p;
+    p = TcParams{};
+    fill_common(p, dtype, g, g.N, pl, status);
+    p.lo_offset = pl.a_bytes + (pl.NT / 64) * pl.Kt * kRowBytes;      // after the A and B slabs
+    p.mode = 2;                                                       // items are (example range, tile) pairs
+    ssum_split(g.B, pl.m_tiles * pl.n_tiles, p.splits, p.per_split);
+    p.sum_out = p.splits > 1 ? reinterpret_cast<float *>(ws_bytes + 2 * ssum_copy_bytes(g)) : acc_w;
+    p.total_tiles = p.splits * pl.m_tiles * pl.n_tiles;
+    return DP_OK;
+}
+
+static SplitSeg split_seg(const void *dY, const float *factor, const ConvGeom &g, void *tc_workspace) {
+    SplitSeg s;
+    s.y = static_cast<const __nv_bfloat16 *>(dY); s.factor = factor;
+    s.per_example = (long long)g.OH * g.OW * g.Kout; s.total8 = s.per_example * g.B / 8;
+    s.hi = static_cast<__nv_bfloat16 *>(tc_workspace);
+    s.lo = reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(tc_workspace) + ssum_copy_bytes(g));
+    return s;
+}
+
 dp_status launch_conv_ssum(int dtype, const void *X, const void *dY, const ConvGeom &g0, const float *factor, float *acc_w,
                            void *tc_workspace, int *status, cudaStream_t stream) {
     if (!tc_clip_scaled_sum(dtype, g0)) return DP_ERR_UNSUPPORTED;
+    dp_status rc = raise_shared_limits();
+    if (rc != DP_OK) return rc;
     const TcProblem pr = tc_problem(dtype, g0);
     const ConvGeom &g = pr.eff;
     const TcPlan pl = make_plan(dtype, g, 4);
-    char *ws_bytes = static_cast<char *>(tc_workspace);
-    __nv_bfloat16 *hi = reinterpret_cast<__nv_bfloat16 *>(ws_bytes), *lo = reinterpret_cast<__nv_bfloat16 *>(ws_bytes + ssum_copy_bytes(g));
-    float *part_ws = reinterpret_cast<float *>(ws_bytes + 2 * ssum_copy_bytes(g));
-    {
-        const long long per_example = (long long)g.OH * g.OW * g.Kout, total8 = per_example * g.B / 8;
-        scale_split_kernel<<<(unsigned)((total8 + 255) / 256), 256, 0, stream>>>(static_cast<const __nv_bfloat16 *>(dY), factor, per_example, total8, hi, lo);
-        DP_LAUNCH_CHECK("scale_split_kernel");
-    }
-    CUtensorMap tmX, tmYhi, tmYlo;
-    if (!encode_nhwc(&tmX, dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&tmYhi, dtype, hi, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY hi)");
-    if (!encode_nhwc(&tmYlo, dtype, lo, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY lo)");
-    TcParams p = {};
-    p.B = g.B; p.Kout = g.Kout; p.Ng = g.N; p.Cin = g.Cin; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
-    p.slab_ch = 64; p.krows = 16;
-    p.a_is_x = pl.a_is_x; p.a_ext = pl.a_ext; p.b_ext = pl.b_ext; p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.NT = pl.NT;
-    p.OWt = pl.OWt; p.OHt = pl.OHt; p.tiles_w = pl.tiles_w; p.Kt = pl.Kt; p.k_tiles = pl.k_tiles;
-    p.stages = pl.stages; p.stage_bytes = pl.stage_bytes; p.a_bytes = pl.a_bytes;
-    p.lo_offset = pl.a_bytes + (pl.NT / 64) * pl.Kt * kRowBytes;      // after the A and B slabs
-    p.mode = 2; p.status = status;                                    // items are (example range, tile) pairs
-    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
-    ssum_split(g.B, pl.m_tiles * pl.n_tiles, p.splits, p.per_split);
-    p.sum_out = p.splits > 1 ? part_ws : acc_w;
-    p.total_tiles = p.splits * pl.m_tiles * pl.n_tiles;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(conv_wgrad_ssum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-    });
-    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
-    const unsigned grid = (unsigned)std::min(p.total_tiles, sm_target());
-    conv_wgrad_ssum_kernel<<<grid, 224, pl.smem, stream>>>(tmX, tmYhi, tmYlo, p);
+    rc = launch_scale_split({split_seg(dY, factor, g, tc_workspace)}, stream);
+    if (rc != DP_OK) return rc;
+    TcTable<TcParams, 3, 1> tab;
+    tab.n = 1; tab.first[0] = 0;
+    rc = fill_ssum(dtype, X, g, pl, acc_w, tc_workspace, status, tab.e[0]);
+    if (rc != DP_OK) return rc;
+    TcParams &p = tab.e[0].p;
+    p.blocks = std::min(p.total_tiles, sm_target());
+    conv_wgrad_ssum_kernel<1><<<(unsigned)p.blocks, 224, pl.smem, stream>>>(tab);
     DP_LAUNCH_CHECK("conv_wgrad_ssum_kernel");
     if (p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g.M * g.N, acc_w, stream);
     return DP_OK;
@@ -2103,34 +2221,34 @@ static void scaled_tiles_split(const ConvGeom &g, const TcPlan &pl, int &splits,
     cluster_split(g.B, pl.m_tiles * pl.n_tiles, g.K, pl.NT, splits, per);
 }
 
+static dp_status fill_scaled_tiles(int dtype, const void *X, const void *dY, const ConvGeom &g, const TcPlan &pl,
+                                   const float *factor, float *acc_w, void *tc_workspace, int *status, ConvEntry &e) {
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    TcParams &p = e.p;
+    p = TcParams{};
+    fill_common(p, dtype, g, g.N, pl, status);
+    p.mode = 3; p.factor = factor; p.cluster = 1;
+    scaled_tiles_split(g, pl, p.splits, p.per_split);
+    p.sum_out = p.splits > 1 ? static_cast<float *>(tc_workspace) : acc_w;
+    p.total_tiles = p.blocks = p.splits * pl.m_tiles * pl.n_tiles;
+    return DP_OK;
+}
+
 dp_status launch_conv_scaled_tiles(int dtype, const void *X, const void *dY, const ConvGeom &g0, const float *factor, float *acc_w,
                                    void *tc_workspace, int *status, cudaStream_t stream) {
     if (!tc_clip_scaled_tiles(dtype, g0)) return DP_ERR_UNSUPPORTED;
+    dp_status rc = raise_shared_limits();
+    if (rc != DP_OK) return rc;
     const TcProblem pr = tc_problem(dtype, g0);
     const ConvGeom &g = pr.eff;
     const TcPlan pl = make_plan(dtype, g, 7);
-    CUtensorMap tmX, tmY;
-    if (!encode_nhwc(&tmX, dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&tmY, dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
-    TcParams p = {};
-    p.B = g.B; p.Kout = g.Kout; p.Ng = g.N; p.Cin = g.Cin; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
-    p.slab_ch = 64; p.krows = 16;
-    p.a_is_x = pl.a_is_x; p.a_ext = pl.a_ext; p.b_ext = pl.b_ext; p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.NT = pl.NT;
-    p.OWt = pl.OWt; p.OHt = pl.OHt; p.tiles_w = pl.tiles_w; p.Kt = pl.Kt; p.k_tiles = pl.k_tiles;
-    p.stages = pl.stages; p.stage_bytes = pl.stage_bytes; p.a_bytes = pl.a_bytes;
-    p.mode = 3; p.status = status; p.factor = factor;
-    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
-    const int tiles = pl.m_tiles * pl.n_tiles;
-    scaled_tiles_split(g, pl, p.splits, p.per_split);
-    p.sum_out = p.splits > 1 ? static_cast<float *>(tc_workspace) : acc_w;
-    p.total_tiles = p.splits * tiles;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(conv_wgrad_clip1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-    });
-    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
-    conv_wgrad_clip1_kernel<<<(unsigned)p.total_tiles, kClipThreads, pl.smem, stream>>>(tmX, tmY, p);
+    TcTable<TcParams, 2, 1> tab;
+    tab.n = 1; tab.first[0] = 0;
+    rc = fill_scaled_tiles(dtype, X, dY, g, pl, factor, acc_w, tc_workspace, status, tab.e[0]);
+    if (rc != DP_OK) return rc;
+    const TcParams &p = tab.e[0].p;
+    conv_wgrad_clip1_kernel<1><<<(unsigned)p.total_tiles, kClipThreads, pl.smem, stream>>>(tab);
     DP_LAUNCH_CHECK("conv_wgrad_clip1_kernel");
     if (p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g.M * g.N, acc_w, stream);
     return DP_OK;
@@ -2178,28 +2296,33 @@ static int gram_describe(int dtype, const ConvGeom &g0, int *out, int n) {
     return 12;
 }
 
-dp_status launch_conv_gram_norm(int dtype, const void *X, const void *dY, const ConvGeom &g0, const TcInlineClip &clipinfo,
-                                float *factor_out, int *status, cudaStream_t stream) {
-    const GramPlan gp = gram_plan(dtype, g0);
-    if (!gp.ok) return DP_ERR_UNSUPPORTED;
+static dp_status fill_gram(int dtype, const void *X, const void *dY, const GramPlan &gp, const TcInlineClip &clipinfo,
+                           float *factor_out, int *status, GramEntry &e) {
     const ConvGeom &g = gp.g;
-    CUtensorMap tmX, tmY;
-    if (!encode_nhwc(&tmX, dtype, X, g.Cin, g.W, g.H, g.B, gp.OWb, gp.OHb, g.stride, gp.pack)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&tmY, dtype, dY, g.Kout, g.OW, g.OH, g.B, gp.OWb, gp.OHb, 1, gp.pack)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
-    GramParams p = {};
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, gp.OWb, gp.OHb, g.stride, gp.pack)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, gp.OWb, gp.OHb, 1, gp.pack)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    GramParams &p = e.p;
+    p = GramParams{};
     p.B = g.B; p.Cin = g.Cin; p.Kout = g.Kout; p.S = g.S; p.taps = g.R * g.S; p.stride = g.stride; p.pad = g.pad;
     p.rows = gp.rows; p.pack = gp.pack; p.m_tiles = gp.m_tiles; p.stages = gp.stages; p.stage_bytes = gp.stage_bytes;
     p.C_l = clipinfo.C_l; p.sqnorm = clipinfo.sqnorm; p.sq_stride = clipinfo.sq_stride; p.clip_out = clipinfo.clip_out;
     p.factor_out = factor_out; p.status = status;
     p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(conv_gram_norm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-    });
-    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
-    const unsigned grid = (unsigned)std::min((g.B + gp.pack - 1) / gp.pack, sm_target());
-    conv_gram_norm_kernel<<<grid, 192, gp.smem, stream>>>(tmX, tmY, p);
+    p.blocks = std::min((g.B + gp.pack - 1) / gp.pack, launch_sms());
+    return DP_OK;
+}
+
+dp_status launch_conv_gram_norm(int dtype, const void *X, const void *dY, const ConvGeom &g0, const TcInlineClip &clipinfo,
+                                float *factor_out, int *status, cudaStream_t stream) {
+    const GramPlan gp = gram_plan(dtype, g0);
+    if (!gp.ok) return DP_ERR_UNSUPPORTED;
+    dp_status rc = raise_shared_limits();
+    if (rc != DP_OK) return rc;
+    TcTable<GramParams, 2, 1> tab;
+    tab.n = 1; tab.first[0] = 0;
+    rc = fill_gram(dtype, X, dY, gp, clipinfo, factor_out, status, tab.e[0]);
+    if (rc != DP_OK) return rc;
+    conv_gram_norm_kernel<1><<<(unsigned)tab.e[0].p.blocks, 192, gp.smem, stream>>>(tab);
     DP_LAUNCH_CHECK("conv_gram_norm_kernel");
     return DP_OK;
 }
@@ -2210,75 +2333,261 @@ bool tc_clip_single_pass(int dtype, const ConvGeom &g0) {
     return pr.ok && encode_fn() && clip1_plan(dtype, g0, pr, pl, g, s2d) && clip1_registers_ok();
 }
 
-dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g0, float *partial, int slots,
-                            const TcInlineClip &clipinfo, float *acc_w, void *tc_workspace, int *status, cudaStream_t stream) {
-    (void)partial; (void)slots;
-    const TcProblem pr = tc_problem(dtype, g0);
-    TcPlan pl; ConvGeom g; bool s2d;
-    if (!pr.ok || !encode_fn() || !clip1_plan(dtype, g0, pr, pl, g, s2d) || !clip1_registers_ok()) return DP_ERR_UNSUPPORTED;
-    char *ws_bytes = static_cast<char *>(tc_workspace);
-    CUtensorMap tmX, tmY;
+// The input as the single-pass kernel reads it: X itself, or its space-to-depth / unfolded copy written to the scratch.
+static dp_status prepare_clip1(int dtype, const void *X, const ConvGeom &g0, const TcProblem &pr, bool s2d, void *tc_workspace,
+                               cudaStream_t stream) {
     if (s2d) {
         const S2dProblem sp = s2d_problem(dtype, g0, pr);
         const long long total = (long long)g0.B * sp.Hs * sp.Ws;
         space_to_depth_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(
-            static_cast<const __nv_bfloat16 *>(X), reinterpret_cast<__nv_bfloat16 *>(ws_bytes), g0, sp.Hs, sp.Ws, total);
+            static_cast<const __nv_bfloat16 *>(X), static_cast<__nv_bfloat16 *>(tc_workspace), g0, sp.Hs, sp.Ws, total);
         DP_LAUNCH_CHECK("space_to_depth_kernel");
+        return DP_OK;
+    }
+    return pr.unfold ? unfold_input(dtype, X, g0, pr, tc_workspace, stream) : DP_OK;
+}
+
+static dp_status fill_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g0, const TcProblem &pr, const ConvGeom &g,
+                            const TcPlan &pl, bool s2d, const TcInlineClip &clipinfo, float *acc_w, void *tc_workspace, int *status,
+                            ConvEntry &e) {
+    char *ws_bytes = static_cast<char *>(tc_workspace);
+    if (s2d) {
+        const S2dProblem sp = s2d_problem(dtype, g0, pr);
         // one operand row per output pixel: 64 values from pixel ow on, pixels 16 values apart
         const cuuint64_t dims[4] = {64, (cuuint64_t)g.OW, (cuuint64_t)sp.Hs, (cuuint64_t)g.B};
         const cuuint64_t strides[3] = {32, (cuuint64_t)sp.Ws * 32, (cuuint64_t)sp.Hs * sp.Ws * 32};
         const cuuint32_t box[4] = {64, (cuuint32_t)pl.OWt, (cuuint32_t)pl.OHt, 1};
         const cuuint32_t estr[4] = {1, 1, 1, 1};
-        if (encode_fn()(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, ws_bytes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (encode_fn()(&e.map[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, ws_bytes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(space-to-depth X)");
-    } else if (pr.unfold) {
-        if (unfold_rows_ok(dtype, g0, pr.n_pad)) {
-            unfold_rows_kernel<__nv_bfloat16, 8><<<dim3(g0.OH, g0.B), 256, unfold_rows_smem(dtype, g0), stream>>>(
-                static_cast<const __nv_bfloat16 *>(X), reinterpret_cast<__nv_bfloat16 *>(ws_bytes), g0, pr.n_pad);
-        } else {
-            const long long total = (long long)g0.B * g0.OH * g0.OW * (pr.n_pad / 8);
-            unfold_small_channels_kernel<__nv_bfloat16, 8><<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(
-                static_cast<const __nv_bfloat16 *>(X), reinterpret_cast<__nv_bfloat16 *>(ws_bytes), g0, pr.n_pad, total);
-        }
-        DP_LAUNCH_CHECK("unfold_small_channels_kernel");
-        X = ws_bytes;
+    } else if (!encode_nhwc(&e.map[0], dtype, pr.unfold ? tc_workspace : X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) {
+        return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
     }
-    float *part_ws = reinterpret_cast<float *>(ws_bytes + unfold_bytes(dtype, g0, pr));
-    if (!s2d && !encode_nhwc(&tmX, dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&tmY, dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
-    TcParams p = {};
-    p.B = g.B; p.Kout = g.Kout; p.Ng = g0.N; p.Cin = g.Cin; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
-    p.n_pad_cols = (g.N != g0.N) ? 1 : 0;
-    p.slab_ch = 64; p.krows = 16;
-    p.a_is_x = pl.a_is_x; p.a_ext = pl.a_ext; p.b_ext = pl.b_ext; p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.NT = pl.NT;
-    p.OWt = pl.OWt; p.OHt = pl.OHt; p.tiles_w = pl.tiles_w; p.Kt = pl.Kt; p.k_tiles = pl.k_tiles;
-    p.stages = pl.stages; p.stage_bytes = pl.stage_bytes; p.a_bytes = pl.a_bytes;
-    p.mode = 3; p.status = status;
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    TcParams &p = e.p;
+    p = TcParams{};
+    fill_common(p, dtype, g, g0.N, pl, status);
+    p.mode = 3;
     if (s2d) { p.s2d_st = g0.stride; p.s2d_R = g0.R; p.s2d_S = g0.S; p.s2d_Cin = g0.Cin; }
-    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
     p.C_l = clipinfo.C_l; p.sqnorm = clipinfo.sqnorm; p.sq_stride = clipinfo.sq_stride; p.clip_out = clipinfo.clip_out;
-    const int cs = pl.m_tiles * pl.n_tiles;
-    cluster_split(g.B, cs, g.K, pl.NT, p.splits, p.per_split);
-    p.sum_out = p.splits > 1 ? part_ws : acc_w;
-    p.total_tiles = p.splits * cs;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(conv_wgrad_clip1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
-    });
-    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
+    p.cluster = pl.m_tiles * pl.n_tiles;
+    cluster_split(g.B, p.cluster, g.K, pl.NT, p.splits, p.per_split);
+    p.sum_out = p.splits > 1 ? reinterpret_cast<float *>(ws_bytes + unfold_bytes(dtype, g0, pr)) : acc_w;
+    p.total_tiles = p.blocks = p.splits * p.cluster;
+    return DP_OK;
+}
+
+template <int N>
+static dp_status launch_clip1_table(const TcTable<TcParams, 2, N> &tab, int cluster, int blocks, size_t smem, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(p.splits * cs)); cfg.blockDim = dim3(kClipThreads); cfg.dynamicSmemBytes = pl.smem; cfg.stream = stream;
+    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(kClipThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_clip1_kernel, tmX, tmY, p);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_clip1_kernel<N>, tab);
     if (le != cudaSuccess) return cuda_fail(le, "conv_wgrad_clip1_kernel");
     DP_LAUNCH_CHECK("conv_wgrad_clip1_kernel");
+    return DP_OK;
+}
+
+dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g0, const TcInlineClip &clipinfo,
+                            float *acc_w, void *tc_workspace, int *status, cudaStream_t stream) {
+    const TcProblem pr = tc_problem(dtype, g0);
+    TcPlan pl; ConvGeom g; bool s2d;
+    if (!pr.ok || !encode_fn() || !clip1_plan(dtype, g0, pr, pl, g, s2d) || !clip1_registers_ok()) return DP_ERR_UNSUPPORTED;
+    dp_status rc = raise_shared_limits();
+    if (rc == DP_OK) rc = prepare_clip1(dtype, X, g0, pr, s2d, tc_workspace, stream);
+    if (rc != DP_OK) return rc;
+    TcTable<TcParams, 2, 1> tab;
+    tab.n = 1; tab.first[0] = 0;
+    rc = fill_clip1(dtype, X, dY, g0, pr, g, pl, s2d, clipinfo, acc_w, tc_workspace, status, tab.e[0]);
+    if (rc != DP_OK) return rc;
+    const TcParams &p = tab.e[0].p;
+    rc = launch_clip1_table<1>(tab, p.cluster, p.blocks, pl.smem, stream);
+    if (rc != DP_OK) return rc;
     if (p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g0.M * g0.N, acc_w, stream);
     return DP_OK;
+}
+
+// ----------------------------------------------------------------------------- batches of layer calls
+// Layers of one kind share a launch.  What a layer needs is cut into blocks that each hold an SM for some tens of
+// microseconds; the blocks of all layers queue up behind one another, longest first, so that the GPU stays full until
+// the last few of them, whatever the size of a single layer.
+int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias) {
+    if (epilogue != DP_EPI_CLIP_ACCUM) return kConvTc;
+    if (has_bias || !single_pass_enabled()) return kConvSingle;
+    if (tc_clip_single_pass(dtype, g)) return kConvClip1;
+    if (tc_clip_scaled_sum(dtype, g) && tc_gram_norm(dtype, g)) return tc_clip_scaled_tiles(dtype, g) ? kConvGramTiles : kConvGramSum;
+    return kConvSingle;
+}
+
+// The longest walk of a block: a third of the GPU's share of all the layers' work (so that the blocks can be spread
+// evenly), within 8 and 60 microseconds (a block costs some 3 to start and end).
+double conv_batch_walk(const std::vector<ConvJob> &jobs) {
+    BatchPlanning planning(120000.0);
+    double cycles = 0.0;
+    for (const ConvJob &j : jobs) {
+        const TcProblem pr = tc_problem(j.dtype, j.g);
+        TcPlan pl; ConvGeom g = pr.eff; bool s2d;
+        if (j.kind == kConvTc) pl = make_plan(j.dtype, g, j.epi == DP_EPI_STORE_NORM ? 0 : 1);
+        else if (j.kind == kConvClip1) clip1_plan(j.dtype, j.g, pr, pl, g, s2d);
+        else if (j.kind == kConvGramTiles) pl = make_plan(j.dtype, g, 7);
+        else continue;
+        cycles += pl.item_cycles * j.g.B * pl.m_tiles * pl.n_tiles;
+    }
+    double walk = 15000.0;
+    while (walk * 2.0 <= std::min(120000.0, cycles / sm_count() / 3.0)) walk *= 2.0;
+    return walk;
+}
+
+template <typename P, int MAPS, int N>
+struct TableQueue {
+    // jobs of one kernel: filled entries with the blocks they take, launched longest blocks first, N layers at a time
+    struct Job { TcEntry<P, MAPS> e; int blocks; size_t smem; double cost; };
+    std::vector<Job> jobs;
+    template <typename F>
+    dp_status launch(F &&go) {
+        std::stable_sort(jobs.begin(), jobs.end(), [](const Job &a, const Job &b) { return a.cost > b.cost; });
+        for (size_t i = 0; i < jobs.size();) {
+            std::unique_ptr<TcTable<P, MAPS, N>> tab(new TcTable<P, MAPS, N>);
+            int blocks = 0;
+            size_t smem = 0;
+            for (tab->n = 0; i < jobs.size() && tab->n < N; ++i) {
+                tab->first[tab->n] = blocks;
+                tab->e[tab->n++] = jobs[i].e;
+                blocks += jobs[i].blocks;
+                smem = std::max(smem, jobs[i].smem);
+            }
+            const dp_status rc = go(*tab, blocks, smem);
+            if (rc != DP_OK) return rc;
+        }
+        return DP_OK;
+    }
+};
+typedef TableQueue<TcParams, 2, kTcLayers> ConvQueue;
+typedef TableQueue<TcParams, 3, kSsumLayers> SsumQueue;
+typedef TableQueue<GramParams, 2, kTcLayers> GramQueue;
+
+// Cluster size of the launch a layer with `tiles` tiles an example joins: sizes that divide one another share one.
+static int launch_cluster(int tiles) { return tiles == 1 || tiles == 2 || tiles == 4 ? 4 : (tiles == 3 || tiles == 6 ? 6 : tiles); }
+
+dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *status, const BatchStreams &streams,
+                            const std::function<dp_status()> &join) {
+    if (jobs.empty()) return join();
+    const cudaStream_t stream = streams.s[BatchStreams::kMain], clusters = streams.s[BatchStreams::kClusters], sums = streams.s[BatchStreams::kSums];
+    BatchPlanning planning(walk);
+    dp_status rc = raise_shared_limits();
+    if (rc != DP_OK) return rc;
+    ConvQueue store[2], clip[kMaxCluster + 1];            // store: bf16 / fp32; clip: by cluster size of the launch
+    GramQueue gram;
+    SsumQueue ssum;
+    std::vector<SplitSeg> splits;
+    std::vector<FoldSeg> folds;
+    for (const ConvJob &j : jobs) {
+        const TcProblem pr = tc_problem(j.dtype, j.g);
+        const ConvGeom &g = pr.eff;
+        const long long P = (long long)j.g.M * j.g.N;
+        if (j.kind == kConvTc) {
+            const TcPlan pl = make_plan(j.dtype, g, j.epi == DP_EPI_STORE_NORM ? 0 : 1);
+            if (!pl.ok) return DP_ERR_UNSUPPORTED;
+            const void *X = j.X;
+            if (pr.unfold) {
+                rc = unfold_input(j.dtype, X, j.g, pr, j.tc_workspace, stream);
+                if (rc != DP_OK) return rc;
+                X = j.tc_workspace;
+            }
+            const TcPublish pub = {j.counter, j.w_slots, j.separate, j.clip.sqnorm, j.clip.sq_stride, nullptr, 0.f, nullptr};
+            ConvQueue::Job q;
+            rc = fill_conv_tc(j.dtype, j.epi, X, j.dY, j.g, pr, pl, j.G_w, j.partial, j.slots, nullptr, nullptr, j.tc_workspace, status, &pub, q.e);
+            if (rc != DP_OK) return rc;
+            TcParams &p = q.e.p;
+            p.run = std::max(1, std::min(p.total_tiles, (int)(walk / pl.item_cycles)));
+            p.blocks = q.blocks = (p.total_tiles + p.run - 1) / p.run;
+            q.smem = pl.smem; q.cost = p.run * pl.item_cycles;
+            store[j.dtype == DP_BF16 ? 0 : 1].jobs.push_back(q);
+        } else if (j.kind == kConvClip1) {
+            TcPlan pl; ConvGeom g1; bool s2d;
+            if (!clip1_plan(j.dtype, j.g, pr, pl, g1, s2d)) return DP_ERR_UNSUPPORTED;
+            rc = prepare_clip1(j.dtype, j.X, j.g, pr, s2d, j.tc_workspace, launch_cluster(pl.m_tiles * pl.n_tiles) > 4 ? clusters : stream);
+            if (rc != DP_OK) return rc;
+            ConvQueue::Job q;
+            rc = fill_clip1(j.dtype, j.X, j.dY, j.g, pr, g1, pl, s2d, j.clip, j.acc_w, j.tc_workspace, status, q.e);
+            if (rc != DP_OK) return rc;
+            TcParams &p = q.e.p;
+            const int tiles = p.cluster, cluster = launch_cluster(tiles), sets = cluster / tiles;
+            p.cluster = cluster;
+            q.blocks = (p.splits + sets - 1) / sets * cluster;
+            q.smem = pl.smem; q.cost = p.per_split * pl.item_cycles;
+            if (p.splits > 1) folds.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+            clip[cluster].jobs.push_back(q);
+        } else {
+            const GramPlan gp = gram_plan(j.dtype, j.g);
+            if (!gp.ok) return DP_ERR_UNSUPPORTED;
+            GramQueue::Job q;
+            rc = fill_gram(j.dtype, j.X, j.dY, gp, j.clip, j.factor, status, q.e);
+            if (rc != DP_OK) return rc;
+            q.blocks = q.e.p.blocks; q.smem = gp.smem;
+            q.cost = (double)(g.Kout / 64 + g.R * g.S * (g.Cin / 64)) * gp.m_tiles * gp.rows;
+            gram.jobs.push_back(q);
+            if (j.kind == kConvGramTiles) {
+                const TcPlan pl = make_plan(j.dtype, g, 7);
+                ConvQueue::Job t;
+                rc = fill_scaled_tiles(j.dtype, j.X, j.dY, g, pl, j.factor, j.acc_w, j.tc_workspace, status, t.e);
+                if (rc != DP_OK) return rc;
+                const TcParams &p = t.e.p;
+                t.blocks = (p.blocks + 3) / 4 * 4;        // joins the launch of the smallest clusters; blocks past the last have no work
+                t.smem = pl.smem; t.cost = p.per_split * pl.item_cycles;
+                if (p.splits > 1) folds.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+                clip[4].jobs.push_back(t);
+            } else {
+                const TcPlan pl = make_plan(j.dtype, g, 4);
+                splits.push_back(split_seg(j.dY, j.factor, g, j.tc_workspace));
+                SsumQueue::Job t;
+                rc = fill_ssum(j.dtype, j.X, g, pl, j.acc_w, j.tc_workspace, status, t.e);
+                if (rc != DP_OK) return rc;
+                TcParams &p = t.e.p;
+                t.blocks = p.blocks = p.total_tiles;
+                t.smem = pl.smem; t.cost = p.per_split * pl.item_cycles;
+                if (p.splits > 1) folds.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+                ssum.jobs.push_back(t);
+            }
+        }
+    }
+    for (int f32 = 0; f32 < 2; ++f32) {
+        rc = store[f32].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
+            if (f32) conv_wgrad_tc_kernel<true, false, kTcLayers><<<(unsigned)blocks, 480, smem, stream>>>(tab);
+            else conv_wgrad_tc_kernel<false, false, kTcLayers><<<(unsigned)blocks, 224, smem, stream>>>(tab);
+            DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
+            return DP_OK;
+        });
+        if (rc != DP_OK) return rc;
+    }
+    rc = gram.launch([&](const TcTable<GramParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
+        conv_gram_norm_kernel<kTcLayers><<<(unsigned)blocks, 192, smem, stream>>>(tab);
+        DP_LAUNCH_CHECK("conv_gram_norm_kernel");
+        return DP_OK;
+    });
+    if (rc == DP_OK && streams.gram_done) {
+        DP_CUDA_TRY(cudaEventRecord(streams.gram_done, stream));
+        DP_CUDA_TRY(cudaStreamWaitEvent(sums, streams.gram_done, 0));
+    }
+    // larger clusters need all their SMs in one GPC and leave some idle: the other streams' launches fill those
+    for (int c = kMaxCluster; c >= 1 && rc == DP_OK; --c)
+        rc = clip[c].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) {
+            return launch_clip1_table<kTcLayers>(tab, c, blocks, smem, c > 4 ? clusters : stream);
+        });
+    if (rc == DP_OK) rc = launch_scale_split(splits, sums);
+    if (rc == DP_OK)
+        rc = ssum.launch([&](const TcTable<TcParams, 3, kSsumLayers> &tab, int blocks, size_t smem) -> dp_status {
+            conv_wgrad_ssum_kernel<kSsumLayers><<<(unsigned)blocks, 224, smem, sums>>>(tab);
+            DP_LAUNCH_CHECK("conv_wgrad_ssum_kernel");
+            return DP_OK;
+        });
+    if (rc == DP_OK) rc = join();
+    if (rc == DP_OK) rc = launch_folds(folds, stream);
+    return rc;
 }
 
 }  // namespace dp

@@ -1,6 +1,8 @@
 // Internal launch interface of the tcgen05 (5th-generation tensor core) per-example conv weight-gradient kernel.
 #pragma once
 #include "wgrad_simple.cuh"
+#include <functional>
+#include <vector>
 
 namespace dp {
 
@@ -10,11 +12,8 @@ bool tc_eligible(int dtype, const ConvGeom &g, int epilogue);
 int tc_norm_slots(int dtype, const ConvGeom &g, int epilogue);
 size_t tc_workspace_bytes(int dtype, const ConvGeom &g, int epilogue);
 // tiling chosen for the layer: {a_is_x, a_ext, b_ext, m_tiles, n_tiles, NT, OWt, OHt, Kt, k_tiles, stages, stage_bytes}
-// acc[i] += sum_s part[s][i] in index order of s (P a multiple of 4)
-dp_status launch_fold_partial_sums(const float *part, int splits, long long P, float *acc, cudaStream_t stream);
 int tc_describe_plan(int dtype, const ConvGeom &g, int epilogue, int *out, int n);
-// When given to a CLIP_ACCUM launch, the kernel derives each example's factor from the norm pass's partial sums
-// itself (threshold C_l) and writes sqnorm[n*sq_stride] and clip_out[n] (optional), so no finalising launch is needed.
+// What a fused clip publishes: factors against C_l, sqnorm[n*sq_stride] and clip_out[n] (optional).
 struct TcInlineClip { float C_l; float *sqnorm; long long sq_stride; float *clip_out; };
 
 // When given to a STORE_NORM / NORM_ONLY launch, the last CTA to finish folds every example's partial squared norms
@@ -27,14 +26,14 @@ struct TcPublish { int *counters; int w_slots; int separate; float *sqnorm; long
 dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY, const ConvGeom &g, float *G_w,
                          float *partial, int slots, const float *factor, float *acc_w, void *tc_workspace,
                          int *status, cudaStream_t stream, bool second_pass = false,
-                         const TcInlineClip *inline_clip = nullptr, const TcPublish *publish = nullptr);
+                         const TcPublish *publish = nullptr);
 
 // The fused clipped sum of a bf16 layer whose per-example gradient fits the tensor memory of one thread-block cluster
 // runs as ONE contraction (norm, factor and scaled sum from the same accumulators); tc_clip_single_pass says whether
-// this layer qualifies.  Writes sqnorm / clip_out like a CLIP_ACCUM launch with TcInlineClip; layers without bias only.
+// this layer qualifies.  Publishes what TcInlineClip names; layers without bias only.
 bool tc_clip_single_pass(int dtype, const ConvGeom &g);
-dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g, float *partial, int slots,
-                            const TcInlineClip &clipinfo, float *acc_w, void *tc_workspace, int *status, cudaStream_t stream);
+dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g, const TcInlineClip &clipinfo,
+                            float *acc_w, void *tc_workspace, int *status, cudaStream_t stream);
 
 // bf16 layers too large for one cluster: after the norm pass has published the factors (factor[2n]), the clipped sum is
 // ONE matrix product over all examples with f_n dY split into hi + lo bf16 copies (kept in tc_workspace).  No bias, not unfolded.
@@ -54,6 +53,41 @@ dp_status launch_conv_scaled_tiles(int dtype, const void *X, const void *dY, con
 bool tc_gram_norm(int dtype, const ConvGeom &g);
 dp_status launch_conv_gram_norm(int dtype, const void *X, const void *dY, const ConvGeom &g, const TcInlineClip &clipinfo,
                                 float *factor_out, int *status, cudaStream_t stream);
+
+// While one of these lives, this thread plans (and launches) for a batch of layer calls: every layer is tiled for least
+// SM time on the whole GPU and no CTA walks through more than `walk_cycles` of one layer.
+struct BatchPlanning {
+    explicit BatchPlanning(double walk_cycles);
+    ~BatchPlanning();
+    double saved;
+};
+
+// One convolution of a batch (tensor-core layers only) and how it is run there.
+enum { kConvSingle = 0, kConvTc, kConvClip1, kConvGramTiles, kConvGramSum };
+struct ConvJob {
+    int kind, dtype, epi;
+    ConvGeom g;
+    const void *X, *dY;
+    float *G_w, *partial;        // stored gradients; per-example partial squared norms [B][slots]
+    int slots, w_slots, separate;
+    int *counter;                // cleared ticket word
+    TcInlineClip clip;           // where norms (and factors) go
+    float *factor;               // [B][2] scratch
+    float *acc_w;
+    void *tc_workspace;
+};
+// kConvSingle: no shared launch takes this layer.
+int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias);
+double conv_batch_walk(const std::vector<ConvJob> &jobs);
+// Streams a batch spreads its independent launches over: s[0] is the caller's, the others are forked from it and joined
+// to it again (ForkedStreams).  All may be one and the same.
+struct BatchStreams {
+    enum { kMain = 0, kClusters, kSums, kAffine, kCount };
+    cudaStream_t s[kCount];
+    cudaEvent_t gram_done;       // null when all streams are one
+};
+dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *status, const BatchStreams &streams,
+                            const std::function<dp_status()> &join);
 
 // Test hook: the number of polls after which a bounded wait of the kernel gives up (0 makes every wait give up at once).
 void set_wait_polls(uint32_t polls);

@@ -307,14 +307,16 @@ class PerLayerClipStep:
         self.acc_w = [views[(li, "w")] for li in range(len(self.layers))]
         self.acc_b = [views.get((li, "b")) for li in range(len(self.layers))]
         self.sq = torch.zeros((B, self.L), dtype=torch.float32, device=device)
-        ws = max([b.dp_workspace_bytes(d, b.DP_EPI_CLIP_ACCUM) for d in self.descs] + [256])
-        self.lanes = max(1, int(lanes))
-        self.ws_lane = _workspaces(ws, self.lanes, device)
-        self.ws = self.ws_lane[0]
         self._col, col = [], 0
         for l in self.layers:
             self._col.append(col)
             col += 2 if l.n_bias else 1
+        self._batches = {}
+        self.batch = self._batch(range(len(self.layers)))
+        ws = max([b.dp_workspace_bytes(d, b.DP_EPI_CLIP_ACCUM) for d in self.descs] + [256, self.batch.workspace_bytes])
+        self.lanes = max(1, int(lanes))
+        self.ws_lane = _workspaces(ws, self.lanes, device)
+        self.ws = self.ws_lane[0]
         self.chunks_done = 0
         self._side = [torch.cuda.Stream(device=device) for _ in range(self.lanes - 1)] if self.lanes > 1 else []
         # layer -> lane: each call goes to the lane with the least work so far (a rough per-call cost is enough)
@@ -334,29 +336,26 @@ class PerLayerClipStep:
                                        b.DP_EPI_CLIP_ACCUM, self.C_l, self.acc_w[li], self.acc_b[li], None,
                                        self.ws_lane[lane], stream=stream), "dp_per_example_wgrad")
 
+    def _batch(self, layers):
+        """The given layers' calls as one batch."""
+        layers = tuple(layers)
+        if layers not in self._batches:
+            batch = b.Batch([self.descs[li] for li in layers], [b.DP_EPI_CLIP_ACCUM] * len(layers))
+            for i, li in enumerate(layers):
+                batch.set(i, sqnorm=self.sq.data_ptr() + 4 * self._col[li], sqnorm_stride=self.L, acc_w=self.acc_w[li],
+                          acc_b=self.acc_b[li])
+            self._batches[layers] = batch
+        return self._batches[layers]
+
     def chunk_calls(self, inputs, only=None):
         """The layer calls of one chunk: in order on the current stream, or forked over the lanes and joined again.
         only: a set of layer indices to restrict the chunk to (measurements of one kind of layer)."""
-        if self.lanes == 1:
-            for li, (X, dY) in enumerate(inputs):
-                if only is None or li in only:
-                    self.wgrad(li, X, dY)
-            return
-        main = torch.cuda.current_stream()
-        fork = torch.cuda.Event()
-        fork.record(main)
-        streams = [main] + self._side
-        for s in self._side:
-            s.wait_event(fork)
-        for li, (X, dY) in enumerate(inputs):
-            if only is not None and li not in only:
-                continue
-            k = self._lane_of[li]
-            self.wgrad(li, X, dY, lane=k, stream=streams[k])
-        for s in self._side:
-            done = torch.cuda.Event()
-            done.record(s)
-            main.wait_event(done)
+        if only is None:
+            batch = self.batch
+        else:
+            layers = [li for li in range(len(self.layers)) if li in only]
+            batch, inputs = self._batch(layers), [inputs[li] for li in layers]
+        b.check(batch.run(inputs, self.C_l, self.ws), "dp_batch_run")
 
     def chunk(self, inputs):
         self.chunk_calls(inputs)
