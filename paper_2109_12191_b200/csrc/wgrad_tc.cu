@@ -14,8 +14,9 @@
 // Two accumulator buffers in TMEM let the epilogue of one tile overlap the main loop of the next.
 // Every wait is bounded: on expiry the CTA sets a status word, drains and returns.
 //
-// fp32 inputs run as split tf32: the tensor core truncates fp32 to tf32, which biases every norm by about
-// 1e-3, so eight more warps write lo = x - hi (hi = x with the low 13 mantissa bits cleared) of each landed
+// fp32 inputs: the tensor core truncates fp32 to tf32, which biases every norm by about 1e-3.  DP_TF32 lets the copies
+// round to tf32 (nearest even) on the way in: TMA's TFLOAT32 element type does that for free, bit for bit like the warps
+// that did it in shared memory before (2.4 us a stage).  DP_F32 runs as split tf32: eight more warps write lo = x - hi (hi = x with the low 13 mantissa bits cleared) of each landed
 // stage into a second buffer of the same layout; x itself stays in place, where the tensor core's own truncation
 // turns it into hi, and the issuer accumulates lo*hi + hi*lo + hi*hi per step.  What is dropped (lo*lo and the truncation of lo) is below 2^-20 relative.
 #include "wgrad_tc.cuh"
@@ -26,6 +27,7 @@
 #include <array>
 #include <map>
 #include <memory>
+#include <numeric>
 
 namespace dp {
 
@@ -55,8 +57,8 @@ struct TcParams {
     int krows;                  // reduction rows per MMA: 16 (bf16) or 8 (tf32)
     int a_is_x, a_ext, b_ext, m_tiles, n_tiles, NT;
     int OWt, OHt, tiles_w, Kt, k_tiles, stages, stage_bytes, a_bytes;
+    int a_group, b_group;       // slabs of A / B that one copy brings (all of one filter tap)
     int lo_offset;              // split tf32: byte offset of the lo copy inside a stage
-    int single_pass;            // fp32 inputs rounded to tf32 (nearest even) in place, one MMA per step, no lo copy
     int mode;                   // 0 store + norm, 1 norm only, 2 clipped sum over a range of examples
     float *G_w;
     float *partial;             // [B][slots], slot = (mt*n_tiles + nt)*4 + epilogue warp
@@ -151,9 +153,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     *abort_flag = 1;
     return false;
 }
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, uint32_t bar, int c0, int c1, int c2, int c3) {
-    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3) : "memory");
+// One lane of a converged warp (the same one every time), and the warp's index as a value the compiler knows to be uniform:
+// with both, the descriptors of a tensor-core instruction are worked out in uniform registers, where it needs them (61
+// cycles an instruction; 107 from inside a branch only one lane takes, which bounded every main loop).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t pred;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+    return pred != 0;
+}
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+// A box of an activation tensor seen as {slab of channels, W, H, B, slabs}: it lands slab after slab, each OWt*OHt rows of
+// 128 bytes, so one copy brings all slabs of an operand that belong to one filter tap.
+__device__ __forceinline__ void tma_load_slabs(uint32_t dst, const CUtensorMap *map, uint32_t bar, int w, int h, int n, int slab) {
+    asm volatile("cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(0), "r"(w), "r"(h), "r"(n), "r"(slab) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols) : "memory");
@@ -237,9 +250,71 @@ __device__ __forceinline__ uint32_t instr_desc(int n_cols, uint32_t fmt) {
     return (1u << 4) | (fmt << 7) | (fmt << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n_cols >> 3) << 17) | ((128u >> 4) << 24);
 }
 
-template <bool TF32, bool CLIP, int N>
-__global__ void __launch_bounds__(TF32 ? 480 : 224, 1)
+// How a finished block of D leaves: to per-example gradients nobody reads soon, to partial sums, or added to the
+// accumulator.  Every element has one owner per launch, so an add needs no order; as a reduction at L2 it does not wait
+// for the old value (reading it back row by row took longer than the tile's whole main loop).
+enum { kPutStream = 0, kPutPlain, kPutAdd };
+__device__ __forceinline__ void red_add(float *dst, float v) {
+    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(dst), "f"(v) : "memory");
+}
+template <int MODE>
+__device__ __forceinline__ void put4(float *dst, const float4 v) {
+    if (MODE == kPutStream) __stcs(reinterpret_cast<float4 *>(dst), v);
+    else if (MODE == kPutPlain) *reinterpret_cast<float4 *>(dst) = v;
+    else asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+// A warp's 32 x 32 block, one row of 32 columns a lane, to 32 rows `ld` floats apart: through 4 KB of shared memory, so that
+// eight lanes write 128 neighbouring bytes of one row (16 bytes a lane of 32 different rows ran at a fraction of the rate).
+// The 16-byte pieces of a row are permuted by its number: both directions are free of bank conflicts.
+template <int MODE, typename V>
+__device__ __forceinline__ void put_rows(float4 *buf, const V &value, int lane, float *dst, long long ld, int rows) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) buf[lane * 8 + (i ^ (lane & 7))] = make_float4(value(4 * i), value(4 * i + 1), value(4 * i + 2), value(4 * i + 3));
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int row = 4 * i + (lane >> 3);
+        const float4 v = buf[row * 8 + ((lane & 7) ^ (row & 7))];
+        if (row < rows) put4<MODE>(dst + (long long)row * ld + 4 * (lane & 7), v);
+    }
+    __syncwarp();
+}
+
+// What a producer warp copies for one operand of a tile: lane o holds the origin of copy o (`group` slabs of one tap).
+// Issuing a copy costs the issuing warp about a hundred cycles and a barrier wait somewhat more, whatever the copy's size,
+// so the fewer copies a stage takes, the smaller the stages (and the shorter their latency) can be.
+struct OperandCopies {
+    int count, slab, dw, dh, mul;
+    uint32_t bytes;             // of one copy
+    __device__ __forceinline__ OperandCopies(const TcParams &p, bool is_x, int slab0, int slabs, int group, int slab_bytes, int lane) {
+        count = slabs / group;
+        bytes = (uint32_t)(group * slab_bytes);
+        slab = slab0 + lane * group; dw = 0; dh = 0; mul = 1;
+        if (is_x) {
+            const int j0 = slab * p.slab_ch;
+            const int tap = j0 / p.Cin;
+            slab = (j0 - tap * p.Cin) / p.slab_ch;
+            const int r = tap / p.S;
+            dw = (tap - r * p.S) - p.pad;
+            dh = r - p.pad;
+            mul = p.stride;
+        }
+    }
+    // the whole warp calls; `leader` issues (origins travel by shuffle, so the copies' operands are uniform)
+    __device__ __forceinline__ void issue(bool leader, const CUtensorMap *map, uint32_t dst, uint32_t bar, int ow0, int oh0, int n) const {
+        for (int o = 0; o < count; ++o) {
+            const int s = __shfl_sync(0xffffffffu, slab, o), w = __shfl_sync(0xffffffffu, dw, o), h = __shfl_sync(0xffffffffu, dh, o);
+            if (leader) tma_load_slabs(dst + (uint32_t)o * bytes, map, bar, ow0 * mul + w, oh0 * mul + h, n, s);
+            __syncwarp();
+        }
+    }
+};
+
+enum { kBf16 = 0, kTf32, kSplit };       // inputs of the tensor cores: bf16, tf32, or fp32 as hi + lo tf32
+template <int ARITH, bool CLIP, int N>
+__global__ void __launch_bounds__(ARITH == kSplit ? 480 : 224, 1)
 conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
+    constexpr bool TF32 = ARITH != kBf16, SPLIT = ARITH == kSplit;
     const int entry = table_entry(tab.first, tab.n, blockIdx.x);
     const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
     const TcParams &p = tab.e[entry].p;
@@ -250,9 +325,9 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], ready_bar[kMaxStages], tmem_full[2], tmem_empty[2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
-    __shared__ float xpose[4][32][33];      // per epilogue warp: 32 x 32 transpose buffer for coalesced row stores
+    __shared__ float4 xpose[4][256];        // per epilogue warp: a 32 x 32 block on its way out (put_rows)
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t tiles_u32 = smem_u32(tiles);
 
@@ -279,10 +354,9 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------------------ TMA producers
-        // Two warps, because issuing a copy costs the issuing warp ~100 cycles: warp 0 loads the A slabs of every
+        // Two warps, so that a stage's copies are issued side by side: warp 0 loads the A slabs of every
         // stage, warp 6 the B slabs; each announces its own bytes on the stage's full barrier (two arrivals).
-        // Lane L owns slab L: it works out its tap shift and channel offset once per tile and then only adds the
-        // pixel-tile origin, so no division sits in the stage loop.
+        const bool leader = elect_one();
         int stage = 0; uint32_t phase = 0;
         bool live = true;
         for (int item = item0; item < item_end && live; item += item_step) {
@@ -290,66 +364,45 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
             const int mt = it.mt, nt = it.nt;
             const int a_slab0 = mt * a_slabs_tile, a_slabs = min(a_slabs_tile, p.a_ext / p.slab_ch - a_slab0);
             const int b_slab0 = nt * b_slabs_tile, b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - b_slab0);
-            const bool is_a = warp == 0;
-            const int local = lane;
-            const bool active = is_a ? (local < a_slabs) : (local < b_slabs);
-            const bool is_x = is_a ? (p.a_is_x != 0) : (p.a_is_x == 0);
-            const int slab = (is_a ? a_slab0 : b_slab0) + local;
-            int c0, dw = 0, dh = 0, mul = 1;
-            if (is_x) {
-                const int j0 = slab * p.slab_ch;
-                const int tap = j0 / p.Cin;
-                c0 = j0 - tap * p.Cin;
-                const int r = tap / p.S;
-                dw = (tap - r * p.S) - p.pad;
-                dh = r - p.pad;
-                mul = p.stride;
-            } else {
-                c0 = slab * p.slab_ch;
-            }
+            const bool is_a = warp == 0, is_x = is_a == (p.a_is_x != 0);
+            const OperandCopies copies(p, is_x, is_a ? a_slab0 : b_slab0, is_a ? a_slabs : b_slabs, is_a ? p.a_group : p.b_group, slab_bytes, lane);
             const CUtensorMap *map = is_x ? &tmX : &tmY;
-            const uint32_t dst_off = (is_a ? 0u : (uint32_t)p.a_bytes) + (uint32_t)(local * slab_bytes);
-            const uint32_t tx_bytes = (uint32_t)((is_a ? a_slabs : b_slabs) * slab_bytes);
+            const uint32_t dst = tiles_u32 + (is_a ? 0u : (uint32_t)p.a_bytes);
+            const uint32_t tx_bytes = (uint32_t)copies.count * copies.bytes;
             for (int n = it.n_lo; n < it.n_hi && live; ++n) {
                 int ow0 = 0, oh0 = 0, tw = 0;
                 for (int kt = 0; kt < p.k_tiles; ++kt) {
-                    bool ok = true;
-                    if (lane == 0) {
-                        ok = mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls);
-                        if (ok) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
-                    }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) { live = false; break; }
-                    if (active)
-                        tma_load_4d(tiles_u32 + stage * p.stage_bytes + dst_off, map, smem_u32(&full_bar[stage]), c0,
-                                    ow0 * mul + dw, oh0 * mul + dh, n);
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls))) { live = false; break; }
+                    if (leader) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
+                    __syncwarp();
+                    copies.issue(leader, map, dst + stage * p.stage_bytes, smem_u32(&full_bar[stage]), ow0, oh0, n);
                     if (++tw == p.tiles_w) { tw = 0; ow0 = 0; oh0 += p.OHt; } else { ow0 += p.OWt; }
                     if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (one lane)
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0;
-            uint32_t acc_phase = 0;  // bit b: phase of accumulator buffer b
-            int buf = 0;
-            bool live = true;
-            const uint64_t desc_base = operand_desc_base<TF32>((uint32_t)slab_bytes);
-            const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
-            const int ksteps = p.Kt / p.krows;
-            constexpr uint32_t kadvance = (uint32_t)((TF32 ? 8 : 16) * kRowBytes) >> 4;   // start-address units of 16 B per MMA step
-            for (int item = item0; item < item_end && live; item += item_step) {
-              const Item it = decode_item(p, item);
-              const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
-              const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, TF32 ? 2u : 1u);
-              for (int n = it.n_lo; n < it.n_hi && live; ++n) {
-                if (!mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls)) { live = false; break; }
+        // ------------------------------------------------------------ MMA issuer: the warp walks together, one lane issues
+        const bool leader = elect_one();
+        int stage = 0; uint32_t phase = 0;
+        uint32_t acc_phase = 0;  // bit b: phase of accumulator buffer b
+        int buf = 0;
+        bool live = true;
+        const uint64_t desc_base = operand_desc_base<TF32>((uint32_t)slab_bytes);
+        const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
+        const int ksteps = p.Kt / p.krows;
+        constexpr uint32_t kadvance = (uint32_t)((TF32 ? 8 : 16) * kRowBytes) >> 4;   // start-address units of 16 B per MMA step
+        for (int item = item0; item < item_end && live; item += item_step) {
+            const Item it = decode_item(p, item);
+            const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
+            const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, TF32 ? 2u : 1u);
+            for (int n = it.n_lo; n < it.n_hi && live; ++n) {
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls))) { live = false; break; }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
                 uint32_t accumulate = 0;
                 for (int kt = 0; kt < p.k_tiles; ++kt) {
-                    if (!mbar_wait(smem_u32(TF32 ? &ready_bar[stage] : &full_bar[stage]), phase, abort_p, p.wait_polls)) { live = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(SPLIT ? &ready_bar[stage] : &full_bar[stage]), phase, abort_p, p.wait_polls))) { live = false; break; }
                     tc_fence_after();
                     const uint32_t a_src = tiles_u32 + stage * p.stage_bytes;
                     // descriptor low words: start address >> 4 in bits 0-13, slab stride >> 4 in bits 16-29
@@ -357,42 +410,39 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                     uint32_t bd = desc_lo | (((a_src + p.a_bytes) & 0x3FFFFu) >> 4);
                     // rows of the A tile past the operand's extent hold whatever the stage held before:
                     // they only feed rows of D that the epilogue never reads
-                    if (TF32 && p.single_pass) {
-#pragma unroll 4
-                        for (int ks = 0; ks < ksteps; ++ks) {
-                            umma<TF32>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);
-                            accumulate = 1;
-                            ad += kadvance; bd += kadvance;
-                        }
-                    } else if (TF32) {
-                        const uint32_t lo = (uint32_t)p.lo_offset >> 4;
+                    if (leader) {
+                        if (SPLIT) {
+                            const uint32_t lo = (uint32_t)p.lo_offset >> 4;
 #pragma unroll 2
-                        for (int ks = 0; ks < ksteps; ++ks) {
-                            umma<TF32>(d_tmem, ad + lo, bd, desc_hi32, idesc, accumulate);      // lo(A) * hi(B)
-                            umma<TF32>(d_tmem, ad, bd + lo, desc_hi32, idesc, 1u);              // hi(A) * lo(B)
-                            umma<TF32>(d_tmem, ad, bd, desc_hi32, idesc, 1u);                   // hi(A) * hi(B)
-                            accumulate = 1;
-                            ad += kadvance; bd += kadvance;
-                        }
-                    } else {
+                            for (int ks = 0; ks < ksteps; ++ks) {
+                                umma<TF32>(d_tmem, ad + lo, bd, desc_hi32, idesc, accumulate);      // lo(A) * hi(B)
+                                umma<TF32>(d_tmem, ad, bd + lo, desc_hi32, idesc, 1u);              // hi(A) * lo(B)
+                                umma<TF32>(d_tmem, ad, bd, desc_hi32, idesc, 1u);                   // hi(A) * hi(B)
+                                accumulate = 1;
+                                ad += kadvance; bd += kadvance;
+                            }
+                        } else {
 #pragma unroll 4
-                        for (int ks = 0; ks < ksteps; ++ks) {
-                            umma<TF32>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);
-                            accumulate = 1;
-                            ad += kadvance; bd += kadvance;
+                            for (int ks = 0; ks < ksteps; ++ks) {
+                                umma<TF32>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);
+                                accumulate = 1;
+                                ad += kadvance; bd += kadvance;
+                            }
                         }
+                        umma_commit(smem_u32(&empty_bar[stage]));      // frees the stage once these MMAs have read it
                     }
-                    umma_commit(smem_u32(&empty_bar[stage]));      // frees the stage once these MMAs have read it
+                    accumulate = 1;
+                    __syncwarp();
                     if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!live) break;
-                umma_commit(smem_u32(&tmem_full[buf]));            // accumulator complete
+                if (leader) umma_commit(smem_u32(&tmem_full[buf]));            // accumulator complete
+                __syncwarp();
                 acc_phase ^= 1u << buf;
                 buf ^= 1;
-              }
             }
         }
-    } else if (TF32 && warp >= 7) {
+    } else if (SPLIT && warp >= 7) {
         // ------------------------------------------------------------ split warps (fp32 inputs only)
         // hi stays where TMA put it, lo goes to the same offset of the stage's second half; both keep the
         // swizzled layout because the split is element-wise on identical relative addresses.
@@ -425,15 +475,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                                 if (i0 + 128 * u < rchunks) x[u] = *reinterpret_cast<const float4 *>(rbase + ((size_t)(i0 + 128 * u) << 4));
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
-                                if (i0 + 128 * u < rchunks && p.single_pass) {
-                                    // round to tf32, nearest even, in place: the tensor core's own truncation then changes nothing
-                                    uint4 b = *reinterpret_cast<const uint4 *>(&x[u]);
-                                    b.x = (b.x + 0xFFFu + ((b.x >> 13) & 1u)) & 0xFFFFE000u;
-                                    b.y = (b.y + 0xFFFu + ((b.y >> 13) & 1u)) & 0xFFFFE000u;
-                                    b.z = (b.z + 0xFFFu + ((b.z >> 13) & 1u)) & 0xFFFFE000u;
-                                    b.w = (b.w + 0xFFFu + ((b.w >> 13) & 1u)) & 0xFFFFE000u;
-                                    *reinterpret_cast<uint4 *>(rbase + ((size_t)(i0 + 128 * u) << 4)) = b;
-                                } else if (i0 + 128 * u < rchunks) {
+                                if (i0 + 128 * u < rchunks) {
                                     uint8_t *ptr = rbase + ((size_t)(i0 + 128 * u) << 4);
                                     float4 hi, lo;
                                     hi.x = __uint_as_float(__float_as_uint(x[u].x) & 0xFFFFE000u); lo.x = x[u].x - hi.x;
@@ -521,20 +563,16 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                             }
                         }
                         if (p.mode == 0 && !p.a_is_x) {
-                            // row = output channel k, tile columns = 32 consecutive j: each lane holds one row, so the
-                            // warp transposes its 32 x 32 block through shared memory and every store instruction then
-                            // writes one 128-byte row segment (scattered 16-byte pieces ran at a fraction of the rate)
-                            float (*xp)[33] = xpose[warp - 2];
+                            // row = output channel k, tile columns = 32 consecutive j: each lane holds one row
+                            const int col0 = nt * p.NT + cc, rows_here = min(32, a_rows - q * 32);
+                            float *dst = Gn + (long long)(mt * 128 + q * 32) * p.Ng + col0;
+                            if (!p.n_pad_cols) {
+                                put_rows<kPutStream>(xpose[warp - 2], [&](int i) { return __uint_as_float(v[i]); }, lane, dst, p.Ng, rows_here);
+                            } else if (lane < rows_here) {           // rows of any length: element by element
 #pragma unroll
-                            for (int i = 0; i < 32; ++i) xp[lane][i] = __uint_as_float(v[i]);
-                            __syncwarp();
-                            const int col = nt * p.NT + cc + lane;
-                            const int rows_here = min(32, a_rows - q * 32);
-                            if (col < p.Ng) {
-                                float *dst = Gn + (long long)(mt * 128 + q * 32) * p.Ng + col;
-                                for (int r = 0; r < rows_here; ++r) __stcs(dst + (long long)r * p.Ng, xp[r][lane]);
+                                for (int i = 0; i < 32; ++i)
+                                    if (col0 + i < p.Ng) dst[(long long)lane * p.Ng + i] = __uint_as_float(v[i]);
                             }
-                            __syncwarp();
                         }
                     };
                     // columns in pairs of 32 with both loads in flight before the wait.  The second load of a tile with
@@ -557,36 +595,27 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
             }
             if (!CLIP && p.counters && lane == 0 && item + item_step >= item_end)
                 __threadfence();          // after this warp's last item: its partial sums are visible to the CTA that folds them
-            if (CLIP && live && row_ok) {
-                // one owner per output element: add straight into the accumulator, or leave a partial sum for the fold
+            if (CLIP && live) {
+                // added to the accumulator, or left as a partial sum for the fold
                 const bool add = p.splits == 1;
                 float *base = p.sum_out + (add ? 0ll : (long long)it.split * p.Kout * p.Ng);
 #pragma unroll
                 for (int c4 = 0; c4 < 4; ++c4) {
                     if (c4 * 32 < n_cols) {
                         const int b_idx = nt * p.NT + c4 * 32;
-                        if (p.a_is_x) {
-                            float *dst = base + (long long)b_idx * p.Ng + a_idx;
+                        auto value = [&](int i) { return run[CLIP ? c4 * 32 + i : 0]; };
+                        if (!p.a_is_x && !p.n_pad_cols) {
+                            float *dst = base + (long long)(mt * 128 + q * 32) * p.Ng + b_idx;
+                            if (add) put_rows<kPutAdd>(xpose[warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
+                            else put_rows<kPutPlain>(xpose[warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
+                        } else if (row_ok) {
+                            const long long step = p.a_is_x ? p.Ng : 1;
+                            float *dst = base + (p.a_is_x ? (long long)b_idx * p.Ng + a_idx : (long long)a_idx * p.Ng + b_idx);
 #pragma unroll
                             for (int i = 0; i < 32; ++i) {
-                                float *e = dst + (long long)i * p.Ng;
-                                const float r = run[CLIP ? c4 * 32 + i : 0];
-                                *e = add ? *e + r : r;
+                                if (!p.a_is_x && b_idx + i >= p.Ng) continue;
+                                if (add) red_add(dst + i * step, value(i)); else dst[i * step] = value(i);
                             }
-                        } else if (!p.n_pad_cols) {
-                            float4 *dst = reinterpret_cast<float4 *>(base + (long long)a_idx * p.Ng + b_idx);
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                float4 r = make_float4(run[CLIP ? c4 * 32 + 4 * i : 0], run[CLIP ? c4 * 32 + 4 * i + 1 : 0],
-                                                       run[CLIP ? c4 * 32 + 4 * i + 2 : 0], run[CLIP ? c4 * 32 + 4 * i + 3 : 0]);
-                                if (add) { const float4 o = dst[i]; r.x += o.x; r.y += o.y; r.z += o.z; r.w += o.w; }
-                                dst[i] = r;
-                            }
-                        } else {
-                            float *dst = base + (long long)a_idx * p.Ng + b_idx;
-#pragma unroll
-                            for (int i = 0; i < 32; ++i)
-                                if (b_idx + i < p.Ng) dst[i] = add ? dst[i] + run[CLIP ? c4 * 32 + i : 0] : run[CLIP ? c4 * 32 + i : 0];
                         }
                     }
                 }
@@ -705,6 +734,20 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     return false;
 }
 
+// Knuth's error-free sum: returns a + b rounded and adds what the rounding lost to `err`.
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    err = __fadd_rn(err, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+    return s;
+}
+__device__ __forceinline__ float sum8(const float4 &x, const float4 &y) {
+    float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
+    const float a = two_sum(x.x, x.y, e0), b = two_sum(x.z, x.w, e1), c = two_sum(y.x, y.y, e2), d = two_sum(y.z, y.w, e3);
+    const float ab = two_sum(a, b, e0), cd = two_sum(c, d, e2);
+    const float s = two_sum(ab, cd, e0);
+    return s + ((e0 + e1) + (e2 + e3));
+}
+
 template <int N>
 __global__ void __launch_bounds__(kClipThreads, 1)
 conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
@@ -715,11 +758,11 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tmem_full[2], tmem_empty[2], norm_bar[4], warp_bar[4];
     __shared__ float warp_part[4][8];                   // [example mod 4][epilogue warp]: this CTA's partial sums
-    __shared__ float norm_part[4][kMaxCluster];         // [example mod 4][source CTA]: every CTA's sum, sent by its first epilogue warp
+    __shared__ __align__(16) float norm_part[4][kMaxCluster];         // [example mod 4][source CTA]: every CTA's sum, sent by its first epilogue warp
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t tiles_u32 = smem_u32(tiles);
     const int cs = p.m_tiles * p.n_tiles;                 // cluster size = tiles of one example's gradient
@@ -740,6 +783,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 2); mbar_init(smem_u32(&empty_bar[s]), 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tmem_full[b]), 1); mbar_init(smem_u32(&tmem_empty[b]), 8); }
         for (int b = 0; b < 4; ++b) { mbar_init(smem_u32(&norm_bar[b]), 1); mbar_init(smem_u32(&warp_bar[b]), 8); }
+        for (int i = 0; i < 4 * kMaxCluster; ++i) norm_part[0][i] = 0.f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), 512);
@@ -759,76 +803,65 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kClipRegsControl));
         if (warp == 0 || warp == 2) {
             // ------------------------------------------------------------ TMA producers (A slabs / B slabs)
-            const bool is_a = warp == 0;
-            const bool active = is_a ? (lane < a_slabs) : (lane < b_slabs);
-            const bool is_x = is_a ? (p.a_is_x != 0) : (p.a_is_x == 0);
-            const int slab = (is_a ? mt * a_slabs_tile : nt * b_slabs_tile) + lane;
-            int c0, dw = 0, dh = 0, mul = 1;
-            if (is_x) {
-                const int j0 = slab * p.slab_ch;
-                const int tap = j0 / p.Cin;
-                c0 = j0 - tap * p.Cin;
-                const int r = tap / p.S;
-                dw = (tap - r * p.S) - p.pad;
-                dh = r - p.pad;
-                mul = p.stride;
-            } else {
-                c0 = slab * p.slab_ch;
-            }
+            const bool leader = elect_one();
+            const bool is_a = warp == 0, is_x = is_a == (p.a_is_x != 0);
+            const OperandCopies copies(p, is_x, is_a ? mt * a_slabs_tile : nt * b_slabs_tile, is_a ? a_slabs : b_slabs,
+                                       is_a ? p.a_group : p.b_group, slab_bytes, lane);
             const CUtensorMap *map = is_x ? &tmX : &tmY;
-            const uint32_t dst_off = (is_a ? 0u : (uint32_t)p.a_bytes) + (uint32_t)(lane * slab_bytes);
-            const uint32_t tx_bytes = (uint32_t)((is_a ? a_slabs : b_slabs) * slab_bytes);
+            const uint32_t dst = tiles_u32 + (is_a ? 0u : (uint32_t)p.a_bytes);
+            const uint32_t tx_bytes = (uint32_t)copies.count * copies.bytes;
+            const int stages = p.stages, stage_bytes = p.stage_bytes, k_tiles = p.k_tiles, tiles_w = p.tiles_w, OWt = p.OWt, OHt = p.OHt;
             int stage = 0; uint32_t phase = 0;
             bool live = true;
             for (int n = n_lo; n < n_hi && live; ++n) {
                 int ow0 = 0, oh0 = 0, tw = 0;
-                for (int kt = 0; kt < p.k_tiles; ++kt) {
-                    bool ok = true;
-                    if (lane == 0) {
-                        ok = mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls);
-                        if (ok) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
-                    }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) { live = false; break; }
-                    if (active)
-                        tma_load_4d(tiles_u32 + stage * p.stage_bytes + dst_off, map, smem_u32(&full_bar[stage]), c0,
-                                    ow0 * mul + dw, oh0 * mul + dh, n);
-                    if (++tw == p.tiles_w) { tw = 0; ow0 = 0; oh0 += p.OHt; } else { ow0 += p.OWt; }
-                    if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+                for (int kt = 0; kt < k_tiles; ++kt) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls))) { live = false; break; }
+                    if (leader) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
+                    __syncwarp();
+                    copies.issue(leader, map, dst + stage * stage_bytes, smem_u32(&full_bar[stage]), ow0, oh0, n);
+                    if (++tw == tiles_w) { tw = 0; ow0 = 0; oh0 += OHt; } else { ow0 += OWt; }
+                    if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
             }
-        } else if (warp == 1 && lane == 0) {
-            // ------------------------------------------------------------ MMA issuer (one lane)
+        } else if (warp == 1) {
+            // ------------------------------------------------------------ MMA issuer: the warp walks together, one lane issues
+            const bool leader = elect_one();
             int stage = 0; uint32_t phase = 0, acc_phase = 0;
             int buf = 0;
             bool live = true;
             const uint64_t desc_base = operand_desc_base<false>((uint32_t)slab_bytes);
             const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
-            const int ksteps = p.Kt / p.krows;
+            const int ksteps = p.Kt / p.krows, k_tiles = p.k_tiles, stages = p.stages, stage_bytes = p.stage_bytes, a_bytes = p.a_bytes;
             constexpr uint32_t kadvance = (uint32_t)(16 * kRowBytes) >> 4;
             const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, 1u);
             for (int n = n_lo; n < n_hi && live; ++n) {
-                if (!mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls)) break;
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls))) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
                 uint32_t accumulate = 0;
-                for (int kt = 0; kt < p.k_tiles; ++kt) {
-                    if (!mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls)) { live = false; break; }
+                for (int kt = 0; kt < k_tiles; ++kt) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls))) { live = false; break; }
                     tc_fence_after();
-                    const uint32_t a_src = tiles_u32 + stage * p.stage_bytes;
+                    const uint32_t a_src = tiles_u32 + stage * stage_bytes;
                     uint32_t ad = desc_lo | ((a_src & 0x3FFFFu) >> 4);
-                    uint32_t bd = desc_lo | (((a_src + p.a_bytes) & 0x3FFFFu) >> 4);
+                    uint32_t bd = desc_lo | (((a_src + a_bytes) & 0x3FFFFu) >> 4);
+                    if (leader) {
 #pragma unroll 4
-                    for (int ks = 0; ks < ksteps; ++ks) {
-                        umma<false>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);
-                        accumulate = 1;
-                        ad += kadvance; bd += kadvance;
+                        for (int ks = 0; ks < ksteps; ++ks) {
+                            umma<false>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);
+                            accumulate = 1;
+                            ad += kadvance; bd += kadvance;
+                        }
+                        umma_commit(smem_u32(&empty_bar[stage]));
                     }
-                    umma_commit(smem_u32(&empty_bar[stage]));
-                    if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+                    accumulate = 1;
+                    __syncwarp();
+                    if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
                 if (!live) break;
-                umma_commit(smem_u32(&tmem_full[buf]));
+                if (leader) umma_commit(smem_u32(&tmem_full[buf]));
+                __syncwarp();
                 acc_phase ^= 1u << buf;
                 buf ^= 1;
             }
@@ -858,6 +891,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         // warp sends only after it has scaled example j + 3, i.e. after every warp of the cluster has sent example
         // j + 3, which each of them did after scaling (and so after reading the slots of) example j + 2 and before it j.
         const int count = n_hi - n_lo;
+        const float threshold = __double2float_rd((double)p.C_l * (double)p.C_l);
         for (int step = 0; known && step < count && live; ++step) {
             // factors known: one read of the finished tile per example, scaled into the running sum
             const int buf = step & 1;
@@ -888,34 +922,38 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                 // finish example step - 1 first: its tile leaves tensor memory before this step's tile is touched, so the
                 // MMAs of the example after this one run while this step's tile is being square-summed
                 const int j = step - 1, n = n_lo + j, buf = j & 1, slot = j & 3;
+                // half of the tile is on its way to registers while the norm is still being exchanged
+                const uint32_t t_addr = tmem_base + (uint32_t)(buf * 256 + half * 128) + ((uint32_t)(q * 32) << 16);
+                uint32_t v0[32], v1[32];
+                tmem_ld32_issue(t_addr, v0);
+                tmem_ld32_issue(t_addr + 32u, v1);
                 const bool all_in = mbar_wait_cluster(smem_u32(&norm_bar[slot]), (uint32_t)((j >> 2) & 1), abort_p, p.wait_polls);
+                // the same tree in every thread of every CTA (slots past the cluster's size hold zeros): all of them apply
+                // the identical factor.  The sum carries its rounding errors along (as good as double, whose pipe is so
+                // narrow that the same tree takes it some 800 cycles on the path every example waits on); the factor
+                // min(1, C_l / sqrt(sn)) is in single precision.
+                const float4 lo = *reinterpret_cast<const float4 *>(norm_part[slot]), hi = *reinterpret_cast<const float4 *>(norm_part[slot] + 4);
+                const float sn = sum8(lo, hi);
+                const float f = (sn <= threshold) ? 1.0f : p.C_l * rsqrtf(sn);
+                tmem_ld_wait32(v0); tmem_ld_wait32(v1);
                 if (!__all_sync(0xffffffffu, all_in)) { live = false; break; }
-                // the same tree in every warp of every CTA (two entries a lane, then a butterfly): all of them apply the
-                // identical factor
-                double sn = lane < cs ? (double)norm_part[slot][lane] : 0.0;
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) sn += __shfl_xor_sync(0xffffffffu, sn, o);      // (at most eight CTAs)
-                sn = __shfl_sync(0xffffffffu, sn, 0);
-                // min(1, C_l / sqrt(sn)) in single precision here: the double-precision square root and division are
-                // some hundreds of cycles on the path every example waits on
-                const float f = (sn <= (double)p.C_l * (double)p.C_l) ? 1.0f : p.C_l / sqrtf((float)sn);
                 if (rank == 0 && e == 0 && lane == 0) {
-                    p.sqnorm[n * p.sq_stride] = (float)sn;
+                    p.sqnorm[n * p.sq_stride] = sn;
                     if (p.clip_out) p.clip_out[n] = f;
                 }
                 // pass 2: scale the tile into the running sum
-                const uint32_t t_addr = tmem_base + (uint32_t)(buf * 256 + half * 128) + ((uint32_t)(q * 32) << 16);
 #pragma unroll
                 for (int c2 = 0; c2 < 2; ++c2) {
                     if (c2 * 64 < my_cols) {
-                        uint32_t v0[32], v1[32];
-                        tmem_ld32_issue(t_addr + (uint32_t)(c2 * 64), v0);
-                        tmem_ld32_issue(t_addr + (uint32_t)(c2 * 64 + 32), v1);
-                        tmem_ld_wait32(v0); tmem_ld_wait32(v1);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) run[c2 * 64 + i] = fmaf(f, __uint_as_float(v0[i]), run[c2 * 64 + i]);
+                        if (c2 == 0 && my_cols > 64) tmem_ld32_issue(t_addr + 64u, v0);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) run[c2 * 64 + 32 + i] = fmaf(f, __uint_as_float(v1[i]), run[c2 * 64 + 32 + i]);
+                        if (c2 == 0 && my_cols > 64) {
+                            tmem_ld32_issue(t_addr + 96u, v1);
+                            tmem_ld_wait32(v0); tmem_ld_wait32(v1);
+                        }
                     }
                 }
                 tc_fence_before();
@@ -963,35 +1001,29 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                 }
             }
         }
-        if (live && row_ok && split < p.splits) {
-            // one owner per output element: add straight into the accumulator, or leave a partial sum for the fold
+        if (live && split < p.splits) {
+            // added to the accumulator, or left as a partial sum for the fold; every tile has been read, so the stages'
+            // memory is free to carry the blocks out
             const bool add = p.splits == 1;
             float *base = p.sum_out + (add ? 0ll : (long long)split * p.Kout * p.Ng);
+            float4 *buf = reinterpret_cast<float4 *>(tiles) + e * 256;
 #pragma unroll
             for (int c4 = 0; c4 < 4; ++c4) {
                 if (c4 * 32 < my_cols) {
                     const int b_idx = nt * p.NT + half * 128 + c4 * 32;
-                    if (p.a_is_x) {
-                        float *dst = base + (long long)b_idx * p.Ng + a_idx;
+                    auto value = [&](int i) { return run[c4 * 32 + i]; };
+                    if (!p.a_is_x && !p.n_pad_cols) {
+                        float *dst = base + (long long)(mt * 128 + q * 32) * p.Ng + b_idx;
+                        if (add) put_rows<kPutAdd>(buf, value, lane, dst, p.Ng, a_rows - q * 32);
+                        else put_rows<kPutPlain>(buf, value, lane, dst, p.Ng, a_rows - q * 32);
+                    } else if (row_ok) {
+                        const long long step = p.a_is_x ? p.Ng : 1;
+                        float *dst = base + (p.a_is_x ? (long long)b_idx * p.Ng + a_idx : (long long)a_idx * p.Ng + b_idx);
 #pragma unroll
                         for (int i = 0; i < 32; ++i) {
-                            float *el = dst + (long long)i * p.Ng;
-                            const float r = run[c4 * 32 + i];
-                            *el = add ? *el + r : r;
+                            if (!p.a_is_x && b_idx + i >= p.Ng) continue;
+                            if (add) red_add(dst + i * step, value(i)); else dst[i * step] = value(i);
                         }
-                    } else if (!p.n_pad_cols) {
-                        float4 *dst = reinterpret_cast<float4 *>(base + (long long)a_idx * p.Ng + b_idx);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            float4 r = make_float4(run[c4 * 32 + 4 * i], run[c4 * 32 + 4 * i + 1], run[c4 * 32 + 4 * i + 2], run[c4 * 32 + 4 * i + 3]);
-                            if (add) { const float4 o = dst[i]; r.x += o.x; r.y += o.y; r.z += o.z; r.w += o.w; }
-                            dst[i] = r;
-                        }
-                    } else {
-                        float *dst = base + (long long)a_idx * p.Ng + b_idx;
-#pragma unroll
-                        for (int i = 0; i < 32; ++i)
-                            if (b_idx + i < p.Ng) dst[i] = add ? dst[i] + run[c4 * 32 + i] : run[c4 * 32 + i];
                     }
                 }
             }
@@ -1031,8 +1063,9 @@ conv_wgrad_ssum_kernel(const __grid_constant__ TcTable<TcParams, 3, N> tab) {
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], tmem_full[2], tmem_empty[2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
+    __shared__ float4 xpose[4][256];        // per epilogue warp: a 32 x 32 block on its way out (put_rows)
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t tiles_u32 = smem_u32(tiles);
 
@@ -1058,95 +1091,77 @@ conv_wgrad_ssum_kernel(const __grid_constant__ TcTable<TcParams, 3, N> tab) {
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------------------ TMA producers
+        const bool leader = elect_one();
+        const bool is_a = warp == 0, is_y = is_a == a_is_y;
         int stage = 0; uint32_t phase = 0;
         bool live = true;
         for (int item = blk; item < p.total_tiles && live; item += p.blocks) {
             const Item it = decode_item(p, item);
-            const int a_slab0 = it.mt * a_slabs_tile, a_slabs = min(a_slabs_tile, p.a_ext / p.slab_ch - a_slab0);
-            const int b_slab0 = it.nt * b_slabs_tile, b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - b_slab0);
-            const bool is_a = warp == 0;
-            const bool is_y = is_a == a_is_y;
-            const int mine = is_a ? a_slabs : b_slabs;       // slabs of this warp's operand; a dY warp issues each twice (hi, lo)
-            const bool second = is_y && lane >= mine;        // lanes [mine, 2*mine) of a dY warp load the lo copies
-            const int local = second ? lane - mine : lane;
-            const bool active = lane < (is_y ? 2 * mine : mine);
-            const int slab = (is_a ? a_slab0 : b_slab0) + local;
-            int c0, dw = 0, dh = 0, mul = 1;
-            if (!is_y) {
-                const int j0 = slab * p.slab_ch;
-                const int tap = j0 / p.Cin;
-                c0 = j0 - tap * p.Cin;
-                const int r = tap / p.S;
-                dw = (tap - r * p.S) - p.pad;
-                dh = r - p.pad;
-                mul = p.stride;
-            } else {
-                c0 = slab * p.slab_ch;
-            }
-            const CUtensorMap *map = !is_y ? &tmX : (second ? &tmYlo : &tmYhi);
-            const uint32_t dst_off = (second ? (uint32_t)p.lo_offset : (is_a ? 0u : (uint32_t)p.a_bytes)) + (uint32_t)(local * slab_bytes);
-            const uint32_t tx_bytes = (uint32_t)((is_y ? 2 * mine : mine) * slab_bytes);
+            const int slab0 = is_a ? it.mt * a_slabs_tile : it.nt * b_slabs_tile;
+            const int slabs = min(is_a ? a_slabs_tile : b_slabs_tile, (is_a ? p.a_ext : p.b_ext) / p.slab_ch - slab0);
+            const OperandCopies copies(p, !is_y, slab0, slabs, is_a ? p.a_group : p.b_group, slab_bytes, lane);
+            const CUtensorMap *map = is_y ? &tmYhi : &tmX;
+            const uint32_t dst = tiles_u32 + (is_a ? 0u : (uint32_t)p.a_bytes), dst_lo = tiles_u32 + (uint32_t)p.lo_offset;
+            const uint32_t tx_bytes = (uint32_t)copies.count * copies.bytes * (is_y ? 2u : 1u);       // dY comes as hi and lo
             for (int n = it.n_lo; n < it.n_hi && live; ++n) {
                 int ow0 = 0, oh0 = 0, tw = 0;
                 for (int kt = 0; kt < p.k_tiles; ++kt) {
-                    bool ok = true;
-                    if (lane == 0) {
-                        ok = mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls);
-                        if (ok) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
-                    }
-                    ok = __shfl_sync(0xffffffffu, ok, 0);
-                    if (!ok) { live = false; break; }
-                    if (active)
-                        tma_load_4d(tiles_u32 + stage * p.stage_bytes + dst_off, map, smem_u32(&full_bar[stage]), c0,
-                                    ow0 * mul + dw, oh0 * mul + dh, n);
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls))) { live = false; break; }
+                    if (leader) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
+                    __syncwarp();
+                    copies.issue(leader, map, dst + stage * p.stage_bytes, smem_u32(&full_bar[stage]), ow0, oh0, n);
+                    if (is_y) copies.issue(leader, &tmYlo, dst_lo + stage * p.stage_bytes, smem_u32(&full_bar[stage]), ow0, oh0, n);
                     if (++tw == p.tiles_w) { tw = 0; ow0 = 0; oh0 += p.OHt; } else { ow0 += p.OWt; }
                     if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (one lane)
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0, acc_phase = 0;
-            int buf = 0;
-            bool live = true;
-            const uint64_t desc_base = operand_desc_base<false>((uint32_t)slab_bytes);
-            const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
-            const int ksteps = p.Kt / p.krows;
-            constexpr uint32_t kadvance = (uint32_t)(16 * kRowBytes) >> 4;
-            for (int item = blk; item < p.total_tiles && live; item += p.blocks) {
-                const Item it = decode_item(p, item);
-                const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
-                const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, 1u);
-                if (!mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls)) break;
+        // ------------------------------------------------------------ MMA issuer: the warp walks together, one lane issues
+        const bool leader = elect_one();
+        int stage = 0; uint32_t phase = 0, acc_phase = 0;
+        int buf = 0;
+        bool live = true;
+        const uint64_t desc_base = operand_desc_base<false>((uint32_t)slab_bytes);
+        const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
+        const int ksteps = p.Kt / p.krows;
+        constexpr uint32_t kadvance = (uint32_t)(16 * kRowBytes) >> 4;
+        for (int item = blk; item < p.total_tiles && live; item += p.blocks) {
+            const Item it = decode_item(p, item);
+            const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - it.nt * b_slabs_tile);
+            const uint32_t idesc = instr_desc(b_slabs * p.slab_ch, 1u);
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls))) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
+            uint32_t accumulate = 0;
+            const int trips = (it.n_hi - it.n_lo) * p.k_tiles;
+            for (int kt = 0; kt < trips; ++kt) {
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls))) { live = false; break; }
                 tc_fence_after();
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * 256);
-                uint32_t accumulate = 0;
-                for (int n = it.n_lo; n < it.n_hi && live; ++n) {
-                    for (int kt = 0; kt < p.k_tiles; ++kt) {
-                        if (!mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls)) { live = false; break; }
-                        tc_fence_after();
-                        const uint32_t src = tiles_u32 + stage * p.stage_bytes;
-                        uint32_t ad = desc_lo | ((src & 0x3FFFFu) >> 4);
-                        uint32_t bd = desc_lo | (((src + p.a_bytes) & 0x3FFFFu) >> 4);
-                        uint32_t ld = desc_lo | (((src + p.lo_offset) & 0x3FFFFu) >> 4);
+                const uint32_t src = tiles_u32 + stage * p.stage_bytes;
+                uint32_t ad = desc_lo | ((src & 0x3FFFFu) >> 4);
+                uint32_t bd = desc_lo | (((src + p.a_bytes) & 0x3FFFFu) >> 4);
+                uint32_t ld = desc_lo | (((src + p.lo_offset) & 0x3FFFFu) >> 4);
+                if (leader) {
 #pragma unroll 2
-                        for (int ks = 0; ks < ksteps; ++ks) {
-                            umma<false>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);                               // X with hi(f dY)
-                            if (a_is_y) umma<false>(d_tmem, ld, bd, desc_hi32, idesc, 1u);                           // X with lo(f dY)
-                            else umma<false>(d_tmem, ad, ld, desc_hi32, idesc, 1u);
-                            accumulate = 1;
-                            ad += kadvance; bd += kadvance; ld += kadvance;
-                        }
-                        umma_commit(smem_u32(&empty_bar[stage]));
-                        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+                    for (int ks = 0; ks < ksteps; ++ks) {
+                        umma<false>(d_tmem, ad, bd, desc_hi32, idesc, accumulate);                               // X with hi(f dY)
+                        if (a_is_y) umma<false>(d_tmem, ld, bd, desc_hi32, idesc, 1u);                           // X with lo(f dY)
+                        else umma<false>(d_tmem, ad, ld, desc_hi32, idesc, 1u);
+                        accumulate = 1;
+                        ad += kadvance; bd += kadvance; ld += kadvance;
                     }
+                    umma_commit(smem_u32(&empty_bar[stage]));
                 }
-                if (!live) break;
-                umma_commit(smem_u32(&tmem_full[buf]));
-                acc_phase ^= 1u << buf;
-                buf ^= 1;
+                accumulate = 1;
+                __syncwarp();
+                if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             }
+            if (!live) break;
+            if (leader) umma_commit(smem_u32(&tmem_full[buf]));
+            __syncwarp();
+            acc_phase ^= 1u << buf;
+            buf ^= 1;
         }
     } else if (warp >= 2 && warp <= 5) {
         // ------------------------------------------------------------ epilogue: one read of the finished tile per item
@@ -1169,23 +1184,17 @@ conv_wgrad_ssum_kernel(const __grid_constant__ TcTable<TcParams, 3, N> tab) {
             const bool add = p.splits == 1;
             float *base = p.sum_out + (add ? 0ll : (long long)it.split * p.Kout * p.Ng);
             auto put = [&](uint32_t (&v)[32], int cc) {
-                if (!row_ok) return;
                 const int b_idx = nt * p.NT + cc;
-                if (p.a_is_x) {
+                auto value = [&](int i) { return __uint_as_float(v[i]); };
+                if (!p.a_is_x) {
+                    float *dst = base + (long long)(mt * 128 + q * 32) * p.Ng + b_idx;
+                    if (add) put_rows<kPutAdd>(xpose[warp - 2], value, lane, dst, p.Ng, a_rows - q * 32);
+                    else put_rows<kPutPlain>(xpose[warp - 2], value, lane, dst, p.Ng, a_rows - q * 32);
+                } else if (row_ok) {
                     float *dst = base + (long long)b_idx * p.Ng + a_idx;
 #pragma unroll
                     for (int i = 0; i < 32; ++i) {
-                        float *el = dst + (long long)i * p.Ng;
-                        const float r = __uint_as_float(v[i]);
-                        *el = add ? *el + r : r;
-                    }
-                } else {
-                    float4 *dst = reinterpret_cast<float4 *>(base + (long long)a_idx * p.Ng + b_idx);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        float4 r = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-                        if (add) { const float4 o = dst[i]; r.x += o.x; r.y += o.y; r.z += o.z; r.w += o.w; }
-                        dst[i] = r;
+                        if (add) red_add(dst + (long long)i * p.Ng, value(i)); else dst[(long long)i * p.Ng] = value(i);
                     }
                 }
             };
@@ -1267,7 +1276,7 @@ conv_gram_norm_kernel(const __grid_constant__ TcTable<GramParams, 2, N> tab) {
     __shared__ __align__(8) uint64_t norm_bar;
     __shared__ double warp_part[4][4];      // [example & 3][quadrant]: a warp may run up to three examples ahead of the one that adds up
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t tiles_u32 = smem_u32(tiles);
 
@@ -1295,52 +1304,50 @@ conv_gram_norm_kernel(const __grid_constant__ TcTable<GramParams, 2, N> tab) {
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer: one box per stage
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0;
-            bool live = true;
-            const uint32_t tx_bytes = (uint32_t)(p.pack * p.rows * kRowBytes);
-            for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
-                for (int mt = 0; mt < p.m_tiles && live; ++mt) {
-                    int tap = 0, cs = 0;
-                    for (int s = 0; s < slabs; ++s) {
-                        if (!mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls)) { live = false; break; }
+        const bool leader = elect_one();
+        int stage = 0; uint32_t phase = 0;
+        bool live = true;
+        const uint32_t tx_bytes = (uint32_t)(p.pack * p.rows * kRowBytes);
+        for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
+            for (int mt = 0; mt < p.m_tiles && live; ++mt) {
+                int r = 0, sx = 0, cs = 0;                   // tap (r, sx) and slab of X
+                for (int s = 0; s < slabs; ++s) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls))) { live = false; break; }
+                    const bool is_y = s < y_slabs;
+                    if (leader) {
                         mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
-                        const uint32_t dst = tiles_u32 + stage * p.stage_bytes;
-                        if (s < y_slabs) {
-                            tma_load_4d(dst, &tmY, smem_u32(&full_bar[stage]), s * 64, 0, 0, n);
-                        } else {
-                            const int r = tap / p.S;
-                            tma_load_4d(dst, &tmX, smem_u32(&full_bar[stage]), cs * 64, (tap - r * p.S) - p.pad, r - p.pad, n);
-                            if (++cs == c_slabs) { cs = 0; ++tap; }
-                        }
-                        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+                        tma_load_slabs(tiles_u32 + stage * p.stage_bytes, is_y ? &tmY : &tmX, smem_u32(&full_bar[stage]), is_y ? 0 : sx - p.pad,
+                                       is_y ? 0 : r - p.pad, n, is_y ? s : cs);
                     }
+                    __syncwarp();
+                    if (!is_y && ++cs == c_slabs) { cs = 0; if (++sx == p.S) { sx = 0; ++r; } }
+                    if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer (one lane)
-        if (lane == 0) {
-            int stage = 0; uint32_t phase = 0, acc_phase = 0;
-            int buf = 0;
-            bool live = true;
-            const uint64_t desc_base = kmajor_desc_base();
-            const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
-            for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
-                for (int mt = 0; mt < p.m_tiles && live; ++mt) {
-                    const int col0 = mt * 128;                       // the tile's columns start at its own first row
-                    const uint32_t idesc = instr_desc_kmajor(p.pack * p.rows - col0);
-                    if (!mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls)) { live = false; break; }
+        // ------------------------------------------------------------ MMA issuer: the warp walks together, one lane issues
+        const bool leader = elect_one();
+        int stage = 0; uint32_t phase = 0, acc_phase = 0;
+        int buf = 0;
+        bool live = true;
+        const uint64_t desc_base = kmajor_desc_base();
+        const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
+        for (int n = blk * p.pack; n < p.B && live; n += p.blocks * p.pack) {
+            for (int mt = 0; mt < p.m_tiles && live; ++mt) {
+                const int col0 = mt * 128;                       // the tile's columns start at its own first row
+                const uint32_t idesc = instr_desc_kmajor(p.pack * p.rows - col0);
+                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&tmem_empty[buf]), ((acc_phase >> buf) & 1u) ^ 1u, abort_p, p.wait_polls))) { live = false; break; }
+                tc_fence_after();
+                const uint32_t d_y = tmem_base + (uint32_t)(buf * 256), d_x = d_y + x_col;
+                for (int s = 0; s < slabs; ++s) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls))) { live = false; break; }
                     tc_fence_after();
-                    const uint32_t d_y = tmem_base + (uint32_t)(buf * 256), d_x = d_y + x_col;
-                    for (int s = 0; s < slabs; ++s) {
-                        if (!mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls)) { live = false; break; }
-                        tc_fence_after();
-                        const uint32_t src = tiles_u32 + stage * p.stage_bytes + (uint32_t)(col0 * kRowBytes);
-                        uint32_t ad = desc_lo | ((src & 0x3FFFFu) >> 4);
-                        const bool is_y = s < y_slabs;
-                        const uint32_t d_tmem = is_y ? d_y : d_x;
-                        uint32_t accumulate = (s == 0 || s == y_slabs) ? 0u : 1u;
+                    const uint32_t src = tiles_u32 + stage * p.stage_bytes + (uint32_t)(col0 * kRowBytes);
+                    uint32_t ad = desc_lo | ((src & 0x3FFFFu) >> 4);
+                    const uint32_t d_tmem = s < y_slabs ? d_y : d_x;
+                    uint32_t accumulate = (s == 0 || s == y_slabs) ? 0u : 1u;
+                    if (leader) {
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks) {             // 64 channels = four steps of 16, 32 bytes apart in the row
                             umma<false>(d_tmem, ad, ad, desc_hi32, idesc, accumulate);
@@ -1348,13 +1355,15 @@ conv_gram_norm_kernel(const __grid_constant__ TcTable<GramParams, 2, N> tab) {
                             ad += 2;
                         }
                         umma_commit(smem_u32(&empty_bar[stage]));
-                        if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                     }
-                    if (!live) break;
-                    umma_commit(smem_u32(&tmem_full[buf]));
-                    acc_phase ^= 1u << buf;
-                    if (nbuf == 2) buf ^= 1;
+                    __syncwarp();
+                    if (++stage == p.stages) { stage = 0; phase ^= 1u; }
                 }
+                if (!live) break;
+                if (leader) umma_commit(smem_u32(&tmem_full[buf]));
+                __syncwarp();
+                acc_phase ^= 1u << buf;
+                if (nbuf == 2) buf ^= 1;
             }
         }
     } else {
@@ -1689,8 +1698,8 @@ static double step_cycles(int dtype, int n_cols, double a_slabs_loaded, double b
         const double smem = 4096.0 + 32.0 * n_cols + 2048.0 * (a_slabs_loaded + b_slabs);
         return std::max(n_cols / 2.0, smem / 128.0);
     }
-    if (dtype == DP_TF32) {   // one MMA per step; the stage is filled once, read once and written back once by the rounding warps
-        const double smem = 4096.0 + 32.0 * n_cols + 1024.0 * (a_slabs_loaded + b_slabs) * 3.0;
+    if (dtype == DP_TF32) {   // one MMA per step of 8 rows
+        const double smem = 4096.0 + 32.0 * n_cols + 1024.0 * (a_slabs_loaded + b_slabs);
         return std::max(n_cols / 2.0, smem / 128.0);
     }
     const double smem = 3.0 * (4096.0 + 32.0 * n_cols) + 1024.0 * (a_slabs_loaded + b_slabs) * 3.0;
@@ -1824,7 +1833,7 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
                     double stage_cost = (double)(Kt / krows) * step + 250.0;
                     // a TMA warp: barrier wait + expect_tx, then one copy per slab it owns (A or B), all latency-bound on that warp
                     stage_cost = std::max(stage_cost, 350.0 + 110.0 * std::max(a_loaded, b_loaded));
-                    if (dtype != DP_BF16)   // split warps, two groups in turn: a fixed fence/hand-over plus their share of the bytes
+                    if (dtype == DP_F32)   // split warps, two groups in turn: a fixed fence/hand-over plus their share of the bytes
                         stage_cost = std::max(stage_cost, 0.5 * (1000.0 + (a_loaded + b_loaded) * Kt * 2.5));
                     double mainloop = stage_cost * tw * th;
                     if (stages < 3) mainloop *= 1.15;
@@ -2007,15 +2016,17 @@ int tc_describe_plan(int dtype, const ConvGeom &g0, int epilogue, int *out, int 
     return 12;
 }
 
-// channels-last [B, H, W, C] tensor, box = {one slab of channels, boxW, boxH, 1 example}; `step` > 1 walks every
-// step-th pixel (the box then spans boxW*step pixels and delivers boxW of them)
-static bool encode_nhwc(CUtensorMap *map, int dtype, const void *base, int C, int W, int H, int Bn, int boxW, int boxH, int step, int boxN = 1) {
-    const cuuint64_t es = (dtype == DP_BF16) ? 2 : 4;
-    const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)Bn};
-    const cuuint64_t strides[3] = {(cuuint64_t)C * es, (cuuint64_t)W * C * es, (cuuint64_t)H * W * C * es};
-    const cuuint32_t box[4] = {(cuuint32_t)(kRowBytes / es), (cuuint32_t)(boxW * step), (cuuint32_t)(boxH * step), (cuuint32_t)boxN};
-    const cuuint32_t estr[4] = {1, (cuuint32_t)step, (cuuint32_t)step, 1};
-    return encode_fn()(map, dtype == DP_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4,
+// channels-last [B, H, W, C] tensor seen as {slab of channels, W, H, B, slabs}; box = {slab, boxW, boxH, boxN, slabs a copy};
+// `step` > 1 walks every step-th pixel (the box then spans boxW*step pixels and delivers boxW of them)
+static bool encode_nhwc(CUtensorMap *map, int dtype, const void *base, int C, int W, int H, int Bn, int boxW, int boxH, int step,
+                        int boxN = 1, int slabs = 1) {
+    const cuuint64_t es = (dtype == DP_BF16) ? 2 : 4, slab_ch = kRowBytes / es;
+    const cuuint64_t dims[5] = {slab_ch, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)Bn, (cuuint64_t)C / slab_ch};
+    const cuuint64_t strides[4] = {(cuuint64_t)C * es, (cuuint64_t)W * C * es, (cuuint64_t)H * W * C * es, kRowBytes};
+    const cuuint32_t box[5] = {(cuuint32_t)slab_ch, (cuuint32_t)(boxW * step), (cuuint32_t)(boxH * step), (cuuint32_t)boxN, (cuuint32_t)slabs};
+    const cuuint32_t estr[5] = {1, (cuuint32_t)step, (cuuint32_t)step, 1, 1};
+    return encode_fn()(map, dtype == DP_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                                             : (dtype == DP_TF32 ? CU_TENSOR_MAP_DATA_TYPE_TFLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32), 5,
                        const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                        dtype == DP_BF16 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -2037,9 +2048,11 @@ static dp_status raise_shared_limits() {
     static cudaError_t err = cudaSuccess;
     std::call_once(once, [] {
         const cudaError_t all[] = {
-            allow_shared(conv_wgrad_tc_kernel<false, false, 1>), allow_shared(conv_wgrad_tc_kernel<false, true, 1>),
-            allow_shared(conv_wgrad_tc_kernel<true, false, 1>), allow_shared(conv_wgrad_tc_kernel<true, true, 1>),
-            allow_shared(conv_wgrad_tc_kernel<false, false, kTcLayers>), allow_shared(conv_wgrad_tc_kernel<true, false, kTcLayers>),
+            allow_shared(conv_wgrad_tc_kernel<kBf16, false, 1>), allow_shared(conv_wgrad_tc_kernel<kBf16, true, 1>),
+            allow_shared(conv_wgrad_tc_kernel<kSplit, false, 1>), allow_shared(conv_wgrad_tc_kernel<kSplit, true, 1>),
+            allow_shared(conv_wgrad_tc_kernel<kBf16, false, kTcLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kTcLayers>),
+            allow_shared(conv_wgrad_tc_kernel<kTf32, false, 1>), allow_shared(conv_wgrad_tc_kernel<kTf32, true, 1>),
+            allow_shared(conv_wgrad_tc_kernel<kTf32, false, kTcLayers>),
             allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
             allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>),
             allow_shared(conv_gram_norm_kernel<1>), allow_shared(conv_gram_norm_kernel<kTcLayers>)};
@@ -2049,6 +2062,15 @@ static dp_status raise_shared_limits() {
     return err == cudaSuccess ? DP_OK : cuda_fail(err, "cudaFuncSetAttribute");
 }
 
+// Slabs one copy brings: neighbours along the channels of one filter tap, a divisor of the tile's and of the tensor's slabs.
+static int slab_group(int dtype, const ConvGeom &g, const TcPlan &pl, bool of_a) {
+    const int slab_ch = (dtype == DP_BF16) ? 64 : 32;
+    const bool is_x = of_a == (pl.a_is_x != 0);
+    return std::gcd((is_x ? g.Cin : g.Kout) / slab_ch, (of_a ? 128 : pl.NT) / slab_ch);
+}
+static int x_group(int dtype, const ConvGeom &g, const TcPlan &pl) { return slab_group(dtype, g, pl, pl.a_is_x != 0); }
+static int y_group(int dtype, const ConvGeom &g, const TcPlan &pl) { return slab_group(dtype, g, pl, pl.a_is_x == 0); }
+
 // what the parameters of every kernel take from the layer and its plan
 static void fill_common(TcParams &p, int dtype, const ConvGeom &g, int Ng, const TcPlan &pl, int *status) {
     p.B = g.B; p.Kout = g.Kout; p.Ng = Ng; p.Cin = g.Cin; p.S = g.S; p.stride = g.stride; p.pad = g.pad;
@@ -2057,6 +2079,7 @@ static void fill_common(TcParams &p, int dtype, const ConvGeom &g, int Ng, const
     p.a_is_x = pl.a_is_x; p.a_ext = pl.a_ext; p.b_ext = pl.b_ext; p.m_tiles = pl.m_tiles; p.n_tiles = pl.n_tiles; p.NT = pl.NT;
     p.OWt = pl.OWt; p.OHt = pl.OHt; p.tiles_w = pl.tiles_w; p.Kt = pl.Kt; p.k_tiles = pl.k_tiles;
     p.stages = pl.stages; p.stage_bytes = pl.stage_bytes; p.a_bytes = pl.a_bytes;
+    p.a_group = slab_group(dtype, g, pl, true); p.b_group = slab_group(dtype, g, pl, false);
     p.status = status;
     p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
 }
@@ -2091,13 +2114,12 @@ static dp_status fill_conv_tc(int dtype, int epilogue, const void *X, const void
                               void *tc_workspace, int *status, const TcPublish *publish, ConvEntry &e) {
     const bool clip = epilogue == DP_EPI_CLIP_ACCUM;
     const ConvGeom &g = pr.eff;
-    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1, 1, y_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
     TcParams &p = e.p;
     p = TcParams{};
     fill_common(p, dtype, g, g0.N, pl, status);
     p.lo_offset = pl.stage_bytes / 2;
-    p.single_pass = (dtype == DP_TF32) ? 1 : 0;
     p.mode = clip ? 2 : (epilogue == DP_EPI_STORE_NORM ? 0 : 1);
     p.G_w = G_w; p.partial = partial; p.slots = slots;
     p.splits = 1; p.per_split = g.B; p.factor = factor; p.sum_out = acc_w;
@@ -2140,11 +2162,14 @@ dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY,
     p.blocks = std::min(p.total_tiles, sm_target());
     const unsigned grid = (unsigned)p.blocks;
     if (dtype == DP_BF16) {
-        if (clip) conv_wgrad_tc_kernel<false, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
-        else conv_wgrad_tc_kernel<false, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        if (clip) conv_wgrad_tc_kernel<kBf16, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        else conv_wgrad_tc_kernel<kBf16, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
+    } else if (dtype == DP_TF32) {
+        if (clip) conv_wgrad_tc_kernel<kTf32, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        else conv_wgrad_tc_kernel<kTf32, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
     } else {
-        if (clip) conv_wgrad_tc_kernel<true, true, 1><<<grid, 480, pl.smem, stream>>>(tab);
-        else conv_wgrad_tc_kernel<true, false, 1><<<grid, 480, pl.smem, stream>>>(tab);
+        if (clip) conv_wgrad_tc_kernel<kSplit, true, 1><<<grid, 480, pl.smem, stream>>>(tab);
+        else conv_wgrad_tc_kernel<kSplit, false, 1><<<grid, 480, pl.smem, stream>>>(tab);
     }
     DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
     if (clip && p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g0.M * g0.N, acc_w, stream);
@@ -2161,9 +2186,9 @@ bool tc_clip_scaled_sum(int dtype, const ConvGeom &g0) {
 static dp_status fill_ssum(int dtype, const void *X, const ConvGeom &g, const TcPlan &pl, float *acc_w, void *tc_workspace,
                            int *status, SsumEntry &e) {
     char *ws_bytes = static_cast<char *>(tc_workspace);
-    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&e.map[1], dtype, ws_bytes, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY hi)");
-    if (!encode_nhwc(&e.map[2], dtype, ws_bytes + ssum_copy_bytes(g), g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY lo)");
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, ws_bytes, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1, 1, y_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY hi)");
+    if (!encode_nhwc(&e.map[2], dtype, ws_bytes + ssum_copy_bytes(g), g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1, 1, y_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY lo)");
     TcParams &p = e.p;
     p = TcParams{};
     fill_common(p, dtype, g, g.N, pl, status);
@@ -2223,8 +2248,8 @@ static void scaled_tiles_split(const ConvGeom &g, const TcPlan &pl, int &splits,
 
 static dp_status fill_scaled_tiles(int dtype, const void *X, const void *dY, const ConvGeom &g, const TcPlan &pl,
                                    const float *factor, float *acc_w, void *tc_workspace, int *status, ConvEntry &e) {
-    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
-    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1, 1, y_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
     TcParams &p = e.p;
     p = TcParams{};
     fill_common(p, dtype, g, g.N, pl, status);
@@ -2354,17 +2379,17 @@ static dp_status fill_clip1(int dtype, const void *X, const void *dY, const Conv
     if (s2d) {
         const S2dProblem sp = s2d_problem(dtype, g0, pr);
         // one operand row per output pixel: 64 values from pixel ow on, pixels 16 values apart
-        const cuuint64_t dims[4] = {64, (cuuint64_t)g.OW, (cuuint64_t)sp.Hs, (cuuint64_t)g.B};
-        const cuuint64_t strides[3] = {32, (cuuint64_t)sp.Ws * 32, (cuuint64_t)sp.Hs * sp.Ws * 32};
-        const cuuint32_t box[4] = {64, (cuuint32_t)pl.OWt, (cuuint32_t)pl.OHt, 1};
-        const cuuint32_t estr[4] = {1, 1, 1, 1};
-        if (encode_fn()(&e.map[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, ws_bytes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        const cuuint64_t dims[5] = {64, (cuuint64_t)g.OW, (cuuint64_t)sp.Hs, (cuuint64_t)g.B, 1};
+        const cuuint64_t strides[4] = {32, (cuuint64_t)sp.Ws * 32, (cuuint64_t)sp.Hs * sp.Ws * 32, (cuuint64_t)g.B * sp.Hs * sp.Ws * 32};
+        const cuuint32_t box[5] = {64, (cuuint32_t)pl.OWt, (cuuint32_t)pl.OHt, 1, 1};
+        const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+        if (encode_fn()(&e.map[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, ws_bytes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(space-to-depth X)");
-    } else if (!encode_nhwc(&e.map[0], dtype, pr.unfold ? tc_workspace : X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride)) {
+    } else if (!encode_nhwc(&e.map[0], dtype, pr.unfold ? tc_workspace : X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) {
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
     }
-    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1)) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
+    if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1, 1, y_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
     TcParams &p = e.p;
     p = TcParams{};
     fill_common(p, dtype, g, g0.N, pl, status);
@@ -2480,7 +2505,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
     BatchPlanning planning(walk);
     dp_status rc = raise_shared_limits();
     if (rc != DP_OK) return rc;
-    ConvQueue store[2], clip[kMaxCluster + 1];            // store: bf16 / fp32; clip: by cluster size of the launch
+    ConvQueue store[3], clip[kMaxCluster + 1];            // store: by element type; clip: by cluster size of the launch
     GramQueue gram;
     SsumQueue ssum;
     std::vector<SplitSeg> splits;
@@ -2506,7 +2531,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             p.run = std::max(1, std::min(p.total_tiles, (int)(walk / pl.item_cycles)));
             p.blocks = q.blocks = (p.total_tiles + p.run - 1) / p.run;
             q.smem = pl.smem; q.cost = p.run * pl.item_cycles;
-            store[j.dtype == DP_BF16 ? 0 : 1].jobs.push_back(q);
+            store[j.dtype].jobs.push_back(q);
         } else if (j.kind == kConvClip1) {
             TcPlan pl; ConvGeom g1; bool s2d;
             if (!clip1_plan(j.dtype, j.g, pr, pl, g1, s2d)) return DP_ERR_UNSUPPORTED;
@@ -2555,10 +2580,11 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             }
         }
     }
-    for (int f32 = 0; f32 < 2; ++f32) {
-        rc = store[f32].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
-            if (f32) conv_wgrad_tc_kernel<true, false, kTcLayers><<<(unsigned)blocks, 480, smem, stream>>>(tab);
-            else conv_wgrad_tc_kernel<false, false, kTcLayers><<<(unsigned)blocks, 224, smem, stream>>>(tab);
+    for (int dtype = 0; dtype < 3; ++dtype) {
+        rc = store[dtype].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
+            if (dtype == DP_BF16) conv_wgrad_tc_kernel<kBf16, false, kTcLayers><<<(unsigned)blocks, 224, smem, stream>>>(tab);
+            else if (dtype == DP_TF32) conv_wgrad_tc_kernel<kTf32, false, kTcLayers><<<(unsigned)blocks, 224, smem, stream>>>(tab);
+            else conv_wgrad_tc_kernel<kSplit, false, kTcLayers><<<(unsigned)blocks, 480, smem, stream>>>(tab);
             DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
             return DP_OK;
         });
