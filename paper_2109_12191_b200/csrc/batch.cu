@@ -151,7 +151,11 @@ static dp_status run_convs(const dp_batch &b, const dp_layer_io *io, float C_l, 
         j.clip = TcInlineClip{C_l, o.sqnorm, o.sqnorm_stride, o.clip_out};
         if (it.desc.has_bias) {
             float *db = it.epi == DP_EPI_STORE_NORM ? o.G_b : reinterpret_cast<float *>(base + it.plan.db_off);
-            const dp_status rc = launch_bias(storage_type(&it.desc), o.dY, j.g, db, j.partial, it.plan.slots, it.plan.w_slots, st);
+            // a bias that is a group of its own and publishes its norm itself need not come before the weights' launch
+            j.bias_apart = j.separate && bias_publishes(storage_type(&it.desc), j.g);
+            const dp_status rc = launch_bias(storage_type(&it.desc), o.dY, j.g, db, j.partial, it.plan.slots, it.plan.w_slots,
+                                             j.bias_apart ? streams.s[BatchStreams::kSums] : st, j.bias_apart ? o.sqnorm + 1 : nullptr,
+                                             o.sqnorm_stride);
             if (rc != DP_OK) return rc;
         }
     }
@@ -224,22 +228,30 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
         DP_CUDA_TRY(cudaEventRecord(b->fork, st));
         for (int i = 1; i < BatchStreams::kCount; ++i) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->fork, 0));
     }
+    // what is not a tensor-core launch of several layers: enqueued behind those, before the streams meet again
+    auto others = [&]() -> dp_status {
+        dp_status rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
+        for (int i = 0; i < n && rc == DP_OK; ++i) {
+            const dp_batch::Item &it = b->items[i];
+            if (it.group >= 0) continue;
+            const LayerBuffers buf = {io[i].X, io[i].dY, io[i].G_w, io[i].G_b, io[i].sqnorm, io[i].sqnorm_stride, io[i].acc_w, io[i].acc_b, io[i].clip_out};
+            rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kAffine]);
+        }
+        return rc;
+    };
+    bool joined = false;
     auto join = [&]() -> dp_status {
-        if (!forked) return DP_OK;
+        if (joined) return DP_OK;
+        joined = true;
+        const dp_status rc = others();
+        if (!forked) return rc;
         for (int i = 1; i < BatchStreams::kCount; ++i) {
             DP_CUDA_TRY(cudaEventRecord(b->done[i], streams.s[i]));
             DP_CUDA_TRY(cudaStreamWaitEvent(st, b->done[i], 0));
         }
-        return DP_OK;
+        return rc;
     };
-    dp_status rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
-    for (int i = 0; i < n && rc == DP_OK; ++i) {
-        const dp_batch::Item &it = b->items[i];
-        if (it.group >= 0) continue;
-        const LayerBuffers buf = {io[i].X, io[i].dY, io[i].G_w, io[i].G_b, io[i].sqnorm, io[i].sqnorm_stride, io[i].acc_w, io[i].acc_b, io[i].clip_out};
-        rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kAffine]);
-    }
-    if (rc == DP_OK) return run_convs(*b, io, C_l, ws, streams, join);
-    (void)join();                        // a launch failed: whatever is enqueued still comes before what follows
+    const dp_status rc = run_convs(*b, io, C_l, ws, streams, join);
+    if (rc != DP_OK) (void)join();       // a launch failed: whatever is enqueued still comes before what follows
     return rc;
 }

@@ -530,7 +530,7 @@ bias_kernel(const T *__restrict__ dY, int K, int Kout, float *__restrict__ db, f
 template <typename T, int VEC>
 __global__ void __launch_bounds__(256)
 bias_vec_kernel(const T *__restrict__ dY, int K, int Kout, float *__restrict__ db, float *__restrict__ partial, int slots,
-                int slot0, int bias_slots) {
+                int slot0, int bias_slots, float *__restrict__ sqnorm, long long sq_stride) {
     extern __shared__ float red[];                     // [rows][Kout]
     __shared__ float scratch[32];
     const int n = blockIdx.x;
@@ -570,6 +570,7 @@ bias_vec_kernel(const T *__restrict__ dY, int K, int Kout, float *__restrict__ d
     }
     sq = block_sum(sq, scratch);
     if (threadIdx.x < bias_slots) partial[(long long)n * slots + slot0 + threadIdx.x] = (threadIdx.x == 0) ? sq : 0.f;
+    if (sqnorm && threadIdx.x == 0) sqnorm[n * sq_stride] = sq;        // the bias is a group of its own: this is its whole norm
 }
 
 // One block per example: weight slots [0, w_slots) and bias slots [w_slots, slots) summed in index order.
@@ -1100,15 +1101,20 @@ dp_status launch_conv_fma(int dtype, int mode, const void *X, const void *dY, co
     return conv_fma_t(mode, static_cast<const __nv_bfloat16 *>(X), static_cast<const __nv_bfloat16 *>(dY), g, G_w, partial, slots, factor, acc_w, sum_ws, st);
 }
 
-dp_status launch_bias(int dtype, const void *dY, const ConvGeom &g, float *db, float *partial, int slots, int slot0,
-                      cudaStream_t st) {
+bool bias_publishes(int dtype, const ConvGeom &g) {
     const int vec = (dtype == DP_F32) ? 4 : 8;
-    if (g.Kout % vec == 0 && g.Kout / vec <= 256 && bias_blocks(g) <= 256) {
+    return g.Kout % vec == 0 && g.Kout / vec <= 256 && bias_blocks(g) <= 256;
+}
+
+dp_status launch_bias(int dtype, const void *dY, const ConvGeom &g, float *db, float *partial, int slots, int slot0,
+                      cudaStream_t st, float *sqnorm, long long sq_stride) {
+    const int vec = (dtype == DP_F32) ? 4 : 8;
+    if (bias_publishes(dtype, g)) {
         const size_t smem = sizeof(float) * (size_t)(256 / (g.Kout / vec)) * g.Kout;
         if (dtype == DP_F32)
-            bias_vec_kernel<float, 4><<<g.B, 256, smem, st>>>(static_cast<const float *>(dY), g.K, g.Kout, db, partial, slots, slot0, bias_blocks(g));
+            bias_vec_kernel<float, 4><<<g.B, 256, smem, st>>>(static_cast<const float *>(dY), g.K, g.Kout, db, partial, slots, slot0, bias_blocks(g), sqnorm, sq_stride);
         else
-            bias_vec_kernel<__nv_bfloat16, 8><<<g.B, 256, smem, st>>>(static_cast<const __nv_bfloat16 *>(dY), g.K, g.Kout, db, partial, slots, slot0, bias_blocks(g));
+            bias_vec_kernel<__nv_bfloat16, 8><<<g.B, 256, smem, st>>>(static_cast<const __nv_bfloat16 *>(dY), g.K, g.Kout, db, partial, slots, slot0, bias_blocks(g), sqnorm, sq_stride);
         DP_LAUNCH_CHECK("bias_vec_kernel");
         return DP_OK;
     }

@@ -37,8 +37,10 @@ dp_status launch_conv_rgb3(int dtype, const void *X, const void *dY, const ConvG
                            int has_bias, int separate, float *sqnorm, long long sq_stride,
                            cudaStream_t stream);
 // db[n,k] = sum over pixels of dY; also sum_k db^2 per block into partial[n*slots + slot0 + block]
+// (and, where bias_publishes() says so, the whole sum to sqnorm[n*sq_stride] when given)
+bool bias_publishes(int dtype, const ConvGeom &g);
 dp_status launch_bias(int dtype, const void *dY, const ConvGeom &g, float *db, float *partial, int slots, int slot0,
-                      cudaStream_t stream);
+                      cudaStream_t stream, float *sqnorm = nullptr, long long sq_stride = 0);
 // folds the partial slots of every example into sqnorm (and clip factors when clip != 0)
 dp_status launch_finalize(const float *partial, int B, int slots, int w_slots, int separate, float *sqnorm,
                           long long sq_stride, int clip, float C_l, float *factor, float *clip_out,

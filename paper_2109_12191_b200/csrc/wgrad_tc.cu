@@ -28,6 +28,7 @@
 #include <map>
 #include <memory>
 #include <numeric>
+#include <cmath>
 
 namespace dp {
 
@@ -75,6 +76,7 @@ struct TcParams {
     // modes 0 / 1 with a ticket: counters[0] counts the CTAs that are done (zero on entry, left at zero); the last
     // one folds every example's slots [0, w_slots) and [w_slots, slots) into sqnorm (two values when `separate`)
     int *counters; int w_slots; int separate;
+    int fold_slots;             // slots that are folded (all of them, or the weights' only)
     float *factor_out;          // with the ticket: also the clip factors against C_l, [B][2] (weight, bias), and clip_out
     // space-to-depth form of a thin strided layer (s2d_st > 0): row j' of D is (r2, s2, dy, dx, c) of the regrouped
     // input and maps to column ((st*r2+dy)*s2d_S + st*s2d+dx)*s2d_Cin + c of the gradient, or to nothing
@@ -87,7 +89,7 @@ struct TcParams {
 
 // A launch serves up to N layers: the table of their tensor maps and parameters travels as a kernel parameter, and every
 // block finds its layer by its index (first[] ascending).  N = 1 for a call on its own.
-constexpr int kTcLayers = 48, kSsumLayers = 40;      // layers per grouped launch: a table stays below the 32 KB a launch may carry
+constexpr int kTcLayers = 54, kSsumLayers = 44;      // layers per grouped launch: a table stays below the 32 KB a launch may carry
 template <typename P, int MAPS>
 struct alignas(64) TcEntry { CUtensorMap map[MAPS]; P p; };
 template <typename P, int MAPS, int N>
@@ -646,7 +648,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                 if (n < p.B) {
                     const float *pn = p.partial + (long long)n * p.slots;
                     for (int i = sub; i < p.w_slots; i += 8) sw += (double)__ldcg(pn + i);
-                    for (int i = p.w_slots + sub; i < p.slots; i += 8) sb += (double)__ldcg(pn + i);
+                    for (int i = p.w_slots + sub; i < p.fold_slots; i += 8) sb += (double)__ldcg(pn + i);
                 }
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) {
@@ -2124,7 +2126,7 @@ static dp_status fill_conv_tc(int dtype, int epilogue, const void *X, const void
     p.G_w = G_w; p.partial = partial; p.slots = slots;
     p.splits = 1; p.per_split = g.B; p.factor = factor; p.sum_out = acc_w;
     if (!clip && publish) {
-        p.counters = publish->counters; p.w_slots = publish->w_slots; p.separate = publish->separate;
+        p.counters = publish->counters; p.w_slots = publish->w_slots; p.separate = publish->separate; p.fold_slots = slots;
         p.sqnorm = publish->sqnorm; p.sq_stride = publish->sq_stride;
         p.factor_out = publish->factor_out; p.C_l = publish->C_l; p.clip_out = publish->clip_out;
     }
@@ -2448,8 +2450,8 @@ int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias) {
     return kConvSingle;
 }
 
-// The longest walk of a block: a third of the GPU's share of all the layers' work (so that the blocks can be spread
-// evenly), within 8 and 60 microseconds (a block costs some 3 to start and end).
+// The longest walk of a block: the GPU's share of all the layers' work in as many rounds of blocks as keep each near 30
+// microseconds (a block costs some 4 to start and end; several rounds even out what the estimates get wrong), at most four.
 double conv_batch_walk(const std::vector<ConvJob> &jobs) {
     BatchPlanning planning(120000.0);
     double cycles = 0.0;
@@ -2462,9 +2464,9 @@ double conv_batch_walk(const std::vector<ConvJob> &jobs) {
         else continue;
         cycles += pl.item_cycles * j.g.B * pl.m_tiles * pl.n_tiles;
     }
-    double walk = 15000.0;
-    while (walk * 2.0 <= std::min(120000.0, cycles / sm_count() / 3.0)) walk *= 2.0;
-    return walk;
+    const double share = cycles / sm_count();
+    const double walk = share / std::max(1.0, std::min(4.0, std::floor(share / 55000.0)));
+    return std::max(8000.0, std::min(120000.0, std::ceil(walk / 1000.0) * 1000.0));
 }
 
 template <typename P, int MAPS, int N>
@@ -2528,6 +2530,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             rc = fill_conv_tc(j.dtype, j.epi, X, j.dY, j.g, pr, pl, j.G_w, j.partial, j.slots, nullptr, nullptr, j.tc_workspace, status, &pub, q.e);
             if (rc != DP_OK) return rc;
             TcParams &p = q.e.p;
+            if (j.bias_apart) { p.separate = 0; p.fold_slots = j.w_slots; }
             p.run = std::max(1, std::min(p.total_tiles, (int)(walk / pl.item_cycles)));
             p.blocks = q.blocks = (p.total_tiles + p.run - 1) / p.run;
             q.smem = pl.smem; q.cost = p.run * pl.item_cycles;

@@ -70,6 +70,7 @@ struct ConvJob {
     const void *X, *dY;
     float *G_w, *partial;        // stored gradients; per-example partial squared norms [B][slots]
     int slots, w_slots, separate;
+    int bias_apart;              // the bias group's norms are somebody else's: fold and publish the weights' only
     int *counter;                // cleared ticket word
     TcInlineClip clip;           // where norms (and factors) go
     float *factor;               // [B][2] scratch

@@ -70,8 +70,8 @@ class GlobalClipStep:
 
     def __init__(self, layers, B, dtype, C, sigma, impl=b.DP_IMPL_AUTO, device="cuda", per_example_noise=False, lanes=1,
                  recompute="none"):
-        """lanes > 1: chunk() spreads the layers' calls over that many CUDA streams (a workspace each) and joins them
-        around the factor computation: the calls write disjoint buffers, so they may overlap."""
+        """The first-pass calls of a chunk run as one batch.  lanes > 1: the second pass of recomputed layers spreads over that
+        many CUDA streams (a workspace each): the calls write disjoint buffers, so they may overlap."""
         self.layers, self.B, self.dtype, self.C, self.sigma = list(layers), B, dtype, float(C), float(sigma)
         self.per_example_noise = bool(per_example_noise)
         self.tensors = _tensors_of(self.layers)
@@ -101,7 +101,13 @@ class GlobalClipStep:
         self._kept = [i for i, k in enumerate(kept) if k]
         self.norms = torch.empty(B, dtype=torch.float32, device=device)
         self.clip = torch.empty(B, dtype=torch.float32, device=device)
-        ws = max([b.dp_workspace_bytes(d, e) for d in self.descs for e in (b.DP_EPI_STORE_NORM, b.DP_EPI_NORM_ONLY, b.DP_EPI_CLIP_ACCUM)] + [256])
+        self.batch = b.Batch(self.descs, [b.DP_EPI_NORM_ONLY if li in self.recompute else b.DP_EPI_STORE_NORM
+                                          for li in range(len(self.layers))])
+        for li, col in enumerate(self._col):
+            self.batch.set(li, sqnorm=self.sq.data_ptr() + 4 * col, sqnorm_stride=self.L, G_w=self.G[col],
+                           G_b=self.G[col + 1] if self.layers[li].n_bias else None)
+        ws = max([b.dp_workspace_bytes(d, e) for d in self.descs for e in (b.DP_EPI_STORE_NORM, b.DP_EPI_NORM_ONLY, b.DP_EPI_CLIP_ACCUM)] +
+                 [256, self.batch.workspace_bytes])
         self.lanes = max(1, min(int(lanes), len(self.layers)))
         self.ws_lane = _workspaces(ws, self.lanes, device)
         self.ws = self.ws_lane[0]
@@ -183,9 +189,8 @@ class GlobalClipStep:
             main.wait_event(done)
 
     def wgrad_all(self, inputs):
-        """Every layer's first-pass call: in order on the current stream, or forked over the lanes and joined."""
-        self._forked([(lambda lane, stream, li=li, X=X, dY=dY: self.wgrad(li, X, dY, lane, stream))
-                      for li, (X, dY) in enumerate(inputs)])
+        """Every layer's first-pass call, as one batch."""
+        b.check(self.batch.run(inputs, 0.0, self.ws), "dp_batch_run")
 
     def clip_accumulate(self, use_epilogue_norms=True, inputs=None):
         """Factors from the norm table, then the clipped sums: over memory for the kept tensors, by a second pass over
@@ -283,9 +288,8 @@ class PerLayerClipStep:
     no per-example gradient is written to memory."""
 
     def __init__(self, layers, B, dtype, C, sigma, impl=b.DP_IMPL_AUTO, device="cuda", lanes=1):
-        """lanes > 1: chunk() spreads the layer calls over that many CUDA streams (each with a workspace of its own).
-        The calls of one chunk touch disjoint outputs, so they may overlap; a chunk of few examples leaves most of
-        the GPU idle inside any single call."""
+        """The layer calls of a chunk run as one batch, whatever `lanes` is; lanes > 1 gives wgrad() that many workspaces for
+        single layer calls that overlap on streams of the caller."""
         self.layers, self.B, self.dtype, self.C, self.sigma = list(layers), B, dtype, float(C), float(sigma)
         self.tensors = _tensors_of(self.layers)
         self.L = len(self.tensors)
@@ -348,7 +352,7 @@ class PerLayerClipStep:
         return self._batches[layers]
 
     def chunk_calls(self, inputs, only=None):
-        """The layer calls of one chunk: in order on the current stream, or forked over the lanes and joined again.
+        """The layer calls of one chunk, as one batch on the current stream.
         only: a set of layer indices to restrict the chunk to (measurements of one kind of layer)."""
         if only is None:
             batch = self.batch
