@@ -8,6 +8,8 @@ from __future__ import annotations
 import ctypes
 import os
 
+import torch
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libdpstep.so")
 
@@ -15,6 +17,14 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2109_12191_b200.build` "
                       "(there is no CPU or PyTorch fallback)")
 _lib = ctypes.CDLL(LIB_PATH)
+
+# The calls of a training step go through a small extension module (marshalling in C); the rest through ctypes.
+from . import _pycall  # noqa: E402
+from ._pycall import (dp_clip_accumulate, dp_clip_accumulate_grouped, dp_clip_accumulate_micro, dp_clip_accumulate_noised,  # noqa: E402,F401
+                      dp_clip_accumulate_static, dp_clip_factors, dp_noise_average, dp_noise_average_sgd, dp_per_example_wgrad,
+                      dp_per_example_wgrad_scaled, dp_scale_accumulate)
+_pycall.set_torch(getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None),
+                  torch.cuda.current_stream)
 
 # enums of dpstep.h
 DP_OK, DP_ERR_INVALID_ARG, DP_ERR_UNSUPPORTED, DP_ERR_WORKSPACE, DP_ERR_CUDA, DP_ERR_TIMEOUT = range(6)
@@ -63,40 +73,14 @@ _dp = ctypes.POINTER(dp_layer_desc)
 _lib.dp_layer_groups.argtypes = [_dp]; _lib.dp_layer_groups.restype = _i
 _lib.dp_workspace_bytes.argtypes = [_dp, _i]; _lib.dp_workspace_bytes.restype = _sz
 _lib.dp_wgrad_uses_tensor_cores.argtypes = [_dp, _i]; _lib.dp_wgrad_uses_tensor_cores.restype = _i
-_lib.dp_per_example_wgrad.argtypes = [_dp, _vp, _vp, _vp, _vp, _vp, _ll, _i, _f, _vp, _vp, _vp, _vp, _sz, _vp]
-_lib.dp_per_example_wgrad.restype = _i
-_lib.dp_per_example_wgrad_scaled.argtypes = [_dp, _vp, _vp, _vp, _vp, _ll, _vp, _vp, _vp, _sz, _vp]
-_lib.dp_per_example_wgrad_scaled.restype = _i
-_lib.dp_clip_factors.argtypes = [_i, _i, _i, _vp, _f, _vp, _vp, _vp]; _lib.dp_clip_factors.restype = _i
-_lib.dp_scale_accumulate.argtypes = [_i, _i, ctypes.POINTER(_vp), ctypes.POINTER(_ll), _vp, _i, ctypes.POINTER(_vp), _vp]
-_lib.dp_scale_accumulate.restype = _i
 _lib.dp_clip_workspace_bytes.argtypes = [_i, _i, ctypes.POINTER(_ll)]; _lib.dp_clip_workspace_bytes.restype = _sz
-_lib.dp_clip_accumulate.argtypes = [_i, _i, _i, ctypes.POINTER(_vp), ctypes.POINTER(_ll), _vp, _f,
-                                    ctypes.POINTER(_vp), _vp, _vp, _vp, _sz, _vp]
-_lib.dp_clip_accumulate.restype = _i
-_lib.dp_clip_accumulate_noised.argtypes = [_i, _i, _i, ctypes.POINTER(_vp), ctypes.POINTER(_ll), ctypes.POINTER(_ll), _vp,
-                                           _f, _f, _ll, _ull, _ull, _ll, ctypes.POINTER(_vp), _vp, _vp, _vp, _sz, _vp]
-_lib.dp_clip_accumulate_noised.restype = _i
 _lib.dp_debug_example_noise_z.argtypes = [_vp, _ll, _ll, _ll, _ull, _ull, _vp]; _lib.dp_debug_example_noise_z.restype = _i
-_lib.dp_clip_accumulate_grouped.argtypes = [_i, _i, _i, ctypes.POINTER(_i), ctypes.POINTER(_vp), ctypes.POINTER(_ll), _vp, _f,
-                                            ctypes.POINTER(_vp), _vp, _vp, _vp, _sz, _vp]
-_lib.dp_clip_accumulate_grouped.restype = _i
-_lib.dp_clip_accumulate_micro.argtypes = [_i, _i, _i, ctypes.POINTER(_vp), ctypes.POINTER(_ll), _f, ctypes.POINTER(_vp), _vp,
-                                          _vp, _vp, _sz, _vp]
-_lib.dp_clip_accumulate_micro.restype = _i
-_lib.dp_clip_accumulate_static.argtypes = [_i, _i, _i, ctypes.POINTER(_vp), ctypes.POINTER(_ll), _vp, _f,
-                                           ctypes.POINTER(_vp), _vp, _vp, _vp]
-_lib.dp_clip_accumulate_static.restype = _i
 _lib.dp_clip_static_scratch_bytes.argtypes = []; _lib.dp_clip_static_scratch_bytes.restype = _sz
-_lib.dp_noise_average.argtypes = [_vp, _ll, _ll, _f, _f, _ll, _ull, _ull, _vp, _vp]; _lib.dp_noise_average.restype = _i
-_lib.dp_noise_average_sgd.argtypes = [_vp, _ll, _ll, _f, _f, _ll, _ull, _ull, _f, _f, _vp, _vp, _vp, _vp]
-_lib.dp_noise_average_sgd.restype = _i
 _lib.dp_debug_philox_raw.argtypes = [_vp, _ll, _ll, _ull, _ull, _vp]; _lib.dp_debug_philox_raw.restype = _i
 _lib.dp_debug_noise_z.argtypes = [_vp, _ll, _ll, _ull, _ull, _vp]; _lib.dp_debug_noise_z.restype = _i
 _lib.dp_batch_create.argtypes = [_i, _dp, ctypes.POINTER(_i), ctypes.POINTER(_vp)]; _lib.dp_batch_create.restype = _i
 _lib.dp_batch_destroy.argtypes = [_vp]; _lib.dp_batch_destroy.restype = None
 _lib.dp_batch_workspace_bytes.argtypes = [_vp]; _lib.dp_batch_workspace_bytes.restype = _sz
-_lib.dp_batch_run.argtypes = [_vp, _vp, _f, _vp, _sz, _vp]; _lib.dp_batch_run.restype = _i
 _lib.dp_wgrad_check.argtypes = [_vp, _vp]; _lib.dp_wgrad_check.restype = _i
 _lib.dp_workspace_init.argtypes = [_vp, _sz, _vp]; _lib.dp_workspace_init.restype = _i
 _lib.dp_debug_set_wait_polls.argtypes = [_ll]; _lib.dp_debug_set_wait_polls.restype = None
@@ -125,7 +109,6 @@ def _nbytes(t):
 
 def _stream(stream):
     if stream is None:
-        import torch
         return torch.cuda.current_stream().cuda_stream
     return getattr(stream, "cuda_stream", stream)
 
@@ -147,114 +130,17 @@ def dp_wgrad_uses_tensor_cores(desc, epilogue):
     return _lib.dp_wgrad_uses_tensor_cores(ctypes.byref(desc), epilogue)
 
 
-def dp_per_example_wgrad(desc, X, dY, G_w, G_b, sqnorm, sqnorm_stride, epilogue, C_l, acc_w, acc_b, clip_out,
-                         workspace, workspace_bytes=None, stream=None):
-    if workspace_bytes is None:
-        workspace_bytes = 0 if workspace is None or isinstance(workspace, int) else _nbytes(workspace)
-    return _lib.dp_per_example_wgrad(ctypes.byref(desc) if desc is not None else None, _ptr(X), _ptr(dY), _ptr(G_w),
-                                     _ptr(G_b), _ptr(sqnorm), sqnorm_stride, epilogue, C_l, _ptr(acc_w), _ptr(acc_b),
-                                     _ptr(clip_out), _ptr(workspace), workspace_bytes, _stream(stream))
-
-
-def dp_per_example_wgrad_scaled(desc, X, dY, factor_w, factor_b, factor_stride, acc_w, acc_b, workspace, workspace_bytes=None,
-                                stream=None):
-    if workspace_bytes is None:
-        workspace_bytes = 0 if workspace is None or isinstance(workspace, int) else _nbytes(workspace)
-    return _lib.dp_per_example_wgrad_scaled(ctypes.byref(desc) if desc is not None else None, _ptr(X), _ptr(dY), _ptr(factor_w),
-                                            _ptr(factor_b), factor_stride, _ptr(acc_w), _ptr(acc_b), _ptr(workspace),
-                                            workspace_bytes, _stream(stream))
-
-
-def dp_clip_factors(mode, B, L, sqnorm, C, norms_out, factors_out, stream=None):
-    return _lib.dp_clip_factors(mode, B, L, _ptr(sqnorm), C, _ptr(norms_out), _ptr(factors_out), _stream(stream))
-
-
-def dp_scale_accumulate(B, G, P_l, factor, per_tensor, acc, stream=None):
-    L = len(P_l)
-    Gp = (_vp * L)(*[_ptr(g) for g in G]) if G is not None else None
-    Ap = (_vp * L)(*[_ptr(a) for a in acc]) if acc is not None else None
-    return _lib.dp_scale_accumulate(B, L, Gp, (_ll * L)(*P_l), _ptr(factor), per_tensor, Ap, _stream(stream))
-
-
 def dp_clip_workspace_bytes(B, P_l):
     L = len(P_l)
     return _lib.dp_clip_workspace_bytes(B, L, (_ll * L)(*P_l))
-
-
-def dp_clip_accumulate(mode, B, G, P_l, sqnorm, C, acc, norms_out, clip_out, workspace, workspace_bytes=None,
-                       stream=None):
-    L = len(P_l)
-    if workspace_bytes is None:
-        workspace_bytes = 0 if workspace is None or isinstance(workspace, int) else _nbytes(workspace)
-    Gp = (_vp * L)(*[_ptr(g) for g in G]) if G is not None else None
-    Ap = (_vp * L)(*[_ptr(a) for a in acc]) if acc is not None else None
-    return _lib.dp_clip_accumulate(mode, B, L, Gp, (_ll * L)(*P_l), _ptr(sqnorm), C, Ap, _ptr(norms_out),
-                                   _ptr(clip_out), _ptr(workspace), workspace_bytes, _stream(stream))
-
-
-def dp_clip_accumulate_noised(mode, B, G, P_l, param_offset_l, sqnorm, C, sigma, total_batch, seed, step, example0, acc,
-                              norms_out, clip_out, workspace, workspace_bytes=None, stream=None):
-    """dp_clip_accumulate with each example's own noise draw added before the sum."""
-    L = len(P_l)
-    if workspace_bytes is None:
-        workspace_bytes = 0 if workspace is None or isinstance(workspace, int) else _nbytes(workspace)
-    Gp = (_vp * L)(*[_ptr(g) for g in G]) if G is not None else None
-    Ap = (_vp * L)(*[_ptr(a) for a in acc]) if acc is not None else None
-    Op = (_ll * L)(*param_offset_l) if param_offset_l is not None else None
-    return _lib.dp_clip_accumulate_noised(mode, B, L, Gp, (_ll * L)(*P_l), Op, _ptr(sqnorm), C, sigma, total_batch, seed,
-                                          step, example0, Ap, _ptr(norms_out), _ptr(clip_out), _ptr(workspace),
-                                          workspace_bytes, _stream(stream))
 
 
 def dp_debug_example_noise_z(z, count, first_index, example, seed, step, stream=None):
     return _lib.dp_debug_example_noise_z(_ptr(z), count, first_index, example, seed, step, _stream(stream))
 
 
-def dp_clip_accumulate_grouped(B, M, group_of, G, P_l, sqnorm, C, acc, norms_out, clip_out, workspace, workspace_bytes=None,
-                               stream=None):
-    """dp_clip_accumulate over M groups of tensors, each clipped to C/sqrt(M)."""
-    L = len(P_l)
-    if workspace_bytes is None:
-        workspace_bytes = 0 if workspace is None or isinstance(workspace, int) else _nbytes(workspace)
-    Gp = (_vp * L)(*[_ptr(g) for g in G]) if G is not None else None
-    Ap = (_vp * L)(*[_ptr(a) for a in acc]) if acc is not None else None
-    go = (_i * L)(*group_of) if group_of is not None else None
-    return _lib.dp_clip_accumulate_grouped(B, L, M, go, Gp, (_ll * L)(*P_l), _ptr(sqnorm), C, Ap, _ptr(norms_out),
-                                           _ptr(clip_out), _ptr(workspace), workspace_bytes, _stream(stream))
-
-
-def dp_clip_accumulate_micro(B, micro, G, P_l, C, acc, norms_out, clip_out, workspace, workspace_bytes=None, stream=None):
-    """Whole-model clipping of the means of runs of `micro` consecutive examples."""
-    L = len(P_l)
-    if workspace_bytes is None:
-        workspace_bytes = 0 if workspace is None or isinstance(workspace, int) else _nbytes(workspace)
-    Gp = (_vp * L)(*[_ptr(g) for g in G]) if G is not None else None
-    Ap = (_vp * L)(*[_ptr(a) for a in acc]) if acc is not None else None
-    return _lib.dp_clip_accumulate_micro(B, L, micro, Gp, (_ll * L)(*P_l), C, Ap, _ptr(norms_out), _ptr(clip_out),
-                                         _ptr(workspace), workspace_bytes, _stream(stream))
-
-
-def dp_clip_accumulate_static(mode, B, G, P_l, sqnorm, C, acc, norms_out, clip_out, stream=None):
-    """dp_clip_accumulate with the library's built-in scratch array instead of a caller workspace."""
-    L = len(P_l)
-    Gp = (_vp * L)(*[_ptr(g) for g in G]) if G is not None else None
-    Ap = (_vp * L)(*[_ptr(a) for a in acc]) if acc is not None else None
-    return _lib.dp_clip_accumulate_static(mode, B, L, Gp, (_ll * L)(*P_l), _ptr(sqnorm), C, Ap, _ptr(norms_out),
-                                          _ptr(clip_out), _stream(stream))
-
-
 def dp_clip_static_scratch_bytes():
     return _lib.dp_clip_static_scratch_bytes()
-
-
-def dp_noise_average(acc, P, param_offset, sigma, C, total_batch, seed, step, out, stream=None):
-    return _lib.dp_noise_average(_ptr(acc), P, param_offset, sigma, C, total_batch, seed, step, _ptr(out), _stream(stream))
-
-
-def dp_noise_average_sgd(acc, P, param_offset, sigma, C, total_batch, seed, step, lr, momentum, theta, momentum_buf=None,
-                         g_out=None, stream=None):
-    return _lib.dp_noise_average_sgd(_ptr(acc), P, param_offset, sigma, C, total_batch, seed, step, lr, momentum,
-                                     _ptr(theta), _ptr(momentum_buf), _ptr(g_out), _stream(stream))
 
 
 class Batch:
@@ -273,9 +159,7 @@ class Batch:
 
     def run(self, inputs, C_l, workspace, stream=None):
         """inputs: (X, dY) of every layer, in order."""
-        for io, (X, dY) in zip(self.io, inputs, strict=True):
-            io.X, io.dY = _ptr(X), _ptr(dY)
-        return _lib.dp_batch_run(self._handle, self.io, C_l, _ptr(workspace), _nbytes(workspace), _stream(stream))
+        return _pycall.batch_run(self._handle.value, self.io, inputs, C_l, workspace, stream)
 
     def __del__(self):
         if getattr(self, "_handle", None) and _lib is not None:       # (module globals go first at interpreter exit)

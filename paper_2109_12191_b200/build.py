@@ -1,14 +1,17 @@
-"""Builds libdpstep.so (the CUDA library behind the C ABI) in-tree with nvcc for sm_100a."""
+"""Builds libdpstep.so (the CUDA library behind the C ABI) in-tree with nvcc for sm_100a, and with gcc the extension module
+through which Python calls it."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdpstep.so")
+EXT = os.path.join(HERE, "_pycall.so")
 
 
 def _nvcc() -> str:
@@ -30,8 +33,22 @@ def needs_build() -> bool:
     return any(os.path.getmtime(p) > t for p in deps)
 
 
+def build_extension(force: bool = False) -> str:
+    """The extension module; found next to the library it is linked against."""
+    deps = [os.path.join(CSRC, "pycall.c"), os.path.join(ROOT, "include", "dpstep.h")]
+    if not force and os.path.exists(EXT) and all(os.path.getmtime(p) <= os.path.getmtime(EXT) for p in deps):
+        return EXT
+    tmp = EXT + f".tmp{os.getpid()}"
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-I", os.path.join(ROOT, "include"), deps[0], "-o", tmp, "-L", HERE, "-l:libdpstep.so", "-Wl,-rpath,$ORIGIN"],
+                   check=True)
+    os.replace(tmp, EXT)
+    return EXT
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
+        build_extension()
         return LIB
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -42,6 +59,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd.insert(2, "-v")
     subprocess.run(cmd, check=True)
     os.replace(tmp, LIB)
+    build_extension(force)
     return LIB
 
 

@@ -25,6 +25,7 @@ struct dp_batch {
     std::vector<int> conv_item;                  // item of every conv
     double walk = 0.0;                           // conv_batch_walk() of all of them
     size_t singles = 0;                          // byte offset of the scratch the single calls share
+    bool used[BatchStreams::kCount] = {};        // streams that have launches of their own
     size_t total = 0;
     // Streams and events of the runs, made on the first run's device; host threads take turns at enqueueing.
     mutable std::mutex mu;
@@ -185,8 +186,17 @@ extern "C" dp_status dp_batch_create(int n, const dp_layer_desc *descs, const in
     plan_affine(*b, off);
     b->singles = off;
     size_t most = 0;
-    for (const auto &it : b->items)
-        if (it.group < 0 && it.plan.total > most) most = it.plan.total;
+    for (const auto &it : b->items) {
+        if (it.group >= 0) continue;
+        most = std::max(most, it.plan.total);
+        b->used[BatchStreams::kAffine] = true;
+    }
+    if (!b->affine.empty()) b->used[BatchStreams::kAffine] = true;
+    for (const ConvJob &j : b->convs) {
+        b->used[BatchStreams::kMain] = true;
+        if (conv_batch_clusters(j, b->walk)) b->used[BatchStreams::kClusters] = true;
+        if (j.kind == kConvGramSum || b->items[b->conv_item[&j - b->convs.data()]].desc.has_bias) b->used[BatchStreams::kSums] = true;
+    }
     b->total = most > kWsHeaderBytes ? round_up(off + most - kWsHeaderBytes, 256) : off;
     *out = b;
     return DP_OK;
@@ -221,12 +231,14 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
     // The launches of different kinds are independent: memory-bound normalisation layers and the blocks of small launches
     // fill what the tensor-core launches leave idle.
     BatchStreams streams;
-    const bool forked = n > 1 && side_streams(*b);
-    for (int i = 0; i < BatchStreams::kCount; ++i) streams.s[i] = forked && i ? b->side[i] : st;
-    streams.gram_done = forked ? b->gram_done : nullptr;
+    // (without convolutions there is nothing to fork from: everything stays on the caller's stream)
+    const bool forked = b->used[BatchStreams::kMain] && (b->used[1] || b->used[2] || b->used[3]) && side_streams(*b);
+    for (int i = 0; i < BatchStreams::kCount; ++i) streams.s[i] = forked && i && b->used[i] ? b->side[i] : st;
+    streams.gram_done = forked && b->used[BatchStreams::kSums] ? b->gram_done : nullptr;
     if (forked) {
         DP_CUDA_TRY(cudaEventRecord(b->fork, st));
-        for (int i = 1; i < BatchStreams::kCount; ++i) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->fork, 0));
+        for (int i = 1; i < BatchStreams::kCount; ++i)
+            if (b->used[i]) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->fork, 0));
     }
     // what is not a tensor-core launch of several layers: enqueued behind those, before the streams meet again
     auto others = [&]() -> dp_status {
@@ -246,6 +258,7 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
         const dp_status rc = others();
         if (!forked) return rc;
         for (int i = 1; i < BatchStreams::kCount; ++i) {
+            if (!b->used[i]) continue;
             DP_CUDA_TRY(cudaEventRecord(b->done[i], streams.s[i]));
             DP_CUDA_TRY(cudaStreamWaitEvent(st, b->done[i], 0));
         }

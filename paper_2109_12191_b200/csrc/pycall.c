@@ -1,0 +1,413 @@
+/* The entry points of dpstep.h as Python functions.  They only marshal arguments: a device pointer may come as a contiguous
+ * torch tensor, an integer address or None.  Written against the CPython API because a training step of a small model is
+ * a handful of calls, and a call through ctypes and Python wrappers costs several times what its launch does
+ * (dp_noise_average_sgd 8.7 us through ctypes, of which the C call 2.4). */
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <stdlib.h>
+#include <string.h>
+#include "dpstep.h"
+
+static PyObject *s_data_ptr, *s_is_contiguous, *s_nbytes, *s_cuda_stream;
+static PyObject *raw_stream, *get_device, *current_stream;      /* torch's, set by set_torch() */
+
+enum { MAX_ARGS = 24 };
+
+/* positional and keyword arguments into `out` by the names in `names`; the first `required` have to be there */
+static int collect(const char *fn, const char *const *names, int n, int required, PyObject *const *args, Py_ssize_t nargs,
+                   PyObject *kwnames, PyObject **out) {
+    if (nargs > n) { PyErr_Format(PyExc_TypeError, "%s() takes at most %d arguments (%zd given)", fn, n, nargs); return -1; }
+    for (int i = 0; i < n; ++i) out[i] = i < nargs ? args[i] : NULL;
+    const Py_ssize_t nkw = kwnames ? PyTuple_GET_SIZE(kwnames) : 0;
+    for (Py_ssize_t k = 0; k < nkw; ++k) {
+        PyObject *key = PyTuple_GET_ITEM(kwnames, k);
+        int i = 0;
+        while (i < n && PyUnicode_CompareWithASCIIString(key, names[i]) != 0) ++i;
+        if (i == n || out[i]) { PyErr_Format(PyExc_TypeError, "%s(): unexpected or repeated argument %R", fn, key); return -1; }
+        out[i] = args[nargs + k];
+    }
+    for (int i = 0; i < n; ++i) {
+        if (!out[i] && i < required) { PyErr_Format(PyExc_TypeError, "%s(): missing argument '%s'", fn, names[i]); return -1; }
+        if (!out[i]) out[i] = Py_None;
+    }
+    return 0;
+}
+
+/* device address of a tensor, an integer or None; -1 with an exception set on failure */
+static int address(PyObject *o, void **p) {
+    if (o == Py_None) { *p = NULL; return 0; }
+    if (PyLong_Check(o)) {
+        *p = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(o);
+        return PyErr_Occurred() ? -1 : 0;
+    }
+    PyObject *args[1] = {o};
+    PyObject *r = PyObject_VectorcallMethod(s_is_contiguous, args, 1 | PY_VECTORCALL_ARGUMENTS_OFFSET, NULL);
+    if (!r) return -1;
+    const int ok = PyObject_IsTrue(r);
+    Py_DECREF(r);
+    if (ok < 0) return -1;
+    if (!ok) { PyErr_SetString(PyExc_ValueError, "tensor must be contiguous"); return -1; }
+    r = PyObject_VectorcallMethod(s_data_ptr, args, 1 | PY_VECTORCALL_ARGUMENTS_OFFSET, NULL);
+    if (!r) return -1;
+    *p = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(r);
+    Py_DECREF(r);
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+static int whole(PyObject *o, long long *v) {
+    if (PyLong_Check(o)) { *v = (long long)PyLong_AsUnsignedLongLongMask(o); return PyErr_Occurred() ? -1 : 0; }
+    PyObject *i = PyNumber_Index(o);
+    if (!i) return -1;
+    *v = (long long)PyLong_AsUnsignedLongLongMask(i);
+    Py_DECREF(i);
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+static int real(PyObject *o, float *v) {
+    const double d = PyFloat_AsDouble(o);
+    if (d == -1.0 && PyErr_Occurred()) return -1;
+    *v = (float)d;
+    return 0;
+}
+
+/* None: the stream torch is on; else an integer handle or a torch stream */
+static int stream_of(PyObject *o, void **p) {
+    PyObject *r;
+    if (o == Py_None && raw_stream) {
+        PyObject *dev = PyObject_CallNoArgs(get_device);
+        if (!dev) return -1;
+        r = PyObject_CallOneArg(raw_stream, dev);
+        Py_DECREF(dev);
+    } else if (o == Py_None) {
+        PyObject *s = current_stream ? PyObject_CallNoArgs(current_stream) : NULL;
+        if (!s) { if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, "set_torch() has not been called"); return -1; }
+        r = PyObject_GetAttr(s, s_cuda_stream);
+        Py_DECREF(s);
+    } else if (PyLong_Check(o)) {
+        r = Py_NewRef(o);
+    } else {
+        r = PyObject_GetAttr(o, s_cuda_stream);
+    }
+    if (!r) return -1;
+    *p = (void *)(uintptr_t)PyLong_AsUnsignedLongLongMask(r);
+    Py_DECREF(r);
+    return PyErr_Occurred() ? -1 : 0;
+}
+
+/* size of a workspace: as given, or that of the tensor (0 for None and addresses) */
+static int bytes_of(PyObject *given, PyObject *workspace, size_t *n) {
+    *n = 0;
+    PyObject *r;
+    if (given != Py_None) r = Py_NewRef(given);
+    else if (workspace == Py_None || PyLong_Check(workspace)) return 0;
+    else r = PyObject_GetAttr(workspace, s_nbytes);
+    if (!r) return -1;
+    long long v;
+    const int rc = whole(r, &v);
+    Py_DECREF(r);
+    *n = (size_t)v;
+    return rc;
+}
+
+/* a ctypes structure (or None) as a pointer to its memory, which outlives the call with the object */
+static int structure(PyObject *o, size_t size, void **p) {
+    *p = NULL;
+    if (o == Py_None) return 0;
+    Py_buffer view;
+    if (PyObject_GetBuffer(o, &view, PyBUF_SIMPLE) < 0) return -1;
+    const int ok = (size_t)view.len >= size;
+    *p = view.buf;
+    PyBuffer_Release(&view);
+    if (!ok) { PyErr_SetString(PyExc_TypeError, "structure too small"); return -1; }
+    return 0;
+}
+
+/* a sequence of addresses / integers (or None) as a C array, freed by the caller; n < 0: any length, written back */
+static int addresses(PyObject *o, Py_ssize_t n, void ***out) {
+    *out = NULL;
+    if (o == Py_None) return 0;
+    PyObject *seq = PySequence_Fast(o, "expected a sequence of tensors");
+    if (!seq) return -1;
+    if (PySequence_Fast_GET_SIZE(seq) < n) { Py_DECREF(seq); PyErr_SetString(PyExc_ValueError, "a tensor list is shorter than P_l"); return -1; }
+    void **a = malloc(sizeof(void *) * (size_t)(n > 0 ? n : 1));
+    int rc = a ? 0 : -1;
+    for (Py_ssize_t i = 0; i < n && rc == 0; ++i) rc = address(PySequence_Fast_GET_ITEM(seq, i), &a[i]);
+    Py_DECREF(seq);
+    if (rc < 0) { free(a); if (!PyErr_Occurred()) PyErr_NoMemory(); return -1; }
+    *out = a;
+    return 0;
+}
+static int wholes(PyObject *o, Py_ssize_t *n, long long **out) {
+    *out = NULL;
+    if (o == Py_None) return 0;
+    PyObject *seq = PySequence_Fast(o, "expected a sequence of integers");
+    if (!seq) return -1;
+    const Py_ssize_t have = PySequence_Fast_GET_SIZE(seq);
+    if (*n < 0) *n = have;
+    long long *a = have >= *n ? malloc(sizeof(long long) * (size_t)(*n > 0 ? *n : 1)) : NULL;
+    int rc = a ? 0 : -1;
+    for (Py_ssize_t i = 0; i < *n && rc == 0; ++i) rc = whole(PySequence_Fast_GET_ITEM(seq, i), &a[i]);
+    Py_DECREF(seq);
+    if (rc < 0) { free(a); if (!PyErr_Occurred()) PyErr_SetString(PyExc_ValueError, "an integer list is shorter than P_l"); return -1; }
+    *out = a;
+    return 0;
+}
+
+#define CALL(rc, expr) do { Py_BEGIN_ALLOW_THREADS rc = (expr); Py_END_ALLOW_THREADS } while (0)
+#define ARGS(fn, required, ...)                                                                                        \
+    static const char *const names[] = {__VA_ARGS__};                                                                  \
+    PyObject *a[MAX_ARGS];                                                                                              \
+    if (collect(fn, names, (int)(sizeof(names) / sizeof(names[0])), required, args, nargs, kwnames, a) < 0) return NULL
+
+static PyObject *per_example_wgrad(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_per_example_wgrad", 13, "desc", "X", "dY", "G_w", "G_b", "sqnorm", "sqnorm_stride", "epilogue", "C_l", "acc_w", "acc_b",
+         "clip_out", "workspace", "workspace_bytes", "stream");
+    void *d, *X, *dY, *G_w, *G_b, *sq, *acc_w, *acc_b, *clip, *ws, *st;
+    long long stride, epi;
+    float C_l;
+    size_t bytes;
+    if (structure(a[0], sizeof(dp_layer_desc), &d) < 0 || address(a[1], &X) < 0 || address(a[2], &dY) < 0 || address(a[3], &G_w) < 0 ||
+        address(a[4], &G_b) < 0 || address(a[5], &sq) < 0 || whole(a[6], &stride) < 0 || whole(a[7], &epi) < 0 || real(a[8], &C_l) < 0 ||
+        address(a[9], &acc_w) < 0 || address(a[10], &acc_b) < 0 || address(a[11], &clip) < 0 || address(a[12], &ws) < 0 ||
+        bytes_of(a[13], a[12], &bytes) < 0 || stream_of(a[14], &st) < 0)
+        return NULL;
+    int rc;
+    CALL(rc, dp_per_example_wgrad(d, X, dY, G_w, G_b, sq, stride, (int)epi, C_l, acc_w, acc_b, clip, ws, bytes, st));
+    return PyLong_FromLong(rc);
+}
+
+static PyObject *per_example_wgrad_scaled(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_per_example_wgrad_scaled", 9, "desc", "X", "dY", "factor_w", "factor_b", "factor_stride", "acc_w", "acc_b", "workspace",
+         "workspace_bytes", "stream");
+    void *d, *X, *dY, *fw, *fb, *acc_w, *acc_b, *ws, *st;
+    long long stride;
+    size_t bytes;
+    if (structure(a[0], sizeof(dp_layer_desc), &d) < 0 || address(a[1], &X) < 0 || address(a[2], &dY) < 0 || address(a[3], &fw) < 0 ||
+        address(a[4], &fb) < 0 || whole(a[5], &stride) < 0 || address(a[6], &acc_w) < 0 || address(a[7], &acc_b) < 0 ||
+        address(a[8], &ws) < 0 || bytes_of(a[9], a[8], &bytes) < 0 || stream_of(a[10], &st) < 0)
+        return NULL;
+    int rc;
+    CALL(rc, dp_per_example_wgrad_scaled(d, X, dY, fw, fb, stride, acc_w, acc_b, ws, bytes, st));
+    return PyLong_FromLong(rc);
+}
+
+static PyObject *clip_factors(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_clip_factors", 7, "mode", "B", "L", "sqnorm", "C", "norms_out", "factors_out", "stream");
+    long long mode, B, L;
+    void *sq, *norms, *factors, *st;
+    float C;
+    if (whole(a[0], &mode) < 0 || whole(a[1], &B) < 0 || whole(a[2], &L) < 0 || address(a[3], &sq) < 0 || real(a[4], &C) < 0 ||
+        address(a[5], &norms) < 0 || address(a[6], &factors) < 0 || stream_of(a[7], &st) < 0)
+        return NULL;
+    int rc;
+    CALL(rc, dp_clip_factors((int)mode, (int)B, (int)L, sq, C, norms, factors, st));
+    return PyLong_FromLong(rc);
+}
+
+/* what the clipped sums over stored gradients share: the tensor lists */
+typedef struct { Py_ssize_t L; long long *P; void **G, **acc; long long *more; } Lists;
+static int lists(PyObject *P_l, PyObject *G, PyObject *acc, PyObject *more, Lists *t) {
+    memset(t, 0, sizeof(*t));
+    t->L = -1;
+    if (wholes(P_l, &t->L, &t->P) < 0) return -1;
+    if (t->L < 0) { PyErr_SetString(PyExc_TypeError, "P_l must be a sequence"); return -1; }
+    if (addresses(G, t->L, &t->G) < 0 || addresses(acc, t->L, &t->acc) < 0) return -1;
+    return wholes(more, &t->L, &t->more);
+}
+static PyObject *done(Lists *t, int failed, int rc) {
+    free(t->P); free(t->G); free(t->acc); free(t->more);
+    return failed ? NULL : PyLong_FromLong(rc);
+}
+
+static PyObject *scale_accumulate(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_scale_accumulate", 6, "B", "G", "P_l", "factor", "per_tensor", "acc", "stream");
+    Lists t;
+    long long B, per;
+    void *factor, *st;
+    int rc = 0;
+    if (lists(a[2], a[1], a[5], Py_None, &t) < 0 || whole(a[0], &B) < 0 || address(a[3], &factor) < 0 || whole(a[4], &per) < 0 ||
+        stream_of(a[6], &st) < 0)
+        return done(&t, 1, 0);
+    CALL(rc, dp_scale_accumulate((int)B, (int)t.L, (const float *const *)t.G, t.P, factor, (int)per, (float *const *)t.acc, st));
+    return done(&t, 0, rc);
+}
+
+static PyObject *clip_accumulate(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_clip_accumulate", 10, "mode", "B", "G", "P_l", "sqnorm", "C", "acc", "norms_out", "clip_out", "workspace", "workspace_bytes",
+         "stream");
+    Lists t;
+    long long mode, B;
+    void *sq, *norms, *clip, *ws, *st;
+    float C;
+    size_t bytes;
+    int rc = 0;
+    if (lists(a[3], a[2], a[6], Py_None, &t) < 0 || whole(a[0], &mode) < 0 || whole(a[1], &B) < 0 || address(a[4], &sq) < 0 ||
+        real(a[5], &C) < 0 || address(a[7], &norms) < 0 || address(a[8], &clip) < 0 || address(a[9], &ws) < 0 ||
+        bytes_of(a[10], a[9], &bytes) < 0 || stream_of(a[11], &st) < 0)
+        return done(&t, 1, 0);
+    CALL(rc, dp_clip_accumulate((int)mode, (int)B, (int)t.L, (const float *const *)t.G, t.P, sq, C, (float *const *)t.acc, norms, clip, ws, bytes, st));
+    return done(&t, 0, rc);
+}
+
+static PyObject *clip_accumulate_static(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_clip_accumulate_static", 9, "mode", "B", "G", "P_l", "sqnorm", "C", "acc", "norms_out", "clip_out", "stream");
+    Lists t;
+    long long mode, B;
+    void *sq, *norms, *clip, *st;
+    float C;
+    int rc = 0;
+    if (lists(a[3], a[2], a[6], Py_None, &t) < 0 || whole(a[0], &mode) < 0 || whole(a[1], &B) < 0 || address(a[4], &sq) < 0 ||
+        real(a[5], &C) < 0 || address(a[7], &norms) < 0 || address(a[8], &clip) < 0 || stream_of(a[9], &st) < 0)
+        return done(&t, 1, 0);
+    CALL(rc, dp_clip_accumulate_static((int)mode, (int)B, (int)t.L, (const float *const *)t.G, t.P, sq, C, (float *const *)t.acc, norms, clip, st));
+    return done(&t, 0, rc);
+}
+
+static PyObject *clip_accumulate_noised(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_clip_accumulate_noised", 16, "mode", "B", "G", "P_l", "param_offset_l", "sqnorm", "C", "sigma", "total_batch", "seed", "step",
+         "example0", "acc", "norms_out", "clip_out", "workspace", "workspace_bytes", "stream");
+    Lists t;
+    long long mode, B, total, seed, step, example0;
+    void *sq, *norms, *clip, *ws, *st;
+    float C, sigma;
+    size_t bytes;
+    int rc = 0;
+    if (lists(a[3], a[2], a[12], a[4], &t) < 0 || whole(a[0], &mode) < 0 || whole(a[1], &B) < 0 || address(a[5], &sq) < 0 ||
+        real(a[6], &C) < 0 || real(a[7], &sigma) < 0 || whole(a[8], &total) < 0 || whole(a[9], &seed) < 0 || whole(a[10], &step) < 0 ||
+        whole(a[11], &example0) < 0 || address(a[13], &norms) < 0 || address(a[14], &clip) < 0 || address(a[15], &ws) < 0 ||
+        bytes_of(a[16], a[15], &bytes) < 0 || stream_of(a[17], &st) < 0)
+        return done(&t, 1, 0);
+    CALL(rc, dp_clip_accumulate_noised((int)mode, (int)B, (int)t.L, (const float *const *)t.G, t.P, t.more, sq, C, sigma, total,
+                                       (unsigned long long)seed, (unsigned long long)step, example0, (float *const *)t.acc, norms, clip, ws, bytes, st));
+    return done(&t, 0, rc);
+}
+
+static PyObject *clip_accumulate_grouped(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_clip_accumulate_grouped", 11, "B", "M", "group_of", "G", "P_l", "sqnorm", "C", "acc", "norms_out", "clip_out", "workspace",
+         "workspace_bytes", "stream");
+    Lists t;
+    long long B, M;
+    void *sq, *norms, *clip, *ws, *st;
+    float C;
+    size_t bytes;
+    int rc = 0, *group_of = NULL;
+    if (lists(a[4], a[3], a[7], a[2], &t) < 0 || whole(a[0], &B) < 0 || whole(a[1], &M) < 0 || address(a[5], &sq) < 0 || real(a[6], &C) < 0 ||
+        address(a[8], &norms) < 0 || address(a[9], &clip) < 0 || address(a[10], &ws) < 0 || bytes_of(a[11], a[10], &bytes) < 0 ||
+        stream_of(a[12], &st) < 0)
+        return done(&t, 1, 0);
+    if (t.more) {
+        group_of = malloc(sizeof(int) * (size_t)(t.L > 0 ? t.L : 1));
+        if (!group_of) { PyErr_NoMemory(); return done(&t, 1, 0); }
+        for (Py_ssize_t i = 0; i < t.L; ++i) group_of[i] = (int)t.more[i];
+    }
+    CALL(rc, dp_clip_accumulate_grouped((int)B, (int)t.L, (int)M, group_of, (const float *const *)t.G, t.P, sq, C, (float *const *)t.acc, norms, clip, ws, bytes, st));
+    free(group_of);
+    return done(&t, 0, rc);
+}
+
+static PyObject *clip_accumulate_micro(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_clip_accumulate_micro", 9, "B", "micro", "G", "P_l", "C", "acc", "norms_out", "clip_out", "workspace", "workspace_bytes", "stream");
+    Lists t;
+    long long B, micro;
+    void *norms, *clip, *ws, *st;
+    float C;
+    size_t bytes;
+    int rc = 0;
+    if (lists(a[3], a[2], a[5], Py_None, &t) < 0 || whole(a[0], &B) < 0 || whole(a[1], &micro) < 0 || real(a[4], &C) < 0 ||
+        address(a[6], &norms) < 0 || address(a[7], &clip) < 0 || address(a[8], &ws) < 0 || bytes_of(a[9], a[8], &bytes) < 0 ||
+        stream_of(a[10], &st) < 0)
+        return done(&t, 1, 0);
+    CALL(rc, dp_clip_accumulate_micro((int)B, (int)t.L, (int)micro, (const float *const *)t.G, t.P, C, (float *const *)t.acc, norms, clip, ws, bytes, st));
+    return done(&t, 0, rc);
+}
+
+static PyObject *noise_average(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_noise_average", 9, "acc", "P", "param_offset", "sigma", "C", "total_batch", "seed", "step", "out", "stream");
+    void *acc, *out, *st;
+    long long P, off, total, seed, step;
+    float sigma, C;
+    if (address(a[0], &acc) < 0 || whole(a[1], &P) < 0 || whole(a[2], &off) < 0 || real(a[3], &sigma) < 0 || real(a[4], &C) < 0 ||
+        whole(a[5], &total) < 0 || whole(a[6], &seed) < 0 || whole(a[7], &step) < 0 || address(a[8], &out) < 0 || stream_of(a[9], &st) < 0)
+        return NULL;
+    int rc;
+    CALL(rc, dp_noise_average(acc, P, off, sigma, C, total, (unsigned long long)seed, (unsigned long long)step, out, st));
+    return PyLong_FromLong(rc);
+}
+
+static PyObject *noise_average_sgd(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_noise_average_sgd", 11, "acc", "P", "param_offset", "sigma", "C", "total_batch", "seed", "step", "lr", "momentum", "theta",
+         "momentum_buf", "g_out", "stream");
+    void *acc, *theta, *mom, *g, *st;
+    long long P, off, total, seed, step;
+    float sigma, C, lr, mu;
+    if (address(a[0], &acc) < 0 || whole(a[1], &P) < 0 || whole(a[2], &off) < 0 || real(a[3], &sigma) < 0 || real(a[4], &C) < 0 ||
+        whole(a[5], &total) < 0 || whole(a[6], &seed) < 0 || whole(a[7], &step) < 0 || real(a[8], &lr) < 0 || real(a[9], &mu) < 0 ||
+        address(a[10], &theta) < 0 || address(a[11], &mom) < 0 || address(a[12], &g) < 0 || stream_of(a[13], &st) < 0)
+        return NULL;
+    int rc;
+    CALL(rc, dp_noise_average_sgd(acc, P, off, sigma, C, total, (unsigned long long)seed, (unsigned long long)step, lr, mu, theta, mom, g, st));
+    return PyLong_FromLong(rc);
+}
+
+/* (batch handle, dp_layer_io array, [(X, dY)] of every layer, C_l, workspace, stream): fills in the inputs and runs */
+static PyObject *batch_run(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("batch_run", 5, "handle", "io", "inputs", "C_l", "workspace", "stream");
+    void *handle, *table, *ws, *st;
+    float C_l;
+    size_t bytes;
+    if (address(a[0], &handle) < 0 || real(a[3], &C_l) < 0 || address(a[4], &ws) < 0 || bytes_of(Py_None, a[4], &bytes) < 0 || stream_of(a[5], &st) < 0)
+        return NULL;
+    Py_buffer view;
+    if (PyObject_GetBuffer(a[1], &view, PyBUF_WRITABLE) < 0) return NULL;
+    table = view.buf;
+    const Py_ssize_t n = view.len / (Py_ssize_t)sizeof(dp_layer_io);
+    PyBuffer_Release(&view);
+    PyObject *seq = PySequence_Fast(a[2], "inputs: expected a sequence of (X, dY)");
+    if (!seq) return NULL;
+    dp_layer_io *io = table;
+    int rc = PySequence_Fast_GET_SIZE(seq) == n ? 0 : -1;
+    if (rc < 0) PyErr_Format(PyExc_ValueError, "inputs: %zd pairs for %zd layers", PySequence_Fast_GET_SIZE(seq), n);
+    for (Py_ssize_t i = 0; i < n && rc == 0; ++i) {
+        PyObject *pair = PySequence_Fast(PySequence_Fast_GET_ITEM(seq, i), "inputs: expected (X, dY)");
+        if (!pair) { rc = -1; break; }
+        void *X = NULL, *dY = NULL;
+        if (PySequence_Fast_GET_SIZE(pair) != 2) { PyErr_SetString(PyExc_ValueError, "inputs: expected (X, dY)"); rc = -1; }
+        if (rc == 0) rc = address(PySequence_Fast_GET_ITEM(pair, 0), &X);
+        if (rc == 0) rc = address(PySequence_Fast_GET_ITEM(pair, 1), &dY);
+        Py_DECREF(pair);
+        io[i].X = X; io[i].dY = dY;
+    }
+    Py_DECREF(seq);
+    if (rc < 0) return NULL;
+    CALL(rc, dp_batch_run(handle, io, C_l, ws, bytes, st));
+    return PyLong_FromLong(rc);
+}
+
+static PyObject *set_torch(PyObject *self, PyObject *const *args, Py_ssize_t nargs) {
+    if (nargs != 3) { PyErr_SetString(PyExc_TypeError, "set_torch(raw_stream, get_device, current_stream)"); return NULL; }
+    Py_XSETREF(raw_stream, args[0] == Py_None ? NULL : Py_NewRef(args[0]));
+    Py_XSETREF(get_device, args[1] == Py_None ? NULL : Py_NewRef(args[1]));
+    Py_XSETREF(current_stream, Py_NewRef(args[2]));
+    if (!raw_stream || !get_device) Py_CLEAR(raw_stream);
+    Py_RETURN_NONE;
+}
+
+#define ENTRY(name, fn) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL | METH_KEYWORDS, NULL}
+static PyMethodDef methods[] = {
+    ENTRY("dp_per_example_wgrad", per_example_wgrad), ENTRY("dp_per_example_wgrad_scaled", per_example_wgrad_scaled),
+    ENTRY("dp_clip_factors", clip_factors), ENTRY("dp_scale_accumulate", scale_accumulate),
+    ENTRY("dp_clip_accumulate", clip_accumulate), ENTRY("dp_clip_accumulate_static", clip_accumulate_static),
+    ENTRY("dp_clip_accumulate_noised", clip_accumulate_noised), ENTRY("dp_clip_accumulate_grouped", clip_accumulate_grouped),
+    ENTRY("dp_clip_accumulate_micro", clip_accumulate_micro), ENTRY("dp_noise_average", noise_average),
+    ENTRY("dp_noise_average_sgd", noise_average_sgd), ENTRY("batch_run", batch_run),
+    {"set_torch", (PyCFunction)(void (*)(void))set_torch, METH_FASTCALL, NULL}, {NULL, NULL, 0, NULL}};
+static struct PyModuleDef module = {PyModuleDef_HEAD_INIT, "_pycall", NULL, -1, methods, NULL, NULL, NULL, NULL};
+
+PyMODINIT_FUNC PyInit__pycall(void) {
+    s_data_ptr = PyUnicode_InternFromString("data_ptr");
+    s_is_contiguous = PyUnicode_InternFromString("is_contiguous");
+    s_nbytes = PyUnicode_InternFromString("nbytes");
+    s_cuda_stream = PyUnicode_InternFromString("cuda_stream");
+    if (!s_data_ptr || !s_is_contiguous || !s_nbytes || !s_cuda_stream) return NULL;
+    return PyModule_Create(&module);
+}

@@ -2500,6 +2500,12 @@ typedef TableQueue<GramParams, 2, kTcLayers> GramQueue;
 // Cluster size of the launch a layer with `tiles` tiles an example joins: sizes that divide one another share one.
 static int launch_cluster(int tiles) { return tiles == 1 || tiles == 2 || tiles == 4 ? 4 : (tiles == 3 || tiles == 6 ? 6 : tiles); }
 
+bool conv_batch_clusters(const ConvJob &j, double walk) {
+    BatchPlanning planning(walk);
+    TcPlan pl; ConvGeom g; bool s2d;
+    return j.kind == kConvClip1 && clip1_plan(j.dtype, j.g, tc_problem(j.dtype, j.g), pl, g, s2d) && launch_cluster(pl.m_tiles * pl.n_tiles) > 4;
+}
+
 dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *status, const BatchStreams &streams,
                             const std::function<dp_status()> &join) {
     if (jobs.empty()) return join();

@@ -80,6 +80,7 @@ struct ConvJob {
 // kConvSingle: no shared launch takes this layer.
 int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias);
 double conv_batch_walk(const std::vector<ConvJob> &jobs);
+bool conv_batch_clusters(const ConvJob &job, double walk);        // runs in a launch of large clusters, on kClusters
 // Streams a batch spreads its independent launches over: s[0] is the caller's, the others are forked from it and joined
 // to it again (ForkedStreams).  All may be one and the same.
 struct BatchStreams {
