@@ -282,6 +282,41 @@ __device__ __forceinline__ void put_rows(float4 *buf, const V &value, int lane, 
     __syncwarp();
 }
 
+// A thread's 32 values along the tile's columns where the block does not go through put_rows: columns of output channels
+// (lanes write neighbouring words), or rows of a length that is no multiple of the vectors.
+template <typename V>
+__device__ __forceinline__ void put_values(const V &value, float *base, bool add, const TcParams &p, int a_idx, int b_idx) {
+    const long long ld = p.Ng;
+    if (p.a_is_x) {
+        float *dst = base + b_idx * ld + a_idx;
+        if (add) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) red_add(dst + i * ld, value(i));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) dst[i * ld] = value(i);
+        }
+    } else {
+        float *dst = base + a_idx * ld + b_idx;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+            if (b_idx + i < p.Ng) { if (add) red_add(dst + i, value(i)); else dst[i] = value(i); }
+    }
+}
+
+// slots first, first + 8, ... below end of an example's partial sums, in order, eight loads in flight
+__device__ __forceinline__ double slot_sum(const float *slots, int first, int end) {
+    double sum = 0.0;
+    for (int i = first; i < end; i += 64) {
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) { v[k] = 0.f; if (i + 8 * k < end) v[k] = __ldcg(slots + i + 8 * k); }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sum += (double)v[k];
+    }
+    return sum;
+}
+
 // What a producer warp copies for one operand of a tile: lane o holds the origin of copy o (`group` slabs of one tap).
 // Issuing a copy costs the issuing warp about a hundred cycles and a barrier wait somewhat more, whatever the copy's size,
 // so the fewer copies a stage takes, the smaller the stages (and the shorter their latency) can be.
@@ -450,6 +485,9 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         // swizzled layout because the split is element-wise on identical relative addresses.
         // The eight warps work as two groups of four that take alternate stages, so the proxy fence that ends one
         // group's stage (it waits for that group's stores to drain) overlaps the other group's loads and stores.
+        // The number of stages is even, so that a slot always belongs to the same group: a group that skipped every other
+        // use of a slot could find the parity of the use before last and take a copy still under way for its own (stages
+        // fill in any order), which with three stages left a launch in some thousands waiting in vain.
         const int group = (warp - 7) >> 2;
         const int tid = (threadIdx.x - 224) & 127;
         int stage = 0; uint32_t phase = 0;
@@ -611,13 +649,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                             if (add) put_rows<kPutAdd>(xpose[warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
                             else put_rows<kPutPlain>(xpose[warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
                         } else if (row_ok) {
-                            const long long step = p.a_is_x ? p.Ng : 1;
-                            float *dst = base + (p.a_is_x ? (long long)b_idx * p.Ng + a_idx : (long long)a_idx * p.Ng + b_idx);
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                if (!p.a_is_x && b_idx + i >= p.Ng) continue;
-                                if (add) red_add(dst + i * step, value(i)); else dst[i * step] = value(i);
-                            }
+                            put_values(value, base, add, p, a_idx, b_idx);
                         }
                     }
                 }
@@ -640,15 +672,16 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         if (last_cta) {
             __threadfence();
             // eight lanes per example (slot i goes to lane i % 8, the eight sums are added by a butterfly), four
-            // examples per warp and trip: the walk is a chain of L2 round trips, so many examples go side by side
+            // examples per warp and trip: the walk is a chain of L2 round trips, so many examples go side by side,
+            // with eight loads of each in flight (one by one, 144 slots an example held the launch up for 2 us)
             const int groups = (int)(blockDim.x >> 3), group = (int)(threadIdx.x >> 3), sub = lane & 7;
             for (int n0 = 0; n0 < p.B; n0 += groups) {     // uniform trip count: the shuffles below need whole warps
                 const int n = n0 + group;
                 double sw = 0.0, sb = 0.0;
                 if (n < p.B) {
                     const float *pn = p.partial + (long long)n * p.slots;
-                    for (int i = sub; i < p.w_slots; i += 8) sw += (double)__ldcg(pn + i);
-                    for (int i = p.w_slots + sub; i < p.fold_slots; i += 8) sb += (double)__ldcg(pn + i);
+                    sw = slot_sum(pn, sub, p.w_slots);
+                    sb = slot_sum(pn, p.w_slots + sub, p.fold_slots);
                 }
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1) {
@@ -1019,13 +1052,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                         if (add) put_rows<kPutAdd>(buf, value, lane, dst, p.Ng, a_rows - q * 32);
                         else put_rows<kPutPlain>(buf, value, lane, dst, p.Ng, a_rows - q * 32);
                     } else if (row_ok) {
-                        const long long step = p.a_is_x ? p.Ng : 1;
-                        float *dst = base + (p.a_is_x ? (long long)b_idx * p.Ng + a_idx : (long long)a_idx * p.Ng + b_idx);
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) {
-                            if (!p.a_is_x && b_idx + i >= p.Ng) continue;
-                            if (add) red_add(dst + i * step, value(i)); else dst[i * step] = value(i);
-                        }
+                        put_values(value, base, add, p, a_idx, b_idx);
                     }
                 }
             }
@@ -1482,28 +1509,39 @@ static dp_status launch_scale_split(const std::vector<SplitSeg> &segs, cudaStrea
     return DP_OK;
 }
 
-// acc[i] += sum over splits of part[s][i], splits in index order; vec: P a multiple of 4 and both 16-byte aligned
+// acc[i] += sum over splits of part[s][i], splits in index order; vec: P a multiple of 4 and both 16-byte aligned.
+// A layer's sums are few (a 64 x 128 gradient is 16 blocks), so what bounds this is one thread's chain of loads: eight
+// in flight and small blocks, which spread over the SMs (30 ranges of such a gradient: 8.4 us with four in flight and
+// 256 threads a block).
+constexpr int kFoldThreads = 128, kFoldAhead = 8;
 struct FoldSeg { const float *part; float *acc; long long P; int splits, vec; };
 struct FoldTable { int n; int first[kTcLayers]; FoldSeg s[kTcLayers]; };
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kFoldThreads)
 fold_partial_sums_kernel(const __grid_constant__ FoldTable tab) {
-    const int entry = table_entry(tab.first, tab.n, blockIdx.x);
-    const FoldSeg &sg = tab.s[entry];
-    const long long P = sg.P, i = ((long long)(blockIdx.x - tab.first[entry]) * 256 + threadIdx.x) * 4;
+    const int entry = tab.n == 1 ? 0 : table_entry(tab.first, tab.n, blockIdx.x);
+    const long long P = tab.s[entry].P, i = ((long long)(blockIdx.x - tab.first[entry]) * kFoldThreads + threadIdx.x) * 4;
+    const float *part = tab.s[entry].part + i;
+    float *acc = tab.s[entry].acc + i;
+    const int splits = tab.s[entry].splits;
     if (i >= P) return;
-    if (sg.vec) {
-        float4 a = *reinterpret_cast<const float4 *>(sg.acc + i);
-#pragma unroll 4
-        for (int s = 0; s < sg.splits; ++s) {
-            const float4 v = __ldcs(reinterpret_cast<const float4 *>(sg.part + (long long)s * P + i));
-            a.x += v.x; a.y += v.y; a.z += v.z; a.w += v.w;
+    if (tab.s[entry].vec) {
+        float4 a = *reinterpret_cast<const float4 *>(acc);
+        for (int s = 0; s < splits; s += kFoldAhead) {
+            float4 v[kFoldAhead];
+#pragma unroll
+            for (int k = 0; k < kFoldAhead; ++k) {
+                v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (s + k < splits) v[k] = __ldcs(reinterpret_cast<const float4 *>(part + (s + k) * P));
+            }
+#pragma unroll
+            for (int k = 0; k < kFoldAhead; ++k) { a.x += v[k].x; a.y += v[k].y; a.z += v[k].z; a.w += v[k].w; }
         }
-        *reinterpret_cast<float4 *>(sg.acc + i) = a;
+        *reinterpret_cast<float4 *>(acc) = a;
     } else {
-        for (long long k = i; k < min(P, i + 4); ++k) {
-            float a = sg.acc[k];
-            for (int s = 0; s < sg.splits; ++s) a += sg.part[(long long)s * P + k];
-            sg.acc[k] = a;
+        for (int k = 0; k < (int)min(P - i, 4ll); ++k) {
+            float a = acc[k];
+            for (int s = 0; s < splits; ++s) a += part[s * P + k];
+            acc[k] = a;
         }
     }
 }
@@ -1518,10 +1556,10 @@ static dp_status launch_folds(const std::vector<FoldSeg> &segs, cudaStream_t str
         for (tab.n = 0; i < segs.size() && tab.n < kTcLayers; ++i) {
             tab.first[tab.n] = (int)blocks;
             tab.s[tab.n++] = segs[i];
-            blocks += (segs[i].P + 1023) / 1024;
+            blocks += (segs[i].P + 4 * kFoldThreads - 1) / (4 * kFoldThreads);
         }
         if (blocks > 0x7fffffffll) return DP_ERR_UNSUPPORTED;
-        fold_partial_sums_kernel<<<(unsigned)blocks, 256, 0, stream>>>(tab);
+        fold_partial_sums_kernel<<<(unsigned)blocks, kFoldThreads, 0, stream>>>(tab);
         DP_LAUNCH_CHECK("fold_partial_sums_kernel");
     }
     return DP_OK;
@@ -1830,6 +1868,7 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
                     int stages = kSmemBudget / stage_bytes;
                     if (stages < 2) continue;
                     if (stages > kMaxStages) stages = kMaxStages;
+                    if (dtype == DP_F32) stages &= ~1;        // each split group has slots of its own (see there)
                     const int tw = (g.OW + OWt - 1) / OWt, th = (g.OH + OHt - 1) / OHt;
                     // a stage: its MMA steps plus the hand-over (barrier wait, commit) of the issuing thread
                     double stage_cost = (double)(Kt / krows) * step + 250.0;
