@@ -4,6 +4,7 @@
 // Formulas: paper section 2 (per-example gradient, its L2 norm, clip) and section 3.5 (per-layer threshold).
 #include "wgrad_simple.cuh"
 #include <math.h>
+#include <mutex>
 
 namespace dp {
 
@@ -314,21 +315,23 @@ dp_status launch_conv_thin(int dtype, const void *X, const void *dY, const ConvG
     return DP_OK;
 }
 
-// 3x3 convolutions on three input channels (image stems), output channels a multiple of 32: one block per example,
-// the zero-padded image in shared memory.  Lane = output pixel (32 consecutive pixels per trip), warp w owns output
-// channels 4w .. 4w+3 of the current group of 32, so a thread keeps a 4 x 27 block of the gradient in registers, every
-// shared-memory word it reads feeds four FMAs, and the 32 lanes read 32 different words (3 floats apart: no bank
-// conflict) instead of one broadcast word.  A trip is short (a few hundred cycles) against the memory latency, so dY
-// streams through a ring of kRgbStages stages of 64 pixels x 32 channels, filled by coalesced asynchronous copies
-// (cp.async, each thread two pieces of four channels per stage) three stages ahead of the arithmetic, one barrier per
-// stage.  Inside a stage the piece of (pixel l, channel quad c) sits at quad position c ^ (l & 7) of its pixel row, so
-// that the 32 lanes of a warp, which read the same quad of 32 different pixels, hit different banks.  The 32 pixel
-// lanes are folded by two shuffle steps and then, in lane order, through shared memory; gradient, bias gradient and
-// the example's squared norms leave from the same pass.
-constexpr int kRgbRed = 113;      // floats per (warp, lane group) in the fold buffer: 4 x 27 weights + 4 bias sums (+1: odd stride)
-constexpr int kRgbStages = 4;     // stages of dY in the ring
-constexpr int kRgbStagePix = 64;  // pixels per stage (two trips)
+// 3x3 convolutions on three input channels (image stems), output channels a multiple of 32: a cluster of one to eight
+// blocks per example, each with a range of output rows.  The zero-padded input rows a block needs sit in shared memory.
+// Lane = output pixel (32 consecutive pixels per trip); warp w owns output channels 8(w%4) .. +7 of the current group of
+// 32 and filter row w/4, i.e. an 8 x 9 block of the gradient in registers as 36 pairs of channels, which the packed
+// FMA takes two at a time.  What bounds it is shared memory and issue alike: 17 wavefronts and 64 instructions for the
+// 72 multiply-adds of a pixel (27 wavefronts, 150 instructions and 16 warps an SM with all 27 columns and four channels
+// a thread: 31 us for 256 examples of 32 x 32, and 23 us for 32, which were 32 blocks).  dY streams through a ring of
+// kRgbStages stages of 128 pixels x 32 channels, filled by coalesced asynchronous copies two stages ahead of the
+// arithmetic, one barrier per stage.  Inside a stage the piece of (pixel l, channel quad c) sits at quad position
+// c ^ (l & 7) of its pixel row, so that the lanes of a warp, which read the same quad of 32 pixels, hit different banks.
+// The 32 pixel lanes are folded by halving (each step a lane keeps half of its values), the blocks of a cluster add
+// their sums through distributed shared memory, in one order; gradient, bias gradient and norms leave from the same pass.
+constexpr int kRgbThreads = 384;  // 12 warps: four channel octets x three filter rows
+constexpr int kRgbStages = 3;     // stages of dY in the ring
+constexpr int kRgbStagePix = 128; // pixels per stage (four trips: a barrier and the copies' addresses every 128 pixels)
 constexpr int kRgbStageFloats = kRgbStagePix * 32;   // ring stride in 4-byte words (bf16 stages use half of it)
+constexpr int kRgbSums = 32 * 27 + 32;               // sums of a group of 32 channels: gradient rows, then bias
 
 template <int BYTES>
 __device__ __forceinline__ void cp_async_zfill(void *smem_dst, const void *src, bool valid) {
@@ -340,131 +343,196 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
+__device__ __forceinline__ unsigned long long pack2(float x, float y) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ void rgb_cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float rgb_peer(const float *mine, unsigned rank) {       // the same word in block `rank` of the cluster
+    unsigned addr = (unsigned)__cvta_generic_to_shared(mine);
+    float v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.f32 %0, [a];\n\t}" : "=f"(v) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+__device__ __forceinline__ double rgb_peer(const double *mine, unsigned rank) {
+    unsigned addr = (unsigned)__cvta_generic_to_shared(mine);
+    double v;
+    asm volatile("{\n\t.reg .b32 a;\n\tmapa.shared::cluster.u32 a, %1, %2;\n\tld.shared::cluster.f64 %0, [a];\n\t}" : "=d"(v) : "r"(addr), "r"(rank) : "memory");
+    return v;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256, 2)
-conv_wgrad_rgb3_kernel(const T *__restrict__ X, const T *__restrict__ dY, const ConvGeom g, float *__restrict__ G_w,
-                       float *__restrict__ db, int has_bias, int separate, float *__restrict__ sqnorm,
-                       long long sq_stride) {
+__global__ void __launch_bounds__(kRgbThreads, 1)
+conv_wgrad_rgb3_kernel(const T *__restrict__ X, const T *__restrict__ dY, const ConvGeom g, int cluster, int rows_per,
+                       float *__restrict__ G_w, float *__restrict__ db, int has_bias, int separate,
+                       float *__restrict__ sqnorm, long long sq_stride) {
     extern __shared__ __align__(16) float rgb_smem[];
     __shared__ double scratch[32];
+    __shared__ float sums[kRgbSums];                         // this block's sums of the current 32 channels
+    __shared__ double norm2[2];
     constexpr int kQuad = 4 * (int)sizeof(T);                // bytes of four output channels of dY
-    const int Hp = g.H + 2 * g.pad, Wp = g.W + 2 * g.pad, row_p = Wp * 3;
-    const int xs_count = Hp * row_p;
-    char *ring = reinterpret_cast<char *>(rgb_smem);         // [kRgbStages][64 pixels][8 quads]; afterwards the fold
-    float *red = rgb_smem;                                   //   buffer [8 warps][8 lane groups][kRgbRed]
-    float *xs = rgb_smem + kRgbStages * kRgbStageFloats;     // [Hp][Wp][3], zero border
-    const int n = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int Wp = g.W + 2 * g.pad, row_p = Wp * 3;
+    char *ring = reinterpret_cast<char *>(rgb_smem);         // [kRgbStages][128 pixels][8 quads]
+    float *xs = rgb_smem + kRgbStages * kRgbStageFloats;     // [input rows of this block][Wp][3], zero border
+    const int n = blockIdx.x / cluster, rank = blockIdx.x - n * cluster;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, oct = w & 3, fr = w >> 2;
+    const int oh0 = min(g.OH, rank * rows_per), oh1 = min(g.OH, oh0 + rows_per);
+    const int pixels = (oh1 - oh0) * g.OW, rows_in = oh1 > oh0 ? (oh1 - oh0 - 1) * g.stride + 3 : 0;
     {
-        const int row_in = g.W * 3;
-        for (int i = threadIdx.x; i < xs_count; i += 256) xs[i] = 0.f;
-        __syncthreads();
+        const int row_in = g.W * 3, ih0 = oh0 * g.stride - g.pad;
         const T *Xn = X + (long long)n * g.H * row_in;
-        for (int i = threadIdx.x; i < g.H * row_in; i += 256) {
-            const int h = i / row_in, rest = i - h * row_in;
-            xs[(h + g.pad) * row_p + g.pad * 3 + rest] = to_float(Xn[i]);
+        for (int i = threadIdx.x; i < rows_in * row_p; i += kRgbThreads) {
+            const int r = i / row_p, c = i - r * row_p - g.pad * 3, ih = ih0 + r;
+            xs[i] = (ih >= 0 && ih < g.H && c >= 0 && c < row_in) ? to_float(Xn[(long long)ih * row_in + c]) : 0.f;
         }
     }
-    float sq = 0.f, sqb = 0.f;
-    const int stages = (g.K + kRgbStagePix - 1) / kRgbStagePix;
-    // copies of this thread: quad cq of pixels cl and cl + 32 of a stage; reads: quad w of pixel lane (+32 on the second trip)
+    const int stages = (pixels + kRgbStagePix - 1) / kRgbStagePix;
+    // copies: thread t < 256 brings quad t%8 of pixels t/8, t/8 + 32, ... of a stage; reads: quads 2*oct and 2*oct + 1 of
+    // pixel `lane` (+32 on each further trip)
     const int cl = threadIdx.x >> 3, cq = threadIdx.x & 7;
     const int copy_off = cl * 8 * kQuad + ((cq ^ (cl & 7)) * kQuad);        // (cl + 32) & 7 == cl & 7
-    const int read_off = lane * 8 * kQuad + ((w ^ (lane & 7)) * kQuad);
+    const int read0 = lane * 8 * kQuad + (((2 * oct) ^ (lane & 7)) * kQuad), read1 = lane * 8 * kQuad + (((2 * oct + 1) ^ (lane & 7)) * kQuad);
+    float sq = 0.f, sqb = 0.f;
     for (int kg = 0; kg < g.Kout / 32; ++kg) {
-        const T *dyp = dY + (long long)n * g.K * g.Kout + kg * 32;
+        const T *dyp = dY + ((long long)n * g.K + (long long)oh0 * g.OW) * g.Kout + kg * 32;
         auto fetch = [&](int stage) {                        // one commit group per stage, also past the end
-            char *dst = ring + (stage % kRgbStages) * (kRgbStageFloats * 4) + copy_off;
+            if (threadIdx.x < 256) {
+                char *dst = ring + (stage % kRgbStages) * (kRgbStageFloats * 4) + copy_off;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int p = stage * kRgbStagePix + cl + 32 * h;
-                const bool valid = stage < stages && p < g.K;
-                cp_async_zfill<kQuad>(dst + h * 32 * 8 * kQuad, dyp + (long long)(valid ? p : 0) * g.Kout + 4 * cq, valid);
+                for (int h = 0; h < kRgbStagePix / 32; ++h) {
+                    const int p = stage * kRgbStagePix + cl + 32 * h;
+                    const bool valid = stage < stages && p < pixels;
+                    cp_async_zfill<kQuad>(dst + h * 32 * 8 * kQuad, dyp + (long long)(valid ? p : 0) * g.Kout + 4 * cq, valid);
+                }
             }
             cp_async_commit();
         };
-        float acc[4][27], bs[4] = {0.f, 0.f, 0.f, 0.f};
+        unsigned long long acc[4][9], bs[4];                 // pairs of channels x columns of this warp's filter row
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
+        for (int k = 0; k < 4; ++k) {
+            bs[k] = 0ull;
 #pragma unroll
-            for (int j = 0; j < 27; ++j) acc[kk][j] = 0.f;
+            for (int q = 0; q < 9; ++q) acc[k][q] = 0ull;
+        }
         for (int t = 0; t < kRgbStages - 1; ++t) fetch(t);
         int oh = lane / g.OW, ow = lane - oh * g.OW;         // pixel of this lane in the current trip
+        const unsigned long long one = pack2(1.f, 1.f);
         for (int st = 0; st < stages; ++st) {
             cp_async_wait<kRgbStages - 2>();                 // this thread's pieces of stage st have landed
             __syncthreads();                                 // ... and everyone's; stage st-1 is no longer read
             fetch(st + kRgbStages - 1);                      // refills the slot of stage st-1
-            const char *src = ring + (st % kRgbStages) * (kRgbStageFloats * 4) + read_off;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float gy[4];
+            const char *src = ring + (st % kRgbStages) * (kRgbStageFloats * 4);
+#pragma unroll 2
+            for (int h = 0; h < kRgbStagePix / 32; ++h) {
+                if (st * kRgbStagePix + 32 * h >= pixels) break;
+                unsigned long long gy[4];
                 if constexpr (sizeof(T) == 4) {
-                    const float4 v = *reinterpret_cast<const float4 *>(src + h * 32 * 8 * kQuad);
-                    gy[0] = v.x; gy[1] = v.y; gy[2] = v.z; gy[3] = v.w;
+                    const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(src + read0 + h * 32 * 8 * kQuad);
+                    const ulonglong2 b = *reinterpret_cast<const ulonglong2 *>(src + read1 + h * 32 * 8 * kQuad);
+                    gy[0] = a.x; gy[1] = a.y; gy[2] = b.x; gy[3] = b.y;
                 } else {
-                    const uint2 v = *reinterpret_cast<const uint2 *>(src + h * 32 * 8 * kQuad);
-                    gy[0] = __uint_as_float(v.x << 16); gy[1] = __uint_as_float(v.x & 0xffff0000u);
-                    gy[2] = __uint_as_float(v.y << 16); gy[3] = __uint_as_float(v.y & 0xffff0000u);
+                    const uint2 a = *reinterpret_cast<const uint2 *>(src + read0 + h * 32 * 8 * kQuad);
+                    const uint2 b = *reinterpret_cast<const uint2 *>(src + read1 + h * 32 * 8 * kQuad);
+                    gy[0] = pack2(__uint_as_float(a.x << 16), __uint_as_float(a.x & 0xffff0000u));
+                    gy[1] = pack2(__uint_as_float(a.y << 16), __uint_as_float(a.y & 0xffff0000u));
+                    gy[2] = pack2(__uint_as_float(b.x << 16), __uint_as_float(b.x & 0xffff0000u));
+                    gy[3] = pack2(__uint_as_float(b.y << 16), __uint_as_float(b.y & 0xffff0000u));
                 }
                 // lanes past the last pixel carry zeros of dY; their patch address is clamped to pixel 0
-                const bool live = st * kRgbStagePix + 32 * h + lane < g.K;
-                const float *patch = xs + (live ? (oh * g.stride * Wp + ow * g.stride) * 3 : 0);
+                const bool live = st * kRgbStagePix + 32 * h + lane < pixels;
+                const float *row = xs + fr * row_p + (live ? oh * g.stride * row_p + ow * g.stride * 3 : 0);
+                float x[9];
 #pragma unroll
-                for (int r = 0; r < 3; ++r) {
-                    float x[9];
+                for (int q = 0; q < 9; ++q) x[q] = row[q];
 #pragma unroll
-                    for (int q = 0; q < 9; ++q) x[q] = patch[r * row_p + q];
+                for (int q = 0; q < 9; ++q) {
+                    const unsigned long long xx = pack2(x[q], x[q]);
 #pragma unroll
-                    for (int q = 0; q < 9; ++q)
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) acc[kk][r * 9 + q] = fmaf(gy[kk], x[q], acc[kk][r * 9 + q]);
+                    for (int k = 0; k < 4; ++k) fma2(acc[k][q], gy[k], xx);
                 }
+                if (fr == 0) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) bs[kk] += gy[kk];
+                    for (int k = 0; k < 4; ++k) fma2(bs[k], gy[k], one);
+                }
                 ow += 32;
                 while (ow >= g.OW) { ow -= g.OW; ++oh; }
             }
         }
         cp_async_wait<0>();
-        __syncthreads();                                     // every thread is done with the ring: it becomes the fold buffer
-        // fold the 32 pixel lanes: two butterfly steps leave eight partial sums (lanes 0..7), added in lane order below
-        float *mine = red + (w * 8 + (lane & 7)) * kRgbRed;
+        // fold the 32 pixel lanes by halving: 80 values (72 sums, 8 bias sums) -> 5, summed over 16 of the lanes, then the last step
+        float v[80];
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
+        for (int k = 0; k < 4; ++k) {
 #pragma unroll
-            for (int j = 0; j < 27; ++j) {
-                float v = acc[kk][j];
-                v += __shfl_xor_sync(0xffffffffu, v, 16);
-                v += __shfl_xor_sync(0xffffffffu, v, 8);
-                if (lane < 8) mine[kk * 27 + j] = v;
+            for (int q = 0; q < 9; ++q) asm("mov.b64 {%0, %1}, %2;" : "=f"(v[(2 * k) * 9 + q]), "=f"(v[(2 * k + 1) * 9 + q]) : "l"(acc[k][q]));
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(v[72 + 2 * k]), "=f"(v[73 + 2 * k]) : "l"(bs[k]));
+        }
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+            const int half = 40 >> s, mask = 16 >> s;
+            const bool up = (lane & mask) != 0;
+#pragma unroll
+            for (int i = 0; i < 40; ++i) {
+                if (i < half) {
+                    const float keep = up ? v[i + half] : v[i], send = up ? v[i] : v[i + half];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
+                }
             }
-            float v = bs[kk];
-            v += __shfl_xor_sync(0xffffffffu, v, 16);
-            v += __shfl_xor_sync(0xffffffffu, v, 8);
-            if (lane < 8) mine[108 + kk] = v;
         }
-        __syncthreads();
-        // entry o of this group of 32 channels is (warp o/108, register o%108) and sits at G_w[n][kg*864 + o]
-        for (int o = threadIdx.x; o < 864; o += 256) {
-            const float *src = red + (o / 108) * 8 * kRgbRed + (o % 108);
-            float v = 0.f;
+        const int base = ((lane & 16) ? 40 : 0) + ((lane & 8) ? 20 : 0) + ((lane & 4) ? 10 : 0) + ((lane & 2) ? 5 : 0);
+        __syncthreads();                                     // sums[] of the previous channels are no longer read
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v += src[q * kRgbRed];
-            if (G_w) G_w[(long long)n * g.Kout * 27 + kg * 864 + o] = v;
-            sq = fmaf(v, v, sq);
+        for (int i = 0; i < 5; ++i) {
+            const float t = v[i] + __shfl_xor_sync(0xffffffffu, v[i], 1);
+            const int e = base + i;                          // 0..71: (channel of the octet, column), 72..79: bias
+            if (!(lane & 1)) {
+                if (e < 72) sums[(8 * oct + e / 9) * 27 + fr * 9 + e % 9] = t;
+                else if (fr == 0) sums[32 * 27 + 8 * oct + e - 72] = t;
+            }
         }
-        if (has_bias && threadIdx.x < 32) {
-            const float *src = red + (threadIdx.x >> 2) * 8 * kRgbRed + 108 + (threadIdx.x & 3);
-            float v = 0.f;
+        if (cluster > 1) rgb_cluster_sync(); else __syncthreads();
+        // block `rank` finishes every cluster-th piece of the sums, adding the blocks in one order
+        for (int o = rank * kRgbThreads + threadIdx.x; o < kRgbSums; o += cluster * kRgbThreads) {
+            float t = sums[o];
+            if (cluster > 1) {
+                float part[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v += src[q * kRgbRed];
-            db[(long long)n * g.Kout + kg * 32 + threadIdx.x] = v;
-            sqb = fmaf(v, v, sqb);
+                for (int c = 0; c < 8; ++c) { part[c] = 0.f; if (c < cluster) part[c] = rgb_peer(&sums[o], (unsigned)c); }
+                t = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+            }
+            if (o < 32 * 27) {
+                if (G_w) G_w[(long long)n * g.Kout * 27 + kg * 864 + o] = t;
+                sq = fmaf(t, t, sq);
+            } else if (has_bias) {
+                db[(long long)n * g.Kout + kg * 32 + o - 864] = t;
+                sqb = fmaf(t, t, sqb);
+            }
         }
-        __syncthreads();
+        if (cluster > 1 && (kg + 1) * 32 < g.Kout) rgb_cluster_sync();       // nobody overwrites its sums while a peer may read them
     }
-    const double sw = block_sum((double)sq, scratch);
-    const double sb = block_sum((double)sqb, scratch);
-    if (threadIdx.x == 0) {
+    const double mw = block_sum((double)sq, scratch), mb = has_bias ? block_sum((double)sqb, scratch) : 0.0;
+    if (threadIdx.x == 0) { norm2[0] = mw; norm2[1] = mb; }
+    if (cluster > 1) rgb_cluster_sync(); else __syncthreads();
+    if (rank == 0 && threadIdx.x == 0) {
+        double sw = norm2[0], sb = norm2[1];
+        if (cluster > 1) {
+            double pw[8], pb[8];
+#pragma unroll
+            for (int c = 1; c < 8; ++c) {
+                pw[c] = pb[c] = 0.0;
+                if (c < cluster) { pw[c] = rgb_peer(&norm2[0], (unsigned)c); pb[c] = rgb_peer(&norm2[1], (unsigned)c); }
+            }
+#pragma unroll
+            for (int c = 1; c < 8; ++c) { sw += pw[c]; sb += pb[c]; }
+        }
         if (separate) {
             sqnorm[n * sq_stride] = (float)sw;
             sqnorm[n * sq_stride + 1] = (float)sb;
@@ -472,31 +540,62 @@ conv_wgrad_rgb3_kernel(const T *__restrict__ X, const T *__restrict__ dY, const 
             sqnorm[n * sq_stride] = (float)(sw + sb);
         }
     }
+    if (cluster > 1) rgb_cluster_sync();                     // block 0 has read its peers: they may leave
 }
 
-static size_t rgb3_smem_bytes(const ConvGeom &g) {
-    static_assert(kRgbStages * kRgbStageFloats >= 8 * 8 * kRgbRed, "the fold buffer reuses the dY ring");
-    const size_t xs = ((size_t)(g.H + 2 * g.pad) * (g.W + 2 * g.pad) * 3 + 3) & ~(size_t)3;
-    return sizeof(float) * (xs + (size_t)kRgbStages * kRgbStageFloats);
+// Blocks per example and output rows per block: as many as run side by side (a cluster needs its SMs at the same time: 32
+// examples of 1024 pixels took 21 us as clusters of eight, of which 15 fit), as long as each keeps 128 pixels, and at
+// least so many that a block's input rows fit beside the ring.
+constexpr size_t kRgbSmemMost = 160 * 1024;
+static size_t rgb3_smem_bytes(const ConvGeom &g, int rows_per) {
+    return sizeof(float) * ((size_t)((rows_per - 1) * g.stride + 3) * (g.W + 2 * g.pad) * 3 + (size_t)kRgbStages * kRgbStageFloats);
+}
+static int rgb3_side_by_side(int cluster) { return cluster == 1 ? sm_count() : (cluster == 2 ? sm_count() / 2 : sm_count() * 4 / 5 / cluster); }
+static bool rgb3_split(const ConvGeom &g, int &cluster, int &rows_per) {
+    bool found = false;
+    for (int c = 1; c <= 8; c *= 2) {
+        const int rows = (g.OH + c - 1) / c;
+        if (rgb3_smem_bytes(g, rows) > kRgbSmemMost) continue;
+        if (found && (g.B > rgb3_side_by_side(c) || (long long)rows * g.OW < 128)) break;
+        cluster = c; rows_per = rows; found = true;
+    }
+    return found;
 }
 
 bool rgb3_conv_eligible(const ConvGeom &g) {
-    return g.R == 3 && g.S == 3 && g.Cin == 3 && g.Kout % 32 == 0 && g.Kout <= 256 && rgb3_smem_bytes(g) <= 47 * 1024;
+    int cluster, rows_per;
+    return g.R == 3 && g.S == 3 && g.Cin == 3 && g.Kout % 32 == 0 && g.Kout <= 256 && g.W <= 512 && g.B <= (1 << 27) && rgb3_split(g, cluster, rows_per);
+}
+
+template <typename T>
+static dp_status launch_rgb3_t(const T *X, const T *dY, const ConvGeom &g, float *G_w, float *db, int has_bias, int separate,
+                               float *sqnorm, long long sq_stride, cudaStream_t st) {
+    int cluster, rows_per;
+    if (!rgb3_split(g, cluster, rows_per)) return DP_ERR_UNSUPPORTED;
+    static std::once_flag once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(once, [] {
+        attr_err = cudaFuncSetAttribute(conv_wgrad_rgb3_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRgbSmemMost);
+    });
+    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(g.B * cluster)); cfg.blockDim = dim3(kRgbThreads);
+    cfg.dynamicSmemBytes = rgb3_smem_bytes(g, rows_per); cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_rgb3_kernel<T>, X, dY, g, cluster, rows_per, G_w, db, has_bias, separate, sqnorm, sq_stride);
+    if (le != cudaSuccess) return cuda_fail(le, "conv_wgrad_rgb3_kernel");
+    DP_LAUNCH_CHECK("conv_wgrad_rgb3_kernel");
+    return DP_OK;
 }
 
 dp_status launch_conv_rgb3(int dtype, const void *X, const void *dY, const ConvGeom &g, float *G_w, float *db,
                            int has_bias, int separate, float *sqnorm, long long sq_stride,
                            cudaStream_t st) {
-    const size_t smem = rgb3_smem_bytes(g);
-    if (dtype == DP_F32)
-        conv_wgrad_rgb3_kernel<float><<<g.B, 256, smem, st>>>(static_cast<const float *>(X), static_cast<const float *>(dY), g,
-                                                              G_w, db, has_bias, separate, sqnorm, sq_stride);
-    else
-        conv_wgrad_rgb3_kernel<__nv_bfloat16><<<g.B, 256, smem, st>>>(static_cast<const __nv_bfloat16 *>(X),
-                                                                      static_cast<const __nv_bfloat16 *>(dY), g, G_w, db,
-                                                                      has_bias, separate, sqnorm, sq_stride);
-    DP_LAUNCH_CHECK("conv_wgrad_rgb3_kernel");
-    return DP_OK;
+    if (dtype == DP_F32) return launch_rgb3_t(static_cast<const float *>(X), static_cast<const float *>(dY), g, G_w, db, has_bias, separate, sqnorm, sq_stride, st);
+    return launch_rgb3_t(static_cast<const __nv_bfloat16 *>(X), static_cast<const __nv_bfloat16 *>(dY), g, G_w, db, has_bias, separate, sqnorm, sq_stride, st);
 }
 
 // db[n, k] = sum over pixels of dY[n, pix, k]; 64 channels x 4 pixel lanes per block, lanes folded in order.
