@@ -2,11 +2,12 @@
 // (paper section 2: sum over the batch of clip(g_j, C); section 3.5: per-group threshold C/sqrt(M)).
 //
 // Three memory-bound stages, all with fixed reduction orders:
-//   1. (only when the caller has no norms) per-block partial sums of squares of every example row,
-//      then one block per (tensor, example) folds the partials;
-//   2. one small kernel turns squared norms into clip factors;
-//   3. every thread owns four neighbouring parameters, streams the B example rows through
-//      registers with 128-bit loads, and touches the accumulator once.
+//   1. (only when the caller has no norms) per-block partial sums of squares of every example row;
+//   2. one small kernel folds the partials, a block per example, and turns squared norms into clip factors;
+//   3. every thread owns four parameters, streams the B example rows through registers with 128-bit loads (or 32-bit
+//      ones where the rows do not start on 16-byte boundaries), and touches the accumulator once.
+// The tensors of a call travel in one table each launch: with 161 tensors in tables of 40 the two passes over 1.6 GB were
+// ten launches, each with a last wave of its own, and took 590 us.
 #include "common.cuh"
 #include "philox.cuh"
 #include <math.h>
@@ -14,18 +15,19 @@
 
 namespace dp {
 
-constexpr int kMaxSeg = 40;          // tensors per launch (table travels as a kernel parameter)
+constexpr int kSmallTable = 16, kLargeTable = 512;   // tensors per launch (the table travels as a kernel parameter, 48 bytes each)
 constexpr int kNormChunk = 8192;     // floats of one example row reduced by one block (stage 1)
 constexpr int kAccCols = 1024;       // parameters per block in stage 3 (256 threads x float4)
 
+template <int N>
 struct SegTable {
-    const float *G[kMaxSeg];         // [B, P] per tensor
-    float *acc[kMaxSeg];             // [P] per tensor
-    long long P[kMaxSeg];
-    int blk_start[kMaxSeg + 1];      // first block of each tensor within this launch
-    int col[kMaxSeg];                // index l of the tensor in the [B, L] norm / factor tables
-    long long part_start[kMaxSeg];   // first partial slot of each tensor within one example's row of partials
-    long long goff[kMaxSeg];         // global index of the tensor's first parameter (per-example noise only)
+    const float *G[N];               // [B, P] per tensor
+    float *acc[N];                   // [P] per tensor
+    long long P[N];
+    long long part_start[N];         // first partial slot of each tensor within one example's row of partials
+    long long goff[N];               // global index of the tensor's first parameter (per-example noise only)
+    int blk_start[N];                // first block of each tensor within this launch
+    int col0;                        // index in the [B, L] norm / factor tables of the first of these consecutive tensors
     int nseg;
 };
 
@@ -37,15 +39,18 @@ struct ExampleNoise {
     uint32_t example0;               // index within the step of this chunk's first example
 };
 
-__device__ __forceinline__ int find_seg(const SegTable &t, int blk) {
-    int s = 0;
-    while (s + 1 < t.nseg && blk >= t.blk_start[s + 1]) ++s;
-    return s;
+template <int N>
+__device__ __forceinline__ int find_seg(const SegTable<N> &t, int blk) {
+    int lo = 0, hi = t.nseg;                                  // the last tensor whose first block is not past blk
+    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (blk >= t.blk_start[mid]) lo = mid; else hi = mid; }
+    return lo;
 }
 
-// stage 1a: partial[n][part_start[seg] + j] = sum of squares of G_seg[n, j*chunk .. (j+1)*chunk)
+// stage 1: partial[n][part_start[seg] + j] = sum of squares of G_seg[n, j*chunk .. (j+1)*chunk); up to three floats before
+// the first 16-byte boundary and after the last one are read alone
+template <int N>
 __global__ void __launch_bounds__(256)
-sqnorm_partial_kernel(const __grid_constant__ SegTable tab, float *__restrict__ partial, long long parts_per_example) {
+sqnorm_partial_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example) {
     __shared__ float scratch[32];
     const int seg = find_seg(tab, blockIdx.x);
     const int j = blockIdx.x - tab.blk_start[seg];
@@ -54,67 +59,26 @@ sqnorm_partial_kernel(const __grid_constant__ SegTable tab, float *__restrict__ 
     const long long c0 = (long long)j * kNormChunk;
     const int len = (int)min((long long)kNormChunk, P - c0);
     const float *row = tab.G[seg] + (long long)n * P + c0;
-    float a = 0.f;
-    if ((reinterpret_cast<uintptr_t>(row) & 15) == 0) {
-        const float4 *row4 = reinterpret_cast<const float4 *>(row);
-        const int n4 = len >> 2;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    const int head = min(len, (int)((0u - (unsigned)(reinterpret_cast<uintptr_t>(row) >> 2)) & 3u));
+    const float4 *row4 = reinterpret_cast<const float4 *>(row + head);
+    const int n4 = (len - head) >> 2, tail = head + 4 * n4;
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll 4
-        for (int i = threadIdx.x; i < n4; i += 256) {
-            const float4 v = __ldg(row4 + i);
-            a0 = fmaf(v.x, v.x, a0); a1 = fmaf(v.y, v.y, a1); a2 = fmaf(v.z, v.z, a2); a3 = fmaf(v.w, v.w, a3);
-        }
-        a = (a0 + a1) + (a2 + a3);
-        for (int i = (n4 << 2) + threadIdx.x; i < len; i += 256) a = fmaf(row[i], row[i], a);
-    } else {
-        for (int i = threadIdx.x; i < len; i += 256) a = fmaf(row[i], row[i], a);
+    for (int i = threadIdx.x; i < n4; i += 256) {
+        const float4 v = __ldg(row4 + i);
+        a0 = fmaf(v.x, v.x, a0); a1 = fmaf(v.y, v.y, a1); a2 = fmaf(v.z, v.z, a2); a3 = fmaf(v.w, v.w, a3);
     }
-    a = block_sum(a, scratch);
+    if ((int)threadIdx.x < head) a0 = fmaf(row[threadIdx.x], row[threadIdx.x], a0);
+    if (tail + (int)threadIdx.x < len) a1 = fmaf(row[tail + threadIdx.x], row[tail + threadIdx.x], a1);
+    const float a = block_sum((a0 + a1) + (a2 + a3), scratch);
     if (threadIdx.x == 0) partial[(long long)n * parts_per_example + tab.part_start[seg] + j] = a;
 }
 
-// stage 1b: sq[n][col[seg]] = sum over the tensor's partials, in index order, in double
-__global__ void __launch_bounds__(128)
-sqnorm_fold_kernel(const __grid_constant__ SegTable tab, const float *__restrict__ partial,
-                   long long parts_per_example, float *__restrict__ sq, int L) {
-    __shared__ double scratch[32];
-    const int seg = blockIdx.x, n = blockIdx.y;
-    const long long nparts = (tab.P[seg] + kNormChunk - 1) / kNormChunk;
-    const float *p = partial + (long long)n * parts_per_example + tab.part_start[seg];
-    double a = 0.0;
-    for (long long i = threadIdx.x; i < nparts; i += 128) a += (double)p[i];
-    a = block_sum(a, scratch);
-    if (threadIdx.x == 0) sq[(long long)n * L + tab.col[seg]] = (float)a;
-}
-
-// stage 2: factors.  GLOBAL: one factor per example from the sum over its L tensors (thread per example).
-// PER_LAYER: one factor per (example, tensor) against C/sqrt(L).
-__global__ void clip_factor_kernel(const float *__restrict__ sq, int B, int L, int per_layer, float C,
-                                   float *__restrict__ factor, float *norms_out, float *clip_out) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (per_layer) {
-        if (idx >= B * L) return;
-        const float thr = (float)((double)C / sqrt((double)L));
-        const double s = (double)sq[idx];
-        const float f = clip_factor(s, thr);
-        factor[idx] = f;
-        if (norms_out) norms_out[idx] = (float)sqrt(s);
-        if (clip_out) clip_out[idx] = f;
-    } else {
-        if (idx >= B) return;
-        double s = 0.0;
-        for (int l = 0; l < L; ++l) s += (double)sq[(long long)idx * L + l];
-        const float f = clip_factor(s, C);
-        factor[idx] = f;
-        if (norms_out) norms_out[idx] = (float)sqrt(s);
-        if (clip_out) clip_out[idx] = f;
-    }
-}
-
-// stage 1a for micro-batch clipping: row j of the partials belongs to the MEAN of examples j*micro .. j*micro+micro-1
+// stage 1 for micro-batch clipping: row j of the partials belongs to the MEAN of examples j*micro .. j*micro+micro-1
 // (the unit that is clipped), so the rows are added before they are squared.
+template <int N>
 __global__ void __launch_bounds__(256)
-sqnorm_partial_micro_kernel(const __grid_constant__ SegTable tab, float *__restrict__ partial,
+sqnorm_partial_micro_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial,
                             long long parts_per_example, int micro) {
     __shared__ float scratch[32];
     const int seg = find_seg(tab, blockIdx.x);
@@ -154,52 +118,119 @@ sqnorm_partial_micro_kernel(const __grid_constant__ SegTable tab, float *__restr
     if (threadIdx.x == 0) partial[(long long)blockIdx.y * parts_per_example + tab.part_start[seg] + j] = a;
 }
 
-// stage 2 for micro-batch clipping: one factor per micro-batch from the norm of its mean; every example of the
-// micro-batch then carries factor / micro, so that stage 3 adds factor * mean.
-__global__ void clip_factor_micro_kernel(const float *__restrict__ sq, int n_micro, int L, int micro, float C,
-                                         float *__restrict__ factor, float *norms_out, float *clip_out) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n_micro) return;
-    double s = 0.0;
-    for (int l = 0; l < L; ++l) s += (double)sq[(long long)j * L + l];
-    const float f = clip_factor(s, C);
-    const float each = f / (float)micro;
-    for (int i = 0; i < micro; ++i) factor[(long long)j * micro + i] = each;
-    if (norms_out) norms_out[j] = (float)sqrt(s);
-    if (clip_out) clip_out[j] = f;
-}
-
-// stage 2 for groups of tensors (section 3.5: M pipeline stages, each clipped to C/sqrt(M)): one block per example
-// sums the squared norms of each group's tensors in tensor order, then every tensor gets its group's factor.
+// stage 2.  A block per row (an example, or a micro-batch): folds the partials of this launch's tensors to squared norms,
+// in double, and after the last table turns the row's norms into factors.
+//   kGlobal   one factor from the sum over the L tensors; the `micro` examples of the row each carry factor / micro, so that
+//             stage 3 adds factor * mean
+//   kPerLayer one factor per tensor against C/sqrt(L)
+//   kGrouped  one factor per group of tensors (section 3.5: M pipeline stages, each clipped to C/sqrt(M))
+// A latency chain: many small loads, so they go side by side over the block (thread per group walking 161 tensors one by
+// one, and a fold launch of its own: 13 us for 16 examples).
+enum { kGlobal = 0, kPerLayer, kGrouped };
+constexpr int kFactorThreads = 256;
+constexpr int kPartsPerWarp = 256;                   // tensors with more partials are folded by the whole block
 constexpr int kMaxGroupedTensors = 1024;
 struct GroupTable {
     int M;
     unsigned short of[kMaxGroupedTensors];   // group of tensor l
 };
-__global__ void __launch_bounds__(128)
-clip_factor_grouped_kernel(const float *__restrict__ sq, int L, const __grid_constant__ GroupTable gt, float C,
-                           float *__restrict__ factor, float *norms_out, float *clip_out) {
-    __shared__ float f_sh[kMaxGroupedTensors];
-    const int n = blockIdx.x;
-    const float thr = (float)((double)C / sqrt((double)gt.M));
-    for (int m = threadIdx.x; m < gt.M; m += 128) {
-        double s = 0.0;
-        for (int l = 0; l < L; ++l)
-            if (gt.of[l] == m) s += (double)sq[(long long)n * L + l];
-        const float f = clip_factor(s, thr);
-        f_sh[m] = f;
-        if (norms_out) norms_out[(long long)n * gt.M + m] = (float)sqrt(s);
-        if (clip_out) clip_out[(long long)n * gt.M + m] = f;
+template <int N, int KIND>
+__global__ void __launch_bounds__(kFactorThreads)
+norm_factor_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ partial, long long parts_per_row,
+                   const float *sq_in, float *sq_ws, int L, int micro, int last, float C, const __grid_constant__ GroupTable gt,
+                   float *__restrict__ factor, float *norms_out, float *clip_out) {
+    __shared__ double scratch[32];
+    __shared__ float f_sh[KIND == kGrouped ? kMaxGroupedTensors : 1];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const long long row = blockIdx.x;
+    if (partial) {
+        float *out = sq_ws + row * L + tab.col0;
+        for (int s = w; s < tab.nseg; s += kFactorThreads / 32) {
+            const long long nparts = (tab.P[s] + kNormChunk - 1) / kNormChunk;
+            if (nparts > kPartsPerWarp) continue;
+            const float *p = partial + row * parts_per_row + tab.part_start[s];
+            double a = 0.0;
+#pragma unroll 4
+            for (int i = lane; i < (int)nparts; i += 32) a += (double)p[i];
+            a = warp_sum(a);
+            if (lane == 0) out[s] = (float)a;
+        }
+        for (int s = 0; s < tab.nseg; ++s) {
+            const long long nparts = (tab.P[s] + kNormChunk - 1) / kNormChunk;
+            if (nparts <= kPartsPerWarp) continue;
+            const float *p = partial + row * parts_per_row + tab.part_start[s];
+            double a = 0.0;
+#pragma unroll 4
+            for (long long i = threadIdx.x; i < nparts; i += kFactorThreads) a += (double)p[i];
+            a = block_sum(a, scratch);
+            if (threadIdx.x == 0) out[s] = (float)a;
+        }
+        if (!last) return;
+        __syncthreads();                             // the norms written above are read below, by other threads of the block
     }
-    __syncthreads();
-    for (int l = threadIdx.x; l < L; l += 128) factor[(long long)n * L + l] = f_sh[gt.of[l]];
+    const float *sq = (partial ? sq_ws : sq_in) + row * L;
+    if (KIND == kGlobal) {
+        double s = 0.0;
+        for (int l = threadIdx.x; l < L; l += kFactorThreads) s += (double)sq[l];
+        s = block_sum(s, scratch);
+        const float f = clip_factor(s, C), each = micro == 1 ? f : f / (float)micro;
+        for (int i = threadIdx.x; i < micro; i += kFactorThreads) factor[row * micro + i] = each;
+        if (threadIdx.x == 0) {
+            if (norms_out) norms_out[row] = (float)sqrt(s);
+            if (clip_out) clip_out[row] = f;
+        }
+    } else if (KIND == kPerLayer) {
+        const float thr = (float)((double)C / sqrt((double)L));
+        for (int l = threadIdx.x; l < L; l += kFactorThreads) {
+            const double s = (double)sq[l];
+            const float f = clip_factor(s, thr);
+            factor[row * L + l] = f;
+            if (norms_out) norms_out[row * L + l] = (float)sqrt(s);
+            if (clip_out) clip_out[row * L + l] = f;
+        }
+    } else {
+        const float thr = (float)((double)C / sqrt((double)gt.M));
+        for (int m = w; m < gt.M; m += kFactorThreads / 32) {
+            double s = 0.0;
+            for (int l = lane; l < L; l += 32)
+                if (gt.of[l] == m) s += (double)sq[l];
+            s = warp_sum(s);
+            if (lane == 0) {
+                const float f = clip_factor(s, thr);
+                f_sh[m] = f;
+                if (norms_out) norms_out[row * gt.M + m] = (float)sqrt(s);
+                if (clip_out) clip_out[row * gt.M + m] = f;
+            }
+        }
+        __syncthreads();
+        for (int l = threadIdx.x; l < L; l += kFactorThreads) factor[row * L + l] = f_sh[gt.of[l]];
+    }
 }
 
-// stage 3: acc[i] += sum_n factor * G[n, i].  factor index: GLOBAL n, PER_LAYER n*L + col.
-template <int UNROLL>
+// stage 2 with the norms given and few of them a row: a thread per example (kGlobal) or per norm (kPerLayer)
+constexpr int kFewTensors = 32;
+__global__ void clip_factor_kernel(const float *__restrict__ sq, int B, int L, int per_layer, float C,
+                                   float *__restrict__ factor, float *norms_out, float *clip_out) {
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (per_layer ? B * L : B)) return;
+    const float thr = per_layer ? (float)((double)C / sqrt((double)L)) : C;
+    double s = 0.0;
+    if (per_layer) s = (double)sq[idx];
+    else
+        for (int l = 0; l < L; ++l) s += (double)sq[(long long)idx * L + l];
+    const float f = clip_factor(s, thr);
+    factor[idx] = f;
+    if (norms_out) norms_out[idx] = (float)sqrt(s);
+    if (clip_out) clip_out[idx] = f;
+}
+
+// stage 3: acc[i] += sum_n factor * G[n, i].  factor index: GLOBAL n, PER_LAYER n*L + col.  Streams B*P floats once; loads
+// past the L1 (evict-first: nothing comes back).
+template <int N>
 __global__ void __launch_bounds__(256)
-scale_accumulate_kernel(const __grid_constant__ SegTable tab, const float *__restrict__ factor, int B, int L,
+scale_accumulate_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
                         int per_layer) {
+    constexpr int kRows = 8;                                   // rows in flight per thread
     __shared__ float f_sh[256];
     const int seg = find_seg(tab, blockIdx.x);
     const long long P = tab.P[seg];
@@ -207,7 +238,7 @@ scale_accumulate_kernel(const __grid_constant__ SegTable tab, const float *__res
     const float *G = tab.G[seg];
     float *acc = tab.acc[seg];
     const int f_stride = per_layer ? L : 1;
-    const int f_off = per_layer ? tab.col[seg] : 0;
+    const int f_off = per_layer ? tab.col0 + seg : 0;
     // vector path needs every row start 16-byte aligned: base aligned and P a multiple of 4
     const bool vec = ((P & 3) == 0) && ((reinterpret_cast<uintptr_t>(G) & 15) == 0) &&
                      ((reinterpret_cast<uintptr_t>(acc) & 15) == 0);
@@ -222,23 +253,19 @@ scale_accumulate_kernel(const __grid_constant__ SegTable tab, const float *__res
             __syncthreads();
             if (live) {
                 const float *g = G + (long long)n0 * P + i;
-                int n = 0;
-                for (; n + UNROLL <= nb; n += UNROLL) {
-                    float4 v[UNROLL];
+                for (int n = 0; n < nb; n += kRows) {
+                    float4 v[kRows];
 #pragma unroll
-                    for (int u = 0; u < UNROLL; ++u)
-                        v[u] = __ldcs(reinterpret_cast<const float4 *>(g + (long long)(n + u) * P));
+                    for (int u = 0; u < kRows; ++u) {
+                        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (n + u < nb) v[u] = __ldcs(reinterpret_cast<const float4 *>(g + (long long)(n + u) * P));
+                    }
 #pragma unroll
-                    for (int u = 0; u < UNROLL; ++u) {
-                        const float f = f_sh[n + u];
+                    for (int u = 0; u < kRows; ++u) {
+                        const float f = n + u < nb ? f_sh[n + u] : 0.f;
                         s.x = fmaf(f, v[u].x, s.x); s.y = fmaf(f, v[u].y, s.y);
                         s.z = fmaf(f, v[u].z, s.z); s.w = fmaf(f, v[u].w, s.w);
                     }
-                }
-                for (; n < nb; ++n) {
-                    const float4 v = __ldcs(reinterpret_cast<const float4 *>(g + (long long)n * P));
-                    const float f = f_sh[n];
-                    s.x = fmaf(f, v.x, s.x); s.y = fmaf(f, v.y, s.y); s.z = fmaf(f, v.z, s.z); s.w = fmaf(f, v.w, s.w);
                 }
             }
         }
@@ -248,106 +275,105 @@ scale_accumulate_kernel(const __grid_constant__ SegTable tab, const float *__res
             *reinterpret_cast<float4 *>(acc + i) = a;
         }
     } else {
+        // rows at any address: columns 256 apart, so that the lanes of a load are neighbours wherever the row starts
         float s[4] = {0.f, 0.f, 0.f, 0.f};
+        const long long left = P - c0 - threadIdx.x;           // column q of this thread exists when 256 q < left
         for (int n0 = 0; n0 < B; n0 += 256) {
             const int nb = min(256, B - n0);
             __syncthreads();
             if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
             __syncthreads();
-            for (int n = 0; n < nb; ++n) {
-                const float f = f_sh[n];
-                const float *g = G + (long long)(n0 + n) * P + c0;
+            const float *g = G + (long long)n0 * P + c0 + threadIdx.x;
+            for (int n = 0; n < nb; n += kRows) {
+                float v[kRows][4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const long long i = threadIdx.x + 256 * q;
-                    if (c0 + i < P) s[q] = fmaf(f, g[i], s[q]);
+                for (int u = 0; u < kRows; ++u)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        v[u][q] = 0.f;
+                        if (n + u < nb && 256 * q < left) v[u][q] = __ldcs(g + (long long)(n + u) * P + 256 * q);
+                    }
+#pragma unroll
+                for (int u = 0; u < kRows; ++u) {
+                    const float f = n + u < nb ? f_sh[n + u] : 0.f;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) s[q] = fmaf(f, v[u][q], s[q]);
                 }
             }
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const long long i = c0 + threadIdx.x + 256 * q;
-            if (i < P) acc[i] += s[q];
-        }
+        for (int q = 0; q < 4; ++q)
+            if (256 * q < left) acc[c0 + threadIdx.x + 256 * q] += s[q];
     }
 }
 
 // stage 3 for small models with many examples: too few 1024-parameter blocks exist to fill the GPU, so a block takes
-// only 128 parameters and splits the example rows over its eight warps (warp w owns rows w, w+8, ...), sixteen rows in
-// flight per thread; the eight partial sums are folded in warp order through shared memory.
+// only 128 parameters and splits the example rows over its eight warps (warp w owns every eighth row), eight rows in
+// flight per thread; the eight partial sums are folded in warp order through shared memory.  The blocks are all resident
+// or nearly so and walk the examples from the last to the first: stage 1 read those rows last, so that most of a gradient
+// up to twice the L2 is still there (256 rows of 175 178 floats, which start at any address: 103 us for the call with four
+// words at a time of one row a thread, in ascending order).
 constexpr int kSplitCols = 128;
+template <int N>
 __global__ void __launch_bounds__(256)
-scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable tab, const float *__restrict__ factor, int B, int L,
+scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
                                  int per_layer) {
+    constexpr int kRows = 8;
     __shared__ float f_sh[256];
-    __shared__ float4 part[8][32];
+    __shared__ float part[8][kSplitCols];
     const int seg = find_seg(tab, blockIdx.x);
     const long long P = tab.P[seg];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const long long i = (long long)(blockIdx.x - tab.blk_start[seg]) * kSplitCols + 4 * lane;
+    const long long c0 = (long long)(blockIdx.x - tab.blk_start[seg]) * kSplitCols;
     const float *G = tab.G[seg];
     float *acc = tab.acc[seg];
     const int f_stride = per_layer ? L : 1;
-    const int f_off = per_layer ? tab.col[seg] : 0;
-    const bool vec = ((P & 3) == 0) && ((reinterpret_cast<uintptr_t>(G) & 15) == 0) &&
-                     ((reinterpret_cast<uintptr_t>(acc) & 15) == 0);
-    const int live = i >= P ? 0 : (int)min(4ll, P - i);           // parameters this thread owns (vec: 0 or 4)
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int n0 = 0; n0 < B; n0 += 256) {
+    const int f_off = per_layer ? tab.col0 + seg : 0;
+    const bool vec = ((P & 3) == 0) && ((reinterpret_cast<uintptr_t>(G) & 15) == 0);
+    // vec: four neighbouring columns of this lane, all or none; otherwise columns 32 apart
+    const long long left = P - c0 - (vec ? 4 * lane : lane);
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int n0 = (B - 1) & ~255; n0 >= 0; n0 -= 256) {
         const int nb = min(256, B - n0);
         __syncthreads();
         if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
         __syncthreads();
-        if (live == 0) continue;
-        const float *g = G + (long long)n0 * P + i;
-        if (vec) {
-            int n = w;
-            for (; n + 8 * 15 < nb; n += 8 * 16) {
-                float4 v[16];
+        if (left <= 0) continue;
+        const float *g = G + (long long)n0 * P + c0 + (vec ? 4 * lane : lane);
+        for (int n = nb - 1 - w; n >= 0; n -= 8 * kRows) {
+            float v[kRows][4];
+            if (vec) {
 #pragma unroll
-                for (int u = 0; u < 16; ++u) v[u] = __ldcs(reinterpret_cast<const float4 *>(g + (long long)(n + 8 * u) * P));
-#pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    const float f = f_sh[n + 8 * u];
-                    s.x = fmaf(f, v[u].x, s.x); s.y = fmaf(f, v[u].y, s.y);
-                    s.z = fmaf(f, v[u].z, s.z); s.w = fmaf(f, v[u].w, s.w);
+                for (int u = 0; u < kRows; ++u) {
+                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (n - 8 * u >= 0) x = __ldcs(reinterpret_cast<const float4 *>(g + (long long)(n - 8 * u) * P));
+                    v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
                 }
+            } else {
+#pragma unroll
+                for (int u = 0; u < kRows; ++u)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        v[u][q] = 0.f;
+                        if (n - 8 * u >= 0 && 32 * q < left) v[u][q] = __ldcs(g + (long long)(n - 8 * u) * P + 32 * q);
+                    }
             }
-            for (; n < nb; n += 8) {
-                const float4 v = __ldcs(reinterpret_cast<const float4 *>(g + (long long)n * P));
-                const float f = f_sh[n];
-                s.x = fmaf(f, v.x, s.x); s.y = fmaf(f, v.y, s.y); s.z = fmaf(f, v.z, s.z); s.w = fmaf(f, v.w, s.w);
-            }
-        } else {
-            for (int n = w; n < nb; n += 8) {
-                const float *row = g + (long long)n * P;
-                const float f = f_sh[n];
-                s.x = fmaf(f, row[0], s.x);
-                if (live > 1) s.y = fmaf(f, row[1], s.y);
-                if (live > 2) s.z = fmaf(f, row[2], s.z);
-                if (live > 3) s.w = fmaf(f, row[3], s.w);
+#pragma unroll
+            for (int u = 0; u < kRows; ++u) {
+                const float f = n - 8 * u >= 0 ? f_sh[n - 8 * u] : 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] = fmaf(f, v[u][q], s[q]);
             }
         }
     }
-    part[w][lane] = s;
-    __syncthreads();
-    if (w == 0 && live > 0) {
-        float4 t = part[0][lane];
 #pragma unroll
-        for (int q = 1; q < 8; ++q) {
-            const float4 v = part[q][lane];
-            t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
-        }
-        if (vec) {
-            float4 a = *reinterpret_cast<const float4 *>(acc + i);
-            a.x += t.x; a.y += t.y; a.z += t.z; a.w += t.w;
-            *reinterpret_cast<float4 *>(acc + i) = a;
-        } else {
-            acc[i] += t.x;
-            if (live > 1) acc[i + 1] += t.y;
-            if (live > 2) acc[i + 2] += t.z;
-            if (live > 3) acc[i + 3] += t.w;
-        }
+    for (int q = 0; q < 4; ++q) part[w][vec ? 4 * lane + q : lane + 32 * q] = s[q];
+    __syncthreads();
+    if (threadIdx.x < kSplitCols && c0 + threadIdx.x < P) {
+        float t = part[0][threadIdx.x];
+#pragma unroll
+        for (int q = 1; q < 8; ++q) t += part[q][threadIdx.x];
+        acc[c0 + threadIdx.x] += t;
     }
 }
 
@@ -355,8 +381,9 @@ scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable tab, const flo
 // Every thread owns the four parameters of one Philox block when the tensor starts on a multiple of four global
 // indices; otherwise each parameter draws its own block and keeps one lane.  Bound by the integer and
 // transcendental work of B*P normals, not by memory.
+template <int N>
 __global__ void __launch_bounds__(256)
-scale_accumulate_noised_kernel(const __grid_constant__ SegTable tab, const float *__restrict__ factor, int B, int L,
+scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
                                int per_layer, const __grid_constant__ ExampleNoise nz) {
     __shared__ float f_sh[256];
     const int seg = find_seg(tab, blockIdx.x);
@@ -366,7 +393,7 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable tab, const float
     float *acc = tab.acc[seg];
     const long long goff = tab.goff[seg];
     const int f_stride = per_layer ? L : 1;
-    const int f_off = per_layer ? tab.col[seg] : 0;
+    const int f_off = per_layer ? tab.col0 + seg : 0;
     const bool vec = ((P & 3) == 0) && ((goff & 3) == 0) && ((reinterpret_cast<uintptr_t>(G) & 15) == 0) &&
                      ((reinterpret_cast<uintptr_t>(acc) & 15) == 0);
     if (vec) {
@@ -478,14 +505,109 @@ struct ClipVariant {
     const float *given_factor = nullptr;   // stage 3 only, with the caller's factors ([B] or [B, L]); no workspace
 };
 
+struct ClipCall {
+    int B, L, per_layer;
+    const float *const *G;
+    const long long *P_l;
+    float *const *acc;
+    const float *sq;                       // given squared norms, or null: `partial` and `sq_ws` receive them
+    float *partial, *sq_ws, *factor_ws;
+    const float *factor;
+    float C;
+    float *norms_out, *clip_out;
+    long long parts_per_example;
+};
+
+static dp_status launch_factors(const ClipCall &c, const ClipVariant &var, cudaStream_t stream);
+
+// The launches of one call, its tensors in tables of N.
+template <int N>
+static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaStream_t stream) {
+    const int B = c.B, L = c.L, micro = var.micro;
+    // A small model gives few wide blocks, and each thread would walk all B rows alone: with many rows the block narrows
+    // to 128 parameters and its warps share the rows (from two rows a warp on where not even two wide blocks an SM exist,
+    // from eight on up to a wave of them).
+    long long wide_blocks = 0;
+    for (int l = 0; l < L; ++l) wide_blocks += (c.P_l[l] + kAccCols - 1) / kAccCols;
+    const bool split = !var.noise && ((B >= 64 && wide_blocks < 8 * sm_count()) || (B >= 16 && wide_blocks < 2 * sm_count()));
+    const int acc_cols = split ? kSplitCols : kAccCols;
+
+    SegTable<N> t;
+    auto fill = [&](int l0, bool norm_blocks, long long &part_cursor) {
+        t.nseg = 0; t.col0 = l0;
+        int blk = 0;
+        for (int l = l0; l < L && t.nseg < N; ++l) {
+            const int s = t.nseg;
+            const long long nparts = (c.P_l[l] + kNormChunk - 1) / kNormChunk;
+            const long long nb = norm_blocks ? nparts : (c.P_l[l] + acc_cols - 1) / acc_cols;
+            if ((long long)blk + nb > 0x7fffffffll) break;
+            t.G[s] = c.G[l]; t.acc[s] = c.acc[l]; t.P[s] = c.P_l[l];
+            t.goff[s] = var.goff_l ? var.goff_l[l] : 0;
+            t.blk_start[s] = blk; t.part_start[s] = part_cursor;
+            part_cursor += nparts; blk += (int)nb; ++t.nseg;
+        }
+        return blk;
+    };
+    if (!var.given_factor && c.sq) {
+        const dp_status rc = launch_factors(c, var, stream);
+        if (rc != DP_OK) return rc;
+    } else if (!var.given_factor) {
+        long long cursor = 0;
+        const unsigned rows = (unsigned)(B / micro);
+        for (int l0 = 0; l0 < L; l0 += t.nseg) {
+            const int blocks = fill(l0, true, cursor);
+            if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
+            if (micro > 1) sqnorm_partial_micro_kernel<N><<<dim3((unsigned)blocks, rows), 256, 0, stream>>>(t, c.partial, c.parts_per_example, micro);
+            else sqnorm_partial_kernel<N><<<dim3((unsigned)blocks, rows), 256, 0, stream>>>(t, c.partial, c.parts_per_example);
+            DP_LAUNCH_CHECK("sqnorm_partial_kernel");
+            const int last = l0 + t.nseg == L;
+            static const GroupTable none = {};
+            const GroupTable &gt = var.groups ? *var.groups : none;
+            if (var.groups)
+                norm_factor_kernel<N, kGrouped><<<rows, kFactorThreads, 0, stream>>>(t, c.partial, c.parts_per_example, nullptr, c.sq_ws, L, micro, last, c.C, gt, c.factor_ws, c.norms_out, c.clip_out);
+            else if (c.per_layer)
+                norm_factor_kernel<N, kPerLayer><<<rows, kFactorThreads, 0, stream>>>(t, c.partial, c.parts_per_example, nullptr, c.sq_ws, L, micro, last, c.C, gt, c.factor_ws, c.norms_out, c.clip_out);
+            else
+                norm_factor_kernel<N, kGlobal><<<rows, kFactorThreads, 0, stream>>>(t, c.partial, c.parts_per_example, nullptr, c.sq_ws, L, micro, last, c.C, gt, c.factor_ws, c.norms_out, c.clip_out);
+            DP_LAUNCH_CHECK("norm_factor_kernel");
+        }
+    }
+    long long cursor = 0;
+    for (int l0 = 0; l0 < L; l0 += t.nseg) {
+        const int blocks = fill(l0, false, cursor);
+        if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
+        if (var.noise) scale_accumulate_noised_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, *var.noise);
+        else if (split) scale_accumulate_rowsplit_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer);
+        else scale_accumulate_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer);
+        DP_LAUNCH_CHECK("scale_accumulate_kernel");
+    }
+    return DP_OK;
+}
+
+// stage 2 from given squared norms
+static dp_status launch_factors(const ClipCall &c, const ClipVariant &var, cudaStream_t stream) {
+    const bool few = !var.groups && (c.per_layer || c.L <= kFewTensors);
+    if (few) {
+        const long long count = c.per_layer ? (long long)c.B * c.L : c.B;
+        clip_factor_kernel<<<(unsigned)((count + 127) / 128), 128, 0, stream>>>(c.sq, c.B, c.L, c.per_layer, c.C, c.factor_ws, c.norms_out, c.clip_out);
+    } else {
+        SegTable<1> t;
+        t.nseg = 0; t.col0 = 0;
+        static const GroupTable none = {};
+        if (var.groups)
+            norm_factor_kernel<1, kGrouped><<<(unsigned)c.B, kFactorThreads, 0, stream>>>(t, nullptr, 0, c.sq, nullptr, c.L, 1, 1, c.C, *var.groups, c.factor_ws, c.norms_out, c.clip_out);
+        else
+            norm_factor_kernel<1, kGlobal><<<(unsigned)c.B, kFactorThreads, 0, stream>>>(t, nullptr, 0, c.sq, nullptr, c.L, 1, 1, c.C, none, c.factor_ws, c.norms_out, c.clip_out);
+    }
+    DP_LAUNCH_CHECK("clip_factor_kernel");
+    return DP_OK;
+}
+
 // Host side of dp_clip_accumulate and its variants.
 static dp_status clip_accumulate_impl(int mode, int B, int L, const float *const *G, const long long *P_l,
                                       const float *sqnorm, float C, float *const *acc, float *norms_out,
                                       float *clip_out, void *workspace, size_t workspace_bytes, void *cuda_stream,
                                       const ClipVariant &var = ClipVariant()) {
-    const ExampleNoise *noise = var.noise;
-    const long long *goff_l = var.goff_l;
-    const int micro = var.micro;
     if (mode != DP_CLIP_GLOBAL && mode != DP_CLIP_PER_LAYER) return DP_ERR_INVALID_ARG;
     if (B <= 0 || L <= 0 || !G || !P_l || !acc || !(C > 0.0f)) return DP_ERR_INVALID_ARG;
     if (B > 65535) return DP_ERR_UNSUPPORTED;
@@ -500,81 +622,18 @@ static dp_status clip_accumulate_impl(int mode, int B, int L, const float *const
     if (!stage3_only && (!workspace || !aligned(workspace, 256) || workspace_bytes < pl.total)) return DP_ERR_WORKSPACE;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     char *ws = static_cast<char *>(workspace);
-    float *partial = stage3_only ? nullptr : reinterpret_cast<float *>(ws + pl.partial_off);
-    float *sq_ws = stage3_only ? nullptr : reinterpret_cast<float *>(ws + pl.sq_off);
-    const float *factor = stage3_only ? var.given_factor : reinterpret_cast<float *>(ws + pl.factor_off);
-    float *factor_ws = stage3_only ? nullptr : reinterpret_cast<float *>(ws + pl.factor_off);
-    const int per_layer = (mode == DP_CLIP_PER_LAYER);
-
-    // tensors go to the kernels in tables of at most kMaxSeg entries
-    long long wide_blocks = 0;
-    for (int l = 0; l < L; ++l) wide_blocks += (P_l[l] + kAccCols - 1) / kAccCols;
-    // A small model gives few blocks, and each thread would walk all B rows alone: with many rows the block narrows
-    // to 128 parameters and its warps share the rows.
-    const bool split = B >= 64 && wide_blocks < 8 * sm_count();
-    const int acc_cols = (split && !noise) ? kSplitCols : kAccCols;
-
-    auto fill = [&](int l0, SegTable &t, bool norm_blocks, long long &part_cursor) {
-        t.nseg = 0;
-        int blk = 0;
-        for (int l = l0; l < L && t.nseg < kMaxSeg; ++l) {
-            const int s = t.nseg++;
-            t.G[s] = G[l]; t.acc[s] = acc[l]; t.P[s] = P_l[l]; t.col[s] = l;
-            t.goff[s] = goff_l ? goff_l[l] : 0;
-            t.blk_start[s] = blk;
-            t.part_start[s] = part_cursor;
-            const long long nparts = (P_l[l] + kNormChunk - 1) / kNormChunk;
-            part_cursor += nparts;
-            const long long nb = norm_blocks ? nparts : (P_l[l] + acc_cols - 1) / acc_cols;
-            if ((long long)blk + nb > 0x7fffffffll) { --t.nseg; part_cursor -= nparts; break; }
-            blk += (int)nb;
-        }
-        t.blk_start[t.nseg] = blk;
-        return blk;
-    };
-
-    const float *sq = sqnorm;
-    if (!sq && !stage3_only) {
-        long long cursor = 0;
-        for (int l0 = 0; l0 < L;) {
-            SegTable t;
-            const int blocks = fill(l0, t, true, cursor);
-            if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
-            if (micro > 1)
-                sqnorm_partial_micro_kernel<<<dim3((unsigned)blocks, (unsigned)(B / micro)), 256, 0, stream>>>(t, partial, pl.parts_per_example, micro);
-            else
-                sqnorm_partial_kernel<<<dim3((unsigned)blocks, (unsigned)B), 256, 0, stream>>>(t, partial, pl.parts_per_example);
-            DP_LAUNCH_CHECK("sqnorm_partial_kernel");
-            sqnorm_fold_kernel<<<dim3((unsigned)t.nseg, (unsigned)(B / micro)), 128, 0, stream>>>(t, partial, pl.parts_per_example, sq_ws, L);
-            DP_LAUNCH_CHECK("sqnorm_fold_kernel");
-            l0 += t.nseg;
-        }
-        sq = sq_ws;
+    ClipCall c = {};
+    c.B = B; c.L = L; c.per_layer = mode == DP_CLIP_PER_LAYER;
+    c.G = G; c.P_l = P_l; c.acc = acc; c.sq = sqnorm; c.C = C; c.norms_out = norms_out; c.clip_out = clip_out;
+    c.parts_per_example = pl.parts_per_example;
+    if (stage3_only) {
+        c.factor = var.given_factor;
+    } else {
+        c.partial = reinterpret_cast<float *>(ws + pl.partial_off);
+        c.sq_ws = reinterpret_cast<float *>(ws + pl.sq_off);
+        c.factor = c.factor_ws = reinterpret_cast<float *>(ws + pl.factor_off);
     }
-    if (!stage3_only) {
-        const long long count = per_layer ? (long long)B * L : B;
-        if (var.groups)
-            clip_factor_grouped_kernel<<<(unsigned)B, 128, 0, stream>>>(sq, L, *var.groups, C, factor_ws, norms_out, clip_out);
-        else if (micro > 1)
-            clip_factor_micro_kernel<<<(unsigned)((B / micro + 127) / 128), 128, 0, stream>>>(sq, B / micro, L, micro, C, factor_ws, norms_out, clip_out);
-        else
-            clip_factor_kernel<<<(unsigned)((count + 127) / 128), 128, 0, stream>>>(sq, B, L, per_layer, C, factor_ws, norms_out, clip_out);
-        DP_LAUNCH_CHECK("clip_factor_kernel");
-    }
-    {
-        long long cursor = 0;
-        for (int l0 = 0; l0 < L;) {
-            SegTable t;
-            const int blocks = fill(l0, t, false, cursor);
-            if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
-            if (noise) scale_accumulate_noised_kernel<<<(unsigned)blocks, 256, 0, stream>>>(t, factor, B, L, per_layer, *noise);
-            else if (split) scale_accumulate_rowsplit_kernel<<<(unsigned)blocks, 256, 0, stream>>>(t, factor, B, L, per_layer);
-            else scale_accumulate_kernel<8><<<(unsigned)blocks, 256, 0, stream>>>(t, factor, B, L, per_layer);
-            DP_LAUNCH_CHECK("scale_accumulate_kernel");
-            l0 += t.nseg;
-        }
-    }
-    return DP_OK;
+    return L <= kSmallTable ? clip_launches<kSmallTable>(c, var, stream) : clip_launches<kLargeTable>(c, var, stream);
 }
 }  // namespace dp
 
@@ -590,12 +649,10 @@ extern "C" dp_status dp_clip_factors(int mode, int B, int L, const float *sqnorm
     if (mode != DP_CLIP_GLOBAL && mode != DP_CLIP_PER_LAYER) return DP_ERR_INVALID_ARG;
     if (B <= 0 || L <= 0 || !sqnorm || !factors_out || !(C > 0.0f)) return DP_ERR_INVALID_ARG;
     if (!dp::aligned(sqnorm, 4) || !dp::aligned(factors_out, 4) || (norms_out && !dp::aligned(norms_out, 4))) return DP_ERR_INVALID_ARG;
-    const int per_layer = (mode == DP_CLIP_PER_LAYER);
-    const long long count = per_layer ? (long long)B * L : B;
-    dp::clip_factor_kernel<<<(unsigned)((count + 127) / 128), 128, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        sqnorm, B, L, per_layer, C, factors_out, norms_out, nullptr);
-    DP_LAUNCH_CHECK("clip_factor_kernel");
-    return DP_OK;
+    dp::ClipCall c = {};
+    c.B = B; c.L = L; c.per_layer = mode == DP_CLIP_PER_LAYER;
+    c.sq = sqnorm; c.C = C; c.factor_ws = factors_out; c.norms_out = norms_out;
+    return dp::launch_factors(c, dp::ClipVariant(), static_cast<cudaStream_t>(cuda_stream));
 }
 
 extern "C" dp_status dp_scale_accumulate(int B, int L, const float *const *G, const long long *P_l, const float *factor,
