@@ -42,10 +42,10 @@ static bool side_streams(const dp_batch &b) {
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
     if (b.device >= 0) return b.device == dev;
     bool ok = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&b.gram_done, cudaEventDisableTiming) == cudaSuccess;
-    for (int i = 1; ok && i < BatchStreams::kCount; ++i)
-        ok = cudaStreamCreateWithFlags(&b.side[i], cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&b.done[i], cudaEventDisableTiming) == cudaSuccess;
+              (!b.used[BatchStreams::kSums] || cudaEventCreateWithFlags(&b.gram_done, cudaEventDisableTiming) == cudaSuccess);
+    for (int i = 1; ok && i < BatchStreams::kCount; ++i)          // (a stream costs some 30 us to make)
+        ok = !b.used[i] || (cudaStreamCreateWithFlags(&b.side[i], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&b.done[i], cudaEventDisableTiming) == cudaSuccess);
     if (!ok) { (void)cudaGetLastError(); return false; }
     b.device = dev;
     return true;
@@ -240,14 +240,16 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
         for (int i = 1; i < BatchStreams::kCount; ++i)
             if (b->used[i]) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->fork, 0));
     }
-    // What is not a tensor-core launch of several layers.  Image stems first: their blocks hold an SM for long, and behind the
-    // tensor-core launch they would be the tail of the chunk (a 64 x 64 stem of 37 examples: 130 us instead of 68 for the
-    // chunk); the rest is small and fills gaps, so it is enqueued last, before the streams meet again.
-    auto singles = [&](bool stems) -> dp_status {
+    // What is not a tensor-core launch of several layers.  Image stems of few examples first: their blocks hold an SM for long,
+    // and behind the tensor-core launch they would be the tail of the chunk (a 38 x 38 stem of 37 examples: 130 us instead
+    // of 68 for the chunk).  The rest fills gaps, so it is enqueued last, before the streams meet again; so are stems of
+    // more examples than SMs, whose second round of blocks would leave SMs idle (256 of 32 x 32: 135 us first, 117 last).
+    auto ahead = [](const dp_batch::Item &it) { return it.plan.use_thin && it.desc.B <= sm_count(); };
+    auto singles = [&](bool first) -> dp_status {
         dp_status rc = DP_OK;
         for (int i = 0; i < n && rc == DP_OK; ++i) {
             const dp_batch::Item &it = b->items[i];
-            if (it.group >= 0 || it.plan.use_thin != stems) continue;
+            if (it.group >= 0 || ahead(it) != first) continue;
             const LayerBuffers buf = {io[i].X, io[i].dY, io[i].G_w, io[i].G_b, io[i].sqnorm, io[i].sqnorm_stride, io[i].acc_w, io[i].acc_b, io[i].clip_out};
             rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kAffine]);
         }
