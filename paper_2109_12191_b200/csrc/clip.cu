@@ -224,12 +224,34 @@ __global__ void clip_factor_kernel(const float *__restrict__ sq, int B, int L, i
     if (clip_out) clip_out[idx] = f;
 }
 
+// Few norms of few examples given: every block of stage 3 works the factors out itself instead of waiting for a launch that
+// does (a warp's worth of double divisions and roots, some half a microsecond, against two for a launch).
+constexpr int kInlineExamples = 32;
+struct InlineFactors {
+    const float *sq;                 // [B, L]; null: the factors are given
+    float C;
+    float *factor, *norms_out, *clip_out;
+};
+__device__ __forceinline__ void stage_factors(float *f_sh, const float *factor, int n0, int nb, int L, int stride, int off, const InlineFactors &in) {
+    const int t = threadIdx.x;
+    if (t >= nb) return;
+    if (!in.sq) { f_sh[t] = factor[(long long)(n0 + t) * stride + off]; return; }
+    double s = 0.0;
+    for (int l = 0; l < L; ++l) s += (double)in.sq[(n0 + t) * L + l];
+    const float f = clip_factor(s, in.C);
+    f_sh[t] = f;
+    if (blockIdx.x) return;
+    in.factor[n0 + t] = f;
+    if (in.norms_out) in.norms_out[n0 + t] = (float)sqrt(s);
+    if (in.clip_out) in.clip_out[n0 + t] = f;
+}
+
 // stage 3: acc[i] += sum_n factor * G[n, i].  factor index: GLOBAL n, PER_LAYER n*L + col.  Streams B*P floats once; loads
 // past the L1 (evict-first: nothing comes back).
 template <int N>
 __global__ void __launch_bounds__(256)
 scale_accumulate_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
-                        int per_layer) {
+                        int per_layer, const __grid_constant__ InlineFactors in) {
     constexpr int kRows = 8;                                   // rows in flight per thread
     __shared__ float f_sh[256];
     const int seg = find_seg(tab, blockIdx.x);
@@ -249,7 +271,7 @@ scale_accumulate_kernel(const __grid_constant__ SegTable<N> tab, const float *__
         for (int n0 = 0; n0 < B; n0 += 256) {
             const int nb = min(256, B - n0);
             __syncthreads();
-            if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
+            stage_factors(f_sh, factor, n0, nb, L, f_stride, f_off, in);
             __syncthreads();
             if (live) {
                 const float *g = G + (long long)n0 * P + i;
@@ -281,7 +303,7 @@ scale_accumulate_kernel(const __grid_constant__ SegTable<N> tab, const float *__
         for (int n0 = 0; n0 < B; n0 += 256) {
             const int nb = min(256, B - n0);
             __syncthreads();
-            if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
+            stage_factors(f_sh, factor, n0, nb, L, f_stride, f_off, in);
             __syncthreads();
             const float *g = G + (long long)n0 * P + c0 + threadIdx.x;
             for (int n = 0; n < nb; n += kRows) {
@@ -317,7 +339,7 @@ constexpr int kSplitCols = 128;
 template <int N>
 __global__ void __launch_bounds__(256)
 scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
-                                 int per_layer) {
+                                 int per_layer, const __grid_constant__ InlineFactors in) {
     constexpr int kRows = 8;
     __shared__ float f_sh[256];
     __shared__ float part[8][kSplitCols];
@@ -336,7 +358,7 @@ scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable<N> tab, const 
     for (int n0 = (B - 1) & ~255; n0 >= 0; n0 -= 256) {
         const int nb = min(256, B - n0);
         __syncthreads();
-        if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
+        stage_factors(f_sh, factor, n0, nb, L, f_stride, f_off, in);
         __syncthreads();
         if (left <= 0) continue;
         const float *g = G + (long long)n0 * P + c0 + (vec ? 4 * lane : lane);
@@ -548,7 +570,10 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
         }
         return blk;
     };
-    if (!var.given_factor && c.sq) {
+    InlineFactors in = {};
+    if (!var.given_factor && c.sq && !var.noise && !var.groups && !c.per_layer && B <= kInlineExamples && L <= kFewTensors) {
+        in = InlineFactors{c.sq, c.C, c.factor_ws, c.norms_out, c.clip_out};
+    } else if (!var.given_factor && c.sq) {
         const dp_status rc = launch_factors(c, var, stream);
         if (rc != DP_OK) return rc;
     } else if (!var.given_factor) {
@@ -577,8 +602,8 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
         const int blocks = fill(l0, false, cursor);
         if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
         if (var.noise) scale_accumulate_noised_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, *var.noise);
-        else if (split) scale_accumulate_rowsplit_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer);
-        else scale_accumulate_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer);
+        else if (split) scale_accumulate_rowsplit_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, in);
+        else scale_accumulate_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, in);
         DP_LAUNCH_CHECK("scale_accumulate_kernel");
     }
     return DP_OK;

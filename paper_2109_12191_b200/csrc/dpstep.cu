@@ -234,11 +234,10 @@ dp_status run_layer(const dp_layer_desc *d, int epi, const LayerBuffers &io, flo
     }
 
     if (d->kind == DP_LAYER_DENSE) {
-        if (epi == DP_EPI_STORE_NORM) {
-            rc = launch_dense_store(storage_type(d), X, dY, d->B, d->C_in, d->K_out, G_w, d->has_bias ? G_b : nullptr, st);
-            if (rc != DP_OK) return rc;
-        }
-        float *db_dst = !d->has_bias ? nullptr : (epi == DP_EPI_STORE_NORM ? G_b : (clip ? db_ws : nullptr));
+        if (epi == DP_EPI_STORE_NORM)
+            return launch_dense_store(storage_type(d), X, dY, d->B, d->C_in, d->K_out, d->has_bias, d->has_bias ? G_b : nullptr, groups == 2,
+                                      sqnorm, sqnorm_stride, G_w, st);
+        float *db_dst = d->has_bias && clip ? db_ws : nullptr;
         rc = launch_dense_norm(storage_type(d), X, dY, d->B, d->C_in, d->K_out, d->has_bias, db_dst, groups == 2, sqnorm,
                                sqnorm_stride, clip, C_l, factor, clip_out, st);
         if (rc != DP_OK || !clip) return rc;

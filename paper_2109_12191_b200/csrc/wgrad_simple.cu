@@ -4,6 +4,7 @@
 // Formulas: paper section 2 (per-example gradient, its L2 norm, clip) and section 3.5 (per-layer threshold).
 #include "wgrad_simple.cuh"
 #include <math.h>
+#include <algorithm>
 #include <mutex>
 
 namespace dp {
@@ -811,41 +812,14 @@ __global__ void expand_factor_kernel(const float *__restrict__ factor_w, const f
 }
 
 // ------------------------------------------------------------------ dense layer
-// G_w[n, o, i] = dY[n, o] * X[n, i]: pure store stream.  One block per (example, output) row of the result,
-// four columns per thread when Cin % 4 == 0.
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(256)
-dense_store_kernel(const T *__restrict__ X, const T *__restrict__ dY, int Cin, int Kout, int rows_per_block,
-                   long long total_rows, float *__restrict__ G_w) {
-    for (int rr = 0; rr < rows_per_block; ++rr) {
-        const long long row = (long long)blockIdx.x * rows_per_block + rr;      // n * Kout + o
-        if (row >= total_rows) return;
-        const long long n = row / Kout;
-        const float gy = to_float(dY[row]);
-        const T *x = X + n * Cin;
-        float *out = G_w + row * Cin;
-        if (VEC) {
-            for (int i = threadIdx.x * 4; i < Cin; i += 1024) {
-                const float4 v = make_float4(gy * to_float(x[i]), gy * to_float(x[i + 1]), gy * to_float(x[i + 2]), gy * to_float(x[i + 3]));
-                __stcs(reinterpret_cast<float4 *>(out + i), v);
-            }
-        } else {
-            for (int i = threadIdx.x; i < Cin; i += 256) out[i] = gy * to_float(x[i]);
-        }
-    }
-}
-
-
-// Dense layer, everything but the outer-product store, one block per example: the rank-1 closed form of the squared
+// Dense layer, everything but the outer-product store, a block for an example: the rank-1 closed form of the squared
 // norm (|dY_n^T X_n|_F^2 = |dY_n|^2 |X_n|^2, bias part |dY_n|^2), the bias gradient db_n = dY_n widened to fp32 (when
 // a destination is given), and the same publishing of norms / clip factors the convolution paths do in a kernel of its own.
 template <typename T>
-__global__ void __launch_bounds__(256)
-dense_norm_kernel(const T *__restrict__ X, const T *__restrict__ dY, int Cin, int Kout, int has_bias, float *__restrict__ db,
-                  int separate, float *__restrict__ sqnorm, long long sq_stride, int clip, float C_l,
-                  float *__restrict__ factor, float *clip_out) {
+__device__ __forceinline__ void dense_norm(int n, const T *__restrict__ X, const T *__restrict__ dY, int Cin, int Kout, int has_bias,
+                                           float *__restrict__ db, int separate, float *__restrict__ sqnorm, long long sq_stride,
+                                           int clip, float C_l, float *__restrict__ factor, float *clip_out) {
     __shared__ double scratch[32];
-    const int n = blockIdx.x;
     double sx = 0.0, sy = 0.0;
     for (int i = threadIdx.x; i < Cin; i += 256) { const double v = to_float(X[(long long)n * Cin + i]); sx += v * v; }
     for (int i = threadIdx.x; i < Kout; i += 256) {
@@ -872,6 +846,44 @@ dense_norm_kernel(const T *__restrict__ X, const T *__restrict__ dY, int Cin, in
             factor[2 * n] = f; factor[2 * n + 1] = f;
             if (clip_out) clip_out[n] = f;
         }
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+dense_norm_kernel(const T *__restrict__ X, const T *__restrict__ dY, int Cin, int Kout, int has_bias, float *__restrict__ db,
+                  int separate, float *__restrict__ sqnorm, long long sq_stride, int clip, float C_l,
+                  float *__restrict__ factor, float *clip_out) {
+    dense_norm(blockIdx.x, X, dY, Cin, Kout, has_bias, db, separate, sqnorm, sq_stride, clip, C_l, factor, clip_out);
+}
+
+// Dense layer with its gradients stored, G_w[n, o, :] = dY[n, o] * X[n, :]: the first B blocks are the norms, the others the
+// outer product.  Bound by the stores.  A thread keeps VEC columns of X and walks down the outputs, so what a block reads
+// is small beside what it writes (a block an output, which reads X again for each, wrote 2048 x 1000 for 16 examples at
+// 4.2 TB/s; and small layers are bound by their launches, of which there were two).
+template <typename T, int VEC>
+__global__ void __launch_bounds__(256)
+dense_store_norm_kernel(const T *__restrict__ X, const T *__restrict__ dY, int B, int Cin, int Kout, int tpc, int outs, int col_blocks,
+                        int out_blocks, int has_bias, float *__restrict__ db, int separate, float *__restrict__ sqnorm,
+                        long long sq_stride, float *__restrict__ G_w) {
+    if ((int)blockIdx.x < B) {
+        dense_norm(blockIdx.x, X, dY, Cin, Kout, has_bias, db, separate, sqnorm, sq_stride, 0, 0.f, (float *)nullptr, (float *)nullptr);
+        return;
+    }
+    const int blk = (int)blockIdx.x - B, cb = blk % col_blocks, rest = blk / col_blocks, ob = rest % out_blocks, n = rest / out_blocks;
+    const int teams = 256 / tpc, team = threadIdx.x / tpc, col = (cb * tpc + threadIdx.x - team * tpc) * VEC;
+    if (team >= teams || col >= Cin) return;
+    const T *x = X + (long long)n * Cin + col, *gy = dY + (long long)n * Kout;
+    float xv[VEC];
+#pragma unroll
+    for (int v = 0; v < VEC; ++v) xv[v] = to_float(x[v]);
+    const int o1 = min(Kout, (ob + 1) * outs);
+    float *out = G_w + (long long)n * Kout * Cin + col;
+#pragma unroll 4
+    for (int o = ob * outs + team; o < o1; o += teams) {
+        const float g = to_float(gy[o]);
+        if constexpr (VEC == 4) __stcs(reinterpret_cast<float4 *>(out + (long long)o * Cin), make_float4(g * xv[0], g * xv[1], g * xv[2], g * xv[3]));
+        else out[(long long)o * Cin] = g * xv[0];
     }
 }
 
@@ -1257,25 +1269,31 @@ dp_status launch_expand_factor(const float *factor_w, const float *factor_b, lon
     return DP_OK;
 }
 
-template <typename T>
-static dp_status dense_store_t(const T *X, const T *dY, int B, int Cin, int Kout, float *G_w, float *G_b, cudaStream_t st) {
-    const bool vec = (Cin & 3) == 0;
-    const long long rows = (long long)B * Kout;
-    // short rows share a block so that every block still moves a few KB
-    const int per_block = Cin >= 1024 ? 1 : (1024 + Cin - 1) / Cin;
-    const long long blocks = (rows + per_block - 1) / per_block;
+template <typename T, int VEC>
+static dp_status dense_store_t(const T *X, const T *dY, int B, int Cin, int Kout, int has_bias, float *db, int separate, float *sqnorm,
+                               long long sq_stride, float *G_w, cudaStream_t st) {
+    const int tpc = std::min(256, (Cin + VEC - 1) / VEC), col_blocks = (Cin + tpc * VEC - 1) / (tpc * VEC), teams = 256 / tpc;
+    // outputs a thread walks through: at most sixteen, fewer while that leaves less than eight blocks an SM
+    const long long units = (long long)B * col_blocks * ((Kout + teams - 1) / teams);
+    const int per = (int)std::max(1ll, std::min(16ll, units / (8ll * sm_count())));
+    const int outs = per * teams, out_blocks = (Kout + outs - 1) / outs;
+    const long long blocks = B + (long long)B * col_blocks * out_blocks;
     if (blocks > 0x7fffffffLL) return DP_ERR_UNSUPPORTED;
-    if (vec) dense_store_kernel<T, true><<<(unsigned)blocks, 256, 0, st>>>(X, dY, Cin, Kout, per_block, rows, G_w);
-    else dense_store_kernel<T, false><<<(unsigned)blocks, 256, 0, st>>>(X, dY, Cin, Kout, per_block, rows, G_w);
-    DP_LAUNCH_CHECK("dense_store_kernel");
-    (void)G_b;      // the bias gradient is written by the norm kernel that every dense call runs
+    dense_store_norm_kernel<T, VEC><<<(unsigned)blocks, 256, 0, st>>>(X, dY, B, Cin, Kout, tpc, outs, col_blocks, out_blocks, has_bias, db, separate, sqnorm, sq_stride, G_w);
+    DP_LAUNCH_CHECK("dense_store_norm_kernel");
     return DP_OK;
 }
 
-dp_status launch_dense_store(int dtype, const void *X, const void *dY, int B, int Cin, int Kout, float *G_w, float *G_b,
-                             cudaStream_t st) {
-    if (dtype == DP_F32) return dense_store_t(static_cast<const float *>(X), static_cast<const float *>(dY), B, Cin, Kout, G_w, G_b, st);
-    return dense_store_t(static_cast<const __nv_bfloat16 *>(X), static_cast<const __nv_bfloat16 *>(dY), B, Cin, Kout, G_w, G_b, st);
+dp_status launch_dense_store(int dtype, const void *X, const void *dY, int B, int Cin, int Kout, int has_bias, float *db, int separate,
+                             float *sqnorm, long long sq_stride, float *G_w, cudaStream_t st) {
+    if (dtype == DP_F32) {
+        const float *x = static_cast<const float *>(X), *y = static_cast<const float *>(dY);
+        return Cin % 4 == 0 ? dense_store_t<float, 4>(x, y, B, Cin, Kout, has_bias, db, separate, sqnorm, sq_stride, G_w, st)
+                            : dense_store_t<float, 1>(x, y, B, Cin, Kout, has_bias, db, separate, sqnorm, sq_stride, G_w, st);
+    }
+    const __nv_bfloat16 *x = static_cast<const __nv_bfloat16 *>(X), *y = static_cast<const __nv_bfloat16 *>(dY);
+    return Cin % 4 == 0 ? dense_store_t<__nv_bfloat16, 4>(x, y, B, Cin, Kout, has_bias, db, separate, sqnorm, sq_stride, G_w, st)
+                        : dense_store_t<__nv_bfloat16, 1>(x, y, B, Cin, Kout, has_bias, db, separate, sqnorm, sq_stride, G_w, st);
 }
 
 dp_status launch_dense_norm(int dtype, const void *X, const void *dY, int B, int Cin, int Kout, int has_bias, float *db,

@@ -57,8 +57,8 @@ dp_status launch_dense_scaled_sum(int dtype, const void *X, const void *dY, cons
 dp_status launch_expand_factor(const float *factor_w, const float *factor_b, long long stride, int B, float *factor2,
                                cudaStream_t stream);
 
-dp_status launch_dense_store(int dtype, const void *X, const void *dY, int B, int Cin, int Kout, float *G_w,
-                             float *G_b, cudaStream_t stream);
+dp_status launch_dense_store(int dtype, const void *X, const void *dY, int B, int Cin, int Kout, int has_bias, float *db, int separate,
+                             float *sqnorm, long long sq_stride, float *G_w, cudaStream_t st);
 // closed-form squared norms (|dY_n|^2 |X_n|^2 and |dY_n|^2), db = dY as fp32 (optional), norms and clip factors published
 dp_status launch_dense_norm(int dtype, const void *X, const void *dY, int B, int Cin, int Kout, int has_bias, float *db,
                             int separate, float *sqnorm, long long sq_stride, int clip, float C_l, float *factor,

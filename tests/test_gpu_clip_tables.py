@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
     ([129, 3, 4100], 17),                 # one column past a narrow block; aligned and unaligned tensors in one launch
     ([127], 300),                         # more rows than one round of factors
     ([8192 * 2 + 1], 65),                 # one float past a chunk of the norms
+    ([40 + l for l in range(32)], 32), ([40 + l for l in range(32)], 33),   # the most whose factors stage 3 works out itself
     ([33 * (l + 1) for l in range(33)], 4),               # more norms than a thread walks alone
 ])
 def test_rows_of_any_length(sizes, Bn, give_norms):
