@@ -547,8 +547,12 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
             const int mt = it.mt, nt = it.nt;
             const int a_rows = min(128, p.a_ext - mt * 128);
             const int n_cols = min(p.NT, p.b_ext - nt * p.NT);
-            const int a_idx = mt * 128 + row;            // index along the A operand's extent
-            const bool row_ok = row < a_rows && (!p.a_is_x || a_idx < p.Ng);
+            int a_idx = mt * 128 + row;                  // index along the A operand's extent
+            bool row_ok = row < a_rows && (!p.a_is_x || a_idx < p.Ng);
+            if (!TF32 && p.s2d_st) {                     // (rows are input columns in this form)
+                a_idx = row < a_rows ? s2d_column(p, a_idx) : -1;
+                row_ok = a_idx >= 0;
+            }
             float run[CLIP ? 128 : 1];                   // clip mode: this thread's row of sum_n f_n D_n (NT <= 128)
             if (CLIP) {
 #pragma unroll
@@ -1808,9 +1812,10 @@ static TcPlan make_plan(int dtype, const ConvGeom &g, int mode) {
 // clusters share the batch, and what is minimised is SM time (clusters x CTAs x time), not the time of one launch
 static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
     const int max_nt = (mode == 2) ? 128 : 256;
-    const bool rows_are_inputs = mode == 6;              // mode 6: mode 3 with the rows of D fixed to the input columns
+    const bool rows_are_inputs = mode == 6 || mode >= 8; // modes 6, 8, 9: modes 3, 0, 1 with the rows of D fixed to the input columns
     const bool any_tiles = mode == 7;                    // mode 7: mode 3 without clusters (factors known): any number of tiles
     if (mode == 6 || mode == 7) mode = 3;
+    if (mode >= 8) mode -= 8;
     TcPlan best; best.ok = false;
     const int slab_ch = (dtype == DP_BF16) ? 64 : 32;
     const int krows = (dtype == DP_BF16) ? 16 : 8;
@@ -1969,6 +1974,22 @@ static bool clip1_plan(int dtype, const ConvGeom &g0, const TcProblem &pr, TcPla
     return pl.ok;
 }
 
+// What the store and norm kernels are given: thin strided layers in space-to-depth form as well, where nothing reads an
+// unfolded copy later on (32 examples of a 7 x 7 stem on 224 x 224: 69 us for the 154 MB copy, 11 for the regrouping).
+struct StoreForm { TcPlan pl; ConvGeom g; bool s2d; };
+static StoreForm store_form(int dtype, const ConvGeom &g0, const TcProblem &pr, int epilogue, bool regroup = true) {
+    StoreForm f = {};
+    const int mode = epilogue == DP_EPI_STORE_NORM ? 0 : 1;
+    const S2dProblem sp = regroup && epilogue != DP_EPI_CLIP_ACCUM ? s2d_problem(dtype, g0, pr) : S2dProblem{};
+    if (sp.ok) {
+        f.pl = make_plan(dtype, sp.eff, mode + 8);
+        if (f.pl.ok) { f.g = sp.eff; f.s2d = true; return f; }
+    }
+    f.g = pr.eff;
+    f.pl = make_plan(dtype, pr.eff, mode);
+    return f;
+}
+
 // clipped-sum mode: how many example ranges each tile is cut into so that every SM has an item
 static void clip_split(const ConvGeom &g, const TcPlan &pl, int &splits, int &per_split) {
     const int tiles = pl.m_tiles * pl.n_tiles;
@@ -1982,7 +2003,7 @@ static void clip_split(const ConvGeom &g, const TcPlan &pl, int &splits, int &pe
 int tc_norm_slots(int dtype, const ConvGeom &g0, int epilogue) {
     const TcProblem pr = tc_problem(dtype, g0);
     if (!pr.ok) return 0;
-    const TcPlan pl = make_plan(dtype, pr.eff, epilogue == DP_EPI_STORE_NORM ? 0 : 1);
+    const TcPlan pl = store_form(dtype, g0, pr, epilogue).pl;
     return pl.ok ? pl.m_tiles * pl.n_tiles * 4 : 0;
 }
 
@@ -2048,7 +2069,7 @@ int tc_describe_plan(int dtype, const ConvGeom &g0, int epilogue, int *out, int 
         ConvGeom g; bool s2d;
         if (!clip1_plan(dtype, g0, pr, pl, g, s2d)) return 0;
     } else {
-        pl = make_plan(dtype, pr.eff, epilogue);
+        pl = epilogue < 2 ? store_form(dtype, g0, pr, epilogue).pl : make_plan(dtype, pr.eff, epilogue);
     }
     if (!pl.ok) return 0;
     const int v[12] = {pl.a_is_x, pl.a_ext, pl.b_ext, pl.m_tiles, pl.n_tiles, pl.NT, pl.OWt, pl.OHt, pl.Kt, pl.k_tiles,
@@ -2149,17 +2170,45 @@ static dp_status unfold_input(int dtype, const void *X, const ConvGeom &g0, cons
     return DP_OK;
 }
 
-// Parameters of the norm / store / two-pass clipped-sum kernel for one layer; X already unfolded where the layer needs it.
+// The input as a kernel reads it: X itself, or its space-to-depth / unfolded copy written to the scratch.
+static dp_status prepare_input(int dtype, const void *X, const ConvGeom &g0, const TcProblem &pr, bool s2d, void *tc_workspace,
+                               cudaStream_t stream) {
+    if (s2d) {
+        const S2dProblem sp = s2d_problem(dtype, g0, pr);
+        const long long total = (long long)g0.B * sp.Hs * sp.Ws;
+        space_to_depth_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(
+            static_cast<const __nv_bfloat16 *>(X), static_cast<__nv_bfloat16 *>(tc_workspace), g0, sp.Hs, sp.Ws, total);
+        DP_LAUNCH_CHECK("space_to_depth_kernel");
+        return DP_OK;
+    }
+    return pr.unfold ? unfold_input(dtype, X, g0, pr, tc_workspace, stream) : DP_OK;
+}
+
+// a space-to-depth copy as the kernels read it: one operand row per output pixel, 64 values from pixel ow on, pixels 16 apart
+static bool encode_s2d(CUtensorMap *map, void *base, const S2dProblem &sp, const TcPlan &pl) {
+    const ConvGeom &g = sp.eff;
+    const cuuint64_t dims[5] = {64, (cuuint64_t)g.OW, (cuuint64_t)sp.Hs, (cuuint64_t)g.B, 1};
+    const cuuint64_t strides[4] = {32, (cuuint64_t)sp.Ws * 32, (cuuint64_t)sp.Hs * sp.Ws * 32, (cuuint64_t)g.B * sp.Hs * sp.Ws * 32};
+    const cuuint32_t box[5] = {64, (cuuint32_t)pl.OWt, (cuuint32_t)pl.OHt, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    return encode_fn()(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                       CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+static void fill_s2d(TcParams &p, const ConvGeom &g0) { p.s2d_st = g0.stride; p.s2d_R = g0.R; p.s2d_S = g0.S; p.s2d_Cin = g0.Cin; }
+
+// Parameters of the norm / store / two-pass clipped-sum kernel for one layer; X already regrouped or unfolded where the layer
+// needs it.
 static dp_status fill_conv_tc(int dtype, int epilogue, const void *X, const void *dY, const ConvGeom &g0, const TcProblem &pr,
-                              const TcPlan &pl, float *G_w, float *partial, int slots, const float *factor, float *acc_w,
+                              const ConvGeom &g, const TcPlan &pl, bool s2d, float *G_w, float *partial, int slots, const float *factor, float *acc_w,
                               void *tc_workspace, int *status, const TcPublish *publish, ConvEntry &e) {
     const bool clip = epilogue == DP_EPI_CLIP_ACCUM;
-    const ConvGeom &g = pr.eff;
-    if (!encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
+    if (s2d ? !encode_s2d(&e.map[0], const_cast<void *>(X), s2d_problem(dtype, g0, pr), pl)
+            : !encode_nhwc(&e.map[0], dtype, X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
     if (!encode_nhwc(&e.map[1], dtype, dY, g.Kout, g.OW, g.OH, g.B, pl.OWt, pl.OHt, 1, 1, y_group(dtype, g, pl))) return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(dY)");
     TcParams &p = e.p;
     p = TcParams{};
     fill_common(p, dtype, g, g0.N, pl, status);
+    if (s2d) fill_s2d(p, g0);
     p.lo_offset = pl.stage_bytes / 2;
     p.mode = clip ? 2 : (epilogue == DP_EPI_STORE_NORM ? 0 : 1);
     p.G_w = G_w; p.partial = partial; p.slots = slots;
@@ -2185,19 +2234,21 @@ dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY,
     const bool clip = epilogue == DP_EPI_CLIP_ACCUM;
     const TcProblem pr = tc_problem(dtype, g0);
     if (!pr.ok || !encode_fn()) return DP_ERR_UNSUPPORTED;
-    const TcPlan pl = make_plan(dtype, pr.eff, clip ? 2 : (epilogue == DP_EPI_STORE_NORM ? 0 : 1));
+    // (the norm pass of a fused clip call leaves its unfolded copy to the second pass, and a single partial sum a tile)
+    const StoreForm form = clip ? StoreForm{make_plan(dtype, pr.eff, 2), pr.eff, false} : store_form(dtype, g0, pr, epilogue, !(publish && publish->factor_out));
+    const TcPlan &pl = form.pl;
     if (!pl.ok) return DP_ERR_UNSUPPORTED;
     dp_status rc = raise_shared_limits();
     if (rc != DP_OK) return rc;
     if (pr.unfold) {
         // in a fused clip call this function runs twice (norm pass, then clipped-sum pass): the unfolded input is
         // rebuilt only by the first of them
-        if (!(clip && second_pass) && (rc = unfold_input(dtype, X, g0, pr, tc_workspace, stream)) != DP_OK) return rc;
+        if (!(clip && second_pass) && (rc = prepare_input(dtype, X, g0, pr, form.s2d, tc_workspace, stream)) != DP_OK) return rc;
         X = tc_workspace;
     }
     TcTable<TcParams, 2, 1> tab;
     tab.n = 1; tab.first[0] = 0;
-    rc = fill_conv_tc(dtype, epilogue, X, dY, g0, pr, pl, G_w, partial, slots, factor, acc_w, tc_workspace, status, publish, tab.e[0]);
+    rc = fill_conv_tc(dtype, epilogue, X, dY, g0, pr, form.g, pl, form.s2d, G_w, partial, slots, factor, acc_w, tc_workspace, status, publish, tab.e[0]);
     if (rc != DP_OK) return rc;
     TcParams &p = tab.e[0].p;
     p.blocks = std::min(p.total_tiles, sm_target());
@@ -2399,33 +2450,12 @@ bool tc_clip_single_pass(int dtype, const ConvGeom &g0) {
     return pr.ok && encode_fn() && clip1_plan(dtype, g0, pr, pl, g, s2d) && clip1_registers_ok();
 }
 
-// The input as the single-pass kernel reads it: X itself, or its space-to-depth / unfolded copy written to the scratch.
-static dp_status prepare_clip1(int dtype, const void *X, const ConvGeom &g0, const TcProblem &pr, bool s2d, void *tc_workspace,
-                               cudaStream_t stream) {
-    if (s2d) {
-        const S2dProblem sp = s2d_problem(dtype, g0, pr);
-        const long long total = (long long)g0.B * sp.Hs * sp.Ws;
-        space_to_depth_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(
-            static_cast<const __nv_bfloat16 *>(X), static_cast<__nv_bfloat16 *>(tc_workspace), g0, sp.Hs, sp.Ws, total);
-        DP_LAUNCH_CHECK("space_to_depth_kernel");
-        return DP_OK;
-    }
-    return pr.unfold ? unfold_input(dtype, X, g0, pr, tc_workspace, stream) : DP_OK;
-}
-
 static dp_status fill_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g0, const TcProblem &pr, const ConvGeom &g,
                             const TcPlan &pl, bool s2d, const TcInlineClip &clipinfo, float *acc_w, void *tc_workspace, int *status,
                             ConvEntry &e) {
     char *ws_bytes = static_cast<char *>(tc_workspace);
     if (s2d) {
-        const S2dProblem sp = s2d_problem(dtype, g0, pr);
-        // one operand row per output pixel: 64 values from pixel ow on, pixels 16 values apart
-        const cuuint64_t dims[5] = {64, (cuuint64_t)g.OW, (cuuint64_t)sp.Hs, (cuuint64_t)g.B, 1};
-        const cuuint64_t strides[4] = {32, (cuuint64_t)sp.Ws * 32, (cuuint64_t)sp.Hs * sp.Ws * 32, (cuuint64_t)g.B * sp.Hs * sp.Ws * 32};
-        const cuuint32_t box[5] = {64, (cuuint32_t)pl.OWt, (cuuint32_t)pl.OHt, 1, 1};
-        const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-        if (encode_fn()(&e.map[0], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, ws_bytes, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                        CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        if (!encode_s2d(&e.map[0], ws_bytes, s2d_problem(dtype, g0, pr), pl))
             return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(space-to-depth X)");
     } else if (!encode_nhwc(&e.map[0], dtype, pr.unfold ? tc_workspace : X, g.Cin, g.W, g.H, g.B, pl.OWt, pl.OHt, g.stride, 1, x_group(dtype, g, pl))) {
         return cuda_fail(cudaErrorInvalidValue, "cuTensorMapEncodeTiled(X)");
@@ -2435,7 +2465,7 @@ static dp_status fill_clip1(int dtype, const void *X, const void *dY, const Conv
     p = TcParams{};
     fill_common(p, dtype, g, g0.N, pl, status);
     p.mode = 3;
-    if (s2d) { p.s2d_st = g0.stride; p.s2d_R = g0.R; p.s2d_S = g0.S; p.s2d_Cin = g0.Cin; }
+    if (s2d) fill_s2d(p, g0);
     p.C_l = clipinfo.C_l; p.sqnorm = clipinfo.sqnorm; p.sq_stride = clipinfo.sq_stride; p.clip_out = clipinfo.clip_out;
     p.cluster = pl.m_tiles * pl.n_tiles;
     cluster_split(g.B, p.cluster, g.K, pl.NT, p.splits, p.per_split);
@@ -2464,7 +2494,7 @@ dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const Conv
     TcPlan pl; ConvGeom g; bool s2d;
     if (!pr.ok || !encode_fn() || !clip1_plan(dtype, g0, pr, pl, g, s2d) || !clip1_registers_ok()) return DP_ERR_UNSUPPORTED;
     dp_status rc = raise_shared_limits();
-    if (rc == DP_OK) rc = prepare_clip1(dtype, X, g0, pr, s2d, tc_workspace, stream);
+    if (rc == DP_OK) rc = prepare_input(dtype, X, g0, pr, s2d, tc_workspace, stream);
     if (rc != DP_OK) return rc;
     TcTable<TcParams, 2, 1> tab;
     tab.n = 1; tab.first[0] = 0;
@@ -2497,7 +2527,7 @@ double conv_batch_walk(const std::vector<ConvJob> &jobs) {
     for (const ConvJob &j : jobs) {
         const TcProblem pr = tc_problem(j.dtype, j.g);
         TcPlan pl; ConvGeom g = pr.eff; bool s2d;
-        if (j.kind == kConvTc) pl = make_plan(j.dtype, g, j.epi == DP_EPI_STORE_NORM ? 0 : 1);
+        if (j.kind == kConvTc) pl = store_form(j.dtype, j.g, pr, j.epi).pl;
         else if (j.kind == kConvClip1) clip1_plan(j.dtype, j.g, pr, pl, g, s2d);
         else if (j.kind == kConvGramTiles) pl = make_plan(j.dtype, g, 7);
         else continue;
@@ -2562,17 +2592,18 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
         const ConvGeom &g = pr.eff;
         const long long P = (long long)j.g.M * j.g.N;
         if (j.kind == kConvTc) {
-            const TcPlan pl = make_plan(j.dtype, g, j.epi == DP_EPI_STORE_NORM ? 0 : 1);
+            const StoreForm form = store_form(j.dtype, j.g, pr, j.epi);
+            const TcPlan &pl = form.pl;
             if (!pl.ok) return DP_ERR_UNSUPPORTED;
             const void *X = j.X;
             if (pr.unfold) {
-                rc = unfold_input(j.dtype, X, j.g, pr, j.tc_workspace, stream);
+                rc = prepare_input(j.dtype, X, j.g, pr, form.s2d, j.tc_workspace, stream);
                 if (rc != DP_OK) return rc;
                 X = j.tc_workspace;
             }
             const TcPublish pub = {j.counter, j.w_slots, j.separate, j.clip.sqnorm, j.clip.sq_stride, nullptr, 0.f, nullptr};
             ConvQueue::Job q;
-            rc = fill_conv_tc(j.dtype, j.epi, X, j.dY, j.g, pr, pl, j.G_w, j.partial, j.slots, nullptr, nullptr, j.tc_workspace, status, &pub, q.e);
+            rc = fill_conv_tc(j.dtype, j.epi, X, j.dY, j.g, pr, form.g, pl, form.s2d, j.G_w, j.partial, j.slots, nullptr, nullptr, j.tc_workspace, status, &pub, q.e);
             if (rc != DP_OK) return rc;
             TcParams &p = q.e.p;
             if (j.bias_apart) { p.separate = 0; p.fold_slots = j.w_slots; }
@@ -2583,7 +2614,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
         } else if (j.kind == kConvClip1) {
             TcPlan pl; ConvGeom g1; bool s2d;
             if (!clip1_plan(j.dtype, j.g, pr, pl, g1, s2d)) return DP_ERR_UNSUPPORTED;
-            rc = prepare_clip1(j.dtype, j.X, j.g, pr, s2d, j.tc_workspace, launch_cluster(pl.m_tiles * pl.n_tiles) > 4 ? clusters : stream);
+            rc = prepare_input(j.dtype, j.X, j.g, pr, s2d, j.tc_workspace, launch_cluster(pl.m_tiles * pl.n_tiles) > 4 ? clusters : stream);
             if (rc != DP_OK) return rc;
             ConvQueue::Job q;
             rc = fill_clip1(j.dtype, j.X, j.dY, j.g, pr, g1, pl, s2d, j.clip, j.acc_w, j.tc_workspace, status, q.e);
