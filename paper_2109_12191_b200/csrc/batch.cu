@@ -3,11 +3,78 @@
 #include "batch.cuh"
 #include "wgrad_tc.cuh"
 #include <algorithm>
+#include <cstddef>
+#include <exception>
 #include <mutex>
 #include <new>
 #include <vector>
 
 using namespace dp;
+
+namespace {
+// Streams and events the runs of a batch fork to.  Making a set costs some 100 us, more than the first run of a small model,
+// so a batch takes one that an earlier batch has given back: a set keeps its order of work, and a new batch's launches at
+// worst queue behind what the old one still has running.  At most kKeptSets wait for a taker.
+struct SideStreams {
+    int device;
+    cudaStream_t stream[BatchStreams::kCount];
+    cudaEvent_t fork, gram_done, done[BatchStreams::kCount];
+};
+constexpr size_t kKeptSets = 8;
+std::mutex kept_mu;
+std::vector<SideStreams *> &kept_sets() { static auto *sets = new std::vector<SideStreams *>; return *sets; }   // outlives every batch
+
+void drop_streams(SideStreams *t) {
+    for (int i = 1; i < BatchStreams::kCount; ++i) {
+        if (t->done[i]) cudaEventDestroy(t->done[i]);
+        if (t->stream[i]) cudaStreamDestroy(t->stream[i]);
+    }
+    if (t->fork) cudaEventDestroy(t->fork);
+    if (t->gram_done) cudaEventDestroy(t->gram_done);
+    delete t;
+}
+// a set on the current device, or null
+SideStreams *take_streams() {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
+    {
+        std::lock_guard<std::mutex> lock(kept_mu);
+        auto &sets = kept_sets();
+        for (size_t i = sets.size(); i-- > 0;) {
+            if (sets[i]->device != dev) continue;
+            SideStreams *t = sets[i];
+            sets.erase(sets.begin() + (std::ptrdiff_t)i);
+            return t;
+        }
+    }
+    SideStreams *t = new (std::nothrow) SideStreams{};
+    if (!t) return nullptr;
+    t->device = dev;
+    bool ok = cudaEventCreateWithFlags(&t->fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&t->gram_done, cudaEventDisableTiming) == cudaSuccess;
+    for (int i = 1; ok && i < BatchStreams::kCount; ++i)
+        ok = cudaStreamCreateWithFlags(&t->stream[i], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&t->done[i], cudaEventDisableTiming) == cudaSuccess;
+    if (ok) return t;
+    (void)cudaGetLastError();
+    drop_streams(t);
+    return nullptr;
+}
+void give_back(SideStreams *t) {
+    bool idle = true;                        // a stream some unfinished capture holds is of no use to others
+    for (int i = 1; i < BatchStreams::kCount; ++i) {
+        cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+        idle = idle && cudaStreamIsCapturing(t->stream[i], &c) == cudaSuccess && c == cudaStreamCaptureStatusNone;
+    }
+    if (idle) {
+        std::lock_guard<std::mutex> lock(kept_mu);
+        auto &sets = kept_sets();
+        if (sets.capacity() < kKeptSets) { try { sets.reserve(kKeptSets); } catch (const std::exception &) {} }
+        if (sets.size() < std::min(kKeptSets, sets.capacity())) { sets.push_back(t); return; }
+    }
+    drop_streams(t);
+}
+}  // namespace
 
 struct dp_batch {
     struct Item {
@@ -27,28 +94,19 @@ struct dp_batch {
     size_t singles = 0;                          // byte offset of the scratch the single calls share
     bool used[BatchStreams::kCount] = {};        // streams that have launches of their own
     size_t total = 0;
-    // Streams and events of the runs, made on the first run's device; host threads take turns at enqueueing.
+    // Taken by the first run, on its device; host threads take turns at enqueueing.
     mutable std::mutex mu;
-    mutable int device = -1;
-    mutable cudaStream_t side[BatchStreams::kCount] = {};
-    mutable cudaEvent_t fork = nullptr, gram_done = nullptr, done[BatchStreams::kCount] = {};
+    mutable SideStreams *side = nullptr;
 };
 
 namespace dp {
 
-// The side streams of a batch, or false where this device is not the one they were made on or they cannot be had.
+// Whether the batch has side streams, on this device.
 static bool side_streams(const dp_batch &b) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (b.device >= 0) return b.device == dev;
-    bool ok = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming) == cudaSuccess &&
-              (!b.used[BatchStreams::kSums] || cudaEventCreateWithFlags(&b.gram_done, cudaEventDisableTiming) == cudaSuccess);
-    for (int i = 1; ok && i < BatchStreams::kCount; ++i)          // (a stream costs some 30 us to make)
-        ok = !b.used[i] || (cudaStreamCreateWithFlags(&b.side[i], cudaStreamNonBlocking) == cudaSuccess &&
-             cudaEventCreateWithFlags(&b.done[i], cudaEventDisableTiming) == cudaSuccess);
-    if (!ok) { (void)cudaGetLastError(); return false; }
-    b.device = dev;
-    return true;
+    if (!b.side) b.side = take_streams();
+    return b.side && b.side->device == dev;
 }
 
 static void plan_affine(dp_batch &b, size_t &off) {
@@ -163,6 +221,34 @@ static dp_status run_convs(const dp_batch &b, const dp_layer_io *io, float C_l, 
     return launch_conv_batch(jobs, b.walk, reinterpret_cast<int *>(ws), streams, join);
 }
 
+static dp_status plan_batch(dp_batch &b, int n, const dp_layer_desc *descs, const int *epilogues) {
+    b.items.resize(n);
+    for (int i = 0; i < n; ++i) {
+        dp_batch::Item &it = b.items[i];
+        it.desc = descs[i]; it.epi = epilogues[i]; it.group = it.slot = -1; it.scratch = 0;
+        make_layer_plan(&it.desc, it.epi, it.plan);
+        if (it.desc.impl == DP_IMPL_TENSOR_CORE && !it.plan.use_tc) return DP_ERR_UNSUPPORTED;
+    }
+    size_t off = kWsHeaderBytes;
+    plan_convs(b, off);
+    plan_affine(b, off);
+    b.singles = off;
+    size_t most = 0;
+    for (const auto &it : b.items) {
+        if (it.group >= 0) continue;
+        most = std::max(most, it.plan.total);
+        b.used[BatchStreams::kAffine] = true;
+    }
+    if (!b.affine.empty()) b.used[BatchStreams::kAffine] = true;
+    for (const ConvJob &j : b.convs) {
+        b.used[BatchStreams::kMain] = true;
+        if (conv_batch_clusters(j, b.walk)) b.used[BatchStreams::kClusters] = true;
+        if (j.kind == kConvGramSum || b.items[b.conv_item[&j - b.convs.data()]].desc.has_bias) b.used[BatchStreams::kSums] = true;
+    }
+    b.total = most > kWsHeaderBytes ? round_up(off + most - kWsHeaderBytes, 256) : off;
+    return DP_OK;
+}
+
 }  // namespace dp
 
 extern "C" dp_status dp_batch_create(int n, const dp_layer_desc *descs, const int *epilogues, dp_batch **out) {
@@ -174,42 +260,20 @@ extern "C" dp_status dp_batch_create(int n, const dp_layer_desc *descs, const in
     }
     dp_batch *b = new (std::nothrow) dp_batch;
     if (!b) return DP_ERR_CUDA;
-    b->items.resize(n);
-    for (int i = 0; i < n; ++i) {
-        dp_batch::Item &it = b->items[i];
-        it.desc = descs[i]; it.epi = epilogues[i]; it.group = it.slot = -1; it.scratch = 0;
-        make_layer_plan(&it.desc, it.epi, it.plan);
-        if (it.desc.impl == DP_IMPL_TENSOR_CORE && !it.plan.use_tc) { delete b; return DP_ERR_UNSUPPORTED; }
+    try {
+        const dp_status rc = plan_batch(*b, n, descs, epilogues);
+        if (rc != DP_OK) { delete b; return rc; }
+    } catch (const std::exception &) {           // out of memory
+        delete b;
+        return DP_ERR_CUDA;
     }
-    size_t off = kWsHeaderBytes;
-    plan_convs(*b, off);
-    plan_affine(*b, off);
-    b->singles = off;
-    size_t most = 0;
-    for (const auto &it : b->items) {
-        if (it.group >= 0) continue;
-        most = std::max(most, it.plan.total);
-        b->used[BatchStreams::kAffine] = true;
-    }
-    if (!b->affine.empty()) b->used[BatchStreams::kAffine] = true;
-    for (const ConvJob &j : b->convs) {
-        b->used[BatchStreams::kMain] = true;
-        if (conv_batch_clusters(j, b->walk)) b->used[BatchStreams::kClusters] = true;
-        if (j.kind == kConvGramSum || b->items[b->conv_item[&j - b->convs.data()]].desc.has_bias) b->used[BatchStreams::kSums] = true;
-    }
-    b->total = most > kWsHeaderBytes ? round_up(off + most - kWsHeaderBytes, 256) : off;
     *out = b;
     return DP_OK;
 }
 
 extern "C" void dp_batch_destroy(dp_batch *b) {
     if (!b) return;
-    for (int i = 0; i < BatchStreams::kCount; ++i) {
-        if (b->done[i]) cudaEventDestroy(b->done[i]);
-        if (b->side[i]) cudaStreamDestroy(b->side[i]);
-    }
-    if (b->fork) cudaEventDestroy(b->fork);
-    if (b->gram_done) cudaEventDestroy(b->gram_done);
+    if (b->side) give_back(b->side);
     delete b;
 }
 
@@ -233,12 +297,12 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
     BatchStreams streams;
     // (without convolutions there is nothing to fork from: everything stays on the caller's stream)
     const bool forked = b->used[BatchStreams::kMain] && (b->used[1] || b->used[2] || b->used[3]) && side_streams(*b);
-    for (int i = 0; i < BatchStreams::kCount; ++i) streams.s[i] = forked && i && b->used[i] ? b->side[i] : st;
-    streams.gram_done = forked && b->used[BatchStreams::kSums] ? b->gram_done : nullptr;
+    for (int i = 0; i < BatchStreams::kCount; ++i) streams.s[i] = forked && i && b->used[i] ? b->side->stream[i] : st;
+    streams.gram_done = forked && b->used[BatchStreams::kSums] ? b->side->gram_done : nullptr;
     if (forked) {
-        DP_CUDA_TRY(cudaEventRecord(b->fork, st));
+        DP_CUDA_TRY(cudaEventRecord(b->side->fork, st));
         for (int i = 1; i < BatchStreams::kCount; ++i)
-            if (b->used[i]) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->fork, 0));
+            if (b->used[i]) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b->side->fork, 0));
     }
     // What is not a tensor-core launch of several layers.  Image stems of few examples first: their blocks hold an SM for long,
     // and behind the tensor-core launch they would be the tail of the chunk (a 38 x 38 stem of 37 examples: 130 us instead
@@ -259,18 +323,28 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
     auto join = [&]() -> dp_status {
         if (joined) return DP_OK;
         joined = true;
-        dp_status rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
-        if (rc == DP_OK) rc = singles(false);
+        dp_status rc;
+        try {
+            rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
+            if (rc == DP_OK) rc = singles(false);
+        } catch (const std::exception &) {       // out of memory: the streams still have to meet
+            rc = DP_ERR_CUDA;
+        }
         if (!forked) return rc;
         for (int i = 1; i < BatchStreams::kCount; ++i) {
             if (!b->used[i]) continue;
-            DP_CUDA_TRY(cudaEventRecord(b->done[i], streams.s[i]));
-            DP_CUDA_TRY(cudaStreamWaitEvent(st, b->done[i], 0));
+            DP_CUDA_TRY(cudaEventRecord(b->side->done[i], streams.s[i]));
+            DP_CUDA_TRY(cudaStreamWaitEvent(st, b->side->done[i], 0));
         }
         return rc;
     };
-    dp_status rc = singles(true);
-    if (rc == DP_OK) rc = run_convs(*b, io, C_l, ws, streams, join);
+    dp_status rc;
+    try {
+        rc = singles(true);
+        if (rc == DP_OK) rc = run_convs(*b, io, C_l, ws, streams, join);
+    } catch (const std::exception &) {           // out of memory
+        rc = DP_ERR_CUDA;
+    }
     if (rc != DP_OK) (void)join();       // a launch failed: whatever is enqueued still comes before what follows
     return rc;
 }
