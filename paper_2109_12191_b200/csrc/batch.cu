@@ -325,8 +325,9 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
         joined = true;
         dp_status rc;
         try {
-            rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
-            if (rc == DP_OK) rc = singles(false);
+            // (singles first: they are short, and behind the normalisation layers they would be the chunk's tail)
+            rc = singles(false);
+            if (rc == DP_OK) rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
         } catch (const std::exception &) {       // out of memory: the streams still have to meet
             rc = DP_ERR_CUDA;
         }
