@@ -128,7 +128,7 @@ sqnorm_partial_micro_kernel(const __grid_constant__ SegTable<N> tab, float *__re
 // shared memory (161 tensors of 16 examples in four groups: 30 us with eight warps and the table read from the parameters).
 enum { kGlobal = 0, kPerLayer, kGrouped };
 constexpr int kFactorThreads = 1024;
-constexpr int kPartsPerWarp = 256;                   // tensors with more partials are folded by the whole block
+constexpr int kPartsPerWarp = 512;                   // tensors with more partials are folded by the whole block
 constexpr int kMaxGroupedTensors = 1024;
 struct GroupTable {
     int M;
@@ -140,6 +140,7 @@ norm_factor_kernel(const __grid_constant__ SegTable<N> tab, const float *__restr
                    const float *sq_in, float *sq_ws, int L, int micro, int last, float C, const __grid_constant__ GroupTable gt,
                    float *__restrict__ factor, float *norms_out, float *clip_out) {
     __shared__ double scratch[32];
+    __shared__ int large;                                // a tensor of this table is left to the whole block
     __shared__ float f_sh[KIND == kGrouped ? kMaxGroupedTensors : 1];
     __shared__ unsigned short of_sh[KIND == kGrouped ? kMaxGroupedTensors : 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -149,25 +150,28 @@ norm_factor_kernel(const __grid_constant__ SegTable<N> tab, const float *__restr
     }
     if (partial) {
         float *out = sq_ws + row * L + tab.col0;
+        if (threadIdx.x == 0) large = 0;
+        __syncthreads();
         for (int s = w; s < tab.nseg; s += kFactorThreads / 32) {
-            const long long nparts = (tab.P[s] + kNormChunk - 1) / kNormChunk;
-            if (nparts > kPartsPerWarp) continue;
+            const int nparts = (int)((tab.P[s] + kNormChunk - 1) / kNormChunk);
+            if (nparts > kPartsPerWarp) { large = 1; continue; }
             const float *p = partial + row * parts_per_row + tab.part_start[s];
-            double a = 0.0;
-#pragma unroll 4
-            for (int i = lane; i < (int)nparts; i += 32) a += (double)p[i];
+            Sum2 a;
+#pragma unroll 8
+            for (int i = lane; i < nparts; i += 32) a.add(p[i]);
             a = warp_sum(a);
-            if (lane == 0) out[s] = (float)a;
+            if (lane == 0) out[s] = (float)a.value();
         }
-        for (int s = 0; s < tab.nseg; ++s) {
-            const long long nparts = (tab.P[s] + kNormChunk - 1) / kNormChunk;
+        __syncthreads();
+        for (int s = 0; large && s < tab.nseg; ++s) {
+            const int nparts = (int)((tab.P[s] + kNormChunk - 1) / kNormChunk);
             if (nparts <= kPartsPerWarp) continue;
             const float *p = partial + row * parts_per_row + tab.part_start[s];
-            double a = 0.0;
+            Sum2 a;
 #pragma unroll 4
-            for (long long i = threadIdx.x; i < nparts; i += kFactorThreads) a += (double)p[i];
-            a = block_sum(a, scratch);
-            if (threadIdx.x == 0) out[s] = (float)a;
+            for (int i = threadIdx.x; i < nparts; i += kFactorThreads) a.add(p[i]);
+            const double t = block_sum(a.value(), scratch);
+            if (threadIdx.x == 0) out[s] = (float)t;
         }
         if (!last) return;
     }
@@ -195,10 +199,11 @@ norm_factor_kernel(const __grid_constant__ SegTable<N> tab, const float *__restr
     } else {
         const float thr = (float)((double)C / sqrt((double)gt.M));
         for (int m = w; m < gt.M; m += kFactorThreads / 32) {
-            double s = 0.0;
+            Sum2 sum;
             for (int l = lane; l < L; l += 32)
-                if (of_sh[l] == m) s += (double)sq[l];
-            s = warp_sum(s);
+                if (of_sh[l] == m) sum.add(sq[l]);
+            sum = warp_sum(sum);
+            const double s = sum.value();
             if (lane == 0) {
                 const float f = clip_factor(s, thr);
                 f_sh[m] = f;

@@ -63,6 +63,30 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// Knuth's error-free sum: returns a + b rounded and adds what the rounding lost to `err`.
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    err = __fadd_rn(err, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+    return s;
+}
+// A sum of floats with its rounding errors (some 46 bits): where the double pipe, a sixty-fourth of the float rate, would be
+// what a kernel waits for.
+struct Sum2 {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) { hi = two_sum(hi, v, lo); }
+    __device__ __forceinline__ void add(const Sum2 &o) { hi = two_sum(hi, o.hi, lo); lo += o.lo; }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+__device__ __forceinline__ Sum2 warp_sum(Sum2 v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        Sum2 w;
+        w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o); w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+        v.add(w);
+    }
+    return v;
+}
+
 // Block-wide sum for blockDim.x a multiple of 32 (<= 1024); every thread gets the result.
 // `scratch` holds at least 32 values.  Fixed order: lanes by butterfly, then warps by butterfly.
 template <typename T>

@@ -773,12 +773,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     return false;
 }
 
-// Knuth's error-free sum: returns a + b rounded and adds what the rounding lost to `err`.
-__device__ __forceinline__ float two_sum(float a, float b, float &err) {
-    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-    err = __fadd_rn(err, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
-    return s;
-}
 __device__ __forceinline__ float sum8(const float4 &x, const float4 &y) {
     float e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;
     const float a = two_sum(x.x, x.y, e0), b = two_sum(x.z, x.w, e1), c = two_sum(y.x, y.y, e2), d = two_sum(y.z, y.w, e3);

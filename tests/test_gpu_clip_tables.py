@@ -21,7 +21,7 @@ def test_rows_of_any_length(sizes, Bn, give_norms):
 
 
 def test_a_tensor_with_more_partials_than_a_warp_folds():
-    sizes = [8192 * 256 + 3, 8192 * 256, 5]
+    sizes = [8192 * 512 + 3, 8192 * 512, 5]
     groups = _spread(3, sizes, 3)
     _check("global", groups, 0.3)
     _check("per_layer", groups, 0.2)
