@@ -90,6 +90,7 @@ struct dp_batch {
     size_t affine_partial = 0;                   // byte offset of the pixel-chunk partials
     std::vector<ConvJob> convs;                  // geometry filled in, buffers per run
     std::vector<int> conv_item;                  // item of every conv
+    int target = 0;                              // SM target the single calls are planned for
     double walk = 0.0;                           // conv_batch_walk() of all of them
     size_t singles = 0;                          // byte offset of the scratch the single calls share
     bool used[BatchStreams::kCount] = {};        // streams that have launches of their own
@@ -171,7 +172,7 @@ static void plan_convs(dp_batch &b, size_t &off) {
     for (size_t i = 0; i < b.items.size(); ++i) {
         dp_batch::Item &it = b.items[i];
         const dp_layer_desc &d = it.desc;
-        if (d.kind != DP_LAYER_CONV2D || !it.plan.use_tc || (int)b.convs.size() >= kWsCounters) continue;
+        if (d.kind != DP_LAYER_CONV2D || !it.plan.use_tc || (int)b.convs.size() >= kWsBatchCounters) continue;
         ConvJob j = {};
         j.g = geom_of(&d); j.dtype = d.dtype; j.epi = it.epi;
         j.kind = conv_batch_kind(d.dtype, j.g, it.epi, d.has_bias != 0);
@@ -206,7 +207,7 @@ static dp_status run_convs(const dp_batch &b, const dp_layer_io *io, float C_l, 
         j.partial = reinterpret_cast<float *>(base + it.plan.partial_off);
         j.factor = reinterpret_cast<float *>(base + it.plan.factor_off);
         j.tc_workspace = base + it.plan.tc_off;
-        j.counter = reinterpret_cast<int *>(ws + kWsCounterOffset) + k;
+        j.counter = reinterpret_cast<int *>(ws + kWsCounterOffset) + (kWsCounters - kWsBatchCounters) + k;
         j.clip = TcInlineClip{C_l, o.sqnorm, o.sqnorm_stride, o.clip_out};
         if (it.desc.has_bias) {
             float *db = it.epi == DP_EPI_STORE_NORM ? o.G_b : reinterpret_cast<float *>(base + it.plan.db_off);
@@ -223,6 +224,7 @@ static dp_status run_convs(const dp_batch &b, const dp_layer_io *io, float C_l, 
 
 static dp_status plan_batch(dp_batch &b, int n, const dp_layer_desc *descs, const int *epilogues) {
     b.items.resize(n);
+    b.target = sm_target_set() ? sm_target() : 0;
     for (int i = 0; i < n; ++i) {
         dp_batch::Item &it = b.items[i];
         it.desc = descs[i]; it.epi = epilogues[i]; it.group = it.slot = -1; it.scratch = 0;
@@ -310,6 +312,9 @@ extern "C" dp_status dp_batch_run(const dp_batch *b, const dp_layer_io *io, floa
     // more examples than SMs, whose second round of blocks would leave SMs idle (256 of 32 x 32: 135 us first, 117 last).
     auto ahead = [](const dp_batch::Item &it) { return it.plan.use_thin && it.desc.B <= sm_count(); };
     auto singles = [&](bool first) -> dp_status {
+        // tiled as their plans were: not as layers of a grouped launch, and for the SM target of that time
+        BatchPlanning alone(0.0);
+        SmTargetScope target(b->target);
         dp_status rc = DP_OK;
         for (int i = 0; i < n && rc == DP_OK; ++i) {
             const dp_batch::Item &it = b->items[i];

@@ -17,6 +17,11 @@ void note_error(const char *message);
 int sm_count();
 // Number of SMs one tensor-core launch should spread over: dp_set_sm_target()'s value, or all of them.
 int sm_target();
+struct SmTargetScope {  // another target (0: none) for this thread while it lives
+    explicit SmTargetScope(int sms);
+    ~SmTargetScope();
+    int saved;
+};
 bool sm_target_set();   // true once dp_set_sm_target() was given a positive value: the caller runs calls side by side
 // false while dp_debug_set_single_pass(0) holds: the fused clipped sum then always runs its two-pass form
 bool single_pass_enabled();
@@ -27,6 +32,7 @@ bool single_pass_enabled();
 constexpr size_t kWsHeaderBytes = 16384;
 constexpr size_t kWsCounterOffset = 256;
 constexpr int kWsCounters = (int)((kWsHeaderBytes - kWsCounterOffset) / sizeof(int));
+constexpr int kWsBatchCounters = 512;    // the last of them belong to the grouped launches of a batch, which run beside single calls
 
 inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) % a) == 0; }
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -75,6 +81,7 @@ struct Sum2 {
     float hi = 0.f, lo = 0.f;
     __device__ __forceinline__ void add(float v) { hi = two_sum(hi, v, lo); }
     __device__ __forceinline__ void add(const Sum2 &o) { hi = two_sum(hi, o.hi, lo); lo += o.lo; }
+    __device__ __forceinline__ void add_square(float v) { const float p = __fmul_rn(v, v); add(p); lo += __fmaf_rn(v, v, -p); }
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 __device__ __forceinline__ Sum2 warp_sum(Sum2 v) {

@@ -25,10 +25,14 @@ static std::atomic<int> g_sm_target{0};
 static std::atomic<int> g_single_pass{1};
 bool single_pass_enabled() { return g_single_pass.load(std::memory_order_relaxed) != 0; }
 
-bool sm_target_set() { return g_sm_target.load(std::memory_order_relaxed) > 0; }
+static thread_local int tl_sm_target = -1;
+SmTargetScope::SmTargetScope(int sms) : saved(tl_sm_target) { tl_sm_target = sms; }
+SmTargetScope::~SmTargetScope() { tl_sm_target = saved; }
+static int raw_sm_target() { return tl_sm_target >= 0 ? tl_sm_target : g_sm_target.load(std::memory_order_relaxed); }
+bool sm_target_set() { return raw_sm_target() > 0; }
 
 int sm_target() {
-    const int all = sm_count(), t = g_sm_target.load(std::memory_order_relaxed);
+    const int all = sm_count(), t = raw_sm_target();
     return (t > 0 && t < all) ? t : all;
 }
 

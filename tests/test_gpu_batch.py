@@ -1,0 +1,70 @@
+"""A batch of layer calls of every kind against the NumPy oracle: layers of one kind share launches, blocks and scratch."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2109_12191_b200 import synth
+from gpu_util import B, TOL_ACC_F32, TOL_FMA, TOL_NORM, dev_inputs, make_desc, oracle_layer, rel_l2, scaled_inputs
+
+pytestmark = pytest.mark.gpu
+
+STORE, NORM, CLIP = 0, 1, 2
+LAYERS = [
+    synth.conv(3, 64, 7, 2, 3, 21, False, "strided stem"), synth.conv(3, 32, 3, 1, 1, 12, True, "stem"),
+    synth.conv(64, 64, 1, 1, 0, 9, False, "one tile"), synth.conv(64, 256, 3, 1, 1, 6, False, "rows of input columns"),
+    synth.conv(128, 384, 1, 1, 0, 7, False, "three tiles"), synth.conv(128, 256, 3, 2, 1, 9, False, "larger clusters"),
+    synth.conv(256, 320, 3, 1, 1, 7, False, "Gram matrices, one product"), synth.conv(256, 256, 3, 1, 1, 13, False, "Gram matrices, tiles"),
+    synth.conv(64, 64, 3, 2, 1, 8, True, "with a bias"), synth.conv(5, 7, 3, 1, 0, 9, True, "nothing aligned"),
+    synth.dense(65, 10, True, "dense"), synth.norm(24, 7), synth.norm(2048, 3), synth.norm(5, 6),
+]
+
+
+@pytest.mark.parametrize("Bn", [1, 5])
+@pytest.mark.parametrize("dtype", ["bf16", "f32", "tf32"])
+@pytest.mark.parametrize("epi,separate", [(STORE, 1), (NORM, 0), (NORM, 1), (CLIP, 0), (CLIP, 1)])
+def test_layers_of_every_kind(epi, separate, dtype, Bn):
+    b = B()
+    inputs = [scaled_inputs(l, Bn, dtype if dtype != "tf32" else "f32", 971, i, spread=True) for i, l in enumerate(LAYERS)]
+    data = [dev_inputs(inp, dtype) for inp in inputs]
+    descs = [make_desc(l, Bn, dtype, 0, separate) for l in LAYERS]
+    groups = [b.dp_layer_groups(d) for d in descs]
+    refs = [oracle_layer(l, inp) for l, inp in zip(LAYERS, inputs)]
+    sqs = []
+    for (dW, db), g in zip(refs, groups):
+        w, v = oracle.sqnorm(dW), (oracle.sqnorm(db) if db is not None else np.zeros(Bn))
+        sqs.append(np.stack([w, v], 1) if g == 2 else (w + v)[:, None])
+    C_l = float(np.sqrt(np.median(np.concatenate([s.ravel() for s in sqs]))))
+    batch = b.Batch(descs, [epi] * len(LAYERS))
+    out = []
+    for i, (l, g) in enumerate(zip(LAYERS, groups)):
+        nan = lambda *shape: torch.full(shape, float("nan"), device="cuda")  # noqa: E731
+        o = dict(sqnorm=nan(Bn, g))
+        if epi == STORE:
+            o["G_w"], o["G_b"] = nan(Bn, l.n_weight), nan(Bn, l.n_bias) if l.n_bias else None
+        if epi == CLIP:
+            o["acc_w"], o["clip_out"] = torch.ones(l.n_weight, device="cuda"), nan(Bn, g)
+            o["acc_b"] = torch.ones(l.n_bias, device="cuda") if l.n_bias else None
+        batch.set(i, sqnorm_stride=g, **o)
+        out.append(o)
+    ws = torch.full((batch.workspace_bytes + 256,), 0xAB, dtype=torch.uint8, device="cuda")
+    b.check(b.dp_workspace_init(ws, batch.workspace_bytes), "dp_workspace_init")
+    try:
+        for target in (0, 40):                               # tickets and scratch are left ready for the next run; plans stay
+            b.check(b.dp_set_sm_target(target), "dp_set_sm_target")
+            b.check(batch.run(data, C_l, ws[:batch.workspace_bytes]), "dp_batch_run")
+    finally:
+        b.dp_set_sm_target(0)
+    b.check(b.dp_wgrad_check(ws), "dp_wgrad_check")
+    assert bool((ws[batch.workspace_bytes:] == 0xAB).all())
+    for l, d, (dW, db), sq, g, o in zip(LAYERS, descs, refs, sqs, groups, out):
+        tol = TOL_ACC_F32 if dtype == "tf32" and b.dp_wgrad_uses_tensor_cores(d, epi) else TOL_FMA
+        np.testing.assert_allclose(o["sqnorm"].cpu().numpy(), sq, rtol=TOL_NORM if tol == TOL_FMA else 1e-3, err_msg=l.name)
+        if epi == STORE:
+            assert rel_l2(o["G_w"].cpu().numpy(), dW) <= tol, l.name
+            assert db is None or rel_l2(o["G_b"].cpu().numpy(), db) <= tol, l.name
+        if epi == CLIP:
+            f = oracle.clip_factor(sq, C_l).reshape(Bn, g)
+            np.testing.assert_allclose(o["clip_out"].cpu().numpy(), f, rtol=TOL_NORM if tol == TOL_FMA else 1e-3, err_msg=l.name)
+            assert rel_l2(o["acc_w"].cpu().numpy(), 1 + 2 * np.einsum("n,np->p", f[:, 0], dW)) <= tol, l.name
+            assert db is None or rel_l2(o["acc_b"].cpu().numpy(), 1 + 2 * np.einsum("n,np->p", f[:, g - 1], db)) <= tol, l.name
