@@ -85,33 +85,48 @@ affine_batch_partial_kernel(const __grid_constant__ AffineGroup grp) {
 }
 
 // Launch 2: block = (layer, example): folds the example's pixel chunks in chunk order, stores its gradients, publishes
-// its squared norms and, for the fused clip, its factors.
+// its squared norms and, for the fused clip, its factors.  A chain of L2 round trips: four channels a thread and eight
+// chunks in flight, and squares summed in floats that carry their rounding errors along, since the double pipe is what the
+// block would wait for (53 layers x 8 examples: 13 us with one channel a thread and double sums).
 __global__ void __launch_bounds__(256)
 affine_batch_fold_kernel(const __grid_constant__ AffineGroup grp) {
-    __shared__ double scratch[32];
+    __shared__ double scratch[2][8];
     const int li = find_layer(grp.start2, grp.n, blockIdx.x);
     const AffineSeg &s = grp.seg[li];
     const int n = blockIdx.x - grp.start2[li], C = s.C, chunks = s.chunks;
     const float *base = grp.partial + s.part_off + (long long)n * chunks * 2 * C;
-    double q[2] = {0.0, 0.0};
-    for (int e = threadIdx.x; e < 2 * C; e += 256) {
-        const int which = e >= C;
-        const float *p = base + e;                        // [chunk][2][C]
-        float a = 0.f;
-        int k = 0;
-        for (; k + 8 <= chunks; k += 8) {                 // eight chunks' loads in flight, added in chunk order
-            float x[8];
+    float *dgamma = s.dgamma + (long long)n * C, *dbeta = s.dbeta + (long long)n * C;
+    Sum2 q[2];
+    for (int e = 4 * threadIdx.x; e < 2 * C; e += 1024) {
+        const bool beta = e >= C;
+        const float4 *p = reinterpret_cast<const float4 *>(base + e);         // [chunk][2][C], C a multiple of four
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int k = 0; k < chunks; k += 8) {
+            float4 x[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = p[(long long)(k + u) * 2 * C];
+            for (int u = 0; u < 8; ++u) {
+                x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (k + u < chunks) x[u] = p[(long long)(k + u) * (C / 2)];
+            }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) a += x[u];
+            for (int u = 0; u < 8; ++u) { a.x += x[u].x; a.y += x[u].y; a.z += x[u].z; a.w += x[u].w; }
         }
-        for (; k < chunks; ++k) a += p[(long long)k * 2 * C];
-        (which ? s.dbeta + (long long)n * C - C : s.dgamma + (long long)n * C)[e] = a;
-        if (which) q[1] += (double)a * a; else q[0] += (double)a * a;
+        *reinterpret_cast<float4 *>(beta ? dbeta + e - C : dgamma + e) = a;
+        Sum2 t;
+        t.add_square(a.x); t.add_square(a.y); t.add_square(a.z); t.add_square(a.w);
+        if (beta) q[1].add(t); else q[0].add(t);
     }
-    const double qg = block_sum(q[0], scratch), qb = block_sum(q[1], scratch);
+    const int warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const Sum2 t = warp_sum(q[k]);
+        if ((threadIdx.x & 31) == 0) scratch[k][warp] = t.value();
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
+    double qg = 0.0, qb = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { qg += scratch[0][i]; qb += scratch[1][i]; }
     float f0 = 1.f, f1 = 1.f;
     if (s.separate) {
         s.sqnorm[n * s.sq_stride] = (float)qg; s.sqnorm[n * s.sq_stride + 1] = (float)qb;
@@ -125,28 +140,35 @@ affine_batch_fold_kernel(const __grid_constant__ AffineGroup grp) {
     if (s.clip) { s.factor[2 * n] = f0; s.factor[2 * n + 1] = f1; }
 }
 
-// Launch 3 (fused clip): block = (layer, 32 of its 2C sums), eight groups of examples folded in group order.
+// Launch 3 (fused clip): block = (layer, 128 of its 2C sums), four a lane, eight groups of examples folded in group order.
+constexpr int kAccumSums = 128;
 __global__ void __launch_bounds__(256)
 affine_batch_accum_kernel(const __grid_constant__ AffineGroup grp) {
-    __shared__ float part[8][32];
+    __shared__ float4 part[8][32];
     const int li = find_layer(grp.start3, grp.n, blockIdx.x);
     const AffineSeg &s = grp.seg[li];
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5, C = s.C;
-    const int e = (blockIdx.x - grp.start3[li]) * 32 + lane;
+    const int e = (blockIdx.x - grp.start3[li]) * kAccumSums + 4 * lane;
     const int which = e >= C, c = which ? e - C : e;
-    float a = 0.f;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
     if (e < 2 * C) {
         const float *v = (which ? s.dbeta : s.dgamma) + c;
-#pragma unroll 8
-        for (int n = q; n < s.B; n += 8) a = fmaf(s.factor[2 * n + which], v[(long long)n * C], a);
+#pragma unroll 4
+        for (int n = q; n < s.B; n += 8) {
+            const float f = s.factor[2 * n + which];
+            const float4 x = *reinterpret_cast<const float4 *>(v + (long long)n * C);
+            a.x = fmaf(f, x.x, a.x); a.y = fmaf(f, x.y, a.y); a.z = fmaf(f, x.z, a.z); a.w = fmaf(f, x.w, a.w);
+        }
     }
     part[q][lane] = a;
     __syncthreads();
     if (q == 0 && e < 2 * C) {
-        float t = part[0][lane];
+        float4 *dst = reinterpret_cast<float4 *>((which ? s.acc_b : s.acc_w) + c);
+        float4 t = part[0][lane], r = *dst;
 #pragma unroll
-        for (int i = 1; i < 8; ++i) t += part[i][lane];
-        (which ? s.acc_b : s.acc_w)[c] += t;
+        for (int i = 1; i < 8; ++i) { const float4 x = part[i][lane]; t.x += x.x; t.y += x.y; t.z += x.z; t.w += x.w; }
+        r.x += t.x; r.y += t.y; r.z += t.z; r.w += t.w;
+        *dst = r;
     }
 }
 
@@ -172,7 +194,7 @@ dp_status launch_affine_batch(int dtype, AffineGroup &grp, cudaStream_t st) {
         grp.start1[i] = b1; grp.start2[i] = b2; grp.start3[i] = b3;
         b1 += s.B * s.chunks * ((s.C / vec + s.tcv - 1) / s.tcv);
         b2 += s.B;
-        b3 += s.clip ? (2 * s.C + 31) / 32 : 0;
+        b3 += s.clip ? (2 * s.C + kAccumSums - 1) / kAccumSums : 0;
         const size_t need = sizeof(float) * (size_t)(256 / s.tcv) * s.tcv * vec * 2;
         if (need > smem) smem = need;
     }

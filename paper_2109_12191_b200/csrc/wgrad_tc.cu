@@ -2580,7 +2580,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
     GramQueue gram;
     SsumQueue ssum;
     std::vector<SplitSeg> splits;
-    std::vector<FoldSeg> folds;
+    std::vector<FoldSeg> folds, folds_clusters, folds_sums;      // by the stream that leaves the partial sums
     for (const ConvJob &j : jobs) {
         const TcProblem pr = tc_problem(j.dtype, j.g);
         const ConvGeom &g = pr.eff;
@@ -2618,7 +2618,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             p.cluster = cluster;
             q.blocks = (p.splits + sets - 1) / sets * cluster;
             q.smem = pl.smem; q.cost = p.per_split * pl.item_cycles;
-            if (p.splits > 1) folds.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+            if (p.splits > 1) (cluster > 4 ? folds_clusters : folds).push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
             clip[cluster].jobs.push_back(q);
         } else {
             const GramPlan gp = gram_plan(j.dtype, j.g);
@@ -2648,7 +2648,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
                 TcParams &p = t.e.p;
                 t.blocks = p.blocks = p.total_tiles;
                 t.smem = pl.smem; t.cost = p.per_split * pl.item_cycles;
-                if (p.splits > 1) folds.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+                if (p.splits > 1) folds_sums.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
                 ssum.jobs.push_back(t);
             }
         }
@@ -2684,9 +2684,11 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             DP_LAUNCH_CHECK("conv_wgrad_ssum_kernel");
             return DP_OK;
         });
-    if (rc == DP_OK) rc = join();
+    // (each stream folds its own: behind the join the fold would be alone on the GPU)
+    if (rc == DP_OK) rc = launch_folds(folds_clusters, clusters);
+    if (rc == DP_OK) rc = launch_folds(folds_sums, sums);
     if (rc == DP_OK) rc = launch_folds(folds, stream);
-    return rc;
+    return rc == DP_OK ? join() : rc;
 }
 
 }  // namespace dp
