@@ -243,6 +243,9 @@ DP_API dp_status dp_clip_accumulate_noised(int mode, int B, int L, const float *
 DP_API dp_status dp_debug_example_noise_z(float *z, long long count, long long first_index, long long example,
                                           unsigned long long seed, unsigned long long step, void *cuda_stream);
 
+/* The start of a step: P floats of zero in `acc`, on the caller's stream. */
+DP_API dp_status dp_accumulator_clear(float *acc, long long P, void *cuda_stream);
+
 /* The two halves of dp_clip_accumulate on their own, for steps that keep only some tensors' per-example gradients in
  * memory and form the others' clipped sums with dp_per_example_wgrad_scaled.
  *

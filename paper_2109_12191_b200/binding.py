@@ -20,7 +20,7 @@ _lib = ctypes.CDLL(LIB_PATH)
 
 # The calls of a training step go through a small extension module (marshalling in C); the rest through ctypes.
 from . import _pycall  # noqa: E402
-from ._pycall import (dp_clip_accumulate, dp_clip_accumulate_grouped, dp_clip_accumulate_micro, dp_clip_accumulate_noised,  # noqa: E402,F401
+from ._pycall import (dp_accumulator_clear, dp_clip_accumulate, dp_clip_accumulate_grouped, dp_clip_accumulate_micro, dp_clip_accumulate_noised,  # noqa: E402,F401
                       dp_clip_accumulate_static, dp_clip_factors, dp_noise_average, dp_noise_average_sgd, dp_per_example_wgrad,
                       dp_per_example_wgrad_scaled, dp_scale_accumulate)
 _pycall.set_torch(getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None),
@@ -42,7 +42,7 @@ EXPORTS = ["dp_layer_groups", "dp_workspace_bytes", "dp_per_example_wgrad", "dp_
            "dp_debug_example_noise_z", "dp_clip_accumulate_grouped", "dp_clip_accumulate_micro",
            "dp_per_example_wgrad_scaled", "dp_clip_factors", "dp_scale_accumulate", "dp_workspace_init",
            "dp_debug_set_wait_polls", "dp_set_sm_target", "dp_debug_set_single_pass", "dp_batch_create",
-           "dp_batch_destroy", "dp_batch_workspace_bytes", "dp_batch_run"]
+           "dp_batch_destroy", "dp_batch_workspace_bytes", "dp_batch_run", "dp_accumulator_clear"]
 
 
 class dp_layer_desc(ctypes.Structure):

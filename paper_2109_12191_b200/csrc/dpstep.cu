@@ -366,6 +366,12 @@ extern "C" dp_status dp_wgrad_check(void *workspace, void *cuda_stream) {
     return DP_ERR_TIMEOUT;
 }
 
+extern "C" dp_status dp_accumulator_clear(float *acc, long long P, void *cuda_stream) {
+    if (!acc || P <= 0 || !aligned(acc, 4)) return DP_ERR_INVALID_ARG;
+    DP_CUDA_TRY(cudaMemsetAsync(acc, 0, sizeof(float) * (size_t)P, static_cast<cudaStream_t>(cuda_stream)));
+    return DP_OK;
+}
+
 extern "C" dp_status dp_set_sm_target(int sms) {
     if (sms < 0) return DP_ERR_INVALID_ARG;
     dp::g_sm_target.store(sms, std::memory_order_relaxed);

@@ -191,6 +191,16 @@ static PyObject *per_example_wgrad_scaled(PyObject *self, PyObject *const *args,
     return PyLong_FromLong(rc);
 }
 
+static PyObject *accumulator_clear(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
+    ARGS("dp_accumulator_clear", 2, "acc", "P", "stream");
+    void *acc, *st;
+    long long P;
+    if (address(a[0], &acc) < 0 || whole(a[1], &P) < 0 || stream_of(a[2], &st) < 0) return NULL;
+    int rc;
+    CALL(rc, dp_accumulator_clear(acc, P, st));
+    return PyLong_FromLong(rc);
+}
+
 static PyObject *clip_factors(PyObject *self, PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames) {
     ARGS("dp_clip_factors", 7, "mode", "B", "L", "sqnorm", "C", "norms_out", "factors_out", "stream");
     long long mode, B, L;
@@ -395,6 +405,7 @@ static PyObject *set_torch(PyObject *self, PyObject *const *args, Py_ssize_t nar
 #define ENTRY(name, fn) {name, (PyCFunction)(void (*)(void))fn, METH_FASTCALL | METH_KEYWORDS, NULL}
 static PyMethodDef methods[] = {
     ENTRY("dp_per_example_wgrad", per_example_wgrad), ENTRY("dp_per_example_wgrad_scaled", per_example_wgrad_scaled),
+    ENTRY("dp_accumulator_clear", accumulator_clear),
     ENTRY("dp_clip_factors", clip_factors), ENTRY("dp_scale_accumulate", scale_accumulate),
     ENTRY("dp_clip_accumulate", clip_accumulate), ENTRY("dp_clip_accumulate_static", clip_accumulate_static),
     ENTRY("dp_clip_accumulate_noised", clip_accumulate_noised), ENTRY("dp_clip_accumulate_grouped", clip_accumulate_grouped),

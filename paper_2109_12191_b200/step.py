@@ -101,6 +101,10 @@ class GlobalClipStep:
         self._kept = [i for i, k in enumerate(kept) if k]
         self.norms = torch.empty(B, dtype=torch.float32, device=device)
         self.clip = torch.empty(B, dtype=torch.float32, device=device)
+        # the buffers stay where they are: their addresses, so that a chunk does not ask every tensor again
+        self._acc_at, self._views_at = self.acc.data_ptr(), [v.data_ptr() for v in self.acc_views]
+        self._G_at = [g.data_ptr() if g is not None else None for g in self.G]
+        self._small_at = (self.sq.data_ptr(), self.norms.data_ptr(), self.clip.data_ptr())
         self.batch = b.Batch(self.descs, [b.DP_EPI_NORM_ONLY if li in self.recompute else b.DP_EPI_STORE_NORM
                                           for li in range(len(self.layers))])
         for li, col in enumerate(self._col):
@@ -113,6 +117,8 @@ class GlobalClipStep:
         self.ws = self.ws_lane[0]
         self._side = [torch.cuda.Stream(device=device) for _ in range(self.lanes - 1)] if self.lanes > 1 else []
         self.clip_ws = torch.empty(max(b.dp_clip_workspace_bytes(B, self.P_l), 256), dtype=torch.uint8, device=device)
+        self._clip_ws_at = (self.clip_ws.data_ptr(), self.clip_ws.numel())
+        self._kept_at = ([self._G_at[i] for i in self._kept], [self.P_l[i] for i in self._kept], [self._views_at[i] for i in self._kept])
         self.chunks_done = 0
 
     def _recompute_set(self, recompute):
@@ -138,7 +144,7 @@ class GlobalClipStep:
 
     def begin(self, total_batch=None, seed=0, step=0, example0=0):
         """Per-example noise needs the step's total batch, its (seed, step) and this rank's first example index up front."""
-        self.acc.zero_()
+        b.check(b.dp_accumulator_clear(self._acc_at, self.P), "dp_accumulator_clear")
         self.chunks_done = 0
         self._noise = _NoiseKey(self.per_example_noise, total_batch, seed, step, example0)
 
@@ -165,8 +171,8 @@ class GlobalClipStep:
 
     def scale_kept(self, stream=None):
         """Clipped sum of the tensors whose per-example gradients are in memory, with the factors in self.clip."""
-        b.check(b.dp_scale_accumulate(self.B, [self.G[i] for i in self._kept], [self.P_l[i] for i in self._kept], self.clip, 0,
-                                      [self.acc_views[i] for i in self._kept], stream=stream), "dp_scale_accumulate")
+        G, P_l, acc = self._kept_at
+        b.check(b.dp_scale_accumulate(self.B, G, P_l, self._small_at[2], 0, acc, stream=stream), "dp_scale_accumulate")
 
     def _forked(self, calls):
         """Runs calls[k](lane, stream) spread over the lanes, joined again on the current stream."""
@@ -195,16 +201,18 @@ class GlobalClipStep:
     def clip_accumulate(self, use_epilogue_norms=True, inputs=None):
         """Factors from the norm table, then the clipped sums: over memory for the kept tensors, by a second pass over
         `inputs` for the recomputed layers."""
-        sq = self.sq if use_epilogue_norms else None
+        sq, norms, clip = self._small_at
+        if not use_epilogue_norms:
+            sq = None
         if self.per_example_noise:
             k = self._noise
-            b.check(b.dp_clip_accumulate_noised(b.DP_CLIP_GLOBAL, self.B, self.G, self.P_l, self.offsets, sq, self.C,
+            b.check(b.dp_clip_accumulate_noised(b.DP_CLIP_GLOBAL, self.B, self._G_at, self.P_l, self.offsets, sq, self.C,
                                                 self.sigma, k.total_batch, k.seed, k.step,
-                                                k.example0 + self.B * self.chunks_done, self.acc_views, self.norms,
-                                                self.clip, self.clip_ws), "dp_clip_accumulate_noised")
+                                                k.example0 + self.B * self.chunks_done, self._views_at, norms,
+                                                clip, *self._clip_ws_at), "dp_clip_accumulate_noised")
         elif not self.recompute:
-            b.check(b.dp_clip_accumulate(b.DP_CLIP_GLOBAL, self.B, self.G, self.P_l, sq, self.C, self.acc_views, self.norms,
-                                         self.clip, self.clip_ws), "dp_clip_accumulate")
+            b.check(b.dp_clip_accumulate(b.DP_CLIP_GLOBAL, self.B, self._G_at, self.P_l, sq, self.C, self._views_at, norms,
+                                         clip, *self._clip_ws_at), "dp_clip_accumulate")
         else:
             if inputs is None:
                 raise ValueError("recomputed layers need the chunk's inputs for their second pass")
@@ -253,10 +261,11 @@ class FlatClipStep:
         self.norms = torch.empty(B, dtype=torch.float32, device=device)
         self.clip = torch.empty(B, dtype=torch.float32, device=device)
         self.ws = torch.empty(max(b.dp_clip_workspace_bytes(B, [P]), 256), dtype=torch.uint8, device=device)
+        self._acc_at = self.acc.data_ptr()
         self.chunks_done = 0
 
     def begin(self, total_batch=None, seed=0, step=0, example0=0):
-        self.acc.zero_()
+        b.check(b.dp_accumulator_clear(self._acc_at, self.P), "dp_accumulator_clear")
         self.chunks_done = 0
         self._noise = _NoiseKey(self.per_example_noise, total_batch, seed, step, example0)
 
@@ -311,6 +320,7 @@ class PerLayerClipStep:
         self.acc_w = [views[(li, "w")] for li in range(len(self.layers))]
         self.acc_b = [views.get((li, "b")) for li in range(len(self.layers))]
         self.sq = torch.zeros((B, self.L), dtype=torch.float32, device=device)
+        self._acc_at = self.acc.data_ptr()
         self._col, col = [], 0
         for l in self.layers:
             self._col.append(col)
@@ -332,7 +342,7 @@ class PerLayerClipStep:
             self._lane_of.append(k)
 
     def begin(self):
-        self.acc.zero_()
+        b.check(b.dp_accumulator_clear(self._acc_at, self.acc.numel()), "dp_accumulator_clear")
         self.chunks_done = 0
 
     def wgrad(self, li, X, dY, lane=0, stream=None):
