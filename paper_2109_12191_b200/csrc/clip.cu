@@ -49,12 +49,10 @@ __device__ __forceinline__ int find_seg(const SegTable<N> &t, int blk) {
 // stage 1: partial[n][part_start[seg] + j] = sum of squares of G_seg[n, j*chunk .. (j+1)*chunk); up to three floats before
 // the first 16-byte boundary and after the last one are read alone
 template <int N>
-__global__ void __launch_bounds__(256)
-sqnorm_partial_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example) {
+__device__ __forceinline__ void sqnorm_partial(const SegTable<N> &tab, int blk, int n, float *__restrict__ partial, long long parts_per_example) {
     __shared__ float scratch[32];
-    const int seg = find_seg(tab, blockIdx.x);
-    const int j = blockIdx.x - tab.blk_start[seg];
-    const int n = blockIdx.y;
+    const int seg = find_seg(tab, blk);
+    const int j = blk - tab.blk_start[seg];
     const long long P = tab.P[seg];
     const long long c0 = (long long)j * kNormChunk;
     const int len = (int)min((long long)kNormChunk, P - c0);
@@ -72,6 +70,12 @@ sqnorm_partial_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict
     if (tail + (int)threadIdx.x < len) a1 = fmaf(row[tail + threadIdx.x], row[tail + threadIdx.x], a1);
     const float a = block_sum((a0 + a1) + (a2 + a3), scratch);
     if (threadIdx.x == 0) partial[(long long)n * parts_per_example + tab.part_start[seg] + j] = a;
+}
+
+template <int N>
+__global__ void __launch_bounds__(256)
+sqnorm_partial_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example) {
+    sqnorm_partial(tab, blockIdx.x, blockIdx.y, partial, parts_per_example);
 }
 
 // stage 1 for micro-batch clipping: row j of the partials belongs to the MEAN of examples j*micro .. j*micro+micro-1
@@ -415,7 +419,7 @@ scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable<N> tab, const 
 template <int N>
 __global__ void __launch_bounds__(256)
 scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
-                               int per_layer, const __grid_constant__ ExampleNoise nz) {
+                               int per_layer, int odd_only, const __grid_constant__ ExampleNoise nz) {
     __shared__ float f_sh[256];
     const int seg = find_seg(tab, blockIdx.x);
     const long long P = tab.P[seg];
@@ -446,8 +450,8 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const fl
                     for (int u = 0; u < 4; ++u) v[u] = __ldcs(reinterpret_cast<const float4 *>(g + (long long)(n + u) * P));
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        float z[4];
-                        example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n + u), block, z);
+                        float z[4] = {0.f, 0.f, 0.f, 0.f};
+                        if ((u & 1) || !odd_only) example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n + u), block, z);
                         const float f = f_sh[n + u];
                         s.x += fmaf(f, v[u].x, nz.sd * z[0]); s.y += fmaf(f, v[u].y, nz.sd * z[1]);
                         s.z += fmaf(f, v[u].z, nz.sd * z[2]); s.w += fmaf(f, v[u].w, nz.sd * z[3]);
@@ -455,8 +459,8 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const fl
                 }
                 for (; n < nb; ++n) {
                     const float4 v = __ldcs(reinterpret_cast<const float4 *>(g + (long long)n * P));
-                    float z[4];
-                    example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n), block, z);
+                    float z[4] = {0.f, 0.f, 0.f, 0.f};
+                    if ((n & 1) || !odd_only) example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n), block, z);
                     const float f = f_sh[n];
                     s.x += fmaf(f, v.x, nz.sd * z[0]); s.y += fmaf(f, v.y, nz.sd * z[1]);
                     s.z += fmaf(f, v.z, nz.sd * z[2]); s.w += fmaf(f, v.w, nz.sd * z[3]);
@@ -496,6 +500,45 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const fl
             if (i < P) acc[i] += s[q];
         }
     }
+}
+
+// Stage 1 with half of the per-example noise: the norm pass waits for memory and the noise for the issue slots, and a draw
+// does not depend on its example's factor.  So the even examples' draws are added here, acc[i] += sd * sum_n z_n(goff + i),
+// by blocks spread evenly among those of the norms (every (ratio + 1)-th), the odd examples' in stage 3 (8 M parameters, 32
+// examples: norms 152 us, then all of the draws with the scaled sum 363).
+template <int N>
+struct NoiseStarts { int first[N]; };                          // first noise block of each tensor, tiles of kAccCols parameters
+template <int N>
+__device__ __forceinline__ bool noise_vec(const SegTable<N> &tab, int seg) {       // four parameters of a Philox block a thread
+    return ((tab.P[seg] & 3) == 0) && ((tab.goff[seg] & 3) == 0) && ((reinterpret_cast<uintptr_t>(tab.G[seg]) & 15) == 0) &&
+           ((reinterpret_cast<uintptr_t>(tab.acc[seg]) & 15) == 0);
+}
+template <int N>
+__global__ void __launch_bounds__(256)
+sqnorm_noise_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example, int norm_blocks,
+                    int B, int noise_blocks, int ratio, const __grid_constant__ NoiseStarts<N> starts, const __grid_constant__ ExampleNoise nz) {
+    const int idx = blockIdx.x, turn = idx / (ratio + 1);
+    if (turn >= noise_blocks || idx - turn * (ratio + 1) != ratio) {
+        const int blk = idx - min(noise_blocks, turn), n = blk / norm_blocks;
+        sqnorm_partial(tab, blk - n * norm_blocks, n, partial, parts_per_example);
+        return;
+    }
+    int lo = 0, hi = tab.nseg;
+    while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (turn >= starts.first[mid]) lo = mid; else hi = mid; }
+    const long long i = (long long)(turn - starts.first[lo]) * kAccCols + 4 * threadIdx.x;
+    if (!noise_vec(tab, lo) || i >= tab.P[lo]) return;         // (tensors off the grid of Philox blocks: all in stage 3)
+    const uint32_t block = (uint32_t)((unsigned long long)(tab.goff[lo] + i) >> 2);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int n = 0; n < B; n += 2) {
+        float z[4];
+        example_normals4(nz.ns, nz.example0 + (uint32_t)n, block, z);
+        s.x = fmaf(nz.sd, z[0], s.x); s.y = fmaf(nz.sd, z[1], s.y); s.z = fmaf(nz.sd, z[2], s.z); s.w = fmaf(nz.sd, z[3], s.w);
+    }
+    float4 *dst = reinterpret_cast<float4 *>(tab.acc[lo] + i);
+    float4 a = *dst;
+    a.x += s.x; a.y += s.y; a.z += s.z; a.w += s.w;
+    *dst = a;
 }
 
 struct ClipPlan {
@@ -563,6 +606,9 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
     const bool split = !var.noise && ((B >= 64 && wide_blocks < 8 * sm_count()) || (B >= 16 && wide_blocks < 2 * sm_count()));
     const int acc_cols = split ? kSplitCols : kAccCols;
 
+    // half of the noise goes with the norm pass where there is one, with at least a block of norms to each of noise
+    const bool halved = var.noise && !c.sq && !var.given_factor && B >= 8 && wide_blocks * (B + 1) <= 0x7fffffffll;
+
     SegTable<N> t;
     auto fill = [&](int l0, bool norm_blocks, long long &part_cursor) {
         t.nseg = 0; t.col0 = l0;
@@ -592,7 +638,13 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
             const int blocks = fill(l0, true, cursor);
             if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
             if (micro > 1) sqnorm_partial_micro_kernel<N><<<dim3((unsigned)blocks, rows), 256, 0, stream>>>(t, c.partial, c.parts_per_example, micro);
-            else sqnorm_partial_kernel<N><<<dim3((unsigned)blocks, rows), 256, 0, stream>>>(t, c.partial, c.parts_per_example);
+            else if (halved) {
+                NoiseStarts<N> starts;
+                long long tiles = 0;
+                for (int s = 0; s < t.nseg; ++s) { starts.first[s] = (int)tiles; tiles += (t.P[s] + kAccCols - 1) / kAccCols; }
+                const int ratio = (int)((long long)blocks * B / tiles);
+                sqnorm_noise_kernel<N><<<(unsigned)((long long)blocks * B + tiles), 256, 0, stream>>>(t, c.partial, c.parts_per_example, blocks, B, (int)tiles, ratio, starts, *var.noise);
+            } else sqnorm_partial_kernel<N><<<dim3((unsigned)blocks, rows), 256, 0, stream>>>(t, c.partial, c.parts_per_example);
             DP_LAUNCH_CHECK("sqnorm_partial_kernel");
             const int last = l0 + t.nseg == L;
             static const GroupTable none = {};
@@ -610,7 +662,7 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
     for (int l0 = 0; l0 < L; l0 += t.nseg) {
         const int blocks = fill(l0, false, cursor);
         if (t.nseg == 0) return DP_ERR_UNSUPPORTED;
-        if (var.noise) scale_accumulate_noised_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, *var.noise);
+        if (var.noise) scale_accumulate_noised_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, halved, *var.noise);
         else if (split) scale_accumulate_rowsplit_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, in);
         else scale_accumulate_kernel<N><<<(unsigned)blocks, 256, 0, stream>>>(t, c.factor, B, L, c.per_layer, in);
         DP_LAUNCH_CHECK("scale_accumulate_kernel");
