@@ -413,93 +413,99 @@ scale_accumulate_rowsplit_kernel(const __grid_constant__ SegTable<N> tab, const 
 }
 
 // stage 3 with per-example noise: acc[i] += sum_n ( factor * G[n, i] + sd * z_{example0+n}(goff + i) ).
-// Every thread owns the four parameters of one Philox block when the tensor starts on a multiple of four global
-// indices; otherwise each parameter draws its own block and keeps one lane.  Bound by the integer and
-// transcendental work of B*P normals, not by memory.
+// Every thread owns the up to four parameters of one Philox block that lie in the tensor, wherever it starts; the rows are
+// read 16 bytes at a time where they start on 16-byte boundaries, else word by word.  Bound by the integer and
+// transcendental work of B*P normals, not by memory (18.8 M parameters of five examples with rows at any address took
+// 673 us with a Philox block for every parameter).
+struct PhiloxLane {                          // this thread's parameters [i + k0, i + k1) of the tensor
+    long long i;
+    int k0, k1;
+    uint32_t block;
+    __device__ __forceinline__ PhiloxLane(long long tile, long long goff, long long P) {
+        i = tile * kAccCols + 4 * threadIdx.x - (goff & 3);
+        k0 = i < 0 ? (int)-i : 0;
+        k1 = (int)max(0ll, min(4ll, P - i));
+        block = (uint32_t)((unsigned long long)(goff + i) >> 2);
+    }
+    __device__ __forceinline__ bool live() const { return k1 > k0; }
+    template <bool VEC>
+    __device__ __forceinline__ float4 load(const float *p) const {
+        if (VEC) return __ldcs(reinterpret_cast<const float4 *>(p));
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k0 == 0) v.x = __ldcs(p);
+        if (k0 <= 1 && k1 > 1) v.y = __ldcs(p + 1);
+        if (k0 <= 2 && k1 > 2) v.z = __ldcs(p + 2);
+        if (k1 > 3) v.w = __ldcs(p + 3);
+        return v;
+    }
+    __device__ __forceinline__ void add(float *acc, const float4 &s, bool vec) const {
+        if (vec) {
+            float4 a = *reinterpret_cast<const float4 *>(acc + i);
+            a.x += s.x; a.y += s.y; a.z += s.z; a.w += s.w;
+            *reinterpret_cast<float4 *>(acc + i) = a;
+            return;
+        }
+        if (k0 == 0) acc[i] += s.x;
+        if (k0 <= 1 && k1 > 1) acc[i + 1] += s.y;
+        if (k0 <= 2 && k1 > 2) acc[i + 2] += s.z;
+        if (k1 > 3) acc[i + 3] += s.w;
+    }
+};
 template <int N>
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ bool noise_vec(const SegTable<N> &tab, int seg) {
+    return ((tab.P[seg] & 3) == 0) && ((tab.goff[seg] & 3) == 0) && ((reinterpret_cast<uintptr_t>(tab.G[seg]) & 15) == 0) &&
+           ((reinterpret_cast<uintptr_t>(tab.acc[seg]) & 15) == 0);
+}
+static long long noise_tiles(long long P, long long goff) { return (P + (goff & 3) + kAccCols - 1) / kAccCols; }
+
+__device__ __forceinline__ void noised_row(float4 &s, float f, const float4 &v, const PhiloxLane &me, bool noisy, uint32_t example, const ExampleNoise &nz) {
+    if (noisy) {
+        float z[4];
+        example_normals4(nz.ns, example, me.block, z);
+        s.x += fmaf(f, v.x, nz.sd * z[0]); s.y += fmaf(f, v.y, nz.sd * z[1]); s.z += fmaf(f, v.z, nz.sd * z[2]); s.w += fmaf(f, v.w, nz.sd * z[3]);
+    } else {
+        s.x = fmaf(f, v.x, s.x); s.y = fmaf(f, v.y, s.y); s.z = fmaf(f, v.z, s.z); s.w = fmaf(f, v.w, s.w);
+    }
+}
+// rows n0 .. n0 + nb of one tensor, four at a time (`g`: this thread's place in row n0)
+template <bool VEC>
+__device__ __forceinline__ void noised_rows(float4 &s, const float *g, const float *f_sh, int n0, int nb, long long P, const PhiloxLane &me,
+                                            int odd_only, const ExampleNoise &nz) {
+    int n = 0;
+    for (; n + 4 <= nb; n += 4) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = me.load<VEC>(g + (long long)(n + u) * P);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) noised_row(s, f_sh[n + u], v[u], me, (u & 1) || !odd_only, nz.example0 + (uint32_t)(n0 + n + u), nz);
+    }
+    for (; n < nb; ++n)
+        noised_row(s, f_sh[n], me.load<VEC>(g + (long long)n * P), me, (n & 1) || !odd_only, nz.example0 + (uint32_t)(n0 + n), nz);
+}
+
+template <int N>
+__global__ void __launch_bounds__(256, 4)
 scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
                                int per_layer, int odd_only, const __grid_constant__ ExampleNoise nz) {
     __shared__ float f_sh[256];
     const int seg = find_seg(tab, blockIdx.x);
     const long long P = tab.P[seg];
-    const long long c0 = (long long)(blockIdx.x - tab.blk_start[seg]) * kAccCols;
-    const float *G = tab.G[seg];
-    float *acc = tab.acc[seg];
-    const long long goff = tab.goff[seg];
     const int f_stride = per_layer ? L : 1;
     const int f_off = per_layer ? tab.col0 + seg : 0;
-    const bool vec = ((P & 3) == 0) && ((goff & 3) == 0) && ((reinterpret_cast<uintptr_t>(G) & 15) == 0) &&
-                     ((reinterpret_cast<uintptr_t>(acc) & 15) == 0);
-    if (vec) {
-        const long long i = c0 + 4 * threadIdx.x;
-        const bool live = i < P;
-        const uint32_t block = (uint32_t)((unsigned long long)(goff + i) >> 2);
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int n0 = 0; n0 < B; n0 += 256) {
-            const int nb = min(256, B - n0);
-            __syncthreads();
-            if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
-            __syncthreads();
-            if (live) {
-                const float *g = G + (long long)n0 * P + i;
-                int n = 0;
-                for (; n + 4 <= nb; n += 4) {
-                    float4 v[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) v[u] = __ldcs(reinterpret_cast<const float4 *>(g + (long long)(n + u) * P));
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        float z[4] = {0.f, 0.f, 0.f, 0.f};
-                        if ((u & 1) || !odd_only) example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n + u), block, z);
-                        const float f = f_sh[n + u];
-                        s.x += fmaf(f, v[u].x, nz.sd * z[0]); s.y += fmaf(f, v[u].y, nz.sd * z[1]);
-                        s.z += fmaf(f, v[u].z, nz.sd * z[2]); s.w += fmaf(f, v[u].w, nz.sd * z[3]);
-                    }
-                }
-                for (; n < nb; ++n) {
-                    const float4 v = __ldcs(reinterpret_cast<const float4 *>(g + (long long)n * P));
-                    float z[4] = {0.f, 0.f, 0.f, 0.f};
-                    if ((n & 1) || !odd_only) example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n), block, z);
-                    const float f = f_sh[n];
-                    s.x += fmaf(f, v.x, nz.sd * z[0]); s.y += fmaf(f, v.y, nz.sd * z[1]);
-                    s.z += fmaf(f, v.z, nz.sd * z[2]); s.w += fmaf(f, v.w, nz.sd * z[3]);
-                }
-            }
-        }
-        if (live) {
-            float4 a = *reinterpret_cast<const float4 *>(acc + i);
-            a.x += s.x; a.y += s.y; a.z += s.z; a.w += s.w;
-            *reinterpret_cast<float4 *>(acc + i) = a;
-        }
-    } else {
-        float s[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int n0 = 0; n0 < B; n0 += 256) {
-            const int nb = min(256, B - n0);
-            __syncthreads();
-            if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
-            __syncthreads();
-            for (int n = 0; n < nb; ++n) {
-                const float f = f_sh[n];
-                const float *g = G + (long long)(n0 + n) * P + c0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const long long i = threadIdx.x + 256 * q;
-                    if (c0 + i < P) {
-                        const unsigned long long gi = (unsigned long long)(goff + c0 + i);
-                        float z[4];
-                        example_normals4(nz.ns, nz.example0 + (uint32_t)(n0 + n), (uint32_t)(gi >> 2), z);
-                        s[q] += fmaf(f, g[i], nz.sd * z[gi & 3]);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const long long i = c0 + threadIdx.x + 256 * q;
-            if (i < P) acc[i] += s[q];
-        }
+    const bool vec = noise_vec(tab, seg);
+    const PhiloxLane me(blockIdx.x - tab.blk_start[seg], tab.goff[seg], P);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int n0 = 0; n0 < B; n0 += 256) {
+        const int nb = min(256, B - n0);
+        __syncthreads();
+        if (threadIdx.x < nb) f_sh[threadIdx.x] = factor[(long long)(n0 + threadIdx.x) * f_stride + f_off];
+        __syncthreads();
+        if (!me.live()) continue;
+        const float *g = tab.G[seg] + (long long)n0 * P + me.i;
+        if (vec) noised_rows<true>(s, g, f_sh, n0, nb, P, me, odd_only, nz);
+        else noised_rows<false>(s, g, f_sh, n0, nb, P, me, odd_only, nz);
     }
+    if (me.live()) me.add(tab.acc[seg], s, vec);
 }
 
 // Stage 1 with half of the per-example noise: the norm pass waits for memory and the noise for the issue slots, and a draw
@@ -509,12 +515,7 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const fl
 template <int N>
 struct NoiseStarts { int first[N]; };                          // first noise block of each tensor, tiles of kAccCols parameters
 template <int N>
-__device__ __forceinline__ bool noise_vec(const SegTable<N> &tab, int seg) {       // four parameters of a Philox block a thread
-    return ((tab.P[seg] & 3) == 0) && ((tab.goff[seg] & 3) == 0) && ((reinterpret_cast<uintptr_t>(tab.G[seg]) & 15) == 0) &&
-           ((reinterpret_cast<uintptr_t>(tab.acc[seg]) & 15) == 0);
-}
-template <int N>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 8)
 sqnorm_noise_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example, int norm_blocks,
                     int B, int noise_blocks, int ratio, const __grid_constant__ NoiseStarts<N> starts, const __grid_constant__ ExampleNoise nz) {
     const int idx = blockIdx.x, turn = idx / (ratio + 1);
@@ -525,20 +526,16 @@ sqnorm_noise_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__
     }
     int lo = 0, hi = tab.nseg;
     while (hi - lo > 1) { const int mid = (lo + hi) >> 1; if (turn >= starts.first[mid]) lo = mid; else hi = mid; }
-    const long long i = (long long)(turn - starts.first[lo]) * kAccCols + 4 * threadIdx.x;
-    if (!noise_vec(tab, lo) || i >= tab.P[lo]) return;         // (tensors off the grid of Philox blocks: all in stage 3)
-    const uint32_t block = (uint32_t)((unsigned long long)(tab.goff[lo] + i) >> 2);
+    const PhiloxLane me(turn - starts.first[lo], tab.goff[lo], tab.P[lo]);
+    if (!me.live()) return;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
+#pragma unroll 1
     for (int n = 0; n < B; n += 2) {
         float z[4];
-        example_normals4(nz.ns, nz.example0 + (uint32_t)n, block, z);
+        example_normals4(nz.ns, nz.example0 + (uint32_t)n, me.block, z);
         s.x = fmaf(nz.sd, z[0], s.x); s.y = fmaf(nz.sd, z[1], s.y); s.z = fmaf(nz.sd, z[2], s.z); s.w = fmaf(nz.sd, z[3], s.w);
     }
-    float4 *dst = reinterpret_cast<float4 *>(tab.acc[lo] + i);
-    float4 a = *dst;
-    a.x += s.x; a.y += s.y; a.z += s.z; a.w += s.w;
-    *dst = a;
+    me.add(tab.acc[lo], s, noise_vec(tab, lo));
 }
 
 struct ClipPlan {
@@ -607,7 +604,7 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
     const int acc_cols = split ? kSplitCols : kAccCols;
 
     // half of the noise goes with the norm pass where there is one, with at least a block of norms to each of noise
-    const bool halved = var.noise && !c.sq && !var.given_factor && B >= 8 && wide_blocks * (B + 1) <= 0x7fffffffll;
+    const bool halved = var.noise && !c.sq && !var.given_factor && B >= 9 && (wide_blocks + L) * (B + 1) <= 0x7fffffffll;
 
     SegTable<N> t;
     auto fill = [&](int l0, bool norm_blocks, long long &part_cursor) {
@@ -616,7 +613,7 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
         for (int l = l0; l < L && t.nseg < N; ++l) {
             const int s = t.nseg;
             const long long nparts = (c.P_l[l] + kNormChunk - 1) / kNormChunk;
-            const long long nb = norm_blocks ? nparts : (c.P_l[l] + acc_cols - 1) / acc_cols;
+            const long long nb = norm_blocks ? nparts : (var.noise ? noise_tiles(c.P_l[l], var.goff_l[l]) : (c.P_l[l] + acc_cols - 1) / acc_cols);
             if ((long long)blk + nb > 0x7fffffffll) break;
             t.G[s] = c.G[l]; t.acc[s] = c.acc[l]; t.P[s] = c.P_l[l];
             t.goff[s] = var.goff_l ? var.goff_l[l] : 0;
@@ -641,8 +638,8 @@ static dp_status clip_launches(const ClipCall &c, const ClipVariant &var, cudaSt
             else if (halved) {
                 NoiseStarts<N> starts;
                 long long tiles = 0;
-                for (int s = 0; s < t.nseg; ++s) { starts.first[s] = (int)tiles; tiles += (t.P[s] + kAccCols - 1) / kAccCols; }
-                const int ratio = (int)((long long)blocks * B / tiles);
+                for (int s = 0; s < t.nseg; ++s) { starts.first[s] = (int)tiles; tiles += noise_tiles(t.P[s], t.goff[s]); }
+                const int ratio = (int)((long long)blocks * B / tiles);       // at least one: a block of norms covers at most nine tiles
                 sqnorm_noise_kernel<N><<<(unsigned)((long long)blocks * B + tiles), 256, 0, stream>>>(t, c.partial, c.parts_per_example, blocks, B, (int)tiles, ratio, starts, *var.noise);
             } else sqnorm_partial_kernel<N><<<dim3((unsigned)blocks, rows), 256, 0, stream>>>(t, c.partial, c.parts_per_example);
             DP_LAUNCH_CHECK("sqnorm_partial_kernel");

@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("Bn,sizes,first,given", [
     (7, [1028], 0, False), (8, [1028], 0, False), (9, [8196], 4, False), (257, [36], 0, False), (33, [1024, 9000, 3, 20], 4, False),
     (8, [4] * 530 + [2052, 5], 0, False), (11, [4096], 0, True),
+    (9, [1025, 1023, 1, 2, 5, 1024], 3, False), (5, [2, 1021, 3], 1, False), (10, [1] * 600 + [1022], 2, False),
 ])
 def test_noise_split_between_the_passes(Bn, sizes, first, given):
     groups, offs = _spread(Bn, sizes, Bn), _offsets(sizes, first)
