@@ -511,7 +511,7 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const fl
 // Stage 1 with half of the per-example noise: the norm pass waits for memory and the noise for the issue slots, and a draw
 // does not depend on its example's factor.  So the even examples' draws are added here, acc[i] += sd * sum_n z_n(goff + i),
 // by blocks spread evenly among those of the norms (every (ratio + 1)-th), the odd examples' in stage 3 (8 M parameters, 32
-// examples: norms 152 us, then all of the draws with the scaled sum 363).
+// examples: norms 152 us, then all of the draws with the scaled sum 363; this way 255 and 220).
 template <int N>
 struct NoiseStarts { int first[N]; };                          // first noise block of each tensor, tiles of kAccCols parameters
 template <int N>
