@@ -50,10 +50,16 @@ SideStreams *take_streams() {
     SideStreams *t = new (std::nothrow) SideStreams{};
     if (!t) return nullptr;
     t->device = dev;
+    // What others wait for, and short launches, take SMs before large clusters do, and those before the caller's stream.
+    int low = 0, high = 0;
+    (void)cudaDeviceGetStreamPriorityRange(&low, &high);
+    int priority[BatchStreams::kCount] = {};
+    priority[BatchStreams::kClusters] = priority[BatchStreams::kClusters6] = high / 2;
+    priority[BatchStreams::kSums] = priority[BatchStreams::kAffine] = high;
     bool ok = cudaEventCreateWithFlags(&t->fork, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&t->gram_done, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 1; ok && i < BatchStreams::kCount; ++i)
-        ok = cudaStreamCreateWithFlags(&t->stream[i], cudaStreamNonBlocking) == cudaSuccess &&
+        ok = cudaStreamCreateWithPriority(&t->stream[i], cudaStreamNonBlocking, priority[i]) == cudaSuccess &&
              cudaEventCreateWithFlags(&t->done[i], cudaEventDisableTiming) == cudaSuccess;
     if (ok) return t;
     (void)cudaGetLastError();
@@ -82,12 +88,14 @@ struct dp_batch {
         int epi;
         WgradPlan plan;
         int group, slot;             // table of its kind and place in it; group < 0: a call of its own
-        int lane;                    // of a call of its own: 0 follows the affine launches' stream, others are the caller's
+        int lane;                    // of a call of its own: 0 has a stream of the batch's, others are the caller's
         size_t scratch;              // byte offset of the layer's own scratch (factors, finished per-example gradients)
     };
     std::vector<Item> items;
     std::vector<AffineGroup> affine;             // shapes filled in, buffers per run
     std::vector<int> affine_dtype;
+    std::vector<char> affine_beside;             // runs beside convolutions
+    bool beside = false;                         // some do
     size_t affine_partial = 0;                   // byte offset of the pixel-chunk partials
     std::vector<ConvJob> convs;                  // geometry filled in, buffers per run
     std::vector<int> conv_item;                  // item of every conv
@@ -159,23 +167,57 @@ static void plan_lanes(dp_batch &b, int lanes) {
     }
 }
 
+static bool affine_of(const dp_layer_desc &d) { return d.kind == DP_LAYER_NORM_AFFINE && affine_batch_eligible(storage_type(&d), d.C_in); }
+static double affine_bytes(const dp_layer_desc &d) { return 2.0 * d.B * d.H * d.W * d.C_in * (storage_type(&d) == DP_F32 ? 4 : 2); }
+// From here on layers run beside the convolutions: the layers of a ResNet of fewer examples are through in the gaps between the
+// launches, and shallower rings of the convolutions cost more than that (3 examples, 120 MB: 162 us, 166 beside; 8 examples,
+// 350 MB: 330 and 328; 22 examples: 534 and 487).
+constexpr double kBesideBytes = 250e6;
+
+// What the convolutions' launches leave the normalisation layers that run beside them, in bytes: some 2.8 TB/s of theirs for the
+// time these take by rates measured on a chunk of ResNet-50 (53 layers x 32 examples: 263 Gflop in 550 us clipped; 16 examples:
+// 133 Gflop and 1.6 GB stored in 430 us).
+static double bytes_beside(const dp_batch &b) {
+    double us = 0.0;
+    for (const ConvJob &j : b.convs) {
+        const double rate = j.dtype == DP_BF16 ? 480e6 : (j.dtype == DP_TF32 ? 200e6 : 90e6);
+        us += 2.0 * j.g.B * j.g.M * j.g.N * j.g.K / rate;
+        if (j.epi == DP_EPI_STORE_NORM) us += 4.0 * j.g.B * j.g.M * j.g.N / 10e6;
+    }
+    return us * 2.8e6;
+}
+
 static void plan_affine(dp_batch &b, size_t &off) {
+    // Layers beside the convolutions as far as these last, the rest at the GPU's full rate, in a form that takes SMs of its own.
+    double room = b.beside ? bytes_beside(b) : 0.0;
+    std::vector<char> beside(b.items.size(), 0);
+    for (size_t i = 0; i < b.items.size(); ++i) {
+        const dp_layer_desc &d = b.items[i].desc;
+        if (!affine_of(d) || affine_bytes(d) > room) continue;
+        beside[i] = 1;
+        room -= affine_bytes(d);
+    }
     size_t partial_floats = 0;
-    for (int dt = 0; dt < 2; ++dt) {
-        const int dtype = dt == 0 ? DP_BF16 : DP_F32;
-        for (auto &it : b.items) {
+    for (int form = 0; form < 4; ++form) {
+        const int dtype = form & 1 ? DP_F32 : DP_BF16;
+        const bool is_beside = form < 2;
+        bool fresh_group = true;
+        for (size_t i = 0; i < b.items.size(); ++i) {
+            dp_batch::Item &it = b.items[i];
             const dp_layer_desc &d = it.desc;
-            if (d.kind != DP_LAYER_NORM_AFFINE || storage_type(&d) != dtype || !affine_batch_eligible(dtype, d.C_in)) continue;
-            if (b.affine.empty() || b.affine_dtype.back() != dtype || b.affine.back().n == kGroupLayers) {
+            if (!affine_of(d) || storage_type(&d) != dtype || (beside[i] != 0) != is_beside) continue;
+            if (fresh_group || b.affine.back().n == kGroupLayers) {
+                fresh_group = false;
                 AffineGroup fresh = {};
                 b.affine.push_back(fresh);
                 b.affine_dtype.push_back(dtype);
+                b.affine_beside.push_back(is_beside);
             }
             AffineGroup &g = b.affine.back();
             it.group = (int)b.affine.size() - 1;
             it.slot = g.n++;
             AffineSeg &s = g.seg[it.slot];
-            affine_batch_shape(dtype, d.B, d.H * d.W, d.C_in, s);
+            affine_batch_shape(dtype, d.B, d.H * d.W, d.C_in, is_beside, s);
             s.clip = it.epi == DP_EPI_CLIP_ACCUM;
             s.separate = groups_of(&d) == 2;
             s.part_off = (long long)partial_floats;
@@ -190,7 +232,9 @@ static void plan_affine(dp_batch &b, size_t &off) {
     off = round_up(off + sizeof(float) * partial_floats, 1024);
 }
 
-static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l, char *ws, cudaStream_t st) {
+// The groups that run beside convolutions (which come after, on other streams) or the others; without streams for that, all.
+enum { kBeside, kApart, kAllGroups };
+static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l, char *ws, int which, cudaStream_t st) {
     if (b.affine.empty()) return DP_OK;
     std::vector<AffineGroup> groups = b.affine;
     for (size_t i = 0; i < b.items.size(); ++i) {
@@ -211,7 +255,9 @@ static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l,
     for (size_t k = 0; k < groups.size(); ++k) {
         groups[k].C_l = C_l;
         groups[k].partial = reinterpret_cast<float *>(ws + b.affine_partial);
-        const dp_status rc = launch_affine_batch(b.affine_dtype[k], groups[k], st);
+        if (which != kAllGroups && (b.affine_beside[k] != 0) != (which == kBeside)) continue;
+        int *tickets = which == kBeside && k < kWsStreams ? reinterpret_cast<int *>(ws + kWsStreamOffset) + 2 * k : nullptr;
+        const dp_status rc = launch_affine_batch(b.affine_dtype[k], groups[k], tickets, st);
         if (rc != DP_OK) return rc;
     }
     return DP_OK;
@@ -232,8 +278,11 @@ static void plan_convs(dp_batch &b, size_t &off) {
         b.conv_item.push_back((int)i);
     }
     if (b.convs.empty()) return;
-    b.walk = conv_batch_walk(b.convs);
-    BatchPlanning planning(b.walk);
+    double bytes = 0.0;
+    for (const auto &it : b.items) bytes += affine_of(it.desc) ? affine_bytes(it.desc) : 0.0;
+    b.beside = bytes >= kBesideBytes;
+    b.walk = conv_batch_walk(b.convs, b.beside);
+    BatchPlanning planning(b.walk, b.beside);
     for (size_t k = 0; k < b.convs.size(); ++k) {
         dp_batch::Item &it = b.items[b.conv_item[k]];
         make_layer_plan(&it.desc, it.epi, it.plan);          // scratch sizes of the tiling a batch uses
@@ -268,7 +317,7 @@ static dp_status run_convs(const dp_batch &b, const dp_layer_io *io, float C_l, 
             if (rc != DP_OK) return rc;
         }
     }
-    return launch_conv_batch(jobs, b.walk, reinterpret_cast<int *>(ws), streams, join);
+    return launch_conv_batch(jobs, b.walk, b.beside, reinterpret_cast<int *>(ws), streams, join);
 }
 
 static dp_status plan_batch(dp_batch &b, int n, const dp_layer_desc *descs, const int *epilogues, int lanes) {
@@ -291,13 +340,13 @@ static dp_status plan_batch(dp_batch &b, int n, const dp_layer_desc *descs, cons
     for (const auto &it : b.items) {
         if (it.group >= 0) continue;
         most = std::max(most, it.plan.total);
-        b.used[BatchStreams::kAffine] = true;
+        b.used[BatchStreams::kSingles] = true;
     }
     if (!b.affine.empty()) b.used[BatchStreams::kAffine] = true;
     for (const ConvJob &j : b.convs) {
         b.used[BatchStreams::kMain] = true;
-        if (conv_batch_clusters(j, b.walk)) b.used[BatchStreams::kClusters] = true;
-        if (j.kind == kConvGramSum || b.items[b.conv_item[&j - b.convs.data()]].desc.has_bias) b.used[BatchStreams::kSums] = true;
+        b.used[conv_cluster_stream(conv_batch_cluster(j, b.walk, b.beside))] = true;
+        if (j.kind == kConvGramSum || j.kind == kConvGramTiles || b.items[b.conv_item[&j - b.convs.data()]].desc.has_bias) b.used[BatchStreams::kSums] = true;
     }
     b.total = most > kWsHeaderBytes ? round_up(off + most - kWsHeaderBytes, 256) : off;
     return DP_OK;
@@ -370,7 +419,7 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
     // fill what the tensor-core launches leave idle.
     BatchStreams streams;
     // (without convolutions there is nothing to fork from: everything stays on the caller's stream)
-    const bool forked = b->used[BatchStreams::kMain] && (b->used[1] || b->used[2] || b->used[3]) && side_streams(*b);
+    const bool forked = b->used[BatchStreams::kMain] && std::find(b->used + 1, b->used + BatchStreams::kCount, true) != b->used + BatchStreams::kCount && side_streams(*b);
     for (int i = 0; i < BatchStreams::kCount; ++i) streams.s[i] = forked && i && b->used[i] ? b->side->stream[i] : st;
     streams.gram_done = forked && b->used[BatchStreams::kSums] ? b->side->gram_done : nullptr;
     if (forked) {
@@ -390,7 +439,7 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
     // more examples than SMs, whose second round of blocks would leave SMs idle (256 of 32 x 32: 135 us first, 117 last).
     auto ahead = [](const dp_batch::Item &it) { return it.plan.use_thin && it.desc.B <= sm_count(); };
     auto singles = [&](bool first) -> dp_status {
-        BatchPlanning alone(0.0);        // tiled as their plans were: not as layers of a grouped launch
+        BatchPlanning alone(0.0, false);        // tiled as their plans were: not as layers of a grouped launch
         SmTargetScope target(b->target);
         dp_status rc = DP_OK;
         for (int i = 0; i < n && rc == DP_OK; ++i) {
@@ -401,7 +450,7 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
                 char *own = static_cast<char *>(lane_workspaces[it.lane - 1]);
                 rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, own, own + kWsHeaderBytes, static_cast<cudaStream_t>(lane_streams[it.lane - 1]));
             } else {
-                rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kAffine]);
+                rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kSingles]);
             }
         }
         return rc;
@@ -414,7 +463,7 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
         try {
             // (singles first: they are short, and behind the normalisation layers they would be the chunk's tail)
             rc = singles(false);
-            if (rc == DP_OK) rc = run_affine(*b, io, C_l, ws, streams.s[BatchStreams::kAffine]);
+            if (rc == DP_OK) rc = run_affine(*b, io, C_l, ws, forked ? kApart : kAllGroups, streams.s[BatchStreams::kAffine]);
         } catch (const std::exception &) {       // out of memory: the streams still have to meet
             rc = DP_ERR_CUDA;
         }
@@ -432,7 +481,9 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
     };
     dp_status rc;
     try {
-        rc = singles(true);
+        // (on every SM before the convolutions' blocks are)
+        rc = forked ? run_affine(*b, io, C_l, ws, kBeside, streams.s[BatchStreams::kAffine]) : DP_OK;
+        if (rc == DP_OK) rc = singles(true);
         if (rc == DP_OK) rc = run_convs(*b, io, C_l, ws, streams, join);
     } catch (const std::exception &) {           // out of memory
         rc = DP_ERR_CUDA;

@@ -26,7 +26,9 @@ struct AffineGroup {
     AffineSeg seg[kGroupLayers];
 };
 bool affine_batch_eligible(int dtype, int C);
-void affine_batch_shape(int dtype, int B, int HW, int C, AffineSeg &s);
-dp_status launch_affine_batch(int dtype, AffineGroup &grp, cudaStream_t st);
+// beside: shaped for the form that runs beside tensor-core launches (any form takes it)
+void affine_batch_shape(int dtype, int B, int HW, int C, bool beside, AffineSeg &s);
+// tickets: two cleared words for the form that runs beside tensor-core launches, which are in later launches; null: the GPU is free
+dp_status launch_affine_batch(int dtype, AffineGroup &grp, int *tickets, cudaStream_t st);
 
 }  // namespace dp

@@ -23,6 +23,8 @@ struct SmTargetScope {  // another target (0: none) for this thread while it liv
     int saved;
 };
 bool sm_target_set();   // true once dp_set_sm_target() was given a positive value: the caller runs calls side by side
+// Polls after which a bounded wait of a kernel gives up.
+uint32_t wait_polls();
 // false while dp_debug_set_single_pass(0) holds: the fused clipped sum then always runs its two-pass form
 bool single_pass_enabled();
 
@@ -30,6 +32,8 @@ bool single_pass_enabled();
 // at byte 0 and, from byte 256, the ticket counters with which the last block to finish a unit of work finds out
 // that it is the last (each kernel leaves its counters at zero again).
 constexpr size_t kWsHeaderBytes = 16384;
+constexpr size_t kWsStreamOffset = 64;   // pairs of words: items taken, blocks done (each kernel leaves them at zero too)
+constexpr int kWsStreams = 8;
 constexpr size_t kWsCounterOffset = 256;
 constexpr int kWsCounters = (int)((kWsHeaderBytes - kWsCounterOffset) / sizeof(int));
 constexpr int kWsBatchCounters = 512;    // the last of them belong to the grouped launches of a batch, which run beside single calls
@@ -56,6 +60,25 @@ void count_launch();
 
 __device__ __forceinline__ float to_float(float v) { return v; }
 __device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
+
+// Two floats that go through the FMA pipe as one instruction: results are those of the separate operations.
+typedef unsigned long long Float2;
+__device__ __forceinline__ Float2 pack2(float lo, float hi) {
+    Float2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(Float2 v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ Float2 fma2(Float2 a, Float2 b, Float2 c) {
+    Float2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ Float2 add2(Float2 a, Float2 b) {
+    Float2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 
 // Sum over the 32 lanes in a fixed butterfly order (same result on every run).
 __device__ __forceinline__ float warp_sum(float v) {

@@ -345,14 +345,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-__device__ __forceinline__ unsigned long long pack2(float x, float y) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a, unsigned long long b) {
-    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
-}
 __device__ __forceinline__ void rgb_cluster_sync() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -458,11 +450,11 @@ conv_wgrad_rgb3_kernel(const T *__restrict__ X, const T *__restrict__ dY, const 
                 for (int q = 0; q < 9; ++q) {
                     const unsigned long long xx = pack2(x[q], x[q]);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) fma2(acc[k][q], gy[k], xx);
+                    for (int k = 0; k < 4; ++k) acc[k][q] = fma2(gy[k], xx, acc[k][q]);
                 }
                 if (fr == 0) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) fma2(bs[k], gy[k], one);
+                    for (int k = 0; k < 4; ++k) bs[k] = fma2(gy[k], one, bs[k]);
                 }
                 ow += 32;
                 while (ow >= g.OW) { ow -= g.OW; ++oh; }

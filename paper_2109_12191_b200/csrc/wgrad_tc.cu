@@ -20,6 +20,7 @@
 // stage into a second buffer of the same layout; x itself stays in place, where the tensor core's own truncation
 // turns it into hi, and the issuer accumulates lo*hi + hi*lo + hi*hi per step.  What is dropped (lo*lo and the truncation of lo) is below 2^-20 relative.
 #include "wgrad_tc.cuh"
+#include "mbar.cuh"
 #include <cuda.h>
 #include <mutex>
 #include <atomic>
@@ -35,10 +36,12 @@ namespace dp {
 constexpr int kRowBytes = 128;         // one pixel's slab of channels: 64 bf16 or 32 fp32/tf32
 constexpr int kMaxStages = 8;
 constexpr int kSmemBudget = 200 * 1024;
+constexpr int kBatchSmem = 176 * 1024;
 constexpr uint32_t kWaitPolls = 1u << 21;   // x ~1 us suspend hint: about two seconds before a wait gives up
 static std::atomic<uint32_t> g_wait_polls{kWaitPolls};
 void set_wait_polls(uint32_t polls) { g_wait_polls.store(polls, std::memory_order_relaxed); }
 uint32_t default_wait_polls() { return kWaitPolls; }
+uint32_t wait_polls() { return g_wait_polls.load(std::memory_order_relaxed); }
 
 struct TcPlan {
     bool ok;
@@ -127,43 +130,6 @@ __device__ __forceinline__ Item decode_item(const TcParams &p, int item) {
 }
 
 // ----------------------------------------------------------------------------- PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-                 "selp.b32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity), "r"(1000u) : "memory");
-    return ok != 0;
-}
-// Bounded wait.  Returns false when the CTA is aborting (this or another wait expired).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t polls) {
-    for (uint32_t it = 0; it < polls; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if ((it & 63u) == 63u && *abort_flag) return false;
-    }
-    *abort_flag = 1;
-    return false;
-}
-// One lane of a converged warp (the same one every time), and the warp's index as a value the compiler knows to be uniform:
-// with both, the descriptors of a tensor-core instruction are worked out in uniform registers, where it needs them (61
-// cycles an instruction; 107 from inside a branch only one lane takes, which bounded every main loop).
-__device__ __forceinline__ bool elect_one() {
-    uint32_t pred;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(pred));
-    return pred != 0;
-}
-__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 // A box of an activation tensor seen as {slab of channels, W, H, B, slabs}: it lands slab after slab, each OWt*OHt rows of
 // 128 bytes, so one copy brings all slabs of an operand that belong to one filter tap.
 __device__ __forceinline__ void tma_load_slabs(uint32_t dst, const CUtensorMap *map, uint32_t bar, int w, int h, int n, int slab) {
@@ -723,10 +689,13 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
 // Roles (384 threads): warp 0 issues the TMA loads of the A slabs, warp 2 those of the B slabs, warp 1 allocates tensor
 // memory and issues the MMAs, warp 3 idles; warps 4-11 are the epilogue: warp w reads TMEM lanes 32*(w%4).. and the
 // 128-column half (w-4)/4 of the tile, so a thread holds 128 running sums.  The first warpgroup gives registers up
-// (setmaxnreg) and the epilogue warpgroups take them: 128*56 + 256*224 = 384*168, the launch's allocation.
+// (setmaxnreg) and the epilogue warpgroups take them: 128*56 + 256*224 = 384*168, the launch's allocation; in a batch
+// 128*40 + 256*208 = 384*152, which leaves a warp of 56 registers a thread to each quarter of the SM (see affine_batch.cu).
 constexpr int kClipThreads = 384;
-constexpr int kClipRegsLaunch = 168, kClipRegsControl = 56, kClipRegsEpilogue = 224;
-static_assert(128 * kClipRegsControl + 256 * kClipRegsEpilogue == kClipThreads * kClipRegsLaunch, "register split must add up");
+template <int N> struct ClipRegs {                   // of a call on its own, and of a batch's launches, which leave some to others
+    static constexpr int kLaunch = N == 1 ? 168 : 152, kControl = N == 1 ? 56 : 40, kEpilogue = N == 1 ? 224 : 208;
+    static_assert(128 * kControl + 256 * kEpilogue == kClipThreads * kLaunch, "register split must add up");
+};
 constexpr int kMaxCluster = 8;
 constexpr int kMaxExamplesPerCluster = 32;   // examples a cluster walks through when an SM target is set (calls run side by side)
 
@@ -772,7 +741,7 @@ __device__ __forceinline__ float sum8(const float4 &x, const float4 &y) {
 }
 
 template <int N>
-__global__ void __launch_bounds__(kClipThreads, 1)
+__global__ void __maxnreg__(ClipRegs<N>::kLaunch)
 conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     const int entry = table_entry(tab.first, tab.n, blockIdx.x);
     const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
@@ -823,7 +792,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - nt * b_slabs_tile);
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kClipRegsControl));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ClipRegs<N>::kControl));
         if (warp == 0 || warp == 2) {
             // ------------------------------------------------------------ TMA producers (A slabs / B slabs)
             const bool leader = elect_one();
@@ -890,7 +859,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
             }
         }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kClipRegsEpilogue));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ClipRegs<N>::kEpilogue));
         // ---------------------------------------------------------------- epilogue (8 warps)
         const int e = warp - 4, q = e & 3, half = e >> 2;
         const int row = q * 32 + lane;
@@ -1744,9 +1713,13 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode);
 // Planning on behalf of a batch of layer calls (this thread): launches hold many layers, so every layer is tiled for
 // least SM time whatever the SM target is, and a CTA walks through at most this many cycles of one layer.
 static thread_local double tl_batch_walk = 0.0;
-BatchPlanning::BatchPlanning(double walk_cycles) : saved(tl_batch_walk) { tl_batch_walk = walk_cycles; }
-BatchPlanning::~BatchPlanning() { tl_batch_walk = saved; }
+static thread_local bool tl_beside = false;
+BatchPlanning::BatchPlanning(double walk_cycles, bool beside) : saved(tl_batch_walk), saved_beside(tl_beside) { tl_batch_walk = walk_cycles; tl_beside = beside; }
+BatchPlanning::~BatchPlanning() { tl_batch_walk = saved; tl_beside = saved_beside; }
 static bool side_by_side() { return tl_batch_walk > 0.0 || sm_target_set(); }
+// What a block's stages may take, with room left for a block of the normalisation layers' where one runs beside it (the kernels of modes
+// 0, 1 and 4 have 16 KB of their own besides).
+static int smem_budget(int mode) { return tl_beside ? (mode == 3 ? kBatchSmem : kBatchSmem - 16 * 1024) : kSmemBudget; }
 static int launch_sms() { return tl_batch_walk > 0.0 ? sm_count() : sm_target(); }
 
 // single-pass clipped sum: how many clusters share the batch and how many examples each walks through
@@ -1785,8 +1758,8 @@ static void cluster_split(int B, int cluster_size, int K, int NT, int &splits, i
 // mode: 0 gradients are stored, 1 norms only, 2 clipped sum (running sum in registers: at most 128 columns per tile)
 static TcPlan make_plan(int dtype, const ConvGeom &g, int mode) {
     static std::mutex mu;
-    static std::map<std::array<int, 13>, TcPlan> memo;
-    const std::array<int, 13> key = {dtype, g.H, g.W, g.Cin, g.Kout, g.R, g.S, g.stride, g.pad, g.B, mode, side_by_side() ? -launch_sms() : launch_sms(), (int)tl_batch_walk};
+    static std::map<std::array<int, 14>, TcPlan> memo;
+    const std::array<int, 14> key = {dtype, g.H, g.W, g.Cin, g.Kout, g.R, g.S, g.stride, g.pad, g.B, mode, side_by_side() ? -launch_sms() : launch_sms(), (int)tl_batch_walk, tl_beside};
     std::lock_guard<std::mutex> lock(mu);
     auto it = memo.find(key);
     if (it != memo.end()) return it->second;
@@ -1824,6 +1797,8 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
             const long long total_tiles = (long long)g.B * m_tiles * n_tiles;
             if (total_tiles > 0x7fffffffLL) continue;
             if (mode == 3 && !any_tiles && m_tiles * n_tiles > kMaxCluster) continue;
+            // (sizes that share no launch with others would be one more to wait for)
+            const double apart = mode == 3 && !any_tiles && tl_batch_walk > 0.0 && (m_tiles * n_tiles == 5 || m_tiles * n_tiles == 7) ? 1.1 : 1.0;
             const int y_slabs = (mode == 4) ? (a_is_x ? NT / slab_ch : a_slabs_tile) : 0;     // second (lo) copy of the dY slabs
             // per-CTA share of (example, tile) units: whole waves of tiles, or in clipped-sum mode an even share of the examples
             // (in a batch other layers fill the last wave)
@@ -1859,7 +1834,7 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
                     const int Kt = OHt * OWt;
                     if (Kt % krows || Kt > 256) continue;
                     const int stage_bytes = (slabs + y_slabs) * Kt * kRowBytes * copies;
-                    int stages = kSmemBudget / stage_bytes;
+                    int stages = smem_budget(mode) / stage_bytes;
                     if (stages < 2) continue;
                     if (stages > kMaxStages) stages = kMaxStages;
                     if (dtype == DP_F32) stages &= ~1;        // each split group has slots of its own (see there)
@@ -1872,7 +1847,7 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
                         stage_cost = std::max(stage_cost, 0.5 * (1000.0 + (a_loaded + b_loaded) * Kt * 2.5));
                     double mainloop = stage_cost * tw * th;
                     if (stages < 3) mainloop *= 1.15;
-                    const double cost = ((std::max(mainloop, epilogue) + 300.0) * waves + (mode == 3 ? 4000.0 : (mode == 4 ? 6000.0 : 0.0))) * sm_share;
+                    const double cost = ((std::max(mainloop, epilogue) + 300.0) * waves + (mode == 3 ? 4000.0 : (mode == 4 ? 6000.0 : 0.0))) * sm_share * apart;
                     if (cost < best_cost) {
                         best_cost = cost;
                         best.ok = true; best.a_is_x = a_is_x; best.a_ext = a_ext; best.b_ext = b_ext;
@@ -1896,13 +1871,13 @@ bool tc_eligible(int dtype, const ConvGeom &g0, int epilogue) {
     return epilogue != DP_EPI_CLIP_ACCUM || make_plan(dtype, pr.eff, 2).ok;
 }
 
-// The single-pass kernel's register split only adds up when the launch allocates kClipRegsLaunch registers a thread.
+// The single-pass kernel's register split only adds up when the launch allocates ClipRegs::kLaunch registers a thread.
 static bool clip1_registers_ok() {
     static int ok = -1;
     if (ok < 0) {
         cudaFuncAttributes attr;
-        ok = (cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<1>) == cudaSuccess && attr.numRegs == kClipRegsLaunch &&
-              cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<kTcLayers>) == cudaSuccess && attr.numRegs == kClipRegsLaunch) ? 1 : 0;
+        ok = (cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<1>) == cudaSuccess && attr.numRegs == ClipRegs<1>::kLaunch &&
+              cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<kTcLayers>) == cudaSuccess && attr.numRegs == ClipRegs<kTcLayers>::kLaunch) ? 1 : 0;
         if (!ok) (void)cudaGetLastError();
     }
     return ok == 1;
@@ -2132,7 +2107,7 @@ static void fill_common(TcParams &p, int dtype, const ConvGeom &g, int Ng, const
     p.stages = pl.stages; p.stage_bytes = pl.stage_bytes; p.a_bytes = pl.a_bytes;
     p.a_group = slab_group(dtype, g, pl, true); p.b_group = slab_group(dtype, g, pl, false);
     p.status = status;
-    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
+    p.wait_polls = wait_polls();
 }
 
 // Layers with few input channels: the unfolded copy of X in the call's scratch.
@@ -2383,7 +2358,7 @@ static GramPlan gram_plan(int dtype, const ConvGeom &g0) {
     gp.pack = (best == 64) ? 2 : 1;
     gp.m_tiles = (best + 127) / 128;
     gp.stage_bytes = gp.m_tiles * 128 * kRowBytes;      // a row tile always reads 128 rows, whatever the box holds
-    gp.stages = std::min(kMaxStages, kSmemBudget / gp.stage_bytes);
+    gp.stages = std::min(kMaxStages, smem_budget(3) / gp.stage_bytes);
     gp.smem = (size_t)gp.stages * gp.stage_bytes + 1024;
     gp.ok = true;
     return gp;
@@ -2413,7 +2388,7 @@ static dp_status fill_gram(int dtype, const void *X, const void *dY, const GramP
     p.rows = gp.rows; p.pack = gp.pack; p.m_tiles = gp.m_tiles; p.stages = gp.stages; p.stage_bytes = gp.stage_bytes;
     p.C_l = clipinfo.C_l; p.sqnorm = clipinfo.sqnorm; p.sq_stride = clipinfo.sq_stride; p.clip_out = clipinfo.clip_out;
     p.factor_out = factor_out; p.status = status;
-    p.wait_polls = g_wait_polls.load(std::memory_order_relaxed);
+    p.wait_polls = wait_polls();
     p.blocks = std::min((g.B + gp.pack - 1) / gp.pack, launch_sms());
     return DP_OK;
 }
@@ -2510,8 +2485,8 @@ int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias) {
 
 // The longest walk of a block: the GPU's share of all the layers' work in as many rounds of blocks as keep each near 30
 // microseconds (a block costs some 4 to start and end; several rounds even out what the estimates get wrong), at most four.
-double conv_batch_walk(const std::vector<ConvJob> &jobs) {
-    BatchPlanning planning(120000.0);
+double conv_batch_walk(const std::vector<ConvJob> &jobs, bool beside) {
+    BatchPlanning planning(120000.0, beside);
     double cycles = 0.0;
     for (const ConvJob &j : jobs) {
         const TcProblem pr = tc_problem(j.dtype, j.g);
@@ -2558,24 +2533,27 @@ typedef TableQueue<GramParams, 2, kTcLayers> GramQueue;
 // Cluster size of the launch a layer with `tiles` tiles an example joins: sizes that divide one another share one.
 static int launch_cluster(int tiles) { return tiles == 1 || tiles == 2 || tiles == 4 ? 4 : (tiles == 3 || tiles == 6 ? 6 : tiles); }
 
-bool conv_batch_clusters(const ConvJob &j, double walk) {
-    BatchPlanning planning(walk);
+int conv_cluster_stream(int cluster) { return cluster > 6 ? BatchStreams::kClusters : (cluster > 4 ? BatchStreams::kClusters6 : BatchStreams::kMain); }
+
+int conv_batch_cluster(const ConvJob &j, double walk, bool beside) {
+    BatchPlanning planning(walk, beside);
     TcPlan pl; ConvGeom g; bool s2d;
-    return j.kind == kConvClip1 && clip1_plan(j.dtype, j.g, tc_problem(j.dtype, j.g), pl, g, s2d) && launch_cluster(pl.m_tiles * pl.n_tiles) > 4;
+    return j.kind == kConvClip1 && clip1_plan(j.dtype, j.g, tc_problem(j.dtype, j.g), pl, g, s2d) ? launch_cluster(pl.m_tiles * pl.n_tiles) : 0;
 }
 
-dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *status, const BatchStreams &streams,
+dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool beside, int *status, const BatchStreams &streams,
                             const std::function<dp_status()> &join) {
     if (jobs.empty()) return join();
-    const cudaStream_t stream = streams.s[BatchStreams::kMain], clusters = streams.s[BatchStreams::kClusters], sums = streams.s[BatchStreams::kSums];
-    BatchPlanning planning(walk);
+    const cudaStream_t stream = streams.s[BatchStreams::kMain], sums = streams.s[BatchStreams::kSums];
+    auto cluster_stream = [&](int cluster) { return streams.s[conv_cluster_stream(cluster)]; };
+    BatchPlanning planning(walk, beside);
     dp_status rc = raise_shared_limits();
     if (rc != DP_OK) return rc;
     ConvQueue store[3], clip[kMaxCluster + 1];            // store: by element type; clip: by cluster size of the launch
     GramQueue gram;
     SsumQueue ssum;
     std::vector<SplitSeg> splits;
-    std::vector<FoldSeg> folds, folds_clusters, folds_sums;      // by the stream that leaves the partial sums
+    std::vector<FoldSeg> folds[BatchStreams::kCount];      // by the stream that leaves the partial sums
     for (const ConvJob &j : jobs) {
         const TcProblem pr = tc_problem(j.dtype, j.g);
         const ConvGeom &g = pr.eff;
@@ -2603,7 +2581,9 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
         } else if (j.kind == kConvClip1) {
             TcPlan pl; ConvGeom g1; bool s2d;
             if (!clip1_plan(j.dtype, j.g, pr, pl, g1, s2d)) return DP_ERR_UNSUPPORTED;
-            rc = prepare_input(j.dtype, j.X, j.g, pr, s2d, j.tc_workspace, launch_cluster(pl.m_tiles * pl.n_tiles) > 4 ? clusters : stream);
+            // (small clusters wait for the sums' stream anyway)
+            const int of = launch_cluster(pl.m_tiles * pl.n_tiles);
+            rc = prepare_input(j.dtype, j.X, j.g, pr, s2d, j.tc_workspace, of > 4 || !streams.gram_done ? cluster_stream(of) : sums);
             if (rc != DP_OK) return rc;
             ConvQueue::Job q;
             rc = fill_clip1(j.dtype, j.X, j.dY, j.g, pr, g1, pl, s2d, j.clip, j.acc_w, j.tc_workspace, status, q.e);
@@ -2613,7 +2593,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             p.cluster = cluster;
             q.blocks = (p.splits + sets - 1) / sets * cluster;
             q.smem = pl.smem; q.cost = p.per_split * pl.item_cycles;
-            if (p.splits > 1) (cluster > 4 ? folds_clusters : folds).push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+            if (p.splits > 1) folds[conv_cluster_stream(cluster)].push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
             clip[cluster].jobs.push_back(q);
         } else {
             const GramPlan gp = gram_plan(j.dtype, j.g);
@@ -2632,7 +2612,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
                 const TcParams &p = t.e.p;
                 t.blocks = (p.blocks + 3) / 4 * 4;        // joins the launch of the smallest clusters; blocks past the last have no work
                 t.smem = pl.smem; t.cost = p.per_split * pl.item_cycles;
-                if (p.splits > 1) folds.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+                if (p.splits > 1) folds[BatchStreams::kMain].push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
                 clip[4].jobs.push_back(t);
             } else {
                 const TcPlan pl = make_plan(j.dtype, g, 4);
@@ -2643,7 +2623,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
                 TcParams &p = t.e.p;
                 t.blocks = p.blocks = p.total_tiles;
                 t.smem = pl.smem; t.cost = p.per_split * pl.item_cycles;
-                if (p.splits > 1) folds_sums.push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+                if (p.splits > 1) folds[BatchStreams::kSums].push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
                 ssum.jobs.push_back(t);
             }
         }
@@ -2658,20 +2638,25 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
         });
         if (rc != DP_OK) return rc;
     }
-    rc = gram.launch([&](const TcTable<GramParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
-        conv_gram_norm_kernel<kTcLayers><<<(unsigned)blocks, 192, smem, stream>>>(tab);
-        DP_LAUNCH_CHECK("conv_gram_norm_kernel");
-        return DP_OK;
-    });
-    if (rc == DP_OK && streams.gram_done) {
-        DP_CUDA_TRY(cudaEventRecord(streams.gram_done, stream));
-        DP_CUDA_TRY(cudaStreamWaitEvent(sums, streams.gram_done, 0));
-    }
-    // larger clusters need all their SMs in one GPC and leave some idle: the other streams' launches fill those
-    for (int c = kMaxCluster; c >= 1 && rc == DP_OK; --c)
-        rc = clip[c].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) {
-            return launch_clip1_table<kTcLayers>(tab, c, blocks, smem, c > 4 ? clusters : stream);
+    // The Gram matrices first: two more launches wait for them.  Larger clusters need all their SMs in one GPC, free at the same
+    // time: behind smaller blocks they would be what the chunk ends with, so they come next, each size on a stream of its own.
+    auto clip_launch = [&](int c) -> dp_status {
+        return clip[c].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) {
+            return launch_clip1_table<kTcLayers>(tab, c, blocks, smem, cluster_stream(c));
         });
+    };
+    if (rc == DP_OK)
+        rc = gram.launch([&](const TcTable<GramParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
+            conv_gram_norm_kernel<kTcLayers><<<(unsigned)blocks, 192, smem, sums>>>(tab);
+            DP_LAUNCH_CHECK("conv_gram_norm_kernel");
+            return DP_OK;
+        });
+    for (int c = kMaxCluster; c > 4 && rc == DP_OK; --c) rc = clip_launch(c);
+    if (rc == DP_OK && streams.gram_done) {
+        DP_CUDA_TRY(cudaEventRecord(streams.gram_done, sums));
+        DP_CUDA_TRY(cudaStreamWaitEvent(stream, streams.gram_done, 0));
+    }
+    for (int c = 4; c >= 1 && rc == DP_OK; --c) rc = clip_launch(c);
     if (rc == DP_OK) rc = launch_scale_split(splits, sums);
     if (rc == DP_OK)
         rc = ssum.launch([&](const TcTable<TcParams, 3, kSsumLayers> &tab, int blocks, size_t smem) -> dp_status {
@@ -2680,9 +2665,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *
             return DP_OK;
         });
     // (each stream folds its own: behind the join the fold would be alone on the GPU)
-    if (rc == DP_OK) rc = launch_folds(folds_clusters, clusters);
-    if (rc == DP_OK) rc = launch_folds(folds_sums, sums);
-    if (rc == DP_OK) rc = launch_folds(folds, stream);
+    for (int i = BatchStreams::kCount - 1; i >= 0 && rc == DP_OK; --i) rc = launch_folds(folds[i], streams.s[i]);
     return rc == DP_OK ? join() : rc;
 }
 

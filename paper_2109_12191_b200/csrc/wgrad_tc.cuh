@@ -55,11 +55,13 @@ dp_status launch_conv_gram_norm(int dtype, const void *X, const void *dY, const 
                                 float *factor_out, int *status, cudaStream_t stream);
 
 // While one of these lives, this thread plans (and launches) for a batch of layer calls: every layer is tiled for least
-// SM time on the whole GPU and no CTA walks through more than `walk_cycles` of one layer.
+// SM time on the whole GPU and no CTA walks through more than `walk_cycles` of one layer.  beside: normalisation layers run
+// on the same SMs at the same time.
 struct BatchPlanning {
-    explicit BatchPlanning(double walk_cycles);
+    BatchPlanning(double walk_cycles, bool beside);
     ~BatchPlanning();
     double saved;
+    bool saved_beside;
 };
 
 // One convolution of a batch (tensor-core layers only) and how it is run there.
@@ -79,16 +81,18 @@ struct ConvJob {
 };
 // kConvSingle: no shared launch takes this layer.
 int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias);
-double conv_batch_walk(const std::vector<ConvJob> &jobs);
-bool conv_batch_clusters(const ConvJob &job, double walk);        // runs in a launch of large clusters, on kClusters
+double conv_batch_walk(const std::vector<ConvJob> &jobs, bool beside);
+int conv_batch_cluster(const ConvJob &job, double walk, bool beside);         // blocks per cluster of the launch it runs in, or 0
+// the stream of a launch of clusters of this size
+int conv_cluster_stream(int cluster);
 // Streams a batch spreads its independent launches over: s[0] is the caller's, the others are forked from it and joined
 // to it again (ForkedStreams).  All may be one and the same.
 struct BatchStreams {
-    enum { kMain = 0, kClusters, kSums, kAffine, kCount };
+    enum { kMain = 0, kClusters, kClusters6, kSums, kAffine, kSingles, kCount };
     cudaStream_t s[kCount];
     cudaEvent_t gram_done;       // null when all streams are one
 };
-dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, int *status, const BatchStreams &streams,
+dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool beside, int *status, const BatchStreams &streams,
                             const std::function<dp_status()> &join);
 
 // Test hook: the number of polls after which a bounded wait of the kernel gives up (0 makes every wait give up at once).

@@ -195,3 +195,43 @@ def test_only_the_first_lane_holds_the_batchs_scratch(kind):
     st.wgrad(largest, X, dY, lane=3)
     torch.cuda.synchronize()
     st.check()
+
+
+@pytest.mark.parametrize("dtype,sizes,Bn", [
+    # one pixel, one vector of channels; several channel blocks, the last one ragged; fewer pixels than a ring's stages hold
+    ("bf16", [(8, 1), (24, 7), (1032, 5), (2048, 3), (512, 9), (64, 20), (2056, 2)], 3),
+    ("f32", [(4, 1), (36, 6), (516, 5), (256, 4), (1024, 3)], 3),
+    ("bf16", [(64, 64)], 40),                                # more items than two for every block
+])
+def test_normalisation_layers_beside_convolutions(dtype, sizes, Bn):
+    """The form for many bytes of them: a last, large layer brings the batch there, and leaves the others in front of it."""
+    b = B()
+    large = synth.norm(64, 64 if Bn > 3 else 512 if dtype == "f32" else 720)
+    layers = [synth.conv(256, 256, 3, 1, 1, 14)] * 4 + [synth.norm(C, H) for C, H in sizes] + [large] * (7 if Bn > 3 else 1)
+    distinct = {}
+    for i, l in enumerate(layers):
+        if l not in distinct and l is not large:
+            inp = scaled_inputs(l, Bn, dtype, 975, i, spread=True)
+            distinct[l] = (inp, dev_inputs(inp, dtype))
+    if large not in distinct:
+        zeros = torch.zeros(large.x_shape(Bn), device="cuda", dtype=torch.bfloat16 if dtype == "bf16" else torch.float32)
+        distinct[large] = (None, (zeros, zeros))
+    data = [distinct[l][1] for l in layers]
+    batch = b.Batch([make_desc(l, Bn, dtype, 0, 1) for l in layers], [NORM] * len(layers))
+    sq = [torch.zeros((Bn, 2), device="cuda") for _ in layers]
+    for i, s in enumerate(sq):
+        batch.set(i, sqnorm=s, sqnorm_stride=2 if layers[i].kind == "norm" else 1)
+    ws = torch.full((batch.workspace_bytes,), 0xAB, dtype=torch.uint8, device="cuda")
+    b.check(b.dp_workspace_init(ws))
+    for _ in range(2):                                       # items are handed out anew
+        for s in sq:
+            s.fill_(float("nan"))
+        b.check(batch.run(data, 1.0, ws))
+        for l, s in zip(layers, sq):
+            inp = distinct[l][0]
+            if l.kind == "norm" and inp is not None:
+                dW, db = oracle_layer(l, inp)
+                np.testing.assert_allclose(s.cpu().numpy(), np.stack([oracle.sqnorm(dW), oracle.sqnorm(db)], 1), rtol=TOL_NORM, err_msg=str(l))
+            elif l.kind == "norm":
+                assert not bool(s.any())
+    b.check(b.dp_wgrad_check(ws))
