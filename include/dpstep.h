@@ -202,7 +202,8 @@ DP_API dp_status dp_per_example_wgrad_scaled(const dp_layer_desc *desc, const vo
                                              float *acc_w, float *acc_b, void *workspace, size_t workspace_bytes,
                                              void *cuda_stream);
 
-/* Bytes of device scratch dp_clip_accumulate needs (per-block partial norms and factors). */
+/* Bytes of device scratch for dp_clip_accumulate: per-block partial norms and factors, and for a single tensor of rows
+ * that can be read once (up to 196 608 floats) partial sums.  Without room for the latter such a call takes the general way. */
 DP_API size_t dp_clip_workspace_bytes(int B, int L, const long long *P_l /* host, [L] */);
 
 /* Norm, clip and accumulate over materialised per-example gradients
@@ -310,8 +311,8 @@ DP_API dp_status dp_clip_accumulate_micro(int B, int L, int micro, const float *
  * dp_clip_static_scratch_bytes() bytes (2 MiB) that every GPU loading the library holds until exit.
  * Arguments and results are those of dp_clip_accumulate without the workspace pair.
  *
- *   - Limit: problems whose dp_clip_workspace_bytes(B, L, P_l) exceeds the array are refused with
- *     DP_ERR_WORKSPACE (dp_last_cuda_error() says why); nothing is launched.
+ *   - Limit: problems whose partial norms and factors exceed the array (4 bytes for every 8192 parameters of a tensor and
+ *     example, and 8 for every tensor and example) are refused with DP_ERR_WORKSPACE (dp_last_cuda_error() says why); nothing is launched.
  *   - Every call looks up the array's device address (cudaGetSymbolAddress, with the caller's device current);
  *     the first look-up on a device loads the library image there, so make that first call outside any stream
  *     capture.  No call allocates or frees memory, and no address is kept across calls.

@@ -10,6 +10,7 @@
 // ten launches, each with a last wave of its own, and took 590 us.
 #include "common.cuh"
 #include "philox.cuh"
+#include "clip_rows.cuh"
 #include <math.h>
 #include <mutex>
 
@@ -565,12 +566,16 @@ static bool plan(int B, int L, const long long *P_l, ClipPlan &pl) {
     return true;
 }
 
+// One tensor whose rows fit the registers of a cluster goes through them in a single read (clip_rows.cu), where its norms
+// are to be computed and the workspace holds the clusters' sums behind the rest.
+static bool single_read(int B, int L, const long long *P_l) { return L == 1 && clip_rows_eligible(B, P_l[0]); }
+
 }  // namespace dp
 
 extern "C" size_t dp_clip_workspace_bytes(int B, int L, const long long *P_l) {
     dp::ClipPlan pl;
     if (B <= 0 || L <= 0 || !P_l || !dp::plan(B, L, P_l, pl)) return 0;
-    return pl.total;
+    return pl.total + (dp::single_read(B, L, P_l) ? dp::clip_rows_workspace_bytes(B, P_l[0]) : 0);
 }
 
 namespace dp {
@@ -712,6 +717,11 @@ static dp_status clip_accumulate_impl(int mode, int B, int L, const float *const
     if (!stage3_only && (!workspace || !aligned(workspace, 256) || workspace_bytes < pl.total)) return DP_ERR_WORKSPACE;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     char *ws = static_cast<char *>(workspace);
+    if (!stage3_only && !sqnorm && !var.noise && !var.groups && var.micro == 1 && single_read(B, L, P_l) &&
+        workspace_bytes >= pl.total + clip_rows_workspace_bytes(B, P_l[0])) {
+        const dp_status rc = launch_clip_rows(G[0], B, P_l[0], C, acc[0], norms_out, clip_out, ws + pl.total, stream);
+        if (rc != DP_ERR_UNSUPPORTED) return rc;
+    }
     ClipCall c = {};
     c.B = B; c.L = L; c.per_layer = mode == DP_CLIP_PER_LAYER;
     c.G = G; c.P_l = P_l; c.acc = acc; c.sq = sqnorm; c.C = C; c.norms_out = norms_out; c.clip_out = clip_out;
@@ -840,9 +850,9 @@ extern "C" dp_status dp_clip_accumulate_static(int mode, int B, int L, const flo
                                                const float *sqnorm, float C, float *const *acc, float *norms_out,
                                                float *clip_out, void *cuda_stream) {
     if (B <= 0 || L <= 0 || !P_l) return DP_ERR_INVALID_ARG;
-    const size_t need = dp_clip_workspace_bytes(B, L, P_l);
-    if (need == 0) return DP_ERR_INVALID_ARG;
-    if (need > dp::kStaticScratchBytes) {
+    dp::ClipPlan pl;
+    if (!dp::plan(B, L, P_l, pl)) return DP_ERR_INVALID_ARG;
+    if (pl.total > dp::kStaticScratchBytes) {
         dp::note_error("dp_clip_accumulate_static: this problem needs more scratch than the built-in 2 MiB array; "
                        "use dp_clip_accumulate with a caller-owned workspace");
         return DP_ERR_WORKSPACE;
