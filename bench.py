@@ -325,19 +325,19 @@ class FlatGrad:
         return 2 * self.P * 4
 
     def roofline(self, dom, totals, prof_steps, peaks):
-        """Per-example noise draws B*P normals per chunk and is bound by the issue of instructions: 46 of a thread per normal
+        """Per-example noise draws B*P normals per chunk and is bound by the issue of instructions: 40 of a thread per normal
         (a quarter of a ten-round Philox block, half a Box-Muller pair, the scaled add, the row's share of the norm pass;
-        counted by ncu: smsp__thread_inst_executed.sum = 12.92 G in the norm pass and 10.72 G in the scaled sum for 512 M
-        normals), so the ceiling is SMs x 128 lanes x SM clock / 46 normals per second."""
+        counted by ncu: 32 x smsp__inst_executed.sum = 2.80 G in the norm pass and 2.35 G in the scaled sum for 128 M
+        normals), so the ceiling is SMs x 128 lanes x SM clock / 40 normals per second."""
         if self.variant != "per_example_noise" or dom != 0:
             return None
         avg_ms_per_chunk = totals[0] / (prof_steps * self.G)
         props = self.torch.cuda.get_device_properties(self.torch.cuda.current_device())
         sms, ghz = props.multi_processor_count, peaks.get("sm_max_mhz", 1965.0) / 1e3
-        peak = sms * 128 * ghz * 1e9 / 46.0 / 1e9
+        peak = sms * 128 * ghz * 1e9 / 40.0 / 1e9
         got = self.B * self.P / (avg_ms_per_chunk / 1e3) / 1e9
         return {"bound": "alu", "achieved": round(got, 1), "peak": round(peak, 1),
-                "peak_source": f"derived: {sms} SMs x 128 lanes x {ghz:.3f} GHz / 46 thread instructions per normal (ncu count)",
+                "peak_source": f"derived: {sms} SMs x 128 lanes x {ghz:.3f} GHz / 40 thread instructions per normal (ncu count)",
                 "unit": "Gnormal/s", "frac": round(got / peak, 4)}
 
     def e2e_prepare(self):

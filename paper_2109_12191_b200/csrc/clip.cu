@@ -49,7 +49,7 @@ __device__ __forceinline__ int find_seg(const SegTable<N> &t, int blk) {
 
 // stage 1: partial[n][part_start[seg] + j] = sum of squares of G_seg[n, j*chunk .. (j+1)*chunk); up to three floats before
 // the first 16-byte boundary and after the last one are read alone
-template <int N>
+template <int AHEAD, int N>
 __device__ __forceinline__ void sqnorm_partial(const SegTable<N> &tab, int blk, int n, float *__restrict__ partial, long long parts_per_example) {
     __shared__ float scratch[32];
     const int seg = find_seg(tab, blk);
@@ -62,10 +62,17 @@ __device__ __forceinline__ void sqnorm_partial(const SegTable<N> &tab, int blk, 
     const float4 *row4 = reinterpret_cast<const float4 *>(row + head);
     const int n4 = (len - head) >> 2, tail = head + 4 * n4;
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 4
-    for (int i = threadIdx.x; i < n4; i += 256) {
-        const float4 v = __ldg(row4 + i);
-        a0 = fmaf(v.x, v.x, a0); a1 = fmaf(v.y, v.y, a1); a2 = fmaf(v.z, v.z, a2); a3 = fmaf(v.w, v.w, a3);
+    for (int i = threadIdx.x; i < n4; i += 256 * AHEAD) {                    // AHEAD loads in flight a thread
+        float4 v[AHEAD];
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i + 256 * u < n4) v[u] = __ldg(row4 + i + 256 * u);
+        }
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) {
+            a0 = fmaf(v[u].x, v[u].x, a0); a1 = fmaf(v[u].y, v[u].y, a1); a2 = fmaf(v[u].z, v[u].z, a2); a3 = fmaf(v[u].w, v[u].w, a3);
+        }
     }
     if ((int)threadIdx.x < head) a0 = fmaf(row[threadIdx.x], row[threadIdx.x], a0);
     if (tail + (int)threadIdx.x < len) a1 = fmaf(row[tail + threadIdx.x], row[tail + threadIdx.x], a1);
@@ -76,7 +83,7 @@ __device__ __forceinline__ void sqnorm_partial(const SegTable<N> &tab, int blk, 
 template <int N>
 __global__ void __launch_bounds__(256)
 sqnorm_partial_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example) {
-    sqnorm_partial(tab, blockIdx.x, blockIdx.y, partial, parts_per_example);
+    sqnorm_partial<4>(tab, blockIdx.x, blockIdx.y, partial, parts_per_example);
 }
 
 // stage 1 for micro-batch clipping: row j of the partials belongs to the MEAN of examples j*micro .. j*micro+micro-1
@@ -492,7 +499,7 @@ __device__ __forceinline__ void noised_rows(float4 &s, const float *g, const flo
 }
 
 template <int N>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256, 6)
 scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const float *__restrict__ factor, int B, int L,
                                int per_layer, int odd_only, const __grid_constant__ ExampleNoise nz) {
     __shared__ float f_sh[256];
@@ -519,17 +526,19 @@ scale_accumulate_noised_kernel(const __grid_constant__ SegTable<N> tab, const fl
 // Stage 1 with half of the per-example noise: the norm pass waits for memory and the noise for the issue slots, and a draw
 // does not depend on its example's factor.  So the even examples' draws are added here, acc[i] += sd * sum_n z_n(goff + i),
 // by blocks spread evenly among those of the norms (every (ratio + 1)-th), the odd examples' in stage 3 (8 M parameters, 32
-// examples: norms 152 us, then all of the draws with the scaled sum 363; this way 255 and 220).
+// examples: norms 152 us, then all of the draws with the scaled sum 363; this way 255 and 220;
+// with the pairs of a draw packed, six blocks an SM in both and eight loads in flight in the blocks of norms, whose few places an SM
+// are what the pass waits for, 227 and 196).
 template <int N>
 struct NoiseStarts { int first[N]; };                          // first noise block of each tensor, tiles of kAccCols parameters
 template <int N>
-__global__ void __launch_bounds__(256, 8)
+__global__ void __launch_bounds__(256, 6)
 sqnorm_noise_kernel(const __grid_constant__ SegTable<N> tab, float *__restrict__ partial, long long parts_per_example, int norm_blocks,
                     int B, int noise_blocks, int ratio, const __grid_constant__ NoiseStarts<N> starts, const __grid_constant__ ExampleNoise nz) {
     const int idx = blockIdx.x, turn = idx / (ratio + 1);
     if (turn >= noise_blocks || idx - turn * (ratio + 1) != ratio) {
         const int blk = idx - min(noise_blocks, turn), n = blk / norm_blocks;
-        sqnorm_partial(tab, blk - n * norm_blocks, n, partial, parts_per_example);
+        sqnorm_partial<8>(tab, blk - n * norm_blocks, n, partial, parts_per_example);
         return;
     }
     int lo = 0, hi = tab.nseg;

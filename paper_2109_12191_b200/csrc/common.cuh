@@ -74,6 +74,12 @@ __device__ __forceinline__ Float2 fma2(Float2 a, Float2 b, Float2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
+__device__ __forceinline__ Float2 mul2(Float2 a, Float2 b) {
+    Float2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ Float2 both2(float v) { return pack2(v, v); }
 __device__ __forceinline__ Float2 add2(Float2 a, Float2 b) {
     Float2 r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));

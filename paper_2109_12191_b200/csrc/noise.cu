@@ -8,9 +8,10 @@ namespace dp {
 
 // A thread block covers kNoiseTile parameters, i.e. kNoiseTile/4 Philox blocks from global index 4*(param_offset/4) on;
 // local index = global - param_offset.  VEC: param_offset % 4 == 0, so a Philox block is one float4.
-// What bounds the kernel is the issue rate (some 45 instructions a normal, of which a third Philox), not the 8 bytes a
+// What bounds the kernel is the issue rate (some 35 instructions a normal, of which a third Philox), not the 8 bytes a
 // parameter it moves: two blocks a thread halve the index arithmetic and give the ten-round chain a second one to
-// overlap with.  25.6 M parameters: 62 us with one block a thread and the library's logf / sincospif.
+// overlap with.  25.6 M parameters: 39 us; 42 with one pair of
+// words at a time, 62 with one block a thread and the library's logf / sincospif.
 constexpr int kNoiseTile = 2048;
 
 template <bool VEC>
