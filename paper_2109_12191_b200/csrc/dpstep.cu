@@ -148,6 +148,14 @@ dp_status check_layer(const dp_layer_desc *d, int epi, const LayerBuffers &io, f
     return DP_OK;
 }
 
+// Norms of a fused clip from the pixel Gram matrices, a block or two examples a block: least SM time where calls run side by
+// side.  A call that has the GPU to itself goes through the tiles on all SMs, unless there are very many of them over few pixels
+// (32 examples of 1 x 1 1024 -> 2048 on 7 x 7: 59 us the call, 68 by tiles; 8 of 3 x 3 512 -> 512 on 7 x 7: 47 and 39; 32 of 3 x 3
+// 256 -> 256 on 14 x 14: 50 and 41).
+static bool clip_norms_from_gram(int dtype, const ConvGeom &g) {
+    return tc_gram_norm(dtype, g) && (sm_target_set() || (g.K <= 64 && (long long)g.B * g.M * g.N >= 24000000));
+}
+
 dp_status run_layer(const dp_layer_desc *d, int epi, const LayerBuffers &io, float C_l, const WgradPlan &pl, char *header,
                     char *scratch, cudaStream_t st) {
     const void *X = io.X, *dY = io.dY;
@@ -205,22 +213,20 @@ dp_status run_layer(const dp_layer_desc *d, int epi, const LayerBuffers &io, flo
         }
         // per-layer clipping: norms of every example first, then the clipped sum with the factors known
         if (pl.use_tc) {
-            if (!d->has_bias && single_pass_enabled() && tc_clip_scaled_sum(d->dtype, g) && tc_gram_norm(d->dtype, g)) {
-                // small planes: norms and factors from the pixel Gram matrices, then the clipped sum as one product
+            const bool one_product = !d->has_bias && single_pass_enabled() && tc_clip_scaled_sum(d->dtype, g);
+            const bool by_tiles = one_product && tc_clip_scaled_tiles(d->dtype, g);      // enough pixels an example: scaled per example out of tensor memory
+            if (one_product && clip_norms_from_gram(d->dtype, g)) {
                 const TcInlineClip ic = {C_l, sqnorm, sqnorm_stride, clip_out};
                 rc = launch_conv_gram_norm(d->dtype, X, dY, g, ic, factor, status, st);
-                if (rc != DP_OK) return rc;
-                if (tc_clip_scaled_tiles(d->dtype, g))     // enough pixels an example: scaled per example out of tensor memory
-                    return launch_conv_scaled_tiles(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
-                return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
+            } else {
+                // the norm pass's last CTA folds the partial norms (bias slots included) into norms and factors
+                const TcPublish pub = {counters, pl.w_slots, groups == 2, sqnorm, sqnorm_stride, factor, C_l, clip_out};
+                rc = launch_conv_tc(d->dtype, DP_EPI_NORM_ONLY, X, dY, g, nullptr, partial, pl.slots, nullptr, nullptr, ws + pl.tc_off,
+                                    status, st, false, &pub);
             }
-            // the norm pass's last CTA folds the partial norms (bias slots included) into norms and factors
-            const TcPublish pub = {counters, pl.w_slots, groups == 2, sqnorm, sqnorm_stride, factor, C_l, clip_out};
-            rc = launch_conv_tc(d->dtype, DP_EPI_NORM_ONLY, X, dY, g, nullptr, partial, pl.slots, nullptr, nullptr, ws + pl.tc_off,
-                                status, st, false, &pub);
             if (rc != DP_OK) return rc;
-            if (!d->has_bias && single_pass_enabled() && tc_clip_scaled_sum(d->dtype, g))
-                return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
+            if (by_tiles) return launch_conv_scaled_tiles(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
+            if (one_product) return launch_conv_ssum(d->dtype, X, dY, g, factor, acc_w, ws + pl.tc_off, status, st);
             rc = launch_conv_tc(d->dtype, DP_EPI_CLIP_ACCUM, X, dY, g, nullptr, partial, pl.slots, factor, acc_w, ws + pl.tc_off,
                                 status, st, true);
             if (rc != DP_OK) return rc;

@@ -52,6 +52,7 @@ struct TcPlan {
     int stages, stage_bytes, a_bytes;
     size_t smem;
     double item_cycles;         // rough time of one (example, tile) item in its CTA
+    int split;                  // modes 0 / 1: blocks that share an item's pixel tiles (conv_wgrad_split_kernel), 1: one does them all
 };
 
 struct TcParams {
@@ -65,7 +66,7 @@ struct TcParams {
     int lo_offset;              // split tf32: byte offset of the lo copy inside a stage
     int mode;                   // 0 store + norm, 1 norm only, 2 clipped sum over a range of examples
     float *G_w;
-    float *partial;             // [B][slots], slot = (mt*n_tiles + nt)*4 + epilogue warp
+    float *partial;             // [B][slots], slot = (mt*n_tiles + nt)*4 + epilogue warp (split items: *split + block)
     int slots;
     int *status;
     uint32_t wait_polls;        // polls after which a wait gives up
@@ -302,11 +303,50 @@ struct OperandCopies {
     }
 };
 
+// The last block to finish: every example's partial squared norms, bias slots included, in slot order; publishes the squared norm(s)
+// and, for a clipped-sum pass that follows, the factors.
+__device__ __forceinline__ void publish_norms(const TcParams &p, int lane) {
+    // eight lanes per example (slot i goes to lane i % 8, the eight sums are added by a butterfly), four
+    // examples per warp and trip: the walk is a chain of L2 round trips, so many examples go side by side,
+    // with eight loads of each in flight (one by one, 144 slots an example held the launch up for 2 us)
+    const int groups = (int)(blockDim.x >> 3), group = (int)(threadIdx.x >> 3), sub = lane & 7;
+    for (int n0 = 0; n0 < p.B; n0 += groups) {     // uniform trip count: the shuffles below need whole warps
+        const int n = n0 + group;
+        double sw = 0.0, sb = 0.0;
+        if (n < p.B) {
+            const float *pn = p.partial + (long long)n * p.slots;
+            sw = slot_sum(pn, sub, p.w_slots);
+            sb = slot_sum(pn, p.w_slots + sub, p.fold_slots);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            sw += __shfl_xor_sync(0xffffffffu, sw, o);
+            sb += __shfl_xor_sync(0xffffffffu, sb, o);
+        }
+        if (n < p.B && sub == 0) {
+            if (p.separate) { p.sqnorm[n * p.sq_stride] = (float)sw; p.sqnorm[n * p.sq_stride + 1] = (float)sb; }
+            else p.sqnorm[n * p.sq_stride] = (float)(sw + sb);
+            if (p.factor_out) {                    // the clipped-sum pass that follows reads its factors here
+                const float fw = clip_factor(p.separate ? sw : sw + sb, p.C_l);
+                const float fb = p.separate ? clip_factor(sb, p.C_l) : fw;
+                p.factor_out[2 * n] = fw; p.factor_out[2 * n + 1] = fb;
+                if (p.clip_out) {
+                    if (p.separate) { p.clip_out[2 * n] = fw; p.clip_out[2 * n + 1] = fb; }
+                    else p.clip_out[n] = fw;
+                }
+            }
+        }
+    }
+}
+
 enum { kBf16 = 0, kTf32, kSplit };       // inputs of the tensor cores: bf16, tf32, or fp32 as hi + lo tf32
-template <int ARITH, bool CLIP, int N>
-__global__ void __launch_bounds__(ARITH == kSplit ? 480 : 224, 1)
+// NORM: norms only, read back by eight warps instead of four (7-10 too): where an example has few pixels the read-back of a tile, a
+// chain of loads from tensor memory and sums, is what the launch waits for.
+template <int ARITH, bool CLIP, int N, bool NORM = false>
+__global__ void __launch_bounds__(ARITH == kSplit ? 480 : (NORM ? 352 : 224), 1)
 conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     constexpr bool TF32 = ARITH != kBf16, SPLIT = ARITH == kSplit;
+    constexpr int READERS = NORM ? 8 : 4;
     const int entry = table_entry(tab.first, tab.n, blockIdx.x);
     const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
     const TcParams &p = tab.e[entry].p;
@@ -317,7 +357,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], ready_bar[kMaxStages], tmem_full[2], tmem_empty[2];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
-    __shared__ float4 xpose[4][256];        // per epilogue warp: a 32 x 32 block on its way out (put_rows)
+    __shared__ float4 xpose[NORM ? 1 : 4][NORM ? 1 : 256];      // per epilogue warp: a 32 x 32 block on its way out (put_rows)
 
     const int warp = uniform_warp(), lane = threadIdx.x & 31;
     uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -331,7 +371,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         for (int s = 0; s < p.stages; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 2); mbar_init(smem_u32(&empty_bar[s]), 1); mbar_init(smem_u32(&ready_bar[s]), 4);
         }
-        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tmem_full[b]), 1); mbar_init(smem_u32(&tmem_empty[b]), 4); }
+        for (int b = 0; b < 2; ++b) { mbar_init(smem_u32(&tmem_full[b]), 1); mbar_init(smem_u32(&tmem_empty[b]), READERS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), 512);
@@ -490,9 +530,9 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                 if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             }
         }
-    } else if (warp >= 2 && warp <= 5) {
-        // ------------------------------------------------------------ epilogue (4 warps, one TMEM lane quadrant each)
-        const int q = warp & 3;
+    } else if ((warp >= 2 && warp <= 5) || (NORM && warp >= 7)) {
+        // ------------------------------------------------------------ epilogue (a TMEM lane quadrant to each warp, or to two)
+        const int q = warp & 3, half = NORM && warp >= 7;
         const int row = q * 32 + lane;
         uint32_t full_phase = 0;     // bit b: parity to wait for on accumulator buffer b
         int buf = 0;
@@ -552,7 +592,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                         if (row_ok) {
 #pragma unroll
                             for (int i = 0; i < 32; ++i) { const float f = __uint_as_float(v[i]); sq4[i & 3] = fmaf(f, f, sq4[i & 3]); }
-                            if (p.mode == 0) {
+                            if (!NORM && p.mode == 0) {
                                 const int b_idx = nt * p.NT + cc;
                                 if (p.a_is_x) {      // row = column j of G, tile column = output channel k: lanes write consecutive j
                                     float *dst = Gn + (long long)b_idx * p.Ng + a_idx;
@@ -561,12 +601,12 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                                 }
                             }
                         }
-                        if (p.mode == 0 && !p.a_is_x) {
+                        if (!NORM && p.mode == 0 && !p.a_is_x) {
                             // row = output channel k, tile columns = 32 consecutive j: each lane holds one row
                             const int col0 = nt * p.NT + cc, rows_here = min(32, a_rows - q * 32);
                             float *dst = Gn + (long long)(mt * 128 + q * 32) * p.Ng + col0;
                             if (!p.n_pad_cols) {
-                                put_rows<kPutStream>(xpose[warp - 2], [&](int i) { return __uint_as_float(v[i]); }, lane, dst, p.Ng, rows_here);
+                                put_rows<kPutStream>(xpose[NORM ? 0 : warp - 2], [&](int i) { return __uint_as_float(v[i]); }, lane, dst, p.Ng, rows_here);
                             } else if (lane < rows_here) {           // rows of any length: element by element
 #pragma unroll
                                 for (int i = 0; i < 32; ++i)
@@ -576,7 +616,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                     };
                     // columns in pairs of 32 with both loads in flight before the wait.  The second load of a tile with
                     // an odd number of 32-column blocks reads columns of this accumulator buffer that nobody uses.
-                    for (int cc = 0; cc < n_cols; cc += 64) {
+                    for (int cc = 64 * half; cc < n_cols; cc += 64 * (READERS / 4)) {
                         uint32_t v0[32], v1[32];
                         tmem_ld32_issue(t_addr + (uint32_t)cc, v0);
                         tmem_ld32_issue(t_addr + (uint32_t)(cc + 32), v1);
@@ -588,7 +628,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                     __syncwarp();
                     if (lane == 0) mbar_arrive(smem_u32(&tmem_empty[buf]));
                     const float sq = warp_sum((sq4[0] + sq4[1]) + (sq4[2] + sq4[3]));
-                    if (lane == 0) p.partial[(long long)n * p.slots + (mt * p.n_tiles + nt) * 4 + q] = sq;
+                    if (lane == 0) p.partial[(long long)n * p.slots + (mt * p.n_tiles + nt) * READERS + half * 4 + q] = sq;
                 }
                 buf ^= 1;
             }
@@ -605,8 +645,8 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
                         auto value = [&](int i) { return run[CLIP ? c4 * 32 + i : 0]; };
                         if (!p.a_is_x && !p.n_pad_cols) {
                             float *dst = base + (long long)(mt * 128 + q * 32) * p.Ng + b_idx;
-                            if (add) put_rows<kPutAdd>(xpose[warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
-                            else put_rows<kPutPlain>(xpose[warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
+                            if (add) put_rows<kPutAdd>(xpose[NORM ? 0 : warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
+                            else put_rows<kPutPlain>(xpose[NORM ? 0 : warp - 2], value, lane, dst, p.Ng, min(32, a_rows - q * 32));
                         } else if (row_ok) {
                             put_values(value, base, add, p, a_idx, b_idx);
                         }
@@ -630,37 +670,7 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
         __syncthreads();
         if (last_cta) {
             __threadfence();
-            // eight lanes per example (slot i goes to lane i % 8, the eight sums are added by a butterfly), four
-            // examples per warp and trip: the walk is a chain of L2 round trips, so many examples go side by side,
-            // with eight loads of each in flight (one by one, 144 slots an example held the launch up for 2 us)
-            const int groups = (int)(blockDim.x >> 3), group = (int)(threadIdx.x >> 3), sub = lane & 7;
-            for (int n0 = 0; n0 < p.B; n0 += groups) {     // uniform trip count: the shuffles below need whole warps
-                const int n = n0 + group;
-                double sw = 0.0, sb = 0.0;
-                if (n < p.B) {
-                    const float *pn = p.partial + (long long)n * p.slots;
-                    sw = slot_sum(pn, sub, p.w_slots);
-                    sb = slot_sum(pn, p.w_slots + sub, p.fold_slots);
-                }
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) {
-                    sw += __shfl_xor_sync(0xffffffffu, sw, o);
-                    sb += __shfl_xor_sync(0xffffffffu, sb, o);
-                }
-                if (n < p.B && sub == 0) {
-                    if (p.separate) { p.sqnorm[n * p.sq_stride] = (float)sw; p.sqnorm[n * p.sq_stride + 1] = (float)sb; }
-                    else p.sqnorm[n * p.sq_stride] = (float)(sw + sb);
-                    if (p.factor_out) {                    // the clipped-sum pass that follows reads its factors here
-                        const float fw = clip_factor(p.separate ? sw : sw + sb, p.C_l);
-                        const float fb = p.separate ? clip_factor(sb, p.C_l) : fw;
-                        p.factor_out[2 * n] = fw; p.factor_out[2 * n + 1] = fb;
-                        if (p.clip_out) {
-                            if (p.separate) { p.clip_out[2 * n] = fw; p.clip_out[2 * n + 1] = fb; }
-                            else p.clip_out[n] = fw;
-                        }
-                    }
-                }
-            }
+            publish_norms(p, lane);
         }
         __syncthreads();
     }
@@ -729,6 +739,192 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     }
     *abort_flag = 1;
     return false;
+}
+
+// ----------------------------------------------------------------------------- pixels of an item shared by a cluster (bf16)
+// Few examples of a layer with few tiles leave most SMs without an item, and a large plane keeps the others busy for long.  Here
+// the blocks of a cluster share the pixel tiles of one (example, tile) item.  Their accumulators meet through shared memory:
+// every block lays its tile out there (the stages are free by then), each takes an equal share of the gradient's rows (or of its
+// columns, where the tile's rows are input columns) and adds that of all blocks in their order, squares and stores it.  What it
+// costs is the tile's way through shared memory, some 2 us.  4 examples of 1 x 1 64 -> 64 on 50 x 50, stored: 14.6 us the call,
+// 10.3 here; norms of 32 of the 7 x 7 stem on 224 x 224: 44 us, 35 on twice the SMs (its overlapping rows come from the L2 at
+// 9 TB/s then, which bounds it).
+// Roles until the accumulators are done: warp 0 / 6 TMA, warp 1 MMA, warps 2-5 read tensor memory; then all warps add up.
+constexpr int kMaxSplit = 8, kSplitPad = 4;                 // floats between rows of a tile in shared memory: no bank conflicts
+__global__ void __launch_bounds__(224, 1)
+conv_wgrad_split_kernel(const __grid_constant__ TcTable<TcParams, 2, 1> tab) {
+    const CUtensorMap &tmX = tab.e[0].map[0], &tmY = tab.e[0].map[1];
+    const TcParams &p = tab.e[0].p;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], done_bar;
+    __shared__ uint32_t tmem_base_slot;
+    __shared__ int abort_flag, last_cta;
+    __shared__ float warp_sq[7];
+
+    const int warp = uniform_warp(), lane = threadIdx.x & 31;
+    uint8_t *tiles = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const uint32_t tiles_u32 = smem_u32(tiles);
+    const int rank = (int)cluster_rank(), split = p.splits;
+    const Item it = decode_item(p, (int)blockIdx.x / split);
+    const int mt = it.mt, nt = it.nt, n = it.n_lo;
+    const int kt0 = (int)((long long)p.k_tiles * rank / split), kt1 = (int)((long long)p.k_tiles * (rank + 1) / split);
+
+    if (threadIdx.x == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmX)) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmY)) : "memory");
+        abort_flag = 0;
+        for (int s = 0; s < p.stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 2); mbar_init(smem_u32(&empty_bar[s]), 1); }
+        mbar_init(smem_u32(&done_bar), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), 256);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_base_slot;
+    volatile int *abort_p = &abort_flag;
+
+    const int slab_bytes = p.Kt * kRowBytes;
+    const int a_slabs = min(128 / p.slab_ch, p.a_ext / p.slab_ch - mt * (128 / p.slab_ch));
+    const int b_slabs = min(p.NT / p.slab_ch, p.b_ext / p.slab_ch - nt * (p.NT / p.slab_ch));
+    const int a_rows = min(128, p.a_ext - mt * 128), n_cols = b_slabs * p.slab_ch;
+    // the tile in shared memory: lines that are contiguous in the gradient, rows of it or (input columns as rows) its columns
+    float *tile = reinterpret_cast<float *>(tiles);
+    const int lines = p.a_is_x ? n_cols : a_rows, width = p.a_is_x ? 128 : n_cols, pitch = width + kSplitPad;
+
+    if (warp == 0 || warp == 6) {
+        const bool leader = elect_one(), is_a = warp == 0, is_x = is_a == (p.a_is_x != 0);
+        const OperandCopies copies(p, is_x, is_a ? mt * (128 / p.slab_ch) : nt * (p.NT / p.slab_ch), is_a ? a_slabs : b_slabs,
+                                   is_a ? p.a_group : p.b_group, slab_bytes, lane);
+        const CUtensorMap *map = is_x ? &tmX : &tmY;
+        const uint32_t dst = tiles_u32 + (is_a ? 0u : (uint32_t)p.a_bytes), tx_bytes = (uint32_t)copies.count * copies.bytes;
+        int stage = 0; uint32_t phase = 0;
+        int tw = kt0 % p.tiles_w, ow0 = tw * p.OWt, oh0 = kt0 / p.tiles_w * p.OHt;
+        for (int kt = kt0; kt < kt1; ++kt) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_p, p.wait_polls))) break;
+            if (leader) mbar_expect_tx(smem_u32(&full_bar[stage]), tx_bytes);
+            __syncwarp();
+            copies.issue(leader, map, dst + stage * p.stage_bytes, smem_u32(&full_bar[stage]), ow0, oh0, n);
+            if (++tw == p.tiles_w) { tw = 0; ow0 = 0; oh0 += p.OHt; } else { ow0 += p.OWt; }
+            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+        }
+    } else if (warp == 1) {
+        const bool leader = elect_one();
+        const uint64_t desc_base = operand_desc_base<false>((uint32_t)slab_bytes);
+        const uint32_t desc_lo = (uint32_t)desc_base, desc_hi32 = (uint32_t)(desc_base >> 32);
+        const int ksteps = p.Kt / p.krows;
+        constexpr uint32_t kadvance = (uint32_t)(16 * kRowBytes) >> 4;
+        const uint32_t idesc = instr_desc(n_cols, 1u);
+        int stage = 0; uint32_t phase = 0, accumulate = 0;
+        bool live = true;
+        for (int kt = kt0; kt < kt1; ++kt) {
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full_bar[stage]), phase, abort_p, p.wait_polls))) { live = false; break; }
+            tc_fence_after();
+            const uint32_t a_src = tiles_u32 + stage * p.stage_bytes;
+            uint32_t ad = desc_lo | ((a_src & 0x3FFFFu) >> 4), bd = desc_lo | (((a_src + p.a_bytes) & 0x3FFFFu) >> 4);
+            if (leader) {
+#pragma unroll 4
+                for (int ks = 0; ks < ksteps; ++ks) {
+                    umma<false>(tmem_base, ad, bd, desc_hi32, idesc, accumulate);
+                    accumulate = 1;
+                    ad += kadvance; bd += kadvance;
+                }
+                umma_commit(smem_u32(&empty_bar[stage]));
+            }
+            accumulate = 1;
+            __syncwarp();
+            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+        }
+        if (live && leader) umma_commit(smem_u32(&done_bar));
+        __syncwarp();
+    } else {
+        const int q = warp & 3, row = q * 32 + lane;
+        // (the last MMA has read its stage: nothing else is left in the stages, whose place the tile takes)
+        if (__all_sync(0xffffffffu, mbar_wait(smem_u32(&done_bar), 0u, abort_p, p.wait_polls))) {
+            tc_fence_after();
+            const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16);
+            for (int cc = 0; cc < n_cols; cc += 64) {                                    // (a multiple of 64)
+                uint32_t v0[32], v1[32];
+                tmem_ld32_issue(t_addr + (uint32_t)cc, v0);
+                tmem_ld32_issue(t_addr + (uint32_t)(cc + 32), v1);
+                tmem_ld_wait32(v0); tmem_ld_wait32(v1);
+                if (p.a_is_x) {
+#pragma unroll
+                    for (int i = 0; i < 32; ++i) { tile[(cc + i) * pitch + row] = __uint_as_float(v0[i]); tile[(cc + 32 + i) * pitch + row] = __uint_as_float(v1[i]); }
+                } else if (row < a_rows) {
+                    float4 *dst = reinterpret_cast<float4 *>(tile + row * pitch + cc);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        dst[i] = make_float4(__uint_as_float(v0[4 * i]), __uint_as_float(v0[4 * i + 1]), __uint_as_float(v0[4 * i + 2]), __uint_as_float(v0[4 * i + 3]));
+                        dst[8 + i] = make_float4(__uint_as_float(v1[4 * i]), __uint_as_float(v1[4 * i + 1]), __uint_as_float(v1[4 * i + 2]), __uint_as_float(v1[4 * i + 3]));
+                    }
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();                                   // every block's tile is in place
+
+    // this block's share of the lines, of all blocks in their order; a thread takes four neighbouring values of a line
+    const int line0 = lines * rank / split, line1 = lines * (rank + 1) / split, quads = width / 4;
+    uint32_t peer[kMaxSplit];
+#pragma unroll
+    for (int r = 0; r < kMaxSplit; ++r) peer[r] = map_to_cta(tiles_u32, (uint32_t)min(r, split - 1));
+    float sq4[4] = {0.f, 0.f, 0.f, 0.f};
+    float *Gn = p.G_w + (long long)n * p.Kout * p.Ng;
+    for (int e = threadIdx.x; e < (line1 - line0) * quads; e += 224) {
+        const int line = line0 + e / quads, x = (e % quads) * 4;
+        const uint32_t off = (uint32_t)(line * pitch + x) * 4u;
+        float4 v[kMaxSplit];
+#pragma unroll
+        for (int r = 0; r < kMaxSplit; ++r)
+            if (r < split)
+                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[r].x), "=f"(v[r].y), "=f"(v[r].z), "=f"(v[r].w) : "r"(peer[r] + off));
+        float a[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+#pragma unroll
+        for (int r = 1; r < kMaxSplit; ++r)
+            if (r < split) { a[0] += v[r].x; a[1] += v[r].y; a[2] += v[r].z; a[3] += v[r].w; }
+        // where the four values lie in the gradient; those that stand for nothing count for nothing
+        const long long row0 = p.a_is_x ? nt * p.NT + line : mt * 128 + line;
+        const int col0 = (p.a_is_x ? mt * 128 : nt * p.NT) + x;
+        const bool whole = !p.s2d_st && col0 + 4 <= p.Ng && (!p.a_is_x || x + 4 <= a_rows);
+        if (whole && !p.n_pad_cols) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) sq4[i] = fmaf(a[i], a[i], sq4[i]);
+            if (p.mode == 0) __stcs(reinterpret_cast<float4 *>(Gn + row0 * p.Ng + col0), make_float4(a[0], a[1], a[2], a[3]));
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                int col = col0 + i;
+                if (p.a_is_x && x + i >= a_rows) col = -1;
+                else if (p.s2d_st) col = s2d_column(p, col);
+                if (col < 0 || col >= p.Ng) continue;
+                sq4[i] = fmaf(a[i], a[i], sq4[i]);
+                if (p.mode == 0) Gn[row0 * p.Ng + col] = a[i];
+            }
+        }
+    }
+    const float sq = warp_sum((sq4[0] + sq4[1]) + (sq4[2] + sq4[3]));
+    if (lane == 0) warp_sq[warp] = sq;
+    __syncthreads();
+    cluster_sync_all();                                   // nobody leaves while a peer may still read its tile
+    if (threadIdx.x == 0) {
+        p.partial[(long long)n * p.slots + (mt * p.n_tiles + nt) * split + rank] =
+            ((warp_sq[0] + warp_sq[1]) + (warp_sq[2] + warp_sq[3])) + ((warp_sq[4] + warp_sq[5]) + warp_sq[6]);
+        __threadfence();
+        last_cta = atomicAdd(&p.counters[0], 1) == p.blocks - 1;
+        if (last_cta) p.counters[0] = 0;
+    }
+    __syncthreads();
+    if (last_cta) { __threadfence(); publish_norms(p, lane); }
+    __syncthreads();
+    if (abort_flag) {
+        if (threadIdx.x == 0) { *p.status = DP_ERR_TIMEOUT; __threadfence(); }
+        __nanosleep(200000);
+        __syncthreads();
+    }
+    if (warp == 1) { tc_fence_after(); tmem_dealloc(tmem_base, 256); }
 }
 
 // sum of non-negative floats with its rounding errors; past the range of float it is infinite, as in plain floats
@@ -1772,6 +1968,17 @@ static TcPlan make_plan(int dtype, const ConvGeom &g, int mode) {
 // work items are (example range, tile) pairs, so the wave count no longer depends on the batch size
 // mode 3 plans the single-pass clipped sum: all tiles of an example in one cluster (at most kMaxCluster of them), the
 // clusters share the batch, and what is minimised is SM time (clusters x CTAs x time), not the time of one launch
+// Rough time of a launch whose items are shared by `by` blocks each: `main` is a block's main loop; loads start from nothing
+// (1500 cycles), the tile goes out of tensor memory (8 a column) and through the cluster (every thread's chain of reads), launch
+// and two cluster barriers take 2500.
+static int max_active_clusters(int cluster_size);
+static double split_cycles(int mode, int items, int by, int NT, double main) {
+    const double places = std::min((double)max_active_clusters(by) * by, (double)launch_sms());
+    const double waves = std::ceil((double)items * by / (std::floor(places / by) * by));
+    return (main + 1500.0 + 8.0 * NT + NT * (5.7 / by + 3.6) + (mode == 0 ? 128.0 * NT * 4.0 / by / 16.0 : 0.0) + 2500.0) * waves;
+}
+static size_t split_smem(int a_is_x, int NT) { return (a_is_x ? NT * (128 + kSplitPad) : 128 * (NT + kSplitPad)) * sizeof(float) + 1024; }
+
 static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
     const int max_nt = (mode == 2) ? 128 : 256;
     const bool rows_are_inputs = mode == 6 || mode >= 8; // modes 6, 8, 9: modes 3, 0, 1 with the rows of D fixed to the input columns
@@ -1786,7 +1993,10 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
     const int sms = launch_sms();
     const int a_slabs_tile = 128 / slab_ch;
     const int copies = (dtype == DP_F32) ? 2 : 1;       // split tf32 keeps a hi and a lo copy of every stage
-    double best_cost = 1e300;
+    double best_cost = 1e300, best_main = 0.0, best_epilogue = 0.0, best_waves = 0.0;
+    TcPlan shared; shared.ok = false;                    // the best form that shares an item's pixels among a cluster
+    double shared_cost = 1e300;
+    const bool may_split = dtype == DP_BF16 && mode <= 1 && !side_by_side();
     for (int a_is_x = rows_are_inputs ? 1 : 0; a_is_x < 2; ++a_is_x) {
         const int a_ext = a_is_x ? g.N : g.M, b_ext = a_is_x ? g.M : g.N;
         for (int NT = slab_ch; NT <= max_nt; NT += slab_ch) {
@@ -1847,21 +2057,37 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
                         stage_cost = std::max(stage_cost, 0.5 * (1000.0 + (a_loaded + b_loaded) * Kt * 2.5));
                     double mainloop = stage_cost * tw * th;
                     if (stages < 3) mainloop *= 1.15;
+                    auto take = [&](TcPlan &t) {
+                        t.ok = true; t.a_is_x = a_is_x; t.a_ext = a_ext; t.b_ext = b_ext;
+                        t.m_tiles = m_tiles; t.n_tiles = n_tiles; t.NT = NT;
+                        t.OWt = OWt; t.OHt = OHt; t.tiles_w = tw; t.tiles_h = th; t.Kt = Kt;
+                        t.k_tiles = tw * th; t.stages = stages; t.stage_bytes = stage_bytes;
+                        t.a_bytes = a_slabs_tile * Kt * kRowBytes;
+                        t.smem = (size_t)stages * stage_bytes + 1024;
+                        t.item_cycles = std::max(mainloop, epilogue) + 300.0;
+                        t.split = 1;
+                    };
+                    for (int by = 2; may_split && by <= std::min(kMaxSplit, tw * th); ++by) {
+                        const double c = split_cycles(mode, g.B * m_tiles * n_tiles, by, NT, stage_cost * ((tw * th + by - 1) / by) * (stages < 3 ? 1.15 : 1.0));
+                        if (c >= shared_cost) continue;
+                        shared_cost = c;
+                        take(shared);
+                        shared.split = by;
+                        shared.smem = std::max(shared.smem, split_smem(a_is_x, NT));
+                    }
                     const double cost = ((std::max(mainloop, epilogue) + 300.0) * waves + (mode == 3 ? 4000.0 : (mode == 4 ? 6000.0 : 0.0))) * sm_share * apart;
                     if (cost < best_cost) {
-                        best_cost = cost;
-                        best.ok = true; best.a_is_x = a_is_x; best.a_ext = a_ext; best.b_ext = b_ext;
-                        best.m_tiles = m_tiles; best.n_tiles = n_tiles; best.NT = NT;
-                        best.OWt = OWt; best.OHt = OHt; best.tiles_w = tw; best.tiles_h = th; best.Kt = Kt;
-                        best.k_tiles = tw * th; best.stages = stages; best.stage_bytes = stage_bytes;
-                        best.a_bytes = a_slabs_tile * Kt * kRowBytes;
-                        best.smem = (size_t)stages * stage_bytes + 1024;
-                        best.item_cycles = std::max(mainloop, epilogue) + 300.0;
+                        best_cost = cost; best_main = mainloop; best_epilogue = epilogue; best_waves = waves;
+                        take(best);
                     }
                 }
             }
         }
     }
+    // (a block's first loads and its last epilogue overlap with nothing; what the memory bounds, two thirds of its rate, stays as it is)
+    const double memory = 2.0 * g.B * ((double)g.H * g.W * g.Cin + (double)g.K * g.Kout) / 2250.0;
+    if (shared.ok && best.ok && std::max(shared_cost, memory) < 0.85 * ((std::max(best_main, best_epilogue) + 300.0) * best_waves + std::min(best_main, best_epilogue) + 1500.0))
+        return shared;
     return best;
 }
 
@@ -1964,11 +2190,17 @@ static void clip_split(const ConvGeom &g, const TcPlan &pl, int &splits, int &pe
     splits = (g.B + per_split - 1) / per_split;
 }
 
+// Eight warps read the tiles of a norm pass back where an example has few pixels (32 examples of 3 x 3 512 -> 512 on 7 x 7: 31 us,
+// 25; on 14 x 14 the same as four, on 50 x 50 3 us of 47 slower), in a call on its own: a batch's launches hold layers that store, too.
+static bool norm_readers(int dtype, int epilogue, const TcPlan &pl) {
+    return dtype == DP_BF16 && epilogue != DP_EPI_STORE_NORM && tl_batch_walk == 0.0 && pl.k_tiles * pl.Kt <= 128;
+}
+
 int tc_norm_slots(int dtype, const ConvGeom &g0, int epilogue) {
     const TcProblem pr = tc_problem(dtype, g0);
     if (!pr.ok) return 0;
     const TcPlan pl = store_form(dtype, g0, pr, epilogue).pl;
-    return pl.ok ? pl.m_tiles * pl.n_tiles * 4 : 0;
+    return pl.ok ? pl.m_tiles * pl.n_tiles * (pl.split > 1 ? pl.split : (norm_readers(dtype, epilogue, pl) ? 8 : 4)) : 0;
 }
 
 static size_t unfold_bytes(int dtype, const ConvGeom &g0, const TcProblem &pr) {
@@ -2079,7 +2311,7 @@ static dp_status raise_shared_limits() {
             allow_shared(conv_wgrad_tc_kernel<kBf16, false, kTcLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kTcLayers>),
             allow_shared(conv_wgrad_tc_kernel<kTf32, false, 1>), allow_shared(conv_wgrad_tc_kernel<kTf32, true, 1>),
             allow_shared(conv_wgrad_tc_kernel<kTf32, false, kTcLayers>),
-            allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
+            allow_shared(conv_wgrad_split_kernel), allow_shared(conv_wgrad_tc_kernel<kBf16, false, 1, true>), allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
             allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>),
             allow_shared(conv_gram_norm_kernel<1>), allow_shared(conv_gram_norm_kernel<kTcLayers>)};
         for (cudaError_t e : all)
@@ -2215,10 +2447,25 @@ dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY,
     rc = fill_conv_tc(dtype, epilogue, X, dY, g0, pr, form.g, pl, form.s2d, G_w, partial, slots, factor, acc_w, tc_workspace, status, publish, tab.e[0]);
     if (rc != DP_OK) return rc;
     TcParams &p = tab.e[0].p;
+    if (!clip && pl.split > 1) {
+        p.splits = pl.split;
+        p.blocks = p.total_tiles * pl.split;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)p.blocks); cfg.blockDim = dim3(224); cfg.dynamicSmemBytes = pl.smem; cfg.stream = stream;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)pl.split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.attrs = at; cfg.numAttrs = 1;
+        const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_split_kernel, tab);
+        if (le != cudaSuccess) return cuda_fail(le, "conv_wgrad_split_kernel");
+        DP_LAUNCH_CHECK("conv_wgrad_split_kernel");
+        return DP_OK;
+    }
     p.blocks = std::min(p.total_tiles, sm_target());
     const unsigned grid = (unsigned)p.blocks;
     if (dtype == DP_BF16) {
         if (clip) conv_wgrad_tc_kernel<kBf16, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        else if (norm_readers(dtype, epilogue, pl)) conv_wgrad_tc_kernel<kBf16, false, 1, true><<<grid, 352, pl.smem, stream>>>(tab);
         else conv_wgrad_tc_kernel<kBf16, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
     } else if (dtype == DP_TF32) {
         if (clip) conv_wgrad_tc_kernel<kTf32, true, 1><<<grid, 224, pl.smem, stream>>>(tab);

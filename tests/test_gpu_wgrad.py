@@ -387,3 +387,25 @@ def test_fused_clip_rerun_is_bit_identical(case, target):
     np.testing.assert_array_equal(one["acc_w"], two["acc_w"])
     np.testing.assert_array_equal(one["sq"], two["sq"])
     np.testing.assert_array_equal(one["clip"], two["clip"])
+
+
+@pytest.mark.parametrize("layer,Bn", [
+    # pixel tiles shared by a cluster: one tile of few rows, rows of input columns, ragged planes, a strided stem, more blocks than tiles
+    (synth.conv(64, 64, 1, 1, 0, 50), 1), (synth.conv(128, 64, 3, 1, 1, 23), 1), (synth.conv(64, 192, 3, 2, 1, 31), 2),
+    (synth.conv(64, 256, 1, 1, 0, 37), 3), (synth.conv(192, 64, 1, 2, 0, 41), 2), (synth.conv(3, 64, 7, 2, 3, 96), 2),
+    (synth.conv(3, 128, 5, 2, 2, 61), 1),
+    # tiles of few pixels read back by eight warps: an odd number of column halves, one example
+    (synth.conv(64, 320, 3, 1, 1, 7), 1), (synth.conv(448, 192, 1, 1, 0, 9), 5), (synth.conv(512, 512, 3, 1, 1, 5), 9),
+])
+@pytest.mark.parametrize("epi", [STORE, NORM, CLIP])
+def test_single_calls_of_few_items_or_few_pixels(layer, Bn, epi):
+    inp = scaled_inputs(layer, Bn, "bf16", 981, Bn, spread=True)
+    dW, _ = oracle_layer(layer, inp)
+    sq = oracle.sqnorm(dW)
+    C_l = float(np.sqrt(np.median(sq)))
+    out = gpu_layer(layer, inp, "bf16", epi, C_l=C_l)
+    np.testing.assert_allclose(out["sq"][:, 0], sq, rtol=TOL_NORM)
+    if epi == STORE:
+        assert rel_l2(out["G_w"], dW) <= TOL_FMA
+    if epi == CLIP:
+        assert rel_l2(out["acc_w"], np.einsum("n,np->p", oracle.clip_factor(sq, C_l), dW)) <= TOL_FMA
