@@ -94,6 +94,7 @@ struct TcParams {
 // A launch serves up to N layers: the table of their tensor maps and parameters travels as a kernel parameter, and every
 // block finds its layer by its index (first[] ascending).  N = 1 for a call on its own.
 constexpr int kTcLayers = 54, kSsumLayers = 44;      // layers per grouped launch: a table stays below the 32 KB a launch may carry
+constexpr int kFewLayers = 4;                        // small models: a table of 2 KB instead of 27, all of which every launch carries
 template <typename P, int MAPS>
 struct alignas(64) TcEntry { CUtensorMap map[MAPS]; P p; };
 template <typename P, int MAPS, int N>
@@ -2311,6 +2312,8 @@ static dp_status raise_shared_limits() {
             allow_shared(conv_wgrad_tc_kernel<kBf16, false, kTcLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kTcLayers>),
             allow_shared(conv_wgrad_tc_kernel<kTf32, false, 1>), allow_shared(conv_wgrad_tc_kernel<kTf32, true, 1>),
             allow_shared(conv_wgrad_tc_kernel<kTf32, false, kTcLayers>),
+            allow_shared(conv_wgrad_tc_kernel<kBf16, false, kFewLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kFewLayers>),
+            allow_shared(conv_wgrad_tc_kernel<kTf32, false, kFewLayers>),
             allow_shared(conv_wgrad_split_kernel), allow_shared(conv_wgrad_tc_kernel<kBf16, false, 1, true>), allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
             allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>),
             allow_shared(conv_gram_norm_kernel<1>), allow_shared(conv_gram_norm_kernel<kTcLayers>)};
@@ -2749,12 +2752,12 @@ double conv_batch_walk(const std::vector<ConvJob> &jobs, bool beside) {
     return std::max(8000.0, std::min(120000.0, std::ceil(walk / 1000.0) * 1000.0));
 }
 
-template <typename P, int MAPS, int N>
+template <typename P, int MAPS, int MOST>
 struct TableQueue {
     // jobs of one kernel: filled entries with the blocks they take, launched longest blocks first, N layers at a time
     struct Job { TcEntry<P, MAPS> e; int blocks; size_t smem; double cost; };
     std::vector<Job> jobs;
-    template <typename F>
+    template <int N = MOST, typename F>
     dp_status launch(F &&go) {
         std::stable_sort(jobs.begin(), jobs.end(), [](const Job &a, const Job &b) { return a.cost > b.cost; });
         for (size_t i = 0; i < jobs.size();) {
@@ -2876,13 +2879,15 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
         }
     }
     for (int dtype = 0; dtype < 3; ++dtype) {
-        rc = store[dtype].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
-            if (dtype == DP_BF16) conv_wgrad_tc_kernel<kBf16, false, kTcLayers><<<(unsigned)blocks, 224, smem, stream>>>(tab);
-            else if (dtype == DP_TF32) conv_wgrad_tc_kernel<kTf32, false, kTcLayers><<<(unsigned)blocks, 224, smem, stream>>>(tab);
-            else conv_wgrad_tc_kernel<kSplit, false, kTcLayers><<<(unsigned)blocks, 480, smem, stream>>>(tab);
+        auto go = [&](const auto &tab, int blocks, size_t smem) -> dp_status {
+            constexpr int N = std::extent<decltype(tab.first)>::value;
+            if (dtype == DP_BF16) conv_wgrad_tc_kernel<kBf16, false, N><<<(unsigned)blocks, 224, smem, stream>>>(tab);
+            else if (dtype == DP_TF32) conv_wgrad_tc_kernel<kTf32, false, N><<<(unsigned)blocks, 224, smem, stream>>>(tab);
+            else conv_wgrad_tc_kernel<kSplit, false, N><<<(unsigned)blocks, 480, smem, stream>>>(tab);
             DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
             return DP_OK;
-        });
+        };
+        rc = store[dtype].jobs.size() <= (size_t)kFewLayers ? store[dtype].launch<kFewLayers>(go) : store[dtype].launch<kTcLayers>(go);
         if (rc != DP_OK) return rc;
     }
     // The Gram matrices first: two more launches wait for them.  Larger clusters need all their SMs in one GPC, free at the same
