@@ -340,7 +340,7 @@ void affine_batch_shape(int dtype, int B, int HW, int C, bool beside, AffineSeg 
     s.chunks = (HW + s.pix - 1) / s.pix;
 }
 
-dp_status launch_affine_batch(int dtype, AffineGroup &grp, int *tickets, cudaStream_t st) {
+dp_status launch_affine_batch(int dtype, AffineGroup &grp, int *tickets, cudaEvent_t begun, cudaStream_t st) {
     const int vec = dtype == DP_F32 ? 4 : 8;
     int b1 = 0, b2 = 0, b3 = 0;
     size_t smem = 0;
@@ -358,8 +358,15 @@ dp_status launch_affine_batch(int dtype, AffineGroup &grp, int *tickets, cudaStr
         const void *kernel = dtype == DP_F32 ? (const void *)affine_batch_stream_kernel<float> : (const void *)affine_batch_stream_kernel<__nv_bfloat16>;
         DP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
         const unsigned grid = (unsigned)(b1 < sm_count() ? b1 : sm_count());
-        if (dtype == DP_F32) affine_batch_stream_kernel<float><<<grid, kStreamThreads, kStreamSmem, st>>>(grp, b1, tickets);
-        else affine_batch_stream_kernel<__nv_bfloat16><<<grid, kStreamThreads, kStreamSmem, st>>>(grp, b1, tickets);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(grid); cfg.blockDim = dim3(kStreamThreads); cfg.dynamicSmemBytes = kStreamSmem; cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeLaunchCompletionEvent;
+        at[0].val.launchCompletionEvent.event = begun; at[0].val.launchCompletionEvent.flags = 0;
+        cfg.attrs = at; cfg.numAttrs = begun ? 1 : 0;
+        const cudaError_t le = dtype == DP_F32 ? cudaLaunchKernelEx(&cfg, affine_batch_stream_kernel<float>, grp, b1, tickets)
+                                               : cudaLaunchKernelEx(&cfg, affine_batch_stream_kernel<__nv_bfloat16>, grp, b1, tickets);
+        if (le != cudaSuccess) return cuda_fail(le, "affine_batch_stream_kernel");
         DP_LAUNCH_CHECK("affine_batch_stream_kernel");
     } else {
         if (dtype == DP_F32) affine_batch_partial_kernel<float, 4><<<(unsigned)b1, 256, smem, st>>>(grp);

@@ -18,7 +18,7 @@ namespace {
 struct SideStreams {
     int device;
     cudaStream_t stream[BatchStreams::kCount];
-    cudaEvent_t fork, gram_done, done[BatchStreams::kCount];
+    cudaEvent_t fork, begun, gate, gram_done, done[BatchStreams::kCount];
 };
 constexpr size_t kKeptSets = 8;
 std::mutex kept_mu;
@@ -30,6 +30,8 @@ void drop_streams(SideStreams *t) {
         if (t->stream[i]) cudaStreamDestroy(t->stream[i]);
     }
     if (t->fork) cudaEventDestroy(t->fork);
+    if (t->begun) cudaEventDestroy(t->begun);
+    if (t->gate) cudaEventDestroy(t->gate);
     if (t->gram_done) cudaEventDestroy(t->gram_done);
     delete t;
 }
@@ -57,6 +59,8 @@ SideStreams *take_streams() {
     priority[BatchStreams::kClusters] = priority[BatchStreams::kClusters6] = high / 2;
     priority[BatchStreams::kSums] = priority[BatchStreams::kAffine] = high;
     bool ok = cudaEventCreateWithFlags(&t->fork, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&t->begun, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&t->gate, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&t->gram_done, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 1; ok && i < BatchStreams::kCount; ++i)
         ok = cudaStreamCreateWithPriority(&t->stream[i], cudaStreamNonBlocking, priority[i]) == cudaSuccess &&
@@ -234,7 +238,7 @@ static void plan_affine(dp_batch &b, size_t &off) {
 
 // The groups that run beside convolutions (which come after, on other streams) or the others; without streams for that, all.
 enum { kBeside, kApart, kAllGroups };
-static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l, char *ws, int which, cudaStream_t st) {
+static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l, char *ws, int which, cudaEvent_t begun, cudaStream_t st) {
     if (b.affine.empty()) return DP_OK;
     std::vector<AffineGroup> groups = b.affine;
     for (size_t i = 0; i < b.items.size(); ++i) {
@@ -257,9 +261,31 @@ static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l,
         groups[k].partial = reinterpret_cast<float *>(ws + b.affine_partial);
         if (which != kAllGroups && (b.affine_beside[k] != 0) != (which == kBeside)) continue;
         int *tickets = which == kBeside && k < kWsStreams ? reinterpret_cast<int *>(ws + kWsStreamOffset) + 2 * k : nullptr;
-        const dp_status rc = launch_affine_batch(b.affine_dtype[k], groups[k], tickets, st);
+        const dp_status rc = launch_affine_batch(b.affine_dtype[k], groups[k], tickets, tickets ? begun : nullptr, st);
+        if (tickets) begun = nullptr;                        // (the first one's)
         if (rc != DP_OK) return rc;
     }
+    return DP_OK;
+}
+
+// Everything else waits until the normalisation layers' blocks are there, one on every SM, while all are still empty.  Started
+// together with other launches they land where room is left: two on one SM, which has none for a convolution's block until they
+// end, or on an SM that a small kernel has left with little shared memory, which is not divided anew while they run.  Chunks of
+// ResNet-50 (32 examples, 32 of them replayed one behind the other) took 771 or 885 us, a run of the program either the one or the
+// other, and 835 without layers beside; 769 this way (on a slower GPU 807 or 921, 851, and 794).  The wait for `begun` ends in a
+// kernel: in a captured graph it is an edge that only kernels may have, and what the streams do next is not always one (without
+// that kernel 795).
+__global__ void batch_gate_kernel() {}
+static dp_status open_gate(const dp_batch &b, const BatchStreams &streams, void *const *lane_streams) {
+    const cudaStream_t st = streams.s[BatchStreams::kMain];
+    DP_CUDA_TRY(cudaStreamWaitEvent(st, b.side->begun, 0));
+    batch_gate_kernel<<<1, 1, 0, st>>>();
+    DP_LAUNCH_CHECK("batch_gate_kernel");
+    DP_CUDA_TRY(cudaEventRecord(b.side->gate, st));
+    for (int i = 1; i < BatchStreams::kCount; ++i)
+        if (b.used[i] && i != BatchStreams::kAffine) DP_CUDA_TRY(cudaStreamWaitEvent(streams.s[i], b.side->gate, 0));
+    for (int k = 1; lane_streams && k < b.lanes; ++k)
+        DP_CUDA_TRY(cudaStreamWaitEvent(static_cast<cudaStream_t>(lane_streams[k - 1]), b.side->gate, 0));
     return DP_OK;
 }
 
@@ -463,7 +489,7 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
         try {
             // (singles first: they are short, and behind the normalisation layers they would be the chunk's tail)
             rc = singles(false);
-            if (rc == DP_OK) rc = run_affine(*b, io, C_l, ws, forked ? kApart : kAllGroups, streams.s[BatchStreams::kAffine]);
+            if (rc == DP_OK) rc = run_affine(*b, io, C_l, ws, forked ? kApart : kAllGroups, nullptr, streams.s[BatchStreams::kAffine]);
         } catch (const std::exception &) {       // out of memory: the streams still have to meet
             rc = DP_ERR_CUDA;
         }
@@ -482,7 +508,9 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
     dp_status rc;
     try {
         // (on every SM before the convolutions' blocks are)
-        rc = forked ? run_affine(*b, io, C_l, ws, kBeside, streams.s[BatchStreams::kAffine]) : DP_OK;
+        const bool beside = forked && std::find(b->affine_beside.begin(), b->affine_beside.end(), 1) != b->affine_beside.end();
+        rc = beside ? run_affine(*b, io, C_l, ws, kBeside, b->side->begun, streams.s[BatchStreams::kAffine]) : DP_OK;
+        if (beside && rc == DP_OK) rc = open_gate(*b, streams, laned ? lane_streams : nullptr);
         if (rc == DP_OK) rc = singles(true);
         if (rc == DP_OK) rc = run_convs(*b, io, C_l, ws, streams, join);
     } catch (const std::exception &) {           // out of memory

@@ -29,6 +29,7 @@ bool affine_batch_eligible(int dtype, int C);
 // beside: shaped for the form that runs beside tensor-core launches (any form takes it)
 void affine_batch_shape(int dtype, int B, int HW, int C, bool beside, AffineSeg &s);
 // tickets: two cleared words for the form that runs beside tensor-core launches, which are in later launches; null: the GPU is free
-dp_status launch_affine_batch(int dtype, AffineGroup &grp, int *tickets, cudaStream_t st);
+// begun (with tickets): recorded when every block of that form runs
+dp_status launch_affine_batch(int dtype, AffineGroup &grp, int *tickets, cudaEvent_t begun, cudaStream_t st);
 
 }  // namespace dp

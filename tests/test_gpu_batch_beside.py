@@ -1,0 +1,61 @@
+"""Normalisation layers that run beside a batch's convolutions: when their blocks start, and their sums under every epilogue."""
+import pytest
+import torch
+
+from paper_2109_12191_b200 import synth
+from gpu_util import B, dev_inputs, make_desc, scaled_inputs
+
+pytestmark = pytest.mark.gpu
+
+STORE, NORM, CLIP = 0, 1, 2
+LARGE = synth.norm(64, 720)                                  # brings a batch of three examples to the form for many bytes
+
+
+def _zeros(layer, Bn, dtype="bf16"):
+    return tuple(torch.zeros(layer.x_shape(Bn), device="cuda", dtype=torch.bfloat16 if dtype == "bf16" else torch.float32) for _ in range(2))
+
+
+@pytest.mark.parametrize("lanes", [1, 2])
+@pytest.mark.parametrize("convs", [
+    [synth.conv(256, 320, 3, 1, 1, 7)],                      # Gram matrices and one product: nothing on the caller's stream itself
+    [synth.conv(3, 64, 7, 2, 3, 21), synth.conv(64, 256, 3, 1, 1, 6), synth.conv(128, 256, 3, 2, 1, 9)],   # a regrouped input, clusters of several sizes
+], ids=["gram", "mixed"])
+def test_blocks_beside_convolutions_start_before_everything_else(convs, lanes):
+    """Captured, the batch has one node that depends on nothing, the launch of those blocks: what started with them took their
+    places on some SMs.  A copy right behind the batch can be captured too, and a replay gives the bits of the plain run."""
+    runtime = pytest.importorskip("cuda.bindings.runtime")
+    b, Bn = B(), 3
+    layers = convs + [synth.norm(64, 20), synth.dense(65, 10, True), synth.dense(33, 7, False), LARGE]
+    data = [_zeros(l, Bn) if l is LARGE else dev_inputs(scaled_inputs(l, Bn, "bf16", 976, i), "bf16") for i, l in enumerate(layers)]
+    batch = b.Batch([make_desc(l, Bn, "bf16") for l in layers], [CLIP] * len(layers), lanes=lanes)
+    assert batch.lanes == lanes
+    sizes = [n for l in layers for n in (l.n_weight, l.n_bias)]
+    ends = torch.tensor([0] + [(n + 3) // 4 * 4 for n in sizes]).cumsum(0).tolist()       # every tensor on a 16-byte boundary
+    acc, sq = torch.zeros(ends[-1], device="cuda"), torch.zeros((len(layers), Bn), device="cuda")
+    parts = [acc[o:o + n] for o, n in zip(ends, sizes)]
+    for i in range(len(layers)):
+        batch.set(i, sqnorm=sq[i], sqnorm_stride=1, acc_w=parts[2 * i], acc_b=parts[2 * i + 1] if parts[2 * i + 1].numel() else None)
+    ws = torch.empty(batch.workspace_bytes, dtype=torch.uint8, device="cuda")
+    b.check(b.dp_workspace_init(ws))
+    if lanes > 1:
+        own = torch.empty(batch.lane_bytes, dtype=torch.uint8, device="cuda")
+        b.check(b.dp_workspace_init(own))
+        batch.use_lanes([torch.cuda.Stream()], [own])
+    copy = torch.empty_like(acc)
+
+    b.check(batch.run(data, 1.0, ws))
+    plain, plain_sq = acc.clone(), sq.clone()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        b.check(batch.run(data, 1.0, ws))
+        copy.copy_(acc)
+    err, _, roots = runtime.cudaGraphGetRootNodes(graph.raw_cuda_graph())
+    assert int(err) == 0 and roots == 1
+    acc.zero_()
+    sq.zero_()
+    graph.instantiate()
+    graph.replay()
+    torch.cuda.synchronize()
+    b.check(b.dp_wgrad_check(ws))
+    assert torch.equal(copy, plain) and torch.equal(sq, plain_sq)
