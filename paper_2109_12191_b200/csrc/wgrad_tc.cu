@@ -700,11 +700,13 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
 // Roles (384 threads): warp 0 issues the TMA loads of the A slabs, warp 2 those of the B slabs, warp 1 allocates tensor
 // memory and issues the MMAs, warp 3 idles; warps 4-11 are the epilogue: warp w reads TMEM lanes 32*(w%4).. and the
 // 128-column half (w-4)/4 of the tile, so a thread holds 128 running sums.  The first warpgroup gives registers up
-// (setmaxnreg) and the epilogue warpgroups take them: 128*56 + 256*224 = 384*168, the launch's allocation; in a batch
-// 128*40 + 256*208 = 384*152, which leaves a warp of 56 registers a thread to each quarter of the SM (see affine_batch.cu).
+// (setmaxnreg) and the epilogue warpgroups take them: 128*56 + 256*224 = 384*168, the launch's allocation; beside normalisation
+// layers 128*24 + 256*216 = 384*152, which leaves a warp of 56 registers a thread to each quarter of the SM (see affine_batch.cu)
+// and keeps all but one value in registers (128*40 + 256*208 spilled ten of the running sums' neighbours: 794 us a chunk of 32
+// ResNet-50 examples, 786 this way).
 constexpr int kClipThreads = 384;
-template <int N> struct ClipRegs {                   // of a call on its own, and of a batch's launches, which leave some to others
-    static constexpr int kLaunch = N == 1 ? 168 : 152, kControl = N == 1 ? 56 : 40, kEpilogue = N == 1 ? 224 : 208;
+template <bool BESIDE> struct ClipRegs {
+    static constexpr int kLaunch = BESIDE ? 152 : 168, kControl = BESIDE ? 24 : 56, kEpilogue = BESIDE ? 216 : 224;
     static_assert(128 * kControl + 256 * kEpilogue == kClipThreads * kLaunch, "register split must add up");
 };
 constexpr int kMaxCluster = 8;
@@ -937,8 +939,8 @@ __device__ __forceinline__ float sum8(const float4 &x, const float4 &y) {
     return s <= kFloatMax ? s + ((e0 + e1) + (e2 + e3)) : s;
 }
 
-template <int N>
-__global__ void __maxnreg__(ClipRegs<N>::kLaunch)
+template <int N, bool BESIDE = false>
+__global__ void __maxnreg__(ClipRegs<BESIDE>::kLaunch)
 conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     const int entry = table_entry(tab.first, tab.n, blockIdx.x);
     const CUtensorMap &tmX = tab.e[entry].map[0], &tmY = tab.e[entry].map[1];
@@ -989,7 +991,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
     const int b_slabs = min(b_slabs_tile, p.b_ext / p.slab_ch - nt * b_slabs_tile);
 
     if (warp < 4) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ClipRegs<N>::kControl));
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ClipRegs<BESIDE>::kControl));
         if (warp == 0 || warp == 2) {
             // ------------------------------------------------------------ TMA producers (A slabs / B slabs)
             const bool leader = elect_one();
@@ -1056,7 +1058,7 @@ conv_wgrad_clip1_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
             }
         }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ClipRegs<N>::kEpilogue));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ClipRegs<BESIDE>::kEpilogue));
         // ---------------------------------------------------------------- epilogue (8 warps)
         const int e = warp - 4, q = e & 3, half = e >> 2;
         const int row = q * 32 + lane;
@@ -2103,8 +2105,9 @@ static bool clip1_registers_ok() {
     static int ok = -1;
     if (ok < 0) {
         cudaFuncAttributes attr;
-        ok = (cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<1>) == cudaSuccess && attr.numRegs == ClipRegs<1>::kLaunch &&
-              cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<kTcLayers>) == cudaSuccess && attr.numRegs == ClipRegs<kTcLayers>::kLaunch) ? 1 : 0;
+        ok = (cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<1>) == cudaSuccess && attr.numRegs == ClipRegs<false>::kLaunch &&
+              cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<kTcLayers>) == cudaSuccess && attr.numRegs == ClipRegs<false>::kLaunch &&
+              cudaFuncGetAttributes(&attr, conv_wgrad_clip1_kernel<kTcLayers, true>) == cudaSuccess && attr.numRegs == ClipRegs<true>::kLaunch) ? 1 : 0;
         if (!ok) (void)cudaGetLastError();
     }
     return ok == 1;
@@ -2315,7 +2318,7 @@ static dp_status raise_shared_limits() {
             allow_shared(conv_wgrad_tc_kernel<kBf16, false, kFewLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kFewLayers>),
             allow_shared(conv_wgrad_tc_kernel<kTf32, false, kFewLayers>),
             allow_shared(conv_wgrad_split_kernel), allow_shared(conv_wgrad_tc_kernel<kBf16, false, 1, true>), allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
-            allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>),
+            allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers, true>),
             allow_shared(conv_gram_norm_kernel<1>), allow_shared(conv_gram_norm_kernel<kTcLayers>)};
         for (cudaError_t e : all)
             if (e != cudaSuccess && err == cudaSuccess) err = e;
@@ -2688,7 +2691,7 @@ static dp_status fill_clip1(int dtype, const void *X, const void *dY, const Conv
     return DP_OK;
 }
 
-template <int N>
+template <int N, bool BESIDE = false>
 static dp_status launch_clip1_table(const TcTable<TcParams, 2, N> &tab, int cluster, int blocks, size_t smem, cudaStream_t stream) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(kClipThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
@@ -2696,7 +2699,7 @@ static dp_status launch_clip1_table(const TcTable<TcParams, 2, N> &tab, int clus
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_clip1_kernel<N>, tab);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_clip1_kernel<N, BESIDE>, tab);
     if (le != cudaSuccess) return cuda_fail(le, "conv_wgrad_clip1_kernel");
     DP_LAUNCH_CHECK("conv_wgrad_clip1_kernel");
     return DP_OK;
@@ -2894,7 +2897,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
     // time: behind smaller blocks they would be what the chunk ends with, so they come next, each size on a stream of its own.
     auto clip_launch = [&](int c) -> dp_status {
         return clip[c].launch([&](const TcTable<TcParams, 2, kTcLayers> &tab, int blocks, size_t smem) {
-            return launch_clip1_table<kTcLayers>(tab, c, blocks, smem, cluster_stream(c));
+            return (beside ? launch_clip1_table<kTcLayers, true> : launch_clip1_table<kTcLayers>)(tab, c, blocks, smem, cluster_stream(c));
         });
     };
     if (rc == DP_OK)

@@ -59,3 +59,38 @@ def test_blocks_beside_convolutions_start_before_everything_else(convs, lanes):
     torch.cuda.synchronize()
     b.check(b.dp_wgrad_check(ws))
     assert torch.equal(copy, plain) and torch.equal(sq, plain_sq)
+
+
+def test_convolutions_with_nothing_beside_keep_their_registers():
+    """Their kernels need not leave any of an SM's registers to others, and put nothing in local memory."""
+    driver = pytest.importorskip("cuda.bindings.driver")
+    b, Bn = B(), 3
+    layers = [synth.conv(64, 64, 1, 1, 0, 9), synth.conv(64, 256, 3, 1, 1, 6), synth.conv(128, 384, 1, 1, 0, 7), synth.conv(128, 256, 3, 2, 1, 9)]
+    data = [dev_inputs(scaled_inputs(l, Bn, "bf16", 977, i), "bf16") for i, l in enumerate(layers)]
+    batch = b.Batch([make_desc(l, Bn, "bf16") for l in layers], [CLIP] * len(layers))
+    acc, sq = [torch.zeros(l.n_weight, device="cuda") for l in layers], torch.zeros((len(layers), Bn), device="cuda")
+    for i, a in enumerate(acc):
+        batch.set(i, sqnorm=sq[i], sqnorm_stride=1, acc_w=a)
+    ws = torch.empty(batch.workspace_bytes, dtype=torch.uint8, device="cuda")
+    b.check(b.dp_workspace_init(ws))
+    b.check(batch.run(data, 1.0, ws))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        b.check(batch.run(data, 1.0, ws))
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    err, _, count = driver.cuGraphGetNodes(raw)
+    err, nodes, count = driver.cuGraphGetNodes(raw, count)
+    assert int(err) == 0 and count >= 3
+    for node in nodes:
+        err, kind = driver.cuGraphNodeGetType(node)
+        if kind != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        err, params = driver.cuGraphKernelNodeGetParams(node)
+        assert int(err) == 0
+        func = params.func
+        if not int(func):
+            err, func = driver.cuKernelGetFunction(params.kern)
+            assert int(err) == 0
+        err, local = driver.cuFuncGetAttribute(driver.CUfunction_attribute.CU_FUNC_ATTRIBUTE_LOCAL_SIZE_BYTES, func)
+        assert int(err) == 0 and local == 0
