@@ -17,6 +17,7 @@ namespace {
 // worst queue behind what the old one still has running.  At most kKeptSets wait for a taker.
 struct SideStreams {
     int device;
+    bool beside;                 // normalisation layers run beside the convolutions
     cudaStream_t stream[BatchStreams::kCount];
     cudaEvent_t fork, begun, gate, gram_done, done[BatchStreams::kCount];
 };
@@ -36,14 +37,14 @@ void drop_streams(SideStreams *t) {
     delete t;
 }
 // a set on the current device, or null
-SideStreams *take_streams() {
+SideStreams *take_streams(bool beside) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     {
         std::lock_guard<std::mutex> lock(kept_mu);
         auto &sets = kept_sets();
         for (size_t i = sets.size(); i-- > 0;) {
-            if (sets[i]->device != dev) continue;
+            if (sets[i]->device != dev || sets[i]->beside != beside) continue;
             SideStreams *t = sets[i];
             sets.erase(sets.begin() + (std::ptrdiff_t)i);
             return t;
@@ -52,9 +53,12 @@ SideStreams *take_streams() {
     SideStreams *t = new (std::nothrow) SideStreams{};
     if (!t) return nullptr;
     t->device = dev;
-    // What others wait for, and short launches, take SMs before large clusters do, and those before the caller's stream.
+    t->beside = beside;
+    // Beside normalisation layers, what others wait for, and short launches, take SMs before large clusters do, and those before
+    // the caller's stream.  Elsewhere the normalisation layers are to fill gaps and not to come first (a chunk of 4 ResNet-50
+    // examples: 167 us with these priorities and single calls on a stream of their own, 155 with neither).
     int low = 0, high = 0;
-    (void)cudaDeviceGetStreamPriorityRange(&low, &high);
+    if (beside) (void)cudaDeviceGetStreamPriorityRange(&low, &high);
     int priority[BatchStreams::kCount] = {};
     priority[BatchStreams::kClusters] = priority[BatchStreams::kClusters6] = high / 2;
     priority[BatchStreams::kSums] = priority[BatchStreams::kAffine] = high;
@@ -99,7 +103,8 @@ struct dp_batch {
     std::vector<AffineGroup> affine;             // shapes filled in, buffers per run
     std::vector<int> affine_dtype;
     std::vector<char> affine_beside;             // runs beside convolutions
-    bool beside = false;                         // some do
+    bool beside = false;                         // planned for some that do
+    int singles_stream = BatchStreams::kSingles; // single calls of lane 0
     size_t affine_partial = 0;                   // byte offset of the pixel-chunk partials
     std::vector<ConvJob> convs;                  // geometry filled in, buffers per run
     std::vector<int> conv_item;                  // item of every conv
@@ -123,7 +128,7 @@ namespace dp {
 static bool side_streams(const dp_batch &b) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    if (!b.side) b.side = take_streams();
+    if (!b.side) b.side = take_streams(b.beside);
     return b.side && b.side->device == dev;
 }
 
@@ -360,18 +365,20 @@ static dp_status plan_batch(dp_batch &b, int n, const dp_layer_desc *descs, cons
         plan_convs(b, off);
         plan_affine(b, off);
     }
+    // (ahead of normalisation layers that run apart from the convolutions, which then do not all start at once)
+    b.singles_stream = b.beside ? BatchStreams::kSingles : BatchStreams::kAffine;
     plan_lanes(b, lanes);
     b.singles = off;
     size_t most = 0;
     for (const auto &it : b.items) {
         if (it.group >= 0) continue;
         most = std::max(most, it.plan.total);
-        b.used[BatchStreams::kSingles] = true;
+        b.used[b.singles_stream] = true;
     }
     if (!b.affine.empty()) b.used[BatchStreams::kAffine] = true;
     for (const ConvJob &j : b.convs) {
         b.used[BatchStreams::kMain] = true;
-        b.used[conv_cluster_stream(conv_batch_cluster(j, b.walk, b.beside))] = true;
+        b.used[conv_cluster_stream(conv_batch_cluster(j, b.walk, b.beside), b.beside)] = true;
         if (j.kind == kConvGramSum || j.kind == kConvGramTiles || b.items[b.conv_item[&j - b.convs.data()]].desc.has_bias) b.used[BatchStreams::kSums] = true;
     }
     b.total = most > kWsHeaderBytes ? round_up(off + most - kWsHeaderBytes, 256) : off;
@@ -476,7 +483,7 @@ extern "C" dp_status dp_batch_run_lanes(const dp_batch *b, const dp_layer_io *io
                 char *own = static_cast<char *>(lane_workspaces[it.lane - 1]);
                 rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, own, own + kWsHeaderBytes, static_cast<cudaStream_t>(lane_streams[it.lane - 1]));
             } else {
-                rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[BatchStreams::kSingles]);
+                rc = run_layer(&it.desc, it.epi, buf, C_l, it.plan, ws, ws + b->singles, streams.s[b->singles_stream]);
             }
         }
         return rc;

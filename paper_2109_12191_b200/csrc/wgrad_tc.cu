@@ -2010,8 +2010,8 @@ static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
             const long long total_tiles = (long long)g.B * m_tiles * n_tiles;
             if (total_tiles > 0x7fffffffLL) continue;
             if (mode == 3 && !any_tiles && m_tiles * n_tiles > kMaxCluster) continue;
-            // (sizes that share no launch with others would be one more to wait for)
-            const double apart = mode == 3 && !any_tiles && tl_batch_walk > 0.0 && (m_tiles * n_tiles == 5 || m_tiles * n_tiles == 7) ? 1.1 : 1.0;
+            // (beside normalisation layers, sizes that share no launch with others would be one more to wait for)
+            const double apart = mode == 3 && !any_tiles && tl_beside && (m_tiles * n_tiles == 5 || m_tiles * n_tiles == 7) ? 1.1 : 1.0;
             const int y_slabs = (mode == 4) ? (a_is_x ? NT / slab_ch : a_slabs_tile) : 0;     // second (lo) copy of the dY slabs
             // per-CTA share of (example, tile) units: whole waves of tiles, or in clipped-sum mode an even share of the examples
             // (in a batch other layers fill the last wave)
@@ -2786,7 +2786,9 @@ typedef TableQueue<GramParams, 2, kTcLayers> GramQueue;
 // Cluster size of the launch a layer with `tiles` tiles an example joins: sizes that divide one another share one.
 static int launch_cluster(int tiles) { return tiles == 1 || tiles == 2 || tiles == 4 ? 4 : (tiles == 3 || tiles == 6 ? 6 : tiles); }
 
-int conv_cluster_stream(int cluster) { return cluster > 6 ? BatchStreams::kClusters : (cluster > 4 ? BatchStreams::kClusters6 : BatchStreams::kMain); }
+int conv_cluster_stream(int cluster, bool beside) {
+    return cluster <= 4 ? BatchStreams::kMain : (beside && cluster <= 6 ? BatchStreams::kClusters6 : BatchStreams::kClusters);
+}
 
 int conv_batch_cluster(const ConvJob &j, double walk, bool beside) {
     BatchPlanning planning(walk, beside);
@@ -2798,7 +2800,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
                             const std::function<dp_status()> &join) {
     if (jobs.empty()) return join();
     const cudaStream_t stream = streams.s[BatchStreams::kMain], sums = streams.s[BatchStreams::kSums];
-    auto cluster_stream = [&](int cluster) { return streams.s[conv_cluster_stream(cluster)]; };
+    auto cluster_stream = [&](int cluster) { return streams.s[conv_cluster_stream(cluster, beside)]; };
     BatchPlanning planning(walk, beside);
     dp_status rc = raise_shared_limits();
     if (rc != DP_OK) return rc;
@@ -2846,7 +2848,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
             p.cluster = cluster;
             q.blocks = (p.splits + sets - 1) / sets * cluster;
             q.smem = pl.smem; q.cost = p.per_split * pl.item_cycles;
-            if (p.splits > 1) folds[conv_cluster_stream(cluster)].push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
+            if (p.splits > 1) folds[conv_cluster_stream(cluster, beside)].push_back(fold_seg(p.sum_out, p.splits, P, j.acc_w));
             clip[cluster].jobs.push_back(q);
         } else {
             const GramPlan gp = gram_plan(j.dtype, j.g);

@@ -84,7 +84,7 @@ int conv_batch_kind(int dtype, const ConvGeom &g, int epilogue, bool has_bias);
 double conv_batch_walk(const std::vector<ConvJob> &jobs, bool beside);
 int conv_batch_cluster(const ConvJob &job, double walk, bool beside);         // blocks per cluster of the launch it runs in, or 0
 // the stream of a launch of clusters of this size
-int conv_cluster_stream(int cluster);
+int conv_cluster_stream(int cluster, bool beside);
 // Streams a batch spreads its independent launches over: s[0] is the caller's, the others are forked from it and joined
 // to it again (ForkedStreams).  All may be one and the same.
 struct BatchStreams {

@@ -94,3 +94,33 @@ def test_convolutions_with_nothing_beside_keep_their_registers():
             assert int(err) == 0
         err, local = driver.cuFuncGetAttribute(driver.CUfunction_attribute.CU_FUNC_ATTRIBUTE_LOCAL_SIZE_BYTES, func)
         assert int(err) == 0 and local == 0
+
+
+def test_normalisation_layers_of_small_batches_fill_gaps():
+    """With few bytes of them nothing runs beside the convolutions, and no launch of the batch comes before the others."""
+    driver = pytest.importorskip("cuda.bindings.driver")
+    b, Bn = B(), 3
+    layers = [synth.conv(64, 64, 1, 1, 0, 9), synth.conv(256, 320, 3, 1, 1, 7), synth.conv(128, 256, 3, 2, 1, 9), synth.norm(64, 20)]
+    data = [dev_inputs(scaled_inputs(l, Bn, "bf16", 978, i), "bf16") for i, l in enumerate(layers)]
+    batch = b.Batch([make_desc(l, Bn, "bf16") for l in layers], [CLIP] * len(layers))
+    acc, sq = [torch.zeros((2, max(l.n_weight, 4)), device="cuda") for l in layers], torch.zeros((len(layers), Bn), device="cuda")
+    for i, l in enumerate(layers):
+        batch.set(i, sqnorm=sq[i], sqnorm_stride=1, acc_w=acc[i][0], acc_b=acc[i][1] if l.n_bias else None)
+    ws = torch.empty(batch.workspace_bytes, dtype=torch.uint8, device="cuda")
+    b.check(b.dp_workspace_init(ws))
+    b.check(batch.run(data, 1.0, ws))
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        b.check(batch.run(data, 1.0, ws))
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    err, _, count = driver.cuGraphGetNodes(raw)
+    err, nodes, count = driver.cuGraphGetNodes(raw, count)
+    priorities = set()
+    for node in nodes:
+        err, kind = driver.cuGraphNodeGetType(node)
+        if kind == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            err, value = driver.cuGraphKernelNodeGetAttribute(node, driver.CUlaunchAttributeID.CU_LAUNCH_ATTRIBUTE_PRIORITY)
+            assert int(err) == 0
+            priorities.add(value.priority)
+    assert len(priorities) == 1
