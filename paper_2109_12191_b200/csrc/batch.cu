@@ -165,8 +165,8 @@ static void plan_lanes(dp_batch &b, int lanes) {
     b.target = sm_target_set() ? sm_target() : 0;
     std::stable_sort(singles.begin(), singles.end(), [&](int x, int y) { return single_cost(b.items[x]) > single_cost(b.items[y]); });
     std::vector<double> load(b.lanes, 0.0);
-    for (const AffineGroup &g : b.affine)                    // these follow lane 0
-        for (int k = 0; k < g.n; ++k) load[0] += (double)g.seg[k].B * g.seg[k].HW * g.seg[k].C * 4.0 / 5e6;
+    for (const AffineGroup &g : b.affine)                    // these follow lane 0, or have a stream of their own
+        for (int k = 0; b.singles_stream == BatchStreams::kAffine && k < g.n; ++k) load[0] += (double)g.seg[k].B * g.seg[k].HW * g.seg[k].C * 4.0 / 5e6;
     for (int i : singles) {
         dp_batch::Item &it = b.items[i];
         make_layer_plan(&it.desc, it.epi, it.plan);          // (for the target)

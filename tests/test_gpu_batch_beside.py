@@ -12,7 +12,8 @@ LARGE = synth.norm(64, 720)                                  # brings a batch of
 
 
 def _zeros(layer, Bn, dtype="bf16"):
-    return tuple(torch.zeros(layer.x_shape(Bn), device="cuda", dtype=torch.bfloat16 if dtype == "bf16" else torch.float32) for _ in range(2))
+    return tuple(torch.zeros(shape, device="cuda", dtype=torch.bfloat16 if dtype == "bf16" else torch.float32)
+                 for shape in (layer.x_shape(Bn), layer.dy_shape(Bn)))
 
 
 @pytest.mark.parametrize("lanes", [1, 2])
@@ -124,3 +125,51 @@ def test_normalisation_layers_of_small_batches_fill_gaps():
             assert int(err) == 0
             priorities.add(value.priority)
     assert len(priorities) == 1
+
+
+@pytest.mark.parametrize("H", [64, 720], ids=["apart", "beside"])
+def test_lanes_count_normalisation_layers_only_where_those_follow_lane_0(H):
+    """Two single calls over two lanes.  Behind large normalisation layers lane 0 would be late, so both take the other lane, one
+    after the other; where those layers have a stream of their own the calls run side by side."""
+    driver = pytest.importorskip("cuda.bindings.driver")
+    b, Bn = B(), 3
+    layers = [synth.conv(256, 256, 3, 1, 1, 14), synth.conv(5, 60, 3, 1, 0, 24), synth.conv(5, 7, 3, 1, 0, 9)] + [synth.norm(64, H)] * (1 if H > 64 else 40)
+    data = [_zeros(l, Bn) for l in layers]
+    descs = [make_desc(l, Bn, "bf16") for l in layers]
+    assert not any(b.dp_wgrad_uses_tensor_cores(d, NORM) for d in descs[1:3])
+    batch = b.Batch(descs, [NORM] * len(descs), lanes=2)
+    assert batch.lanes == 2
+    sq = torch.full((len(layers), Bn), 7.0, device="cuda")
+    for i in range(len(layers)):
+        batch.set(i, sqnorm=sq[i], sqnorm_stride=1)
+    ws = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in (batch.workspace_bytes, batch.lane_bytes)]
+    for w in ws:
+        b.check(b.dp_workspace_init(w))
+    batch.use_lanes([torch.cuda.Stream()], [ws[1]])
+    b.check(batch.run(data, 1.0, ws[0]))
+    torch.cuda.synchronize()
+    assert not bool(sq.any())
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        b.check(batch.run(data, 1.0, ws[0]))
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    err, _, _, _, count = driver.cuGraphGetEdges_v2(raw)
+    err, start, end, _, count = driver.cuGraphGetEdges_v2(raw, count)
+    assert int(err) == 0
+    before = {}
+    for a, z in zip(start, end):
+        before.setdefault(int(z), []).append(a)
+
+    def name(node):
+        err, kind = driver.cuGraphNodeGetType(node)
+        if kind != driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            return b""
+        err, params = driver.cuGraphKernelNodeGetParams(node)
+        return driver.cuKernelGetName(params.kern)[1] if int(params.kern) else driver.cuFuncGetName(params.func)[1]
+
+    def follows_one(node):
+        return any(b"conv_wgrad_fma" in name(a) or follows_one(a) for a in before.get(int(node), []))
+
+    own = {int(n): n for n in list(start) + list(end) if b"conv_wgrad_fma" in name(n)}
+    assert len(own) == 2
+    assert sum(follows_one(n) for n in own.values()) == (0 if H > 64 else 1)
