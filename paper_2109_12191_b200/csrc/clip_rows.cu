@@ -11,7 +11,7 @@
 #include "mbar.cuh"
 #include <math.h>
 #include <algorithm>
-#include <mutex>
+#include <atomic>
 
 namespace dp {
 
@@ -284,37 +284,43 @@ size_t clip_rows_workspace_bytes(int B, long long P) {
     return p.clusters > 1 ? sizeof(float) * (size_t)p.clusters * (size_t)P : 0;
 }
 
-// Clusters of this size that the GPU holds at once (one block an SM, all of a cluster in one GPC); 0: none, and the caller takes another way.
+// The limit on dynamic shared memory belongs to a function in one context: it is raised for every launch (60 ns), in whichever
+// context and on whichever device is current.
+static bool rows_shared(RowsKernel kernel) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem) == cudaSuccess) return true;
+    (void)cudaGetLastError();
+    return false;
+}
+
+// Clusters of this size that the current device holds at once (one block an SM, all of a cluster in one GPC); 0: none, and the
+// caller takes another way.
 static int rows_resident(int cluster) {
-    static std::mutex mu;
-    static int cached[kRowsMaxCluster + 1] = {0};        // one more than that
-    std::lock_guard<std::mutex> lock(mu);
-    if (!cached[cluster]) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(cluster * 64)); cfg.blockDim = dim3(kRowsThreads); cfg.dynamicSmemBytes = kRowsSmem;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.attrs = at; cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, rows_kernel(kRowsKernels - 1), &cfg) != cudaSuccess || n < 0) { (void)cudaGetLastError(); n = 0; }
-        cached[cluster] = n + 1;
+    static std::atomic<int> cached[64][kRowsMaxCluster + 1];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) { (void)cudaGetLastError(); return 0; }
+    if (dev < 64) {
+        const int n = cached[dev][cluster].load(std::memory_order_relaxed);
+        if (n > 0) return n;
     }
-    return cached[cluster] - 1;
+    const RowsKernel kernel = rows_kernel(kRowsKernels - 1);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cluster * 64)); cfg.blockDim = dim3(kRowsThreads); cfg.dynamicSmemBytes = kRowsSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (!rows_shared(kernel) || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 0) { (void)cudaGetLastError(); return 0; }
+    if (dev < 64) cached[dev][cluster].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 dp_status launch_clip_rows(const float *G, int B, long long P, float C, float *acc, float *norms_out, float *clip_out,
                            void *workspace, cudaStream_t stream) {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        for (int i = 0; i < kRowsKernels && err == cudaSuccess; ++i)
-            err = cudaFuncSetAttribute(rows_kernel(i), cudaFuncAttributeMaxDynamicSharedMemorySize, kRowsSmem);
-    });
-    if (err != cudaSuccess) return cuda_fail(err, "cudaFuncSetAttribute");
     RowsPlan p = rows_plan(B, P);
+    const RowsKernel kernel = rows_kernel(rows_kernel_for(p.slice));
     const int resident = rows_resident(p.cluster);
-    if (resident < 1) return DP_ERR_UNSUPPORTED;
+    if (resident < 1 || !rows_shared(kernel)) return DP_ERR_UNSUPPORTED;
     p.clusters = std::min(p.clusters, resident);
     RowsArgs a = {};
     a.G = G; a.P = P; a.B = B; a.clusters = p.clusters; a.slice = p.slice;
@@ -331,7 +337,7 @@ dp_status launch_clip_rows(const float *G, int B, long long P, float C, float *a
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)p.cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, rows_kernel(rows_kernel_for(p.slice)), a);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, a);
     if (le != cudaSuccess) return cuda_fail(le, "clip_rows_kernel");
     DP_LAUNCH_CHECK("clip_rows_kernel");
     if (p.clusters > 1) {
