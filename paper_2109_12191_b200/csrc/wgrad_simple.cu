@@ -6,7 +6,6 @@
 #include "affine.cuh"
 #include <math.h>
 #include <algorithm>
-#include <mutex>
 
 namespace dp {
 
@@ -566,12 +565,8 @@ static dp_status launch_rgb3_t(const T *X, const T *dY, const ConvGeom &g, float
                                float *sqnorm, long long sq_stride, cudaStream_t st) {
     int cluster, rows_per;
     if (!rgb3_split(g, cluster, rows_per)) return DP_ERR_UNSUPPORTED;
-    static std::once_flag once;
-    static cudaError_t attr_err = cudaSuccess;
-    std::call_once(once, [] {
-        attr_err = cudaFuncSetAttribute(conv_wgrad_rgb3_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRgbSmemMost);
-    });
-    if (attr_err != cudaSuccess) return cuda_fail(attr_err, "cudaFuncSetAttribute");
+    // (the limit belongs to a function in one context: raised for every launch)
+    DP_CUDA_TRY(cudaFuncSetAttribute(conv_wgrad_rgb3_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRgbSmemMost));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(g.B * cluster)); cfg.blockDim = dim3(kRgbThreads);
     cfg.dynamicSmemBytes = rgb3_smem_bytes(g, rows_per); cfg.stream = st;

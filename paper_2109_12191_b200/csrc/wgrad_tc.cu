@@ -2116,24 +2116,24 @@ static bool clip1_registers_ok() {
 // How many clusters of this size the GPU can hold at once (a cluster needs all its SMs free in one GPC at the same
 // time, so this is less than SMs / size); more clusters than that would run as a second wave.  Unknown (no device): no cap.
 static int max_active_clusters(int cluster_size) {
-    static std::mutex mu;
-    static int cached[kMaxCluster + 1] = {0};
+    static std::atomic<int> cached[64][kMaxCluster + 1];
+    int dev = -1;
     if (cluster_size < 1 || cluster_size > kMaxCluster) return 1 << 30;
-    std::lock_guard<std::mutex> lock(mu);
-    if (cached[cluster_size] == 0) {
-        int n = 0;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(cluster_size * 64)); cfg.blockDim = dim3(kClipThreads); cfg.dynamicSmemBytes = kSmemBudget + 1024;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)cluster_size; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.attrs = at; cfg.numAttrs = 1;
-        const bool ok = cudaFuncSetAttribute(conv_wgrad_clip1_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048) == cudaSuccess &&
-                        cudaOccupancyMaxActiveClusters(&n, conv_wgrad_clip1_kernel<1>, &cfg) == cudaSuccess && n > 0;
-        if (!ok) (void)cudaGetLastError();
-        cached[cluster_size] = ok ? n : -1;
-    }
-    return cached[cluster_size] > 0 ? cached[cluster_size] : 1 << 30;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { (void)cudaGetLastError(); return 1 << 30; }
+    const int known = cached[dev][cluster_size].load(std::memory_order_relaxed);
+    if (known) return known;
+    int n = 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cluster_size * 64)); cfg.blockDim = dim3(kClipThreads); cfg.dynamicSmemBytes = kSmemBudget + 1024;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster_size; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    const bool ok = cudaFuncSetAttribute(conv_wgrad_clip1_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, conv_wgrad_clip1_kernel<1>, &cfg) == cudaSuccess && n > 0;
+    if (!ok) { (void)cudaGetLastError(); return 1 << 30; }
+    cached[dev][cluster_size].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 // Thin strided layers (a 7 x 7 stride-2 stem on RGB) in space-to-depth form, see space_to_depth_kernel: the geometry the
@@ -2300,30 +2300,32 @@ typedef TcEntry<TcParams, 3> SsumEntry;
 typedef TcEntry<GramParams, 2> GramEntry;
 static_assert(sizeof(TcTable<TcParams, 3, kSsumLayers>) <= 32000 && sizeof(TcTable<TcParams, 2, kTcLayers>) <= 32000, "kernel parameters are limited to 32764 bytes");
 
+// The limit on dynamic shared memory belongs to a function in one context: it is raised for every launch (60 ns), in whichever
+// context and on whichever device is current.
 template <typename K>
 static cudaError_t allow_shared(K kernel) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048);
 }
-// Raised once per process, for every form of the kernels at once.
-static dp_status raise_shared_limits() {
-    static std::once_flag once;
-    static cudaError_t err = cudaSuccess;
-    std::call_once(once, [] {
-        const cudaError_t all[] = {
-            allow_shared(conv_wgrad_tc_kernel<kBf16, false, 1>), allow_shared(conv_wgrad_tc_kernel<kBf16, true, 1>),
-            allow_shared(conv_wgrad_tc_kernel<kSplit, false, 1>), allow_shared(conv_wgrad_tc_kernel<kSplit, true, 1>),
-            allow_shared(conv_wgrad_tc_kernel<kBf16, false, kTcLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kTcLayers>),
-            allow_shared(conv_wgrad_tc_kernel<kTf32, false, 1>), allow_shared(conv_wgrad_tc_kernel<kTf32, true, 1>),
-            allow_shared(conv_wgrad_tc_kernel<kTf32, false, kTcLayers>),
-            allow_shared(conv_wgrad_tc_kernel<kBf16, false, kFewLayers>), allow_shared(conv_wgrad_tc_kernel<kSplit, false, kFewLayers>),
-            allow_shared(conv_wgrad_tc_kernel<kTf32, false, kFewLayers>),
-            allow_shared(conv_wgrad_split_kernel), allow_shared(conv_wgrad_tc_kernel<kBf16, false, 1, true>), allow_shared(conv_wgrad_ssum_kernel<1>), allow_shared(conv_wgrad_ssum_kernel<kSsumLayers>),
-            allow_shared(conv_wgrad_clip1_kernel<1>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers>), allow_shared(conv_wgrad_clip1_kernel<kTcLayers, true>),
-            allow_shared(conv_gram_norm_kernel<1>), allow_shared(conv_gram_norm_kernel<kTcLayers>)};
-        for (cudaError_t e : all)
-            if (e != cudaSuccess && err == cudaSuccess) err = e;
-    });
-    return err == cudaSuccess ? DP_OK : cuda_fail(err, "cudaFuncSetAttribute");
+template <typename TABLE>
+static dp_status launch_table(void (*kernel)(const TABLE), const char *name, const TABLE &tab, int blocks, int threads, size_t smem, cudaStream_t stream) {
+    DP_CUDA_TRY(allow_shared(kernel));
+    kernel<<<(unsigned)blocks, (unsigned)threads, smem, stream>>>(tab);
+    DP_LAUNCH_CHECK(name);
+    return DP_OK;
+}
+template <typename TABLE>
+static dp_status launch_table_clusters(void (*kernel)(const TABLE), const char *name, const TABLE &tab, int cluster, int blocks, int threads, size_t smem, cudaStream_t stream) {
+    DP_CUDA_TRY(allow_shared(kernel));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, tab);
+    if (le != cudaSuccess) return cuda_fail(le, name);
+    DP_LAUNCH_CHECK(name);
+    return DP_OK;
 }
 
 // Slabs one copy brings: neighbours along the channels of one filter tap, a divisor of the tile's and of the tensor's slabs.
@@ -2440,8 +2442,7 @@ dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY,
     const StoreForm form = clip ? StoreForm{make_plan(dtype, pr.eff, 2), pr.eff, false} : store_form(dtype, g0, pr, epilogue, !(publish && publish->factor_out));
     const TcPlan &pl = form.pl;
     if (!pl.ok) return DP_ERR_UNSUPPORTED;
-    dp_status rc = raise_shared_limits();
-    if (rc != DP_OK) return rc;
+    dp_status rc = DP_OK;
     if (pr.unfold) {
         // in a fused clip call this function runs twice (norm pass, then clipped-sum pass): the unfolded input is
         // rebuilt only by the first of them
@@ -2456,31 +2457,22 @@ dp_status launch_conv_tc(int dtype, int epilogue, const void *X, const void *dY,
     if (!clip && pl.split > 1) {
         p.splits = pl.split;
         p.blocks = p.total_tiles * pl.split;
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)p.blocks); cfg.blockDim = dim3(224); cfg.dynamicSmemBytes = pl.smem; cfg.stream = stream;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)pl.split; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        cfg.attrs = at; cfg.numAttrs = 1;
-        const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_split_kernel, tab);
-        if (le != cudaSuccess) return cuda_fail(le, "conv_wgrad_split_kernel");
-        DP_LAUNCH_CHECK("conv_wgrad_split_kernel");
-        return DP_OK;
+        return launch_table_clusters(conv_wgrad_split_kernel, "conv_wgrad_split_kernel", tab, pl.split, p.blocks, 224, pl.smem, stream);
     }
     p.blocks = std::min(p.total_tiles, sm_target());
-    const unsigned grid = (unsigned)p.blocks;
+    auto go = [&](void (*kernel)(const TcTable<TcParams, 2, 1>), int threads) {
+        return launch_table(kernel, "conv_wgrad_tc_kernel", tab, p.blocks, threads, pl.smem, stream);
+    };
     if (dtype == DP_BF16) {
-        if (clip) conv_wgrad_tc_kernel<kBf16, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
-        else if (norm_readers(dtype, epilogue, pl)) conv_wgrad_tc_kernel<kBf16, false, 1, true><<<grid, 352, pl.smem, stream>>>(tab);
-        else conv_wgrad_tc_kernel<kBf16, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        if (clip) rc = go(conv_wgrad_tc_kernel<kBf16, true, 1>, 224);
+        else if (norm_readers(dtype, epilogue, pl)) rc = go(conv_wgrad_tc_kernel<kBf16, false, 1, true>, 352);
+        else rc = go(conv_wgrad_tc_kernel<kBf16, false, 1>, 224);
     } else if (dtype == DP_TF32) {
-        if (clip) conv_wgrad_tc_kernel<kTf32, true, 1><<<grid, 224, pl.smem, stream>>>(tab);
-        else conv_wgrad_tc_kernel<kTf32, false, 1><<<grid, 224, pl.smem, stream>>>(tab);
+        rc = clip ? go(conv_wgrad_tc_kernel<kTf32, true, 1>, 224) : go(conv_wgrad_tc_kernel<kTf32, false, 1>, 224);
     } else {
-        if (clip) conv_wgrad_tc_kernel<kSplit, true, 1><<<grid, 480, pl.smem, stream>>>(tab);
-        else conv_wgrad_tc_kernel<kSplit, false, 1><<<grid, 480, pl.smem, stream>>>(tab);
+        rc = clip ? go(conv_wgrad_tc_kernel<kSplit, true, 1>, 480) : go(conv_wgrad_tc_kernel<kSplit, false, 1>, 480);
     }
-    DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
+    if (rc != DP_OK) return rc;
     if (clip && p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g0.M * g0.N, acc_w, stream);
     return DP_OK;
 }
@@ -2521,12 +2513,10 @@ static SplitSeg split_seg(const void *dY, const float *factor, const ConvGeom &g
 dp_status launch_conv_ssum(int dtype, const void *X, const void *dY, const ConvGeom &g0, const float *factor, float *acc_w,
                            void *tc_workspace, int *status, cudaStream_t stream) {
     if (!tc_clip_scaled_sum(dtype, g0)) return DP_ERR_UNSUPPORTED;
-    dp_status rc = raise_shared_limits();
-    if (rc != DP_OK) return rc;
     const TcProblem pr = tc_problem(dtype, g0);
     const ConvGeom &g = pr.eff;
     const TcPlan pl = make_plan(dtype, g, 4);
-    rc = launch_scale_split({split_seg(dY, factor, g, tc_workspace)}, stream);
+    dp_status rc = launch_scale_split({split_seg(dY, factor, g, tc_workspace)}, stream);
     if (rc != DP_OK) return rc;
     TcTable<TcParams, 3, 1> tab;
     tab.n = 1; tab.first[0] = 0;
@@ -2534,8 +2524,8 @@ dp_status launch_conv_ssum(int dtype, const void *X, const void *dY, const ConvG
     if (rc != DP_OK) return rc;
     TcParams &p = tab.e[0].p;
     p.blocks = std::min(p.total_tiles, sm_target());
-    conv_wgrad_ssum_kernel<1><<<(unsigned)p.blocks, 224, pl.smem, stream>>>(tab);
-    DP_LAUNCH_CHECK("conv_wgrad_ssum_kernel");
+    rc = launch_table(conv_wgrad_ssum_kernel<1>, "conv_wgrad_ssum_kernel", tab, p.blocks, 224, pl.smem, stream);
+    if (rc != DP_OK) return rc;
     if (p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g.M * g.N, acc_w, stream);
     return DP_OK;
 }
@@ -2572,18 +2562,16 @@ static dp_status fill_scaled_tiles(int dtype, const void *X, const void *dY, con
 dp_status launch_conv_scaled_tiles(int dtype, const void *X, const void *dY, const ConvGeom &g0, const float *factor, float *acc_w,
                                    void *tc_workspace, int *status, cudaStream_t stream) {
     if (!tc_clip_scaled_tiles(dtype, g0)) return DP_ERR_UNSUPPORTED;
-    dp_status rc = raise_shared_limits();
-    if (rc != DP_OK) return rc;
     const TcProblem pr = tc_problem(dtype, g0);
     const ConvGeom &g = pr.eff;
     const TcPlan pl = make_plan(dtype, g, 7);
     TcTable<TcParams, 2, 1> tab;
     tab.n = 1; tab.first[0] = 0;
-    rc = fill_scaled_tiles(dtype, X, dY, g, pl, factor, acc_w, tc_workspace, status, tab.e[0]);
+    dp_status rc = fill_scaled_tiles(dtype, X, dY, g, pl, factor, acc_w, tc_workspace, status, tab.e[0]);
     if (rc != DP_OK) return rc;
     const TcParams &p = tab.e[0].p;
-    conv_wgrad_clip1_kernel<1><<<(unsigned)p.total_tiles, kClipThreads, pl.smem, stream>>>(tab);
-    DP_LAUNCH_CHECK("conv_wgrad_clip1_kernel");
+    rc = launch_table(conv_wgrad_clip1_kernel<1>, "conv_wgrad_clip1_kernel", tab, p.total_tiles, kClipThreads, pl.smem, stream);
+    if (rc != DP_OK) return rc;
     if (p.splits > 1) return launch_fold_partial_sums(p.sum_out, p.splits, (long long)g.M * g.N, acc_w, stream);
     return DP_OK;
 }
@@ -2650,15 +2638,11 @@ dp_status launch_conv_gram_norm(int dtype, const void *X, const void *dY, const 
                                 float *factor_out, int *status, cudaStream_t stream) {
     const GramPlan gp = gram_plan(dtype, g0);
     if (!gp.ok) return DP_ERR_UNSUPPORTED;
-    dp_status rc = raise_shared_limits();
-    if (rc != DP_OK) return rc;
     TcTable<GramParams, 2, 1> tab;
     tab.n = 1; tab.first[0] = 0;
-    rc = fill_gram(dtype, X, dY, gp, clipinfo, factor_out, status, tab.e[0]);
+    const dp_status rc = fill_gram(dtype, X, dY, gp, clipinfo, factor_out, status, tab.e[0]);
     if (rc != DP_OK) return rc;
-    conv_gram_norm_kernel<1><<<(unsigned)tab.e[0].p.blocks, 192, gp.smem, stream>>>(tab);
-    DP_LAUNCH_CHECK("conv_gram_norm_kernel");
-    return DP_OK;
+    return launch_table(conv_gram_norm_kernel<1>, "conv_gram_norm_kernel", tab, tab.e[0].p.blocks, 192, gp.smem, stream);
 }
 
 bool tc_clip_single_pass(int dtype, const ConvGeom &g0) {
@@ -2693,16 +2677,7 @@ static dp_status fill_clip1(int dtype, const void *X, const void *dY, const Conv
 
 template <int N, bool BESIDE = false>
 static dp_status launch_clip1_table(const TcTable<TcParams, 2, N> &tab, int cluster, int blocks, size_t smem, cudaStream_t stream) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(kClipThreads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
-    const cudaError_t le = cudaLaunchKernelEx(&cfg, conv_wgrad_clip1_kernel<N, BESIDE>, tab);
-    if (le != cudaSuccess) return cuda_fail(le, "conv_wgrad_clip1_kernel");
-    DP_LAUNCH_CHECK("conv_wgrad_clip1_kernel");
-    return DP_OK;
+    return launch_table_clusters(conv_wgrad_clip1_kernel<N, BESIDE>, "conv_wgrad_clip1_kernel", tab, cluster, blocks, kClipThreads, smem, stream);
 }
 
 dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const ConvGeom &g0, const TcInlineClip &clipinfo,
@@ -2710,8 +2685,7 @@ dp_status launch_conv_clip1(int dtype, const void *X, const void *dY, const Conv
     const TcProblem pr = tc_problem(dtype, g0);
     TcPlan pl; ConvGeom g; bool s2d;
     if (!pr.ok || !encode_fn() || !clip1_plan(dtype, g0, pr, pl, g, s2d) || !clip1_registers_ok()) return DP_ERR_UNSUPPORTED;
-    dp_status rc = raise_shared_limits();
-    if (rc == DP_OK) rc = prepare_input(dtype, X, g0, pr, s2d, tc_workspace, stream);
+    dp_status rc = prepare_input(dtype, X, g0, pr, s2d, tc_workspace, stream);
     if (rc != DP_OK) return rc;
     TcTable<TcParams, 2, 1> tab;
     tab.n = 1; tab.first[0] = 0;
@@ -2802,8 +2776,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
     const cudaStream_t stream = streams.s[BatchStreams::kMain], sums = streams.s[BatchStreams::kSums];
     auto cluster_stream = [&](int cluster) { return streams.s[conv_cluster_stream(cluster, beside)]; };
     BatchPlanning planning(walk, beside);
-    dp_status rc = raise_shared_limits();
-    if (rc != DP_OK) return rc;
+    dp_status rc = DP_OK;
     ConvQueue store[3], clip[kMaxCluster + 1];            // store: by element type; clip: by cluster size of the launch
     GramQueue gram;
     SsumQueue ssum;
@@ -2886,11 +2859,8 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
     for (int dtype = 0; dtype < 3; ++dtype) {
         auto go = [&](const auto &tab, int blocks, size_t smem) -> dp_status {
             constexpr int N = std::extent<decltype(tab.first)>::value;
-            if (dtype == DP_BF16) conv_wgrad_tc_kernel<kBf16, false, N><<<(unsigned)blocks, 224, smem, stream>>>(tab);
-            else if (dtype == DP_TF32) conv_wgrad_tc_kernel<kTf32, false, N><<<(unsigned)blocks, 224, smem, stream>>>(tab);
-            else conv_wgrad_tc_kernel<kSplit, false, N><<<(unsigned)blocks, 480, smem, stream>>>(tab);
-            DP_LAUNCH_CHECK("conv_wgrad_tc_kernel");
-            return DP_OK;
+            const auto kernel = dtype == DP_BF16 ? conv_wgrad_tc_kernel<kBf16, false, N> : (dtype == DP_TF32 ? conv_wgrad_tc_kernel<kTf32, false, N> : conv_wgrad_tc_kernel<kSplit, false, N>);
+            return launch_table(kernel, "conv_wgrad_tc_kernel", tab, blocks, dtype == DP_F32 ? 480 : 224, smem, stream);
         };
         rc = store[dtype].jobs.size() <= (size_t)kFewLayers ? store[dtype].launch<kFewLayers>(go) : store[dtype].launch<kTcLayers>(go);
         if (rc != DP_OK) return rc;
@@ -2904,9 +2874,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
     };
     if (rc == DP_OK)
         rc = gram.launch([&](const TcTable<GramParams, 2, kTcLayers> &tab, int blocks, size_t smem) -> dp_status {
-            conv_gram_norm_kernel<kTcLayers><<<(unsigned)blocks, 192, smem, sums>>>(tab);
-            DP_LAUNCH_CHECK("conv_gram_norm_kernel");
-            return DP_OK;
+            return launch_table(conv_gram_norm_kernel<kTcLayers>, "conv_gram_norm_kernel", tab, blocks, 192, smem, sums);
         });
     for (int c = kMaxCluster; c > 4 && rc == DP_OK; --c) rc = clip_launch(c);
     if (rc == DP_OK && streams.gram_done) {
@@ -2917,9 +2885,7 @@ dp_status launch_conv_batch(const std::vector<ConvJob> &jobs, double walk, bool 
     if (rc == DP_OK) rc = launch_scale_split(splits, sums);
     if (rc == DP_OK)
         rc = ssum.launch([&](const TcTable<TcParams, 3, kSsumLayers> &tab, int blocks, size_t smem) -> dp_status {
-            conv_wgrad_ssum_kernel<kSsumLayers><<<(unsigned)blocks, 224, smem, sums>>>(tab);
-            DP_LAUNCH_CHECK("conv_wgrad_ssum_kernel");
-            return DP_OK;
+            return launch_table(conv_wgrad_ssum_kernel<kSsumLayers>, "conv_wgrad_ssum_kernel", tab, blocks, 224, smem, sums);
         });
     // (each stream folds its own: behind the join the fold would be alone on the GPU)
     for (int i = BatchStreams::kCount - 1; i >= 0 && rc == DP_OK; --i) rc = launch_folds(folds[i], streams.s[i]);

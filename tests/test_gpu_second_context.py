@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 PROGRAM = r"""
-import ctypes, sys
+import sys
 import numpy as np
 from cuda.bindings import driver as cu
 from paper_2109_12191_b200 import binding as b
@@ -49,13 +49,60 @@ def clip(static):
     ref = (np.minimum(1.0, 50.0 / np.linalg.norm(d, axis=1))[:, None] * d).sum(0)
     assert np.linalg.norm(to_host(acc, P) - ref) <= 2e-5 * np.linalg.norm(ref)
 
-CALLS = {"clip": lambda: clip(False), "clip_static": lambda: clip(True)}
+LAYERS = {                                                   # C_in, K_out, size, R, stride, pad
+    "stem": (3, 64, 40, 3, 1, 1), "one_tile": (64, 64, 9, 1, 1, 0), "clusters": (128, 256, 9, 3, 2, 1), "gram": (256, 320, 7, 3, 1, 1),
+    "shared_pixels": (64, 64, 50, 1, 1, 0),
+}
+kept = []
+
+class Memory:                                                # what a batch asks of its workspace
+    def __init__(self, nbytes):
+        self.nbytes, self.address = nbytes, to_gpu(np.zeros(nbytes, np.uint8))
+    def is_contiguous(self):
+        return True
+    def data_ptr(self):
+        return self.address
+
+def layer(name, dtype, seed):
+    Cin, K, H, R, stride, pad = LAYERS[name]
+    Bn, OH = 3, (H + 2 * pad - R) // stride + 1
+    rng = np.random.default_rng(seed)
+    X, dY = (rng.standard_normal(n, dtype=np.float32) for n in (Bn * H * H * Cin, Bn * OH * OH * K))
+    if dtype == b.DP_BF16:
+        X, dY = ((t.view(np.uint32) >> 16).astype(np.uint16) for t in (X, dY))
+    return b.make_desc(b.DP_LAYER_CONV2D, dtype, Bn, Cin, K, H, H, R, R, stride, pad), to_gpu(X), to_gpu(dY), Bn, K * R * R * Cin
+
+def conv(name, dtype, epi):
+    d, X, dY, Bn, P = layer(name, dtype, 2)
+    G, sq, acc = to_gpu(np.zeros((Bn, P), np.float32)), to_gpu(np.zeros(Bn, np.float32)), to_gpu(np.zeros(P, np.float32))
+    n = b.dp_workspace_bytes(d, epi)
+    ws = to_gpu(np.zeros(n, np.uint8))
+    b.check(b.dp_per_example_wgrad(d, X, dY, G, None, sq, 1, epi, 1.0, acc, None, None, ws, n, stream=0))
+    ok(cu.cuCtxSynchronize())
+    return np.concatenate([to_host(t, k).ravel() for t, k in ((G, Bn * P), (sq, Bn), (acc, P))])
+
+def batch():
+    parts = [layer(name, b.DP_BF16, 3) for name in LAYERS]
+    made = b.Batch([p[0] for p in parts], [b.DP_EPI_CLIP_ACCUM] * len(parts))
+    kept.append(made)                                        # its streams stay with their context
+    out = [(to_gpu(np.zeros(P, np.float32)), to_gpu(np.zeros(Bn, np.float32)), P, Bn) for _, _, _, Bn, P in parts]
+    for i, (acc, sq, _, _) in enumerate(out):
+        made.set(i, acc_w=acc, sqnorm=sq, sqnorm_stride=1)
+    b.check(made.run([(X, dY) for _, X, dY, _, _ in parts], 1.0, Memory(made.workspace_bytes), stream=0))
+    ok(cu.cuCtxSynchronize())
+    return np.concatenate([to_host(a, n) for acc, sq, P, Bn in out for a, n in ((acc, P), (sq, Bn))])
+
+def convs(dtype):
+    return np.concatenate([conv(name, dtype, epi) for name in LAYERS for epi in range(3)])
+
+CALLS = {"convs_bf16": lambda: convs(b.DP_BF16), "convs_f32": lambda: convs(b.DP_F32), "convs_tf32": lambda: convs(b.DP_TF32), "batch": batch,
+         "clip": lambda: clip(False), "clip_static": lambda: clip(True)}
 first = ok(cu.cuDevicePrimaryCtxRetain(device))
 ok(cu.cuCtxSetCurrent(first))
-CALLS[sys.argv[1]]()
+before = CALLS[sys.argv[1]]()
 second = ok(cu.cuCtxCreate(0, device))                       # current from here on
-buffers.clear()
-CALLS[sys.argv[1]]()
+after = CALLS[sys.argv[1]]()
+assert before is None or (np.array_equal(before, after) and np.all(np.isfinite(after)) and np.any(after))
 print("done")
 """
 
@@ -68,4 +115,9 @@ def run(call):
 
 @pytest.mark.parametrize("call", ["clip", "clip_static"])
 def test_flat_gradients(call):
+    run(call)
+
+
+@pytest.mark.parametrize("call", ["convs_bf16", "convs_f32", "convs_tf32", "batch"])
+def test_weight_gradients(call):
     run(call)
