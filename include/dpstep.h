@@ -222,7 +222,11 @@ DP_API size_t dp_clip_workspace_bytes(int B, int L, const long long *P_l /* host
  *   acc      host array of L device pointers, acc[l] = [P_l] fp32, read-modify-write.
  *   norms_out  optional device fp32: GLOBAL [B] whole-gradient L2 norms; PER_LAYER [B, L].
  *   clip_out   optional device fp32, same shape: the factors applied.
- *   workspace  at least dp_clip_workspace_bytes(B, L, P_l) bytes, 256-byte aligned. */
+ *   workspace  at least dp_clip_workspace_bytes(B, L, P_l) bytes, 256-byte aligned.
+ *
+ * A single tensor whose rows are read once goes through kernels that wait for copies and for one another, for about two
+ * seconds at most.  Should a wait give up (there is no status word here), all of acc[0] is NaN, and so are the norms and
+ * factors of the examples concerned. */
 DP_API dp_status dp_clip_accumulate(int mode, int B, int L, const float *const *G, const long long *P_l,
                              const float *sqnorm, float C, float *const *acc,
                              float *norms_out, float *clip_out,
@@ -379,8 +383,8 @@ DP_API dp_status dp_wgrad_check(void *workspace, void *cuda_stream);
  * lets layers whose per-example gradient fits one thread-block cluster run the single-pass form.  Process-wide. */
 DP_API void dp_debug_set_single_pass(int on);
 
-/* Test hook: the number of polls (each about a microsecond) after which the bounded waits of the tensor-core kernel
- * give up; 0 makes every wait give up before anything is copied or multiplied, a negative value restores the
+/* Test hook: the number of polls (each about a microsecond) after which the bounded waits of the tensor-core kernels and
+ * of dp_clip_accumulate give up; 0 makes every wait give up before anything is copied or multiplied, a negative value restores the
  * default (about two seconds).  Process-wide; applies to launches enqueued afterwards. */
 DP_API void dp_debug_set_wait_polls(long long polls);
 

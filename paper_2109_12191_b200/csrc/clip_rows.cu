@@ -45,10 +45,11 @@ struct RowsArgs {
     uint32_t polls;
 };
 
-// What the threads of a block wait for.  After one wait has given up the others do soon and the block runs through to its end
-// on whatever shared memory holds: every barrier is still met.
-__device__ __forceinline__ void rows_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t polls) {
-    if (!mbar_try_wait(bar, parity) && !*abort_flag) (void)mbar_wait(bar, parity, abort_flag, polls);
+// What the threads of a block wait for.  A thread whose wait gave up runs through to the end and waits for, arms, frees and sends
+// nothing more; others miss what it would have sent and give up as well.  What they all compute from then on is thrown away.
+// (Leaving the loops instead takes a vote a wait: 54.0 us for 256 rows of 175 178, 52.2 this way.)
+__device__ __forceinline__ bool rows_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, uint32_t polls) {
+    return mbar_try_wait(bar, parity) || (!*abort_flag && mbar_wait(bar, parity, abort_flag, polls));
 }
 __device__ __forceinline__ bool rows_try_peers(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -89,7 +90,7 @@ clip_rows_kernel(const RowsArgs a) {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
     // the last warp: row n on its way to a buffer
-    auto load = [&](int n, int buffer) {
+    auto load = [&](int n, int buffer, bool live) {
         const uintptr_t first = (uintptr_t)a.G, end = (uintptr_t)(a.G + (long long)a.B * a.P);
         const uintptr_t lo = (uintptr_t)(a.G + n * a.P + c0), hi = lo + 4 * (uintptr_t)len;
         uint8_t *buf = rows_sh + buffer * a.stride;
@@ -98,12 +99,12 @@ clip_rows_kernel(const RowsArgs a) {
         if (from < first || to > end) {                                          // words at the matrix's very ends
             if (from < first) from += 16;
             if (to > end) to -= 16;
-            if (lo + 4 * lane < min(from, hi)) *reinterpret_cast<float *>(buf + (lo + 4 * lane - at)) = *reinterpret_cast<const float *>(lo + 4 * lane);
+            if (live && lo + 4 * lane < min(from, hi)) *reinterpret_cast<float *>(buf + (lo + 4 * lane - at)) = *reinterpret_cast<const float *>(lo + 4 * lane);
             const uintptr_t tail = max(max(to, from), lo);
-            if (tail + 4 * lane < hi) *reinterpret_cast<float *>(buf + (tail + 4 * lane - at)) = *reinterpret_cast<const float *>(tail + 4 * lane);
+            if (live && tail + 4 * lane < hi) *reinterpret_cast<float *>(buf + (tail + 4 * lane - at)) = *reinterpret_cast<const float *>(tail + 4 * lane);
             __syncwarp();
         }
-        if (lane == 0) {
+        if (lane == 0 && live) {
             const uint32_t bytes = len > 0 && to > from ? (uint32_t)(to - from) : 0u, bar = smem_u32(&full[buffer]);
             mbar_expect_tx(bar, bytes);
             if (bytes)
@@ -115,21 +116,22 @@ clip_rows_kernel(const RowsArgs a) {
     int ahead = cluster, ahead_buffer = 0;           // the next row to load, and where to
     uint32_t ahead_phase = 0;
     if (warp == kRowsWarps - 1)
-        for (int s = 0; s < a.buffers && ahead < a.B; ++s, ahead += a.clusters) load(ahead, s);
+        for (int s = 0; s < a.buffers && ahead < a.B; ++s, ahead += a.clusters) load(ahead, s, true);
 
     float acc[V];
 #pragma unroll
     for (int i = 0; i < V; ++i) acc[i] = 0.f;
     int buffer = 0; uint32_t phase = 0;
     int turn = 0;
+    bool live = true;
     for (int n0 = cluster; n0 < a.B; n0 += R * a.clusters, ++turn) {
         const int rows = min(R, (a.B - n0 + a.clusters - 1) / a.clusters), half = turn & 1;
-        if (t == 0) mbar_expect_tx(smem_u32(&sums_in[half]), 4u * kRowsWarps * blocks * (uint32_t)rows);
+        if (t == 0 && live) mbar_expect_tx(smem_u32(&sums_in[half]), 4u * kRowsWarps * blocks * (uint32_t)rows);
         float v[R][V];
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (r < rows) {
-                rows_wait(smem_u32(&full[buffer]), phase, abort_p, a.polls);
+                live = live && rows_wait(smem_u32(&full[buffer]), phase, abort_p, a.polls);
                 const uint32_t shift = (uint32_t)(((uintptr_t)a.G >> 2) + (long long)(n0 + r * a.clusters) * a.P + c0) & (kRowsLine / 4 - 1);
                 const float *x = reinterpret_cast<const float *>(rows_sh + buffer * a.stride) + shift + t;
                 float sq[4] = {0.f, 0.f, 0.f, 0.f};
@@ -138,11 +140,11 @@ clip_rows_kernel(const RowsArgs a) {
 #pragma unroll
                 for (int i = 0; i < V; ++i) sq[i & 3] = fmaf(v[r][i], v[r][i], sq[i & 3]);
                 __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&empty[buffer]));
+                if (lane == 0 && live) mbar_arrive(smem_u32(&empty[buffer]));
                 if (++buffer == a.buffers) { buffer = 0; phase ^= 1u; }
                 // every warp's sum goes to all blocks of the cluster by itself: no block adds its own up first
                 const float sum = warp_sum((sq[0] + sq[1]) + (sq[2] + sq[3]));
-                if (lane < (int)blocks)
+                if (lane < (int)blocks && live)
                     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
                                  ::"r"(rows_peer(&sums[half][r][rank * kRowsWarps + warp], lane)), "r"(__float_as_uint(sum)),
                                  "r"(rows_peer(&sums_in[half], lane)) : "memory");
@@ -150,19 +152,19 @@ clip_rows_kernel(const RowsArgs a) {
         }
         if (warp == kRowsWarps - 1) {
             for (int r = 0; r < rows && ahead < a.B; ++r, ahead += a.clusters) {
-                rows_wait(smem_u32(&empty[ahead_buffer]), ahead_phase, abort_p, a.polls);
+                live = live && rows_wait(smem_u32(&empty[ahead_buffer]), ahead_phase, abort_p, a.polls);
                 __syncwarp();
-                if (!*abort_p) load(ahead, ahead_buffer);
+                load(ahead, ahead_buffer, live);
                 if (++ahead_buffer == a.buffers) { ahead_buffer = 0; ahead_phase ^= 1u; }
             }
         }
         // (a warp sends the sums of turn j + 2 after it has those of turn j + 1 from all, who send them after reading turn j's)
         bool arrived = false;
-        for (uint32_t it = 0; it < a.polls && !arrived; ++it) {
+        for (uint32_t it = 0; live && it < a.polls && !arrived; ++it) {
             arrived = rows_try_peers(smem_u32(&sums_in[half]), (uint32_t)(turn >> 1) & 1u);
             if ((it & 63u) == 63u && *abort_p) break;
         }
-        if (!arrived) *abort_p = 1;
+        if (!arrived) { *abort_p = 1; live = false; }
         __syncwarp();
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -184,17 +186,29 @@ clip_rows_kernel(const RowsArgs a) {
         }
     }
     __syncthreads();
-    if (abort_flag) __nanosleep(200000);             // copies still in flight land before shared memory is released
+    if (*abort_p) {
+        __nanosleep(200000);                         // copies still in flight land before shared memory is released
+        if (t < (int)blocks) asm volatile("st.shared::cluster.u32 [%0], 1;" ::"r"(rows_peer(&abort_flag, t)) : "memory");
+    }
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // nobody leaves while a peer may still send to it
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const bool failed = *abort_p != 0;               // here or in a peer
     float *out = a.out + (a.clusters > 1 ? cluster * a.P : 0ll) + c0 + t;
 #pragma unroll
     for (int i = 0; i < V; ++i) {
         if (i * kRowsThreads + t < len) {
-            const float v = abort_flag ? __int_as_float(0x7fffffff) : acc[i];
+            const float v = failed ? __int_as_float(0x7fffffff) : acc[i];
             if (a.clusters > 1) out[i * kRowsThreads] = v;
             else out[i * kRowsThreads] += v;
         }
+    }
+    if (failed) {
+        for (int n = cluster + t * a.clusters; rank == 0 && n < a.B; n += kRowsThreads * a.clusters) {
+            if (a.norms_out) a.norms_out[n] = __int_as_float(0x7fffffff);
+            if (a.clip_out) a.clip_out[n] = __int_as_float(0x7fffffff);
+        }
+        __nanosleep(200000);                         // sums that peers had on their way
     }
 }
 
