@@ -102,6 +102,7 @@ clip_rows_kernel(const RowsArgs a) {
             if (live && lo + 4 * lane < min(from, hi)) *reinterpret_cast<float *>(buf + (lo + 4 * lane - at)) = *reinterpret_cast<const float *>(lo + 4 * lane);
             const uintptr_t tail = max(max(to, from), lo);
             if (live && tail + 4 * lane < hi) *reinterpret_cast<float *>(buf + (tail + 4 * lane - at)) = *reinterpret_cast<const float *>(tail + 4 * lane);
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // before a bulk copy overwrites them one day
             __syncwarp();
         }
         if (lane == 0 && live) {
