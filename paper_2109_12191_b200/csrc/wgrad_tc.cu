@@ -867,7 +867,11 @@ conv_wgrad_split_kernel(const __grid_constant__ TcTable<TcParams, 2, 1> tab) {
     }
     tc_fence_before();
     __syncthreads();
+    // A block whose wait gave up has no tile to add: the whole cluster leaves its share of the gradient alone and NaN for a norm.
+    if (*abort_p && (int)threadIdx.x < split) asm volatile("st.shared::cluster.u32 [%0], 1;" ::"r"(map_to_cta(smem_u32(&abort_flag), threadIdx.x)) : "memory");
+    __syncwarp();
     cluster_sync_all();                                   // every block's tile is in place
+    const bool failed = *abort_p != 0;                    // here or in a peer
 
     // this block's share of the lines, of all blocks in their order; a thread takes four neighbouring values of a line
     const int line0 = lines * rank / split, line1 = lines * (rank + 1) / split, quads = width / 4;
@@ -876,7 +880,7 @@ conv_wgrad_split_kernel(const __grid_constant__ TcTable<TcParams, 2, 1> tab) {
     for (int r = 0; r < kMaxSplit; ++r) peer[r] = map_to_cta(tiles_u32, (uint32_t)min(r, split - 1));
     float sq4[4] = {0.f, 0.f, 0.f, 0.f};
     float *Gn = p.G_w + (long long)n * p.Kout * p.Ng;
-    for (int e = threadIdx.x; e < (line1 - line0) * quads; e += 224) {
+    for (int e = threadIdx.x; !failed && e < (line1 - line0) * quads; e += 224) {
         const int line = line0 + e / quads, x = (e % quads) * 4;
         const uint32_t off = (uint32_t)(line * pitch + x) * 4u;
         float4 v[kMaxSplit];
@@ -909,7 +913,7 @@ conv_wgrad_split_kernel(const __grid_constant__ TcTable<TcParams, 2, 1> tab) {
         }
     }
     const float sq = warp_sum((sq4[0] + sq4[1]) + (sq4[2] + sq4[3]));
-    if (lane == 0) warp_sq[warp] = sq;
+    if (lane == 0) warp_sq[warp] = failed ? __int_as_float(0x7fffffff) : sq;
     __syncthreads();
     cluster_sync_all();                                   // nobody leaves while a peer may still read its tile
     if (threadIdx.x == 0) {

@@ -113,3 +113,25 @@ def scaled_inputs(layer, Bn, dtype, *key, spread=True):
             inp["dY_bits"], dY = synth.round_to_bf16(dY)
         inp["dY"] = dY
     return inp
+
+
+def kernels_of(run):
+    """Names of the kernels that run() launches, which is captured and not executed."""
+    import pytest
+    driver = pytest.importorskip("cuda.bindings.driver")
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        run()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    _, _, count = driver.cuGraphGetNodes(raw)
+    err, nodes, count = driver.cuGraphGetNodes(raw, count)
+    assert int(err) == 0
+    names = []
+    for node in nodes:
+        _, kind = driver.cuGraphNodeGetType(node)
+        if kind == driver.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            _, params = driver.cuGraphKernelNodeGetParams(node)
+            err, name = driver.cuKernelGetName(params.kern) if int(params.kern) else driver.cuFuncGetName(params.func)
+            assert int(err) == 0
+            names.append(name.decode())
+    return names
