@@ -1,9 +1,11 @@
 """Normalisation layers that run beside a batch's convolutions: when their blocks start, and their sums under every epilogue."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2109_12191_b200 import synth
-from gpu_util import B, dev_inputs, make_desc, scaled_inputs
+from gpu_util import B, TOL_FMA, TOL_NORM, dev_inputs, kernels_of, make_desc, oracle_layer, rel_l2, scaled_inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -173,3 +175,51 @@ def test_lanes_count_normalisation_layers_only_where_those_follow_lane_0(H):
     own = {int(n): n for n in list(start) + list(end) if b"conv_wgrad_fma" in name(n)}
     assert len(own) == 2
     assert sum(follows_one(n) for n in own.values()) == (0 if H > 64 else 1)
+
+
+@pytest.mark.parametrize("epi,separate", [(STORE, 1), (CLIP, 0), (CLIP, 1)])
+@pytest.mark.parametrize("dtype,sizes,Bn", [
+    # one pixel, one vector of channels; several channel blocks, the last one ragged; fewer pixels than a ring's stages hold
+    ("bf16", [(8, 1), (24, 7), (1032, 5), (2048, 3), (512, 9), (64, 20), (2056, 2)], 3),
+    ("f32", [(4, 1), (36, 6), (516, 5), (256, 4), (1024, 3)], 3),
+])
+def test_gradients_and_clipped_sums_of_layers_beside_convolutions(dtype, sizes, Bn, epi, separate):
+    b = B()
+    large = LARGE if dtype == "bf16" else synth.norm(64, 512)
+    norms = [synth.norm(C, H) for C, H in sizes]
+    layers = [synth.conv(256, 256, 3, 1, 1, 14)] * 4 + norms + [large]
+    inputs = [scaled_inputs(l, Bn, dtype, 979, i) if l in norms else None for i, l in enumerate(layers)]
+    data = [_zeros(l, Bn, dtype) if inp is None else dev_inputs(inp, dtype) for l, inp in zip(layers, inputs)]
+    refs = [oracle_layer(l, inp) if inp is not None else None for l, inp in zip(layers, inputs)]
+    sqs = [None if r is None else np.stack([oracle.sqnorm(r[0]), oracle.sqnorm(r[1])], 1) for r in refs]
+    sqs = [s if s is None or separate else s.sum(1, keepdims=True) for s in sqs]
+    C_l = float(np.sqrt(np.median(np.concatenate([s.ravel() for s in sqs if s is not None]))))
+    batch = b.Batch([make_desc(l, Bn, dtype, 0, separate) for l in layers], [epi if l.kind == "norm" else NORM for l in layers])
+    out = []
+    for i, l in enumerate(layers):
+        g = 1 + separate if l.kind == "norm" else 1
+        o = dict(sqnorm=torch.full((Bn, g), float("nan"), device="cuda"))
+        if l.kind == "norm" and epi == STORE:
+            o.update(G_w=torch.full((Bn, l.n_weight), float("nan"), device="cuda"), G_b=torch.full((Bn, l.n_bias), float("nan"), device="cuda"))
+        if l.kind == "norm" and epi == CLIP:
+            o.update(acc_w=torch.ones(l.n_weight, device="cuda"), acc_b=torch.ones(l.n_bias, device="cuda"), clip_out=torch.full((Bn, g), float("nan"), device="cuda"))
+        batch.set(i, sqnorm_stride=g, **o)
+        out.append(o)
+    ws = torch.full((batch.workspace_bytes + 256,), 0xAB, dtype=torch.uint8, device="cuda")
+    b.check(b.dp_workspace_init(ws, batch.workspace_bytes))
+    for _ in range(2):                                       # items are handed out anew
+        b.check(batch.run(data, C_l, ws[:batch.workspace_bytes]))
+    b.check(b.dp_wgrad_check(ws))
+    assert any("affine_batch_stream_kernel" in name for name in kernels_of(lambda: b.check(batch.run(data, C_l, ws[:batch.workspace_bytes]))))
+    assert bool((ws[batch.workspace_bytes:] == 0xAB).all())
+    for l, ref, sq, o in zip(layers, refs, sqs, out):
+        if ref is None:
+            continue
+        np.testing.assert_allclose(o["sqnorm"].cpu().numpy(), sq, rtol=TOL_NORM, err_msg=str(l))
+        if epi == STORE:
+            assert rel_l2(o["G_w"].cpu().numpy(), ref[0]) <= TOL_FMA and rel_l2(o["G_b"].cpu().numpy(), ref[1]) <= TOL_FMA, str(l)
+        else:
+            f = oracle.clip_factor(sq, C_l).reshape(Bn, -1)
+            np.testing.assert_allclose(o["clip_out"].cpu().numpy(), f, rtol=TOL_NORM, err_msg=str(l))
+            assert rel_l2(o["acc_w"].cpu().numpy(), 1 + 2 * np.einsum("n,np->p", f[:, 0], ref[0])) <= TOL_FMA, str(l)
+            assert rel_l2(o["acc_b"].cpu().numpy(), 1 + 2 * np.einsum("n,np->p", f[:, -1], ref[1])) <= TOL_FMA, str(l)

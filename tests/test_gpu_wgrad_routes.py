@@ -75,3 +75,45 @@ def test_pixels_shared_by_a_cluster_with_waits_that_give_up(layer, Bn, epi):
     sq, _, *G = call.times_out()
     assert bool(torch.isnan(sq).all())
     assert all(bool((g == -7.0).all()) for g in G)
+
+
+GRAM_CONVS = [
+    # gradients too large for a cluster, output planes of at most 256 pixels: two row tiles, the second with 96 rows, with 16; one row
+    # tile, mostly zero rows; strided taps; strided 1 x 1; flattened pixels, 196 -> 208 rows; exactly 256 pixels
+    synth.conv(128, 256, 3, 1, 1, 14), synth.conv(128, 256, 3, 1, 1, 10), synth.conv(128, 256, 3, 1, 1, 5), synth.conv(128, 256, 3, 2, 1, 14),
+    synth.conv(512, 1024, 1, 2, 0, 14), synth.conv(1024, 512, 1, 1, 0, 14), synth.conv(256, 1152, 1, 1, 0, 16),
+]
+
+
+@pytest.fixture
+def side_by_side():
+    b = B()
+    b.check(b.dp_set_sm_target(torch.cuda.get_device_properties(0).multi_processor_count))
+    yield
+    b.check(b.dp_set_sm_target(0))
+
+
+@pytest.mark.parametrize("layer", GRAM_CONVS)
+def test_norms_from_gram_matrices_side_by_side(layer, side_by_side):
+    """Calls that run side by side with others take their norms from the Gram matrices of the pixels."""
+    call = Call(layer, 5, "bf16", CLIP, 983)
+    call()
+    call.is_right()
+    assert any("conv_gram_norm_kernel" in name for name in kernels_of(call))
+
+
+def test_gram_matrices_with_waits_that_give_up(side_by_side):
+    call = Call(GRAM_CONVS[0], 3, "bf16", CLIP, 984)
+    call()
+    torch.cuda.synchronize()
+    assert any("conv_gram_norm_kernel" in name for name in kernels_of(call))
+    call.times_out()
+
+
+@pytest.mark.parametrize("Bn,gram", [(10, False), (11, True)])
+def test_norms_of_very_many_tiles_over_few_pixels(Bn, gram):
+    """512 x 4608 entries an example over 25 pixels: by tiles up to 24 million of them, from Gram matrices past that."""
+    call = Call(synth.conv(512, 512, 3, 1, 1, 5), Bn, "bf16", CLIP, 985)
+    call()
+    call.is_right()
+    assert any("conv_gram_norm_kernel" in name for name in kernels_of(call)) == gram
