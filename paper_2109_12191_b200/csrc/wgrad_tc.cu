@@ -1984,7 +1984,13 @@ static double split_cycles(int mode, int items, int by, int NT, double main) {
     const double waves = std::ceil((double)items * by / (std::floor(places / by) * by));
     return (main + 1500.0 + 8.0 * NT + NT * (5.7 / by + 3.6) + (mode == 0 ? 128.0 * NT * 4.0 / by / 16.0 : 0.0) + 2500.0) * waves;
 }
-static size_t split_smem(int a_is_x, int NT) { return (a_is_x ? NT * (128 + kSplitPad) : 128 * (NT + kSplitPad)) * sizeof(float) + 1024; }
+// At least a third of an SM's shared memory: two blocks, of 256 columns of tensor memory each, on an SM at most.  A third would wait
+// for columns with its cluster waiting for it, and clusters that hold columns might wait for one another.  (Their registers keep a
+// third one out as well, 112 a thread as compiled now.)
+constexpr size_t kSplitSmemLeast = 77 * 1024;
+static size_t split_smem(int a_is_x, int NT) {
+    return std::max(kSplitSmemLeast, (a_is_x ? NT * (128 + kSplitPad) : 128 * (NT + kSplitPad)) * sizeof(float) + 1024);
+}
 
 static TcPlan search_plan(int dtype, const ConvGeom &g, int mode) {
     const int max_nt = (mode == 2) ? 128 : 256;
