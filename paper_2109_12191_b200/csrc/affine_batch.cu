@@ -61,7 +61,8 @@ affine_batch_partial_kernel(const __grid_constant__ AffineGroup grp) {
 // and reads its own vectors, so that nobody waits for anybody (a warp that filled the ring by bulk copies through barriers
 // took 1200 cycles a stage).  Items (an example's pixel chunk, some 130 KB) come from a counter, since SMs stream at the rate
 // their convolutions leave them.  What bounds it is the one warp a quarter: 460 us alone for the 53 layers of 32 examples of
-// ResNet-50 against 240 in the form above, but the chunk with its convolutions goes from 878 to 788 us.
+// ResNet-50 against 240 in the form above, but the chunk with its convolutions goes from 833 to 759 us.  (At 56 registers the bf16
+// form spills six words.)
 constexpr int kStreamThreads = 128, kStreamStages = 5;
 constexpr int kStreamVecs = 2;                               // vectors of X and of dY that a thread has in a stage, of neighbouring pixel rows
 constexpr int kStreamBytes = kStreamVecs * kStreamThreads * 16;

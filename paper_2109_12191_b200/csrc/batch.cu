@@ -178,9 +178,9 @@ static void plan_lanes(dp_batch &b, int lanes) {
 
 static bool affine_of(const dp_layer_desc &d) { return d.kind == DP_LAYER_NORM_AFFINE && affine_batch_eligible(storage_type(&d), d.C_in); }
 static double affine_bytes(const dp_layer_desc &d) { return 2.0 * d.B * d.H * d.W * d.C_in * (storage_type(&d) == DP_F32 ? 4 : 2); }
-// From here on layers run beside the convolutions: the layers of a ResNet of fewer examples are through in the gaps between the
-// launches, and shallower rings of the convolutions cost more than that (3 examples, 120 MB: 162 us, 166 beside; 8 examples,
-// 350 MB: 330 and 328; 22 examples: 534 and 487).
+// From here on layers run beside the convolutions: the layers of a ResNet-50 of fewer examples are through in the gaps between the
+// launches, and shallower rings of the convolutions cost more than that.  Chunks of 3, 4, 5, 6, 8 and 12 examples (133, 178, 222,
+// 267, 356 and 533 MB of these layers): 136, 154, 180, 214, 255 and 358 us, with the layers beside 144, 152, 177, 188, 242 and 330.
 constexpr double kBesideBytes = 250e6;
 
 // What the convolutions' launches leave the normalisation layers that run beside them, in bytes: some 2.8 TB/s of theirs for the
@@ -276,10 +276,10 @@ static dp_status run_affine(const dp_batch &b, const dp_layer_io *io, float C_l,
 // Everything else waits until the normalisation layers' blocks are there, one on every SM, while all are still empty.  Started
 // together with other launches they land where room is left: two on one SM, which has none for a convolution's block until they
 // end, or on an SM that a small kernel has left with little shared memory, which is not divided anew while they run.  Chunks of
-// ResNet-50 (32 examples, 32 of them replayed one behind the other) took 771 or 885 us, a run of the program either the one or the
-// other, and 835 without layers beside; 769 this way (on a slower GPU 807 or 921, 851, and 794).  The wait for `begun` ends in a
-// kernel: in a captured graph it is an edge that only kernels may have, and what the streams do next is not always one (without
-// that kernel 795).
+// ResNet-50 (32 examples, 32 of them replayed one behind the other) took 771 or 889 us, a run of the program either the one or the
+// other, and 833 without layers beside; 759 this way (on a slower GPU 807 or 921, 851, and 786).  The wait for `begun` ends in a
+// kernel: in a captured graph it is an edge that only kernels may have, and what the streams do next is not always one (with the
+// streams waiting themselves: the same time).
 __global__ void batch_gate_kernel() {}
 static dp_status open_gate(const dp_batch &b, const BatchStreams &streams, void *const *lane_streams) {
     const cudaStream_t st = streams.s[BatchStreams::kMain];

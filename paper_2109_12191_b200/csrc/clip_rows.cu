@@ -4,7 +4,7 @@
 // up to some hundred thousand floats fits the registers of a thread-block cluster: a bulk copy brings it to shared
 // memory, which is free for another row as soon as it is in registers; it is square-summed there, the cluster's blocks exchange their
 // sums through distributed shared memory, and it is scaled into running sums, also in registers, while the next rows arrive.
-// Bound by memory where rows are long; the exchange takes about a microsecond, so short rows go several at a time.
+// Bound by memory where rows are long; the exchange takes some two microseconds, so short rows go several at a time.
 // 256 rows of 175 178 floats, rows at any address: 60 us for the three launches that read twice, 45 here (38 for the rows,
 // 4.7 TB/s from the 120 SMs that clusters of eight find room on); 600 MB of them 189 and 116.
 #include "clip_rows.cuh"
@@ -283,10 +283,10 @@ static RowsPlan rows_plan(int B, long long P) {
 }
 
 // Rows up to what the registers of a cluster hold.  In the middle, rows of a few blocks and not many of them, every cluster has
-// one or two and the two passes, the second from the L2, are quicker (50 rows of 98 304: 17 us, 21 in a single read; 150 rows: 29
-// and 27; 457 rows: 65 and 45).  On either side of it the single read is, also where the L2 holds everything: short rows
-// are too narrow for the passes over columns (12 500 rows of 2001: 293 us, 99 here), long ones fill the GPU (38 rows of 131 071:
-// 22 us, 17 here).
+// one or two and the two passes, the second from the L2, are quicker (50 rows of 98 304: 14 us, 21 in a single read; 130 rows: 18
+// and 21; 150 rows, 59 MB: 19 and 22; 457 rows: 60 and 45).  On either side of it the single read is, also where the L2 holds
+// everything: short rows are too narrow for the passes over columns (12 500 rows of 2001: 293 us, 99 here), long ones fill the GPU
+// (38 rows of 131 071: 22 us, 17 here).
 constexpr long long kRowsShort = 12288, kRowsLong = 98304, kRowsFewBytes = 6000000, kRowsManyBytes = 60000000;
 bool clip_rows_eligible(int B, long long P) {
     const long long bytes = 4ll * B * P;

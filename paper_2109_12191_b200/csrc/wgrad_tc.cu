@@ -702,8 +702,8 @@ conv_wgrad_tc_kernel(const __grid_constant__ TcTable<TcParams, 2, N> tab) {
 // 128-column half (w-4)/4 of the tile, so a thread holds 128 running sums.  The first warpgroup gives registers up
 // (setmaxnreg) and the epilogue warpgroups take them: 128*56 + 256*224 = 384*168, the launch's allocation; beside normalisation
 // layers 128*24 + 256*216 = 384*152, which leaves a warp of 56 registers a thread to each quarter of the SM (see affine_batch.cu)
-// and keeps all but one value in registers (128*40 + 256*208 spilled ten of the running sums' neighbours: 794 us a chunk of 32
-// ResNet-50 examples, 786 this way).
+// and keeps all but one value in registers (128*40 + 256*208 spilled ten values: 794 us a chunk of 32 ResNet-50 examples on
+// the GPU that takes 786 this way).
 constexpr int kClipThreads = 384;
 template <bool BESIDE> struct ClipRegs {
     static constexpr int kLaunch = BESIDE ? 152 : 168, kControl = BESIDE ? 24 : 56, kEpilogue = BESIDE ? 216 : 224;
