@@ -383,7 +383,7 @@ class PerLayer:
         only = os.environ.get("DP_BENCH_ONLY")           # experiments: time one layer kind alone ("conv", "norm")
         if only:
             self.layers = [l for l in self.layers if l.kind == only]
-        # the layer calls of a chunk are one batch, planned for the whole GPU, whose launches fork over four streams; the
+        # the layer calls of a chunk are one batch, planned for the whole GPU, whose launches fork over six streams; the
         # only layer without a shared launch is the classifier, so that lanes and an SM target would change nothing
         self.lanes = int(os.environ.get("DP_BENCH_LANES", "1"))
         self.sm_target = int(os.environ.get("DP_BENCH_SM_TARGET", "0"))
@@ -424,7 +424,7 @@ class PerLayer:
         return {"workload": self.workload_text(self.layers, self.step_obj.L),
                 "examples_per_step": self.examples_per_step, "params": self.step_obj.P,
                 "l2": f"one chunk of inputs is {self.in_bytes / 1e9:.2f} GB, far larger than L2",
-                "streams": 3 + self.step_obj.batch.lanes, "sm_target": self.sm_target}
+                "streams": 5 + self.step_obj.batch.lanes, "sm_target": self.sm_target}
 
     def run(self, i, rec=None):
         """With a recorder the calls run one after the other on one stream so that each can be timed; otherwise a

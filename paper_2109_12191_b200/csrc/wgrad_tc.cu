@@ -1986,7 +1986,7 @@ static double split_cycles(int mode, int items, int by, int NT, double main) {
 }
 // At least a third of an SM's shared memory: two blocks, of 256 columns of tensor memory each, on an SM at most.  A third would wait
 // for columns with its cluster waiting for it, and clusters that hold columns might wait for one another.  (Their registers keep a
-// third one out as well, 112 a thread as compiled now.)
+// third one out as well, as compiled now.)
 constexpr size_t kSplitSmemLeast = 77 * 1024;
 static size_t split_smem(int a_is_x, int NT) {
     return std::max(kSplitSmemLeast, (a_is_x ? NT * (128 + kSplitPad) : 128 * (NT + kSplitPad)) * sizeof(float) + 1024);
